@@ -491,7 +491,7 @@ HDG_API int hdg_learned_loss_grad_dev(hdg_handle *h, const float *R, int n, floa
 #define HDG_IMEX_ARS3  3   /* ARS3(4,4,3): four implicit stages with a_ii = 1/2                        */
 /* Store the Coriolis field of the explicit term (host array [n_vertices], P1
  * per cell like hdg_params.f_vertex; NULL: no rotation) and allocate the
- * stage buffers (3 + 10 state vectors of n_cells * 3 n_p doubles).
+ * stage buffers (2 + 10 state vectors of n_cells * 3 n_p doubles).
  * HDG_EINVAL if the handle was set up with a non-zero f_vertex. */
 HDG_API int hdg_imex_init(hdg_handle *h, const double *f_vertex);
 /* The stage rates of a state (device pointers, caller layouts u [N][2][n_p],

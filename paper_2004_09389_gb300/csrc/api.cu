@@ -1208,7 +1208,7 @@ void free_handle(hdg_handle *h) {
     for (auto *p_ : h->gal.w) cudaFree(p_);
     if (h->prof.evict_buf) cudaFree(h->prof.evict_buf);
     if (h->prof.evict_sink) cudaFree(h->prof.evict_sink);
-    dfree(h->d_ref); dfree(h->d_X); dfree(h->d_fcell); dfree(h->d_facet_of); dfree(h->d_flip);
+    dfree(h->d_ref); dfree(h->d_nref); dfree(h->d_X); dfree(h->d_fcell); dfree(h->d_facet_of); dfree(h->d_flip);
     dfree(h->d_facet_cell); dfree(h->d_facet_edge); dfree(h->d_facet_verts); dfree(h->d_v2f_ptr); dfree(h->d_v2f);
     dfree(h->d_nbr); dfree(h->d_Xb); dfree(h->d_Rm); dfree(h->d_W); dfree(h->d_Scell); dfree(h->d_Sval);
     dfree(h->d_Xb2); dfree(h->d_Rm2); dfree(h->d_W2); dfree(h->d_Sval2);
@@ -1406,6 +1406,7 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     const HostMesh &hm = h->hm;
     RefElem re = build_ref_elem(h->p);
     TRY(upload(&h->d_ref, re.packed(), s));
+    TRY(upload(&h->d_nref, build_nodal_ref(h->p).packed(), s));
     TRY(upload(&h->d_X, hm.X, s));
     std::vector<double> fcell(size_t(h->N) * 3, 0.0);
     if (prm->f_vertex)

@@ -49,6 +49,55 @@ inline RefOffsets ref_offsets(int p) {
     return o;
 }
 
+// The same element in function space, every matrix multiplied by the inverse
+// reference mass matrix, so that it maps nodal values to nodal values and |det J|
+// drops out (Dx, Dy: derivatives of the basis at the nodes, M^-1 Dxi and M^-1
+// Deta without a solve).  About 0.45 of the entries of Dx and Dy vanish
+// (nodal_dx_nonzero, nodal_dy_nonzero).
+struct NodalRef {
+    std::vector<double> Dx, Dy;     // [n][n]     d_xi phi_b, d_eta phi_b at node a
+    std::vector<double> lift;       // [3][n][pp] M^-1 N_i
+    std::vector<double> ML1, ML2;   // [n][n]     M^-1 ML_1, M^-1 ML_2: multiplication by L_1, L_2 (L_0 = 1 - L_1 - L_2)
+    // packed copy for the device: Dx | Dy | lift | ML1 | ML2
+    std::vector<double> packed() const;
+};
+NodalRef build_nodal_ref(int p);
+struct NodalOffsets {
+    int Dx, Dy, lift, ML1, ML2, total;
+};
+__host__ __device__ constexpr NodalOffsets nodal_offsets(int p) {
+    const int n = (p + 1) * (p + 2) / 2, nn = n * n;
+    return NodalOffsets{0, nn, 2 * nn, 2 * nn + 3 * n * (p + 1), 3 * nn + 3 * n * (p + 1), 4 * nn + 3 * n * (p + 1)};
+}
+// lattice index b (row) of cell node k of degree p; a = k - row start, c = p - a - b
+__host__ __device__ constexpr int node_b(int p, int k) {
+    int b = 0;
+    while (k > p - b) {
+        k -= p - b + 1;
+        ++b;
+    }
+    return b;
+}
+__host__ __device__ constexpr int node_a(int p, int k) {
+    int b = 0;
+    while (k > p - b) {
+        k -= p - b + 1;
+        ++b;
+    }
+    return k;
+}
+// Whether d_xi phi_j (d_eta phi_j) at node i can be non-zero.  phi_j = F_c(L0) F_a(L1)
+// F_b(L2) with F_k(m / p) = binomial(m, k), zero for m < k: d_xi leaves F_b(L2) alone, so
+// it vanishes where b_i < b_j, and where both other factors do; d_eta likewise with a.
+__host__ __device__ constexpr bool nodal_dx_nonzero(int p, int i, int j) {
+    return node_b(p, i) >= node_b(p, j) &&
+           !(node_a(p, i) < node_a(p, j) && node_a(p, i) + node_b(p, i) > node_a(p, j) + node_b(p, j));
+}
+__host__ __device__ constexpr bool nodal_dy_nonzero(int p, int i, int j) {
+    return node_a(p, i) >= node_a(p, j) &&
+           !(node_b(p, i) < node_b(p, j) && node_a(p, i) + node_b(p, i) > node_a(p, j) + node_b(p, j));
+}
+
 // ---------------------------------------------------------------- host mesh data
 // Patches of the fused P1 smoothing kernels between a level (fine) and the
 // next coarser one.  The coarse vertices are split into nb spatially compact
@@ -200,10 +249,9 @@ struct Imex {
     bool has_f = false;          // explicit Coriolis term present
     size_t nq = 0;               // doubles of one state vector: N * 3 * n_p (u part, then h part)
     double *fcell = nullptr;     // [N][3] Coriolis at the cell vertices (explicit term)
-    double *minv = nullptr;      // [n_p][n_p] inverse of the reference mass matrix
     double *lam = nullptr;       // [PP][NF] upwind trace of the DG state
     double *lam_out = nullptr;   // [NF][PP] trace solution of a stage solve
-    double *buf = nullptr;       // (3 + 2 kImexMaxStages) state vectors
+    double *buf = nullptr;       // (2 + 2 kImexMaxStages) state vectors
 };
 
 // per-iteration readback of the Krylov driver (pinned host copy)
@@ -223,6 +271,17 @@ struct ReadBack {
 };
 
 #ifdef __CUDACC__
+// f(integral_constant<int, 0>) ... f(integral_constant<int, N - 1>): a loop whose
+// index is a constant expression in the body (zero entries left out at compile time)
+template <class F, int... I>
+__device__ __forceinline__ void static_for_seq(F &f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F &&f) {
+    static_for_seq(f, std::make_integer_sequence<int, N>{});
+}
+
 // The last block of a grid-wide reduction: out[i] = sum over b < nb of
 // partial[i * nb + b] for i < k, in a fixed order.  The warps are shared out
 // among the vectors (all of them for one vector, half each for two, ...);
@@ -543,6 +602,7 @@ struct hdg_handle {
 
     // device mesh / geometry
     double *d_ref = nullptr;        // packed reference matrices
+    double *d_nref = nullptr;       // packed nodal reference matrices (NodalRef)
     double *d_X = nullptr;          // [N][3][2]
     double *d_fcell = nullptr;      // [N][3] Coriolis at the cell vertices
     int32_t *d_facet_of = nullptr, *d_flip = nullptr;   // [N][3]
@@ -654,8 +714,8 @@ cudaError_t noalloc_prepare(hdg_handle *h);
 // read a buffer larger than L2 so that the next kernel's data comes from DRAM (k_measure.cu)
 cudaError_t launch_l2_evict(const void *buf, size_t bytes, uint32_t *sink, cudaStream_t s);
 
-// IMEX rates (k_imex.cu): upwind trace of the state, then M^-1 N(q) (nu, nh;
-// skipped when null) and M^-1 L(q) (lu, lh) per cell
+// IMEX rates (k_imex.cu): M^-1 N(q) (nu and, when given, nh = 0) and M^-1 L(q)
+// (lu, lh; from the upwind trace of the state) per cell, each skipped when null
 cudaError_t launch_imex_rates(hdg_handle *h, const double *u, const double *hh, double *nu, double *nh, double *lu,
                               double *lh);
 void imex_release(hdg_handle *h);

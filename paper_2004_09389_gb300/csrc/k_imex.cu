@@ -37,20 +37,20 @@ __device__ __forceinline__ int edge_node(int i, int j) {
     return b * (P + 1) - b * (b - 1) / 2 + a;
 }
 
-// outward unit normal of edge i of a counter-clockwise cell with local vertices x[6]
-__device__ __forceinline__ void edge_normal(const double *x, int i, double &nx, double &ny, double &len) {
+// tangent of edge i (from local vertex (i+1)%3 to (i+2)%3) of a cell with
+// local vertices x[6]; (ty, -tx) is its outward normal times its length
+__device__ __forceinline__ void edge_tangent(const double *x, int i, double &tx, double &ty) {
     const int v1 = (i + 1) % 3, v2 = (i + 2) % 3;
-    const double tx = x[2 * v2] - x[2 * v1], ty = x[2 * v2 + 1] - x[2 * v1 + 1];
-    len = sqrt(tx * tx + ty * ty);
-    nx = ty / len;
-    ny = -tx / len;
+    tx = x[2 * v2] - x[2 * v1];
+    ty = x[2 * v2 + 1] - x[2 * v1 + 1];
 }
 
-// lambda at the p+1 trace nodes of every facet (internal layout [PP][NF])
+// lambda at the p+1 trace nodes of every facet (internal layout [PP][NF]);
+// c = H / (2 tau_s)
 template <int P>
 __global__ void upwind_trace_kernel(int NF, const int32_t *__restrict__ fcell, const int32_t *__restrict__ fedge,
                                     const int32_t *__restrict__ flip, const double *__restrict__ X,
-                                    const double *__restrict__ u, const double *__restrict__ h, double H, double ts,
+                                    const double *__restrict__ u, const double *__restrict__ h, double c,
                                     double *__restrict__ lam) {
     constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -64,14 +64,14 @@ __global__ void upwind_trace_kernel(int NF, const int32_t *__restrict__ fcell, c
         double x[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) x[k] = X[size_t(K) * 6 + k];
-        double nx, ny, len;
-        edge_normal(x, i, nx, ny, len);
+        double tx, ty;
+        edge_tangent(x, i, tx, ty);
+        const double w = c / sqrt(tx * tx + ty * ty), wx = w * ty, wy = -w * tx;
 #pragma unroll
         for (int r = 0; r < PP; ++r) {
             const int node = edge_node<P>(i, fl ? P - r : r);
             const double hv = h[size_t(K) * NP + node];
-            const double un = nx * u[size_t(K) * 2 * NP + node] + ny * u[size_t(K) * 2 * NP + NP + node];
-            v[r] += 0.5 * hv + (H / (2.0 * ts)) * un;
+            v[r] = fma(wx, u[size_t(K) * 2 * NP + node], fma(wy, u[size_t(K) * 2 * NP + NP + node], fma(0.5, hv, v[r])));
         }
     }
 #pragma unroll
@@ -81,153 +81,190 @@ __global__ void upwind_trace_kernel(int NF, const int32_t *__restrict__ fcell, c
 struct RateArgs {
     int N, NF;
     double g, H, ts;
-    const double *ref;       // packed reference matrices
-    const double *minv;      // [NP][NP] inverse of the reference mass matrix
+    const double *nref;      // packed nodal reference matrices
     const double *X;         // [N][3][2]
     const double *fcell;     // [N][3] Coriolis at the cell's vertices (P1), or null
     const int32_t *facet_of, *flip;
     const double *lam;       // [PP][NF]
     const double *u, *h;     // state
-    double *nu, *nh;         // M^-1 N(q) (u and h parts), or null
-    double *lu, *lh;         // M^-1 L(q)
+    double *nu, *nh;         // M^-1 N(q): u part (N kernels), h part (zero, when given)
+    double *lu, *lh;         // M^-1 L(q) (L kernels)
 };
 
-// one thread per cell: the cell's rows of L(q) and N(q), then the inverse
-// cell mass matrix (M_K = |det J| M_ref)
-template <int P>
-__global__ void __launch_bounds__(128) imex_rates_kernel(RateArgs a) {
-    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2;
-    constexpr int oM = 0, oML = oM + NP * NP, oDxi = oML + 3 * NP * NP, oDeta = oDxi + NP * NP,
-                  oE = oDeta + NP * NP, oN = oE + 3 * NP * NP, oM1 = oN + 3 * NP * PP, oEnd = oM1 + PP * PP;
-    __shared__ double ref[oEnd];
-    __shared__ double minv[NP * NP];
-    for (int k = threadIdx.x; k < oEnd; k += blockDim.x) ref[k] = a.ref[k];
-    for (int k = threadIdx.x; k < NP * NP; k += blockDim.x) minv[k] = a.minv[k];
+// The rates of 64 cells per block, one thread per cell, in function space (every
+// matrix of the reference element multiplied by M_ref^-1 on the host, so no mass
+// solve is left and |det J| drops out).  L is integrated by parts to the strong
+// form, whose facet terms all act on the jump d = h - lambda: with
+// s_i = lift_i d_i / |det J| (t the edge tangent, J^-T = j),
+//   l~_u = -g grad h + g sum_i (t_y, -t_x)_i s_i,
+//   l~_h = -H div u - tau_s sum_i |e_i| s_i,
+// div u through the contravariant components (two matrix products, not four),
+// and n~ through f's P1 form f_0 + (f_1 - f_0) L_1 + (f_2 - f_0) L_2.
+// What bounds it is the FP64 pipe (1.05 TFLOP/s measured): about 570 FMAs per cell
+// for L and 430 for N at p = 3 (no derivative entry that vanishes is multiplied)
+// against about 3,500 FP64 operations in the weak form with a mass solve per
+// field (554 us per launch on the r = 6 sphere, 81,920 cells, p = 3).  An ARS2
+// step there went from 4,596 to 3,250 us with these rates, the first stage's
+// unused l~ left out and the combinations below.  Cells are staged through shared memory
+// (odd stride: no bank conflicts) so that global reads and writes coalesce.
+constexpr int kRateCells = 64;
+template <int P, bool L, bool N>
+__global__ void __launch_bounds__(kRateCells) imex_rates_kernel(RateArgs a) {
+    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, LD = NK | 1;
+    constexpr NodalOffsets O = nodal_offsets(P);
+    __shared__ double ref[O.total];
+    __shared__ double sS[kRateCells * LD];
+    const int t = threadIdx.x;
+    const int K0 = blockIdx.x * kRateCells, nc = min(kRateCells, a.N - K0);
+    for (int k = t; k < O.total; k += kRateCells) ref[k] = a.nref[k];
+    for (int k = t; k < nc * 2 * NP; k += kRateCells) sS[(k / (2 * NP)) * LD + k % (2 * NP)] = a.u[size_t(K0) * 2 * NP + k];
+    if (L)
+        for (int k = t; k < nc * NP; k += kRateCells) sS[(k / NP) * LD + 2 * NP + k % NP] = a.h[size_t(K0) * NP + k];
     __syncthreads();
-    const int K = blockIdx.x * blockDim.x + threadIdx.x;
-    if (K >= a.N) return;
-    double x[6];
+    const int K = K0 + t;
+    const bool on = t < nc;
+    double *q = sS + t * LD;                  // this thread's cell: the state, then its rates
+    double ux[NP], uy[NP];
+    if (on) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) x[k] = a.X[size_t(K) * 6 + k];
-    const double J00 = x[2] - x[0], J01 = x[4] - x[0], J10 = x[3] - x[1], J11 = x[5] - x[1];
-    const double det = J00 * J11 - J01 * J10;
-    // J^-T: d/dx = j00 d/dxi + j01 d/deta, d/dy = j10 d/dxi + j11 d/deta
-    const double j00 = J11 / det, j01 = -J10 / det, j10 = -J01 / det, j11 = J00 / det;
-    double ux[NP], uy[NP], hh[NP];
-#pragma unroll
-    for (int b = 0; b < NP; ++b) {
-        ux[b] = a.u[size_t(K) * 2 * NP + b];
-        uy[b] = a.u[size_t(K) * 2 * NP + NP + b];
-        hh[b] = a.h[size_t(K) * NP + b];
-    }
-    double lam[3][PP], nrm[3][2], len[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        edge_normal(x, i, nrm[i][0], nrm[i][1], len[i]);
-        const int f = a.facet_of[3 * K + i], fl = a.flip[3 * K + i];
-#pragma unroll
-        for (int j = 0; j < PP; ++j) lam[i][j] = a.lam[size_t(fl ? P - j : j) * a.NF + f];
-    }
-    const double g = a.g, H = a.H, ts = a.ts;
-    // L(q) rows, tested against phi_a
-    double Lx[NP], Ly[NP], Lh[NP];
-#pragma unroll
-    for (int ia = 0; ia < NP; ++ia) {
-        double lx = 0.0, ly = 0.0, lh = 0.0;
-#pragma unroll
-        for (int ib = 0; ib < NP; ++ib) {
-            // g (h, d_x phi_a) = g sum_b h_b int phi_b d_x phi_a
-            const double dxi_ba = ref[oDxi + ib * NP + ia], deta_ba = ref[oDeta + ib * NP + ia];
-            lx = fma(g * det * (j00 * dxi_ba + j01 * deta_ba), hh[ib], lx);
-            ly = fma(g * det * (j10 * dxi_ba + j11 * deta_ba), hh[ib], ly);
-            // -H (div u, phi_a) = -H sum_b (u_x,b int phi_a d_x phi_b + u_y,b int phi_a d_y phi_b)
-            const double dxi_ab = ref[oDxi + ia * NP + ib], deta_ab = ref[oDeta + ia * NP + ib];
-            lh = fma(-H * det * (j00 * dxi_ab + j01 * deta_ab), ux[ib], lh);
-            lh = fma(-H * det * (j10 * dxi_ab + j11 * deta_ab), uy[ib], lh);
-            // -tau_s <h, phi_a>_dK
-            double e = 0.0;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) e = fma(len[i], ref[oE + (i * NP + ia) * NP + ib], e);
-            lh = fma(-ts * e, hh[ib], lh);
+        for (int b = 0; b < NP; ++b) {
+            ux[b] = q[b];
+            uy[b] = q[NP + b];
         }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            double nl = 0.0;
-#pragma unroll
-            for (int j = 0; j < PP; ++j) nl = fma(ref[oN + (i * NP + ia) * PP + j], lam[i][j], nl);
-            nl *= len[i];
-            lx = fma(-g * nrm[i][0], nl, lx);      // -g <lambda, w.n>
-            ly = fma(-g * nrm[i][1], nl, ly);
-            lh = fma(ts, nl, lh);                  // + tau_s <lambda, psi>
-        }
-        Lx[ia] = lx;
-        Ly[ia] = ly;
-        Lh[ia] = lh;
     }
-    // M_K^-1 = M_ref^-1 / det
-    const double s = 1.0 / det;
+    if constexpr (L) {
+        if (on) {
+            double x[6];
 #pragma unroll
-    for (int ia = 0; ia < NP; ++ia) {
-        double vx = 0.0, vy = 0.0, vh = 0.0;
+            for (int k = 0; k < 6; ++k) x[k] = a.X[size_t(K) * 6 + k];
+            const double J00 = x[2] - x[0], J01 = x[4] - x[0], J10 = x[3] - x[1], J11 = x[5] - x[1];
+            const double s = 1.0 / (J00 * J11 - J01 * J10);
+            // J^-T: d/dx = j00 d/dxi + j01 d/deta, d/dy = j10 d/dxi + j11 d/deta
+            const double j00 = J11 * s, j01 = -J10 * s, j10 = -J01 * s, j11 = J00 * s;
+            double hh[NP], d[3][PP], wx[3], wy[3], wh[3];
 #pragma unroll
-        for (int ib = 0; ib < NP; ++ib) {
-            const double mi = minv[ia * NP + ib];
-            vx = fma(mi, Lx[ib], vx);
-            vy = fma(mi, Ly[ib], vy);
-            vh = fma(mi, Lh[ib], vh);
+            for (int b = 0; b < NP; ++b) hh[b] = q[2 * NP + b];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                double tx, ty;
+                edge_tangent(x, i, tx, ty);
+                wx[i] = a.g * ty;
+                wy[i] = -a.g * tx;
+                wh[i] = -a.ts * sqrt(tx * tx + ty * ty);
+                const int f = a.facet_of[3 * K + i], fl = a.flip[3 * K + i];
+#pragma unroll
+                for (int j = 0; j < PP; ++j)
+                    d[i][j] = s * (hh[edge_node<P>(i, j)] - a.lam[size_t(fl ? P - j : j) * a.NF + f]);
+            }
+            const double g00 = -a.g * j00, g01 = -a.g * j01, g10 = -a.g * j10, g11 = -a.g * j11;
+            // the contravariant velocity times -H
+            double c1[NP], c2[NP];
+#pragma unroll
+            for (int b = 0; b < NP; ++b) {
+                c1[b] = -a.H * fma(j00, ux[b], j10 * uy[b]);
+                c2[b] = -a.H * fma(j01, ux[b], j11 * uy[b]);
+            }
+            static_for<NP>([&](auto ia_) {
+                constexpr int ia = decltype(ia_)::value;
+                double hx = 0.0, hy = 0.0, lh = 0.0;
+                static_for<NP>([&](auto ib_) {
+                    constexpr int ib = decltype(ib_)::value;
+                    if constexpr (nodal_dx_nonzero(P, ia, ib)) {
+                        const double m = ref[O.Dx + ia * NP + ib];
+                        hx = fma(m, hh[ib], hx);
+                        lh = fma(m, c1[ib], lh);
+                    }
+                    if constexpr (nodal_dy_nonzero(P, ia, ib)) {
+                        const double m = ref[O.Dy + ia * NP + ib];
+                        hy = fma(m, hh[ib], hy);
+                        lh = fma(m, c2[ib], lh);
+                    }
+                });
+                double lx = fma(g00, hx, g01 * hy), ly = fma(g10, hx, g11 * hy);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    double si = 0.0;
+#pragma unroll
+                    for (int j = 0; j < PP; ++j) si = fma(ref[O.lift + (i * NP + ia) * PP + j], d[i][j], si);
+                    lx = fma(wx[i], si, lx);
+                    ly = fma(wy[i], si, ly);
+                    lh = fma(wh[i], si, lh);
+                }
+                q[ia] = lx;
+                q[NP + ia] = ly;
+                q[2 * NP + ia] = lh;
+            });
         }
-        a.lu[size_t(K) * 2 * NP + ia] = s * vx;
-        a.lu[size_t(K) * 2 * NP + NP + ia] = s * vy;
-        a.lh[size_t(K) * NP + ia] = s * vh;
+        __syncthreads();
+        for (int k = t; k < nc * 2 * NP; k += kRateCells)
+            a.lu[size_t(K0) * 2 * NP + k] = sS[(k / (2 * NP)) * LD + k % (2 * NP)];
+        for (int k = t; k < nc * NP; k += kRateCells) a.lh[size_t(K0) * NP + k] = sS[(k / NP) * LD + 2 * NP + k % NP];
+        if constexpr (N) __syncthreads();
     }
-    if (!a.nu) return;
-    // N(q) = -(f u_perp, w): x row +(f u_y, phi_a), y row -(f u_x, phi_a); f is P1
-    double f0 = a.fcell[size_t(K) * 3], f1 = a.fcell[size_t(K) * 3 + 1], f2 = a.fcell[size_t(K) * 3 + 2];
+    if constexpr (N) {
+        if (on) {
+            // (n~_x, n~_y) = (F u_y, -F u_x), F the projected multiplication by f
+            const double f0 = a.fcell[size_t(K) * 3];
+            const double f1 = a.fcell[size_t(K) * 3 + 1] - f0, f2 = a.fcell[size_t(K) * 3 + 2] - f0;
 #pragma unroll
-    for (int ia = 0; ia < NP; ++ia) {
-        double nx = 0.0, ny = 0.0;
+            for (int ia = 0; ia < NP; ++ia) {
+                double nx = f0 * uy[ia], ny = f0 * ux[ia];
 #pragma unroll
-        for (int ib = 0; ib < NP; ++ib) {
-            const double mf = det * (f0 * ref[oML + ia * NP + ib] + f1 * ref[oML + NP * NP + ia * NP + ib] +
-                                     f2 * ref[oML + 2 * NP * NP + ia * NP + ib]);
-            nx = fma(mf, uy[ib], nx);
-            ny = fma(-mf, ux[ib], ny);
+                for (int ib = 0; ib < NP; ++ib) {
+                    const double m = fma(f1, ref[O.ML1 + ia * NP + ib], f2 * ref[O.ML2 + ia * NP + ib]);
+                    nx = fma(m, uy[ib], nx);
+                    ny = fma(m, ux[ib], ny);
+                }
+                q[ia] = nx;
+                q[NP + ia] = -ny;
+            }
         }
-        Lx[ia] = nx;
-        Ly[ia] = ny;
-    }
-#pragma unroll
-    for (int ia = 0; ia < NP; ++ia) {
-        double vx = 0.0, vy = 0.0;
-#pragma unroll
-        for (int ib = 0; ib < NP; ++ib) {
-            const double mi = minv[ia * NP + ib];
-            vx = fma(mi, Lx[ib], vx);
-            vy = fma(mi, Ly[ib], vy);
-        }
-        a.nu[size_t(K) * 2 * NP + ia] = s * vx;
-        a.nu[size_t(K) * 2 * NP + NP + ia] = s * vy;
-        a.nh[size_t(K) * NP + ia] = 0.0;
+        __syncthreads();
+        for (int k = t; k < nc * 2 * NP; k += kRateCells)
+            a.nu[size_t(K0) * 2 * NP + k] = sS[(k / (2 * NP)) * LD + k % (2 * NP)];
+        if (a.nh)
+            for (int k = t; k < nc * NP; k += kRateCells) a.nh[size_t(K0) * NP + k] = 0.0;
     }
 }
 
-// out = q0 + dt sum_j (cn[j] n~_j + cl[j] l~_j), over whole state vectors
-// (u part then h part, n entries); coefficients that are 0 are skipped
+// out = q0 + dt sum_j c_j x_j over a whole state (u part of nu entries, then h
+// part; q0 and out in two pieces each, which may be the caller's); terms j < kn
+// are rates n~, whose h part is zero and not read.  Only the terms with a
+// non-zero coefficient are passed.  Four entries per thread, a block width
+// apart, so that their loads overlap.
 struct Combo {
-    int k;
-    double cn[8], cl[8];
-    const double *n[8], *l[8];
+    int k = 0, kn = 0;
+    double c[2 * kImexMaxStages];
+    const double *x[2 * kImexMaxStages];
 };
-__global__ void imex_combine_kernel(size_t n, const double *__restrict__ q0, Combo c, double dt,
-                                    double *__restrict__ out) {
-    const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double acc = 0.0;
-    for (int j = 0; j < c.k; ++j) {
-        if (c.cn[j] != 0.0) acc = fma(c.cn[j], c.n[j][i], acc);
-        if (c.cl[j] != 0.0) acc = fma(c.cl[j], c.l[j][i], acc);
+constexpr int kCombU = 4;
+__global__ void __launch_bounds__(256) imex_combine_kernel(size_t nu, size_t n, const double *q0u, const double *q0h,
+                                                           Combo c, double dt, double *outu, double *outh) {
+    const size_t i0 = size_t(blockIdx.x) * blockDim.x * kCombU + threadIdx.x;
+    double q[kCombU], acc[kCombU];
+#pragma unroll
+    for (int u = 0; u < kCombU; ++u) {
+        const size_t i = i0 + size_t(u) * blockDim.x;
+        q[u] = i < nu ? q0u[i] : i < n ? q0h[i - nu] : 0.0;
+        acc[u] = 0.0;
     }
-    out[i] = fma(dt, acc, q0[i]);
+    for (int j = 0; j < c.k; ++j) {
+        const double cj = c.c[j];
+        const double *x = c.x[j];
+        const size_t m = j < c.kn ? nu : n;
+#pragma unroll
+        for (int u = 0; u < kCombU; ++u) {
+            const size_t i = i0 + size_t(u) * blockDim.x;
+            if (i < m) acc[u] = fma(cj, x[i], acc[u]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kCombU; ++u) {
+        const size_t i = i0 + size_t(u) * blockDim.x;
+        const double v = fma(dt, acc[u], q[u]);
+        if (i < nu) outu[i] = v;
+        else if (i < n) outh[i - nu] = v;
+    }
 }
 
 // Butcher tableaux (explicit a, implicit a~, weights b, b~) of Sec. 5.1
@@ -290,14 +327,23 @@ Tableau tableau(int scheme, double theta) {
 cudaError_t launch_imex_rates(hdg_handle *h, const double *u, const double *hh, double *nu, double *nh, double *lu,
                               double *lh) {
     Imex &I = h->imex;
+    RateArgs a{h->N, h->NF, h->prm.g, h->prm.H, h->tau_s, h->d_nref, h->d_X, I.fcell, h->d_facet_of,
+               h->d_flip, I.lam, u, hh, nu, nh, lu, lh};
+    const unsigned nb = nblocks(h->N, kRateCells);
+    if (!lu) {
+        HDG_DISPATCH_P(h->p, (imex_rates_kernel<P, false, true><<<nb, kRateCells, 0, h->stream>>>(a)));
+        return cudaGetLastError();
+    }
     HDG_DISPATCH_P(h->p, (upwind_trace_kernel<P><<<nblocks(h->NF, 256), 256, 0, h->stream>>>(
-                             h->NF, h->d_facet_cell, h->d_facet_edge, h->d_flip, h->d_X, u, hh, h->prm.H, h->tau_s,
-                             I.lam)));
+                             h->NF, h->d_facet_cell, h->d_facet_edge, h->d_flip, h->d_X, u, hh,
+                             h->prm.H / (2.0 * h->tau_s), I.lam)));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    RateArgs a{h->N, h->NF, h->prm.g, h->prm.H, h->tau_s, h->d_ref, I.minv, h->d_X, I.fcell, h->d_facet_of,
-               h->d_flip, I.lam, u, hh, nu, nh, lu, lh};
-    HDG_DISPATCH_P(h->p, (imex_rates_kernel<P><<<nblocks(h->N, 128), 128, 0, h->stream>>>(a)));
+    if (nu) {
+        HDG_DISPATCH_P(h->p, (imex_rates_kernel<P, true, true><<<nb, kRateCells, 0, h->stream>>>(a)));
+    } else {
+        HDG_DISPATCH_P(h->p, (imex_rates_kernel<P, true, false><<<nb, kRateCells, 0, h->stream>>>(a)));
+    }
     return cudaGetLastError();
 }
 
@@ -313,7 +359,7 @@ int imex_fail(hdg_handle *h, int code, const std::string &msg) {
 }
 
 void imex_free(Imex &I) {
-    for (double **p : {&I.fcell, &I.minv, &I.lam, &I.lam_out, &I.buf})
+    for (double **p : {&I.fcell, &I.lam, &I.lam_out, &I.buf})
         if (*p) {
             cudaFree(*p);
             *p = nullptr;
@@ -336,33 +382,6 @@ extern "C" int hdg_imex_init(hdg_handle *h, const double *f_vertex) {
     Imex &I = h->imex;
     imex_free(I);
     const size_t N = h->N, np = h->np, nq = N * 3 * np;
-    // inverse reference mass matrix (Gauss-Jordan with partial pivoting, host)
-    RefElem re = build_ref_elem(h->p);
-    const int n = int(np);
-    std::vector<double> A(re.M), inv(size_t(n) * n, 0.0);
-    for (int i = 0; i < n; ++i) inv[size_t(i) * n + i] = 1.0;
-    for (int k = 0; k < n; ++k) {
-        int piv = k;
-        for (int r = k + 1; r < n; ++r)
-            if (std::fabs(A[size_t(r) * n + k]) > std::fabs(A[size_t(piv) * n + k])) piv = r;
-        for (int c = 0; c < n; ++c) {
-            std::swap(A[size_t(k) * n + c], A[size_t(piv) * n + c]);
-            std::swap(inv[size_t(k) * n + c], inv[size_t(piv) * n + c]);
-        }
-        const double d = 1.0 / A[size_t(k) * n + k];
-        for (int c = 0; c < n; ++c) {
-            A[size_t(k) * n + c] *= d;
-            inv[size_t(k) * n + c] *= d;
-        }
-        for (int r = 0; r < n; ++r)
-            if (r != k) {
-                const double f = A[size_t(r) * n + k];
-                for (int c = 0; c < n; ++c) {
-                    A[size_t(r) * n + c] -= f * A[size_t(k) * n + c];
-                    inv[size_t(r) * n + c] -= f * inv[size_t(k) * n + c];
-                }
-            }
-    }
     std::vector<double> fcell(N * 3, 0.0);
     I.has_f = false;
     if (f_vertex)
@@ -371,19 +390,16 @@ extern "C" int hdg_imex_init(hdg_handle *h, const double *f_vertex) {
                 fcell[K * 3 + i] = f_vertex[h->hm.cells[3 * K + i]];
                 if (fcell[K * 3 + i] != 0.0) I.has_f = true;
             }
-    // state buffers: 3 + 2 * kImexMaxStages state vectors (stage state, stage
-    // right-hand side, a copy of q0, the two rates of every stage)
+    // state buffers: 2 + 2 * kImexMaxStages state vectors (stage state, stage
+    // right-hand side, the two rates of every stage)
     I.nq = nq;
-    const size_t nbuf = size_t(3 + 2 * kImexMaxStages) * nq;
+    const size_t nbuf = size_t(2 + 2 * kImexMaxStages) * nq;
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&I.fcell), sizeof(double) * N * 3);
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&I.minv), sizeof(double) * np * np);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&I.lam), sizeof(double) * size_t(h->NT));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&I.lam_out), sizeof(double) * size_t(h->NT));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&I.buf), sizeof(double) * nbuf);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(I.fcell, fcell.data(), sizeof(double) * N * 3, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(I.minv, inv.data(), sizeof(double) * np * np, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         imex_free(I);
@@ -425,38 +441,45 @@ extern "C" int hdg_imex_step_dev(hdg_handle *h, int scheme, double theta, double
         if (rc) return rc;
     }
     const size_t nq = I.nq, nu_ = size_t(h->N) * 2 * h->np;
-    double *Q = I.buf, *R = I.buf + nq, *q0k = I.buf + 2 * nq;
+    double *Q = I.buf, *R = I.buf + nq;
     double *rn[kImexMaxStages], *rl[kImexMaxStages];
     for (int i = 0; i < kImexMaxStages; ++i) {
-        rn[i] = I.buf + (3 + 2 * i) * nq;
-        rl[i] = I.buf + (4 + 2 * i) * nq;
+        rn[i] = I.buf + (2 + 2 * i) * nq;
+        rl[i] = I.buf + (3 + 2 * i) * nq;
     }
     cudaStream_t s = h->stream;
-    // q0 as one contiguous state vector (u part, then h part)
-    cudaError_t e = cudaMemcpyAsync(q0k, u, sizeof(double) * nu_, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(q0k + nu_, hh, sizeof(double) * (nq - nu_), cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return imex_fail(h, HDG_ECUDA, std::string("hdg_imex_step_dev: ") + cudaGetErrorString(e));
     hdg_solve_info acc{};
     int status = HDG_OK;
     const bool expl_f = I.has_f;
+    // out = q0 + dt sum_{j < n} (a_j n~_j + at_j l~_j), the terms whose coefficient is zero
+    // left out; q0 stays in the caller's u, h until the last combination replaces it
+    auto combine = [&](int n, const double *a_, const double *at_, double *ou, double *oh) {
+        Combo c;
+        for (int j = 0; expl_f && j < n; ++j)
+            if (a_[j] != 0.0) {
+                c.c[c.k] = a_[j];
+                c.x[c.k++] = rn[j];
+            }
+        c.kn = c.k;
+        for (int j = 0; j < n; ++j)
+            if (at_[j] != 0.0) {
+                c.c[c.k] = at_[j];
+                c.x[c.k++] = rl[j];
+            }
+        return account_launch(h, HDG_PROF_IMEX, 1, [&]() {
+            imex_combine_kernel<<<nblocks(nq, 256 * kCombU), 256, 0, s>>>(nu_, nq, u, hh, c, dt, ou, oh);
+            return cudaGetLastError();
+        });
+    };
+    cudaError_t e = cudaSuccess;
     for (int i = 0; i < T.s; ++i) {
         // stage right-hand side r_i = q0 + dt sum_{j<i} (a_ij n~_j + a~_ij l~_j)
-        Combo c{};
-        c.k = i;
-        for (int j = 0; j < i; ++j) {
-            c.cn[j] = expl_f ? T.a[i][j] : 0.0;
-            c.cl[j] = T.at[i][j];
-            c.n[j] = rn[j];
-            c.l[j] = rl[j];
-        }
-        double *Qi;
+        const double *Qu, *Qh;
         if (i == 0 && T.at[0][0] == 0.0) {
-            Qi = q0k;                                   // explicit first stage: Q_1 = q0
+            Qu = u;                                     // explicit first stage: Q_1 = q0
+            Qh = hh;
         } else {
-            e = account_launch(h, HDG_PROF_IMEX, 1, [&]() {
-                imex_combine_kernel<<<nblocks(nq, 256), 256, 0, s>>>(nq, q0k, c, dt, R);
-                return cudaGetLastError();
-            });
+            e = combine(i, T.a[i], T.at[i], R, R + nu_);
             if (e != cudaSuccess) return imex_fail(h, HDG_ECUDA, std::string("imex combine: ") + cudaGetErrorString(e));
             if (T.at[i][i] != 0.0) {
                 hdg_solve_info si{};
@@ -471,15 +494,24 @@ extern "C" int hdg_imex_step_dev(hdg_handle *h, int scheme, double theta, double
                 const bool kz = solve_kept_z(h);
                 rc = hdg_recover_dev(h, kz ? nullptr : R, kz ? nullptr : R + nu_, nullptr, Q, Q + nu_);
                 if (rc) return rc;
-                Qi = Q;
+                Qu = Q;
             } else {
-                Qi = R;                                 // M Q = M r: a mass solve in function space
+                Qu = R;                                 // M Q = M r: a mass solve in function space
             }
+            Qh = Qu + nu_;
         }
-        // the stage's rates n~(Q_i), l~(Q_i)
-        e = account_launch(h, HDG_PROF_IMEX, 2, [&]() {
-            return launch_imex_rates(h, Qi, Qi + nu_, expl_f ? rn[i] : nullptr, expl_f ? rn[i] + nu_ : nullptr,
-                                     rl[i], rl[i] + nu_);
+        // the stage's rates n~(Q_i), l~(Q_i), those that a later stage or the new state takes
+        // (ARS2 never uses the first stage's l~: its weight and its column are zero)
+        bool need_n = T.b[i] != 0.0, need_l = T.bt[i] != 0.0;
+        for (int j = i + 1; j < T.s; ++j) {
+            need_n |= T.a[j][i] != 0.0;
+            need_l |= T.at[j][i] != 0.0;
+        }
+        need_n &= expl_f;
+        if (!need_n && !need_l) continue;
+        e = account_launch(h, HDG_PROF_IMEX, need_l ? 2 : 1, [&]() {
+            return launch_imex_rates(h, Qu, Qh, need_n ? rn[i] : nullptr, nullptr, need_l ? rl[i] : nullptr,
+                                     need_l ? rl[i] + nu_ : nullptr);
         });
         if (e != cudaSuccess) return imex_fail(h, HDG_ECUDA, std::string("imex rates: ") + cudaGetErrorString(e));
     }
@@ -489,20 +521,7 @@ extern "C" int hdg_imex_step_dev(hdg_handle *h, int scheme, double theta, double
         return status;
     }
     // q1 = q0 + dt sum_i (b_i n~_i + b~_i l~_i), written into the caller's u, h
-    Combo c{};
-    c.k = T.s;
-    for (int j = 0; j < T.s; ++j) {
-        c.cn[j] = expl_f ? T.b[j] : 0.0;
-        c.cl[j] = T.bt[j];
-        c.n[j] = rn[j];
-        c.l[j] = rl[j];
-    }
-    e = account_launch(h, HDG_PROF_IMEX, 1, [&]() {
-        imex_combine_kernel<<<nblocks(nq, 256), 256, 0, s>>>(nq, q0k, c, dt, R);
-        return cudaGetLastError();
-    });
-    if (e == cudaSuccess) e = cudaMemcpyAsync(u, R, sizeof(double) * nu_, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hh, R + nu_, sizeof(double) * (nq - nu_), cudaMemcpyDeviceToDevice, s);
+    e = combine(T.s, T.b, T.bt, u, hh);
     if (e != cudaSuccess) return imex_fail(h, HDG_ECUDA, std::string("hdg_imex_step_dev: ") + cudaGetErrorString(e));
     acc.status = status;
     if (info) *info = acc;

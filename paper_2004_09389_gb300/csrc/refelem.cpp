@@ -11,6 +11,7 @@
 #include "common.h"
 
 #include <cmath>
+#include <utility>
 
 namespace hdg {
 
@@ -146,6 +147,72 @@ RefElem build_ref_elem(int p) {
             for (int k = 0; k < pp; ++k)
                 r.M1[j * pp + k] += ew[q] * trace_basis(p, j, ex[q]) * trace_basis(p, k, ex[q]);
     return r;
+}
+
+NodalRef build_nodal_ref(int p) {
+    const RefElem re = build_ref_elem(p);
+    const int n = re.n, pp = re.pp;
+    NodalRef r;
+    r.Dx.assign(size_t(n) * n, 0.0);
+    r.Dy.assign(size_t(n) * n, 0.0);
+    std::vector<double> v, dx, dy;
+    int k = 0;
+    for (int b = 0; b <= p; ++b)
+        for (int a = 0; a <= p - b; ++a, ++k) {
+            eval_basis(p, double(a) / p, double(b) / p, v, dx, dy);
+            for (int j = 0; j < n; ++j) {
+                // the entries that nodal_dx_nonzero / nodal_dy_nonzero leave out vanish identically
+                r.Dx[size_t(k) * n + j] = dx[j];
+                r.Dy[size_t(k) * n + j] = dy[j];
+            }
+        }
+    // [lift | ML1 | ML2] = M^-1 [N_0 | N_1 | N_2 | ML_1 | ML_2]: Gauss-Jordan with
+    // partial pivoting in extended precision, rounded once
+    const int w = 3 * pp + 2 * n;
+    std::vector<long double> A(size_t(n) * n), B(size_t(n) * w);
+    for (int i = 0; i < n; ++i) {
+        for (int j = 0; j < n; ++j) A[size_t(i) * n + j] = re.M[size_t(i) * n + j];
+        for (int e = 0; e < 3; ++e)
+            for (int j = 0; j < pp; ++j)
+                B[size_t(i) * w + e * pp + j] = re.N[(size_t(e) * n + i) * pp + j];
+        for (int l = 0; l < 2; ++l)
+            for (int j = 0; j < n; ++j)
+                B[size_t(i) * w + 3 * pp + l * n + j] = re.ML[(size_t(l + 1) * n + i) * n + j];
+    }
+    for (int c = 0; c < n; ++c) {
+        int piv = c;
+        for (int i = c + 1; i < n; ++i)
+            if (std::fabs(A[size_t(i) * n + c]) > std::fabs(A[size_t(piv) * n + c])) piv = i;
+        for (int j = 0; j < n; ++j) std::swap(A[size_t(c) * n + j], A[size_t(piv) * n + j]);
+        for (int j = 0; j < w; ++j) std::swap(B[size_t(c) * w + j], B[size_t(piv) * w + j]);
+        const long double d = 1.0L / A[size_t(c) * n + c];
+        for (int j = 0; j < n; ++j) A[size_t(c) * n + j] *= d;
+        for (int j = 0; j < w; ++j) B[size_t(c) * w + j] *= d;
+        for (int i = 0; i < n; ++i) {
+            if (i == c) continue;
+            const long double f = A[size_t(i) * n + c];
+            for (int j = 0; j < n; ++j) A[size_t(i) * n + j] -= f * A[size_t(c) * n + j];
+            for (int j = 0; j < w; ++j) B[size_t(i) * w + j] -= f * B[size_t(c) * w + j];
+        }
+    }
+    r.lift.assign(size_t(3) * n * pp, 0.0);
+    r.ML1.assign(size_t(n) * n, 0.0);
+    r.ML2.assign(size_t(n) * n, 0.0);
+    for (int i = 0; i < n; ++i) {
+        for (int e = 0; e < 3; ++e)
+            for (int j = 0; j < pp; ++j) r.lift[(size_t(e) * n + i) * pp + j] = double(B[size_t(i) * w + e * pp + j]);
+        for (int j = 0; j < n; ++j) {
+            r.ML1[size_t(i) * n + j] = double(B[size_t(i) * w + 3 * pp + j]);
+            r.ML2[size_t(i) * n + j] = double(B[size_t(i) * w + 3 * pp + n + j]);
+        }
+    }
+    return r;
+}
+
+std::vector<double> NodalRef::packed() const {
+    std::vector<double> out;
+    for (const std::vector<double> *m : {&Dx, &Dy, &lift, &ML1, &ML2}) out.insert(out.end(), m->begin(), m->end());
+    return out;
 }
 
 std::vector<double> RefElem::packed() const {
