@@ -211,7 +211,8 @@ HDG_API int hdg_setup(const hdg_mesh_desc *mesh, const hdg_params *prm, void *st
  * C_K A_K^-1 M_K; then the facet-row trace operator (the S_K summed onto the
  * facets), the inverted facet diagonal blocks of the block-Jacobi smoother and
  * the P1 level operators (Eq. coarse_problem_upwind, divided by tau).
- * FP64 handles eliminate in FP64.  Handles in HDG_MIXED_FP32 / HDG_MIXED_BF16,
+ * FP64 handles eliminate in FP64 (velocity first, then the n_p x n_p height
+ * system).  Handles in HDG_MIXED_FP32 / HDG_MIXED_BF16,
  * which use these matrices only as two-float pairs, invert A_K in FP32 and
  * refine A_K^-1 [B_K | M_K] twice with two-float residuals (about 48-bit
  * results, written directly as the pairs); the environment variable

@@ -1414,6 +1414,7 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
             for (int i = 0; i < 3; ++i) {
                 fcell[size_t(K) * 3 + i] = prm->f_vertex[hm.cells[3 * K + i]];
                 if (fcell[size_t(K) * 3 + i] != 0.0) h->has_f = true;
+                if (!(fcell[size_t(K) * 3 + i] == fcell[size_t(K) * 3])) h->f_const = false;
             }
     TRY(upload(&h->d_fcell, fcell, s));
     TRY(upload(&h->d_facet_of, hm.facet_of, s));

@@ -58,16 +58,18 @@ struct NodalRef {
     std::vector<double> Dx, Dy;     // [n][n]     d_xi phi_b, d_eta phi_b at node a
     std::vector<double> lift;       // [3][n][pp] M^-1 N_i
     std::vector<double> ML1, ML2;   // [n][n]     M^-1 ML_1, M^-1 ML_2: multiplication by L_1, L_2 (L_0 = 1 - L_1 - L_2)
-    // packed copy for the device: Dx | Dy | lift | ML1 | ML2
+    std::vector<double> Wx, Wy;     // [n][n]     -M^-1 Dxi^T, -M^-1 Deta^T: the weak derivatives (dense)
+    // packed copy for the device: Dx | Dy | lift | ML1 | ML2 | Wx | Wy
     std::vector<double> packed() const;
 };
 NodalRef build_nodal_ref(int p);
 struct NodalOffsets {
-    int Dx, Dy, lift, ML1, ML2, total;
+    int Dx, Dy, lift, ML1, ML2, Wx, Wy, total;
 };
 __host__ __device__ constexpr NodalOffsets nodal_offsets(int p) {
     const int n = (p + 1) * (p + 2) / 2, nn = n * n;
-    return NodalOffsets{0, nn, 2 * nn, 2 * nn + 3 * n * (p + 1), 3 * nn + 3 * n * (p + 1), 4 * nn + 3 * n * (p + 1)};
+    const int l = 3 * n * (p + 1);
+    return NodalOffsets{0, nn, 2 * nn, 2 * nn + l, 3 * nn + l, 4 * nn + l, 5 * nn + l, 6 * nn + l};
 }
 // lattice index b (row) of cell node k of degree p; a = k - row start, c = p - a - b
 __host__ __device__ constexpr int node_b(int p, int k) {
@@ -96,6 +98,17 @@ __host__ __device__ constexpr bool nodal_dx_nonzero(int p, int i, int j) {
 __host__ __device__ constexpr bool nodal_dy_nonzero(int p, int i, int j) {
     return node_a(p, i) >= node_a(p, j) &&
            !(node_b(p, i) < node_b(p, j) && node_a(p, i) + node_b(p, i) > node_a(p, j) + node_b(p, j));
+}
+
+// cell node at position j of edge i (from local vertex (i+1)%3 to (i+2)%3), and the
+// position of cell node k on edge i, -1 if it is not on that edge
+__host__ __device__ constexpr int edge_cell_node(int p, int i, int j) {
+    const int a = i == 0 ? p - j : i == 1 ? 0 : j, b = i == 0 ? j : i == 1 ? p - j : 0;
+    return b * (p + 1) - b * (b - 1) / 2 + a;
+}
+__host__ __device__ constexpr int node_edge_pos(int p, int i, int k) {
+    const int a = node_a(p, k), b = node_b(p, k);
+    return i == 0 ? (a + b == p ? b : -1) : i == 1 ? (a == 0 ? p - b : -1) : (b == 0 ? a : -1);
 }
 
 // ---------------------------------------------------------------- host mesh data
@@ -655,6 +668,7 @@ struct hdg_handle {
     std::vector<std::complex<double>> cheb_c_ritz;
     std::vector<double> cheb_c_omega, cheb_c_beta;
     bool has_f = false;               // a non-zero Coriolis field was given to hdg_setup
+    bool f_const = true;              // the field is constant on every cell (none, or an f-plane)
     // Chebyshev smoother (smoother 1): the ellipse, the Ritz values it was
     // fitted to, and per step k the sweep coefficients omega_k (of D^-1 r)
     // and beta_k (of x_k - x_{k-1})

@@ -1,20 +1,21 @@
 // Static condensation (Sec. 4.2) and assembly of the facet-row trace operator.
 //
-// Per cell K (one CTA per cell), with u_perp = (-u_y, u_x), the cell rows of
-// the upwind HDG form (Eq. bilinear_HDG_upwind, ABCM split of Eq. ABCMform /
-// App. B, Coriolis implicit) are assembled in the integrated-by-parts form
+// Per cell K, with u_perp = (-u_y, u_x), the cell rows of the upwind HDG form
+// (Eq. bilinear_HDG_upwind, ABCM split of Eq. ABCMform / App. B, Coriolis implicit)
+// in the integrated-by-parts form
 //   momentum: (u,w) + tau (f u_perp, w) - tau g (h, div w)         + tau g <lambda, w.n>
 //   mass:     (h,psi) + tau H (div u, psi) + tau tau_s <h, psi>_dK - tau tau_s <lambda, psi>
 //   facet:    <H u.n + tau_s h, mu> - tau_s <lambda, mu>
 // i.e. A_K q + B_K lambda = Mass_K r on the cell and C_K q - Mt_K lambda on its
-// facets.  The momentum rows are scaled by H/g: the scaled A_K has the
-// positive-definite symmetric part  diag((H/g) M, M + tau tau_s E)  (the
-// Coriolis and the tau H div coupling are skew after scaling), so every
-// leading minor is non-zero and Gauss-Jordan elimination needs no pivoting.
-// Elimination of [A | B | Mass] gives X_B = A^-1 B and R_M = A^-1 Mass; then
+// facets, are condensed to X_B = A^-1 B, R_M = A^-1 Mass and
 //   S_K = Mt_K + C_K X_B      (the cell's part of Eq. schur_system)
 //   W_K = C_K R_M             (step 1: g = sum_K P_K^T W_K r_K)
-// and R_M, X_B serve step 3 (Eq. reconstruct_solution): q = R_M r - X_B lambda_K.
+// R_M and X_B serve step 3 (Eq. reconstruct_solution): q = R_M r - X_B lambda_K.
+// FP64 handles eliminate the velocity first, in function space (condense_nodal_kernel);
+// the two-float handles invert A_K in FP32 and refine (condense_mp_kernel), the momentum
+// rows scaled by H/g: the scaled A_K has the positive-definite symmetric part
+// diag((H/g) M, M + tau tau_s E) (the Coriolis and the tau H div coupling are skew after
+// scaling), so every leading minor is non-zero and no pivoting is needed.
 #include "common.h"
 
 #include <cstdlib>
@@ -135,74 +136,441 @@ __device__ __forceinline__ void cell_system(const CondenseArgs &a, int K, double
 
 }
 
-template <int P>
-__global__ void __launch_bounds__(kCondenseThreads) condense_kernel(CondenseArgs a) {
-    using S = Sz<P>;
-    constexpr int NP = S::NP, NK = S::NK, M = S::M, PP = S::PP, LDA = S::LDA;
-    constexpr int oM = 0, oML = oM + NP * NP, oDxi = oML + 3 * NP * NP, oDeta = oDxi + NP * NP,
-                  oE = oDeta + NP * NP, oN = oE + 3 * NP * NP, oM1 = oN + 3 * NP * PP;
-    extern __shared__ double smem[];
-    double *Aug = smem;                 // [NK][LDA]
-    double *Cm = Aug + NK * LDA;        // [M][NK]
-    double *prow = Cm + M * NK;         // [LDA]
-    double *fac = prow + LDA;           // [NK]
-    __shared__ double geo[16];          // detJ, Jit[4], len[3], nrm[6], pad
-    __shared__ double fK[3];
-    __shared__ int bad;
+// ---------------------------------------------------------------- condensation in function space
+// Every cell matrix multiplied by M_K^-1, so that the cell equations act on
+// nodal values and the reference matrices are the same for every cell:
+//   u + tau F u_perp + tau g G h = r_u - b_u,   h + tau H div u + tau tau_s E h = r_h - b_h
+// with F the projected multiplication by f, G the weak gradient, E the lifted edge
+// traces and (b_u, b_h) = B^ lambda.  With R = (I + tau F J)^-1 = [P Q; -Q P],
+// P = (I + tau^2 F^2)^-1, Q = tau F P, the velocity is eliminated first,
+//   T = tau g R G,   S = I + tau tau_s E - tau H div T,   h = S^-1 (r_h - tau H div R r_u),
+//   u = R r_u - T h,
+// so that a cell takes two inverses of n_p x n_p instead of one of 3 n_p x 3 n_p.
+// Where f is constant on every cell (FC; decided at set-up), F = f and P, Q are
+// numbers: one inverse.  X_B = A^-1 B, R_M = A^-1 Mass, S_K = Mt_K + C X_B and
+// W_K = C R_M follow column by column.
+//
+// One thread per column of a cell, kCondCells<P> cells per block with the cell as
+// the fastest thread index (shared-memory reads without bank conflicts, global
+// writes in runs of neighbouring cells).  The FP64 pipe is the bound (1.05 TFLOP/s
+// measured, one warp instruction in about 77 cycles per scheduler), so the split is
+// the one that keeps the warps full: at p = 3 8 x 10 columns in the first phase and
+// 8 x 12 in the second, of 96 threads.  The elimination of the whole augmented cell
+// system [A | B | Mass], one cell per block with two barriers per pivot, took 1,466 us
+// on 18,432 cells at p = 2; a change of the time step followed by a solve and recovery
+// there went from 3,014 to 1,965 us.
+template <int P> constexpr int kCondCells = P == 1 ? 16 : P == 2 ? 10 : P == 3 ? 8 : 6;
+constexpr int kCondThreads = 96;
 
-    const int K = blockIdx.x;
-    const int tid = threadIdx.x;
-    const double *ref = a.ref;
-    const double ts = a.tau_s;
-    if (tid == 0) bad = 0;
-    cell_system<P>(a, K, Aug, Cm, geo, fK);
+struct NodalArgs {
+    int N;
+    double tau, g, H, ts;
+    const double *nref;     // packed nodal reference matrices
+    const double *M1;       // [PP][PP] edge mass matrix
+    const double *X;        // [N][3][2]
+    const double *fcell;    // [N][3]
+    double *Xb, *Rm, *W, *Scell;
+    int32_t *status;
+};
 
-    // ---- Gauss-Jordan elimination, no pivoting (see the header comment)
-    for (int k = 0; k < NK; ++k) {
-        const double piv = Aug[k * LDA + k];
-        if (!(fabs(piv) > 1e-300)) {
-            if (tid == 0) bad = 1;
-        }
-        const double pinv = 1.0 / piv;
-        for (int c = k + 1 + tid; c < LDA; c += blockDim.x) prow[c] = Aug[k * LDA + c] * pinv;
-        for (int r = tid; r < NK; r += blockDim.x) fac[r] = Aug[r * LDA + k];
+// In-place inverse of the n x n matrices A[(i * n + j) * CC + c] of the block's cells
+// by Gauss-Jordan elimination with partial pivoting; thread (c, j) owns column j.
+// Every thread of the block calls it (on: the thread owns a column); piv is shared
+// scratch [n][CC].  Sets bad on a zero pivot.
+template <int n, int CC>
+__device__ __forceinline__ void block_inverse(double *A, int c, int j, bool on, int *piv, int *bad) {
+    for (int k = 0; k < n; ++k) {
         __syncthreads();
-        const int W = LDA - k - 1;
-        for (int idx = tid; idx < NK * W; idx += blockDim.x) {
-            const int r = idx / W, c = k + 1 + idx % W;
-            if (r == k) Aug[r * LDA + c] = prow[c];
-            else Aug[r * LDA + c] -= fac[r] * prow[c];
+        double f[n];
+        int p = k;
+        if (on) {
+            // the pivot row by magnitude (the high words order like the values)
+            int best = -1;
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                f[i] = A[(i * n + k) * CC + c];
+                const int m = __double2hiint(f[i]) & 0x7fffffff;
+                if (i >= k && m > best) {
+                    best = m;
+                    p = i;
+                }
+            }
+        }
+        __syncthreads();                       // column k has been read
+        if (on) {
+            double d = 0.0, fk = 0.0;
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                if (i == p) d = f[i];
+                if (i == k) fk = f[i];
+            }
+            if (!(fabs(d) > 1e-300)) *bad = 1;
+            const double r = 1.0 / d;
+            double *a = A + j * CC + c;
+            const double akj = a[k * n * CC], apj = a[p * n * CC];
+            if (p != k) a[p * n * CC] = akj;   // the rows swapped
+            const double row = j == k ? r : apj * r;
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                const double fi = i == p ? fk : f[i];   // column k after the swap
+                const double aij = a[i * n * CC];
+                a[i * n * CC] = i == k ? row : j == k ? -fi * r : fma(-fi, row, aij);
+            }
+            if (j == 0) piv[k * CC + c] = p;
+        }
+    }
+    __syncthreads();
+    // the row swaps, undone on the columns in reverse order: column j goes to place q
+    double col[n];
+    int q = j;
+    if (on) {
+        for (int k = n - 1; k >= 0; --k) {
+            const int p = piv[k * CC + c];
+            q = q == k ? p : q == p ? k : q;
+        }
+#pragma unroll
+        for (int i = 0; i < n; ++i) col[i] = A[(i * n + j) * CC + c];
+    }
+    __syncthreads();
+    if (on) {
+#pragma unroll
+        for (int i = 0; i < n; ++i) A[(i * n + q) * CC + c] = col[i];
+    }
+    __syncthreads();
+}
+
+// Keeps the compiler from moving shared-memory loads of later rows above this point
+// (at p = 4 it would otherwise hold whole matrices in registers and spill).
+__device__ __forceinline__ void row_fence() { asm volatile("" ::: "memory"); }
+
+// rh += div of the contravariant velocity of (wx, wy) scaled by the weights g00 .. g11
+// (nodal derivatives, the entries that vanish left out)
+template <int P>
+__device__ __forceinline__ void add_div(const double *ref, double g00, double g01, double g10, double g11,
+                                        const double (&wx)[Sz<P>::NP], const double (&wy)[Sz<P>::NP],
+                                        double (&rh)[Sz<P>::NP]) {
+    constexpr int NP = Sz<P>::NP;
+    constexpr NodalOffsets O = nodal_offsets(P);
+    double c1[NP], c2[NP];
+#pragma unroll
+    for (int b = 0; b < NP; ++b) {
+        c1[b] = fma(g00, wx[b], g10 * wy[b]);
+        c2[b] = fma(g01, wx[b], g11 * wy[b]);
+    }
+    static_for<NP>([&](auto ia_) {
+        constexpr int ia = decltype(ia_)::value;
+        row_fence();
+        static_for<NP>([&](auto ib_) {
+            constexpr int ib = decltype(ib_)::value;
+            if constexpr (nodal_dx_nonzero(P, ia, ib)) rh[ia] = fma(ref[O.Dx + ia * NP + ib], c1[ib], rh[ia]);
+            if constexpr (nodal_dy_nonzero(P, ia, ib)) rh[ia] = fma(ref[O.Dy + ia * NP + ib], c2[ib], rh[ia]);
+        });
+    });
+}
+
+// h = S^-1 rh and (wx, wy) -= T h, cell c of the block's matrices.  So non-null: S
+// itself, for one step of iterative refinement of h.  The explicit inverse alone
+// leaves S_K about 20 times less exact than an elimination of the whole cell system
+// (p = 3, Courant 16: S_K applied to a nearly constant trace off by 1e-12 instead of
+// 7e-14); one step brings it to 2e-14.
+template <int NP, int CC>
+__device__ __forceinline__ void back_substitute(const double *Ss, const double *So, const double *Ts, int c,
+                                                const double (&rh)[NP], double (&wx)[NP], double (&wy)[NP],
+                                                double (&h)[NP]) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) v = fma(Ss[(i * NP + k) * CC + c], rh[k], v);
+        h[i] = v;
+    }
+    if (So) {
+        double res[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            row_fence();
+            double v = rh[i];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) v = fma(-So[(i * NP + k) * CC + c], h[k], v);
+            res[i] = v;
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            row_fence();
+            double v = h[i];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) v = fma(Ss[(i * NP + k) * CC + c], res[k], v);
+            h[i] = v;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            wx[i] = fma(-Ts[(i * NP + k) * CC + c], h[k], wx[i]);
+            wy[i] = fma(-Ts[((NP + i) * NP + k) * CC + c], h[k], wy[i]);
+        }
+    }
+}
+
+// row (edge e, node jj) of C q into out[row * ld]; diag is added to the rows of edge e0
+// (diag times column jj0 of the edge mass matrix; e0 = -1: nothing)
+template <int P>
+__device__ __forceinline__ void c_rows(const double *m1, const double (&wn)[3][3], const double (&qx)[Sz<P>::NP],
+                                       const double (&qy)[Sz<P>::NP], const double (&qh)[Sz<P>::NP], int e0, int jj0,
+                                       double diag, double *out, size_t ld) {
+    constexpr int PP = P + 1;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        row_fence();
+        double fl[PP];
+#pragma unroll
+        for (int jb = 0; jb < PP; ++jb) {
+            const int b = edge_cell_node(P, e, jb);
+            fl[jb] = fma(wn[e][0], qx[b], fma(wn[e][1], qy[b], wn[e][2] * qh[b]));
+        }
+#pragma unroll
+        for (int jj = 0; jj < PP; ++jj) {
+            double v = e == e0 ? diag * m1[jj * PP + jj0] : 0.0;
+#pragma unroll
+            for (int jb = 0; jb < PP; ++jb) v = fma(m1[jb * PP + jj], fl[jb], v);
+            out[size_t(e * PP + jj) * ld] = v;
+        }
+    }
+}
+
+// shared memory of the kernel below, in doubles
+template <int P, bool FC>
+struct CondSmem {
+    static constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NN = NP * NP, CC = kCondCells<P>;
+    static constexpr int oRef = 0, oM1 = nodal_offsets(P).total, oGeo = oM1 + PP * PP;
+    static constexpr int nGeo = 4 + 9 + 2 + 3;                     // j, edge weights, R (FC), f
+    static constexpr int oS = oGeo + nGeo * CC, oT = oS + NN * CC, oSo = oT + 2 * NN * CC, oP = oSo + NN * CC;
+    static constexpr int oQ = oP + (FC ? 0 : NN * CC), total = oQ + (FC ? 0 : NN * CC);
+};
+
+template <int P, bool FC>
+__global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs a) {
+    using L = CondSmem<P, FC>;
+    constexpr int PP = P + 1, NP = L::NP, NK = 3 * NP, M = 3 * PP, CC = L::CC;
+    constexpr NodalOffsets O = nodal_offsets(P);
+    extern __shared__ double sm[];
+    double *ref = sm + L::oRef, *m1 = sm + L::oM1, *geo = sm + L::oGeo;
+    double *Ss = sm + L::oS, *Ts = sm + L::oT, *So = sm + L::oSo, *Ps = sm + L::oP, *Qs = sm + L::oQ;
+    __shared__ int piv[NP * CC];
+    __shared__ int bad;
+    const int t = threadIdx.x, c = t % CC, j = t / CC;
+    const int K = blockIdx.x * CC + c;
+    const bool cell = K < a.N, on = cell && j < NP;
+    if (t == 0) bad = 0;
+    for (int k = t; k < O.total; k += kCondThreads) ref[k] = a.nref[k];
+    for (int k = t; k < PP * PP; k += kCondThreads) m1[k] = a.M1[k];
+    // geometry of the cell, [entry][CC]: J^-T (0..3), per edge 1/det times (t_y, -t_x, |e|)
+    // (4..12), P and Q where f is constant on the cell (13, 14), tau times f_0, f_1 - f_0,
+    // f_2 - f_0 (15..17)
+    if (cell && j == 0) {
+        const double *x = a.X + size_t(K) * 6;
+        const double J00 = x[2] - x[0], J01 = x[4] - x[0], J10 = x[3] - x[1], J11 = x[5] - x[1];
+        const double s = 1.0 / (J00 * J11 - J01 * J10);
+        geo[0 * CC + c] = J11 * s;
+        geo[1 * CC + c] = -J10 * s;
+        geo[2 * CC + c] = -J01 * s;
+        geo[3 * CC + c] = J00 * s;
+        for (int i = 0; i < 3; ++i) {
+            const int v1 = (i + 1) % 3, v2 = (i + 2) % 3;
+            const double tx = x[2 * v2] - x[2 * v1], ty = x[2 * v2 + 1] - x[2 * v1 + 1];
+            geo[(4 + 3 * i) * CC + c] = s * ty;
+            geo[(5 + 3 * i) * CC + c] = -s * tx;
+            geo[(6 + 3 * i) * CC + c] = s * sqrt(tx * tx + ty * ty);
+        }
+        const double f0 = a.fcell[size_t(K) * 3];
+        const double f = a.tau * f0, kap = 1.0 / fma(f, f, 1.0);
+        geo[13 * CC + c] = kap;
+        geo[14 * CC + c] = f * kap;
+        geo[15 * CC + c] = f;
+        geo[16 * CC + c] = a.tau * (a.fcell[size_t(K) * 3 + 1] - f0);
+        geo[17 * CC + c] = a.tau * (a.fcell[size_t(K) * 3 + 2] - f0);
+    }
+    __syncthreads();
+    const double tg = a.tau * a.g, tH = a.tau * a.H;
+    const double j00 = geo[0 * CC + c], j01 = geo[1 * CC + c], j10 = geo[2 * CC + c], j11 = geo[3 * CC + c];
+
+    // ---- R: P and Q (f varying over the cell); tau F waits in T's place
+    if constexpr (!FC) {
+        double col[NP];
+        if (on) {
+            const double f0 = geo[15 * CC + c], f1 = geo[16 * CC + c], f2 = geo[17 * CC + c];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                col[i] = fma(f1, ref[O.ML1 + i * NP + j], f2 * ref[O.ML2 + i * NP + j]);
+                if (i == j) col[i] += f0;
+                Ts[(i * NP + j) * CC + c] = col[i];
+            }
+        }
+        __syncthreads();
+        if (on) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                row_fence();
+                double v = i == j ? 1.0 : 0.0;
+#pragma unroll
+                for (int k = 0; k < NP; ++k) v = fma(Ts[(i * NP + k) * CC + c], col[k], v);
+                Ps[(i * NP + j) * CC + c] = v;
+            }
+        }
+        block_inverse<NP, CC>(Ps, c, j, on, piv, &bad);
+        if (on) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) col[i] = Ps[(i * NP + j) * CC + c];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                row_fence();
+                double v = 0.0;
+#pragma unroll
+                for (int k = 0; k < NP; ++k) v = fma(Ts[(i * NP + k) * CC + c], col[k], v);
+                Qs[(i * NP + j) * CC + c] = v;
+            }
         }
         __syncthreads();
     }
+    const double kap = geo[13 * CC + c], fk = geo[14 * CC + c];
+
+    // ---- T = tau g R G and S, column j
+    if (on) {
+        double tx[NP], ty[NP], s[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) tx[i] = ty[i] = 0.0;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            row_fence();
+            const double wx = ref[O.Wx + k * NP + j], wy = ref[O.Wy + k * NP + j];
+            const double gx = tg * fma(j00, wx, j01 * wy), gy = tg * fma(j10, wx, j11 * wy);
+            if constexpr (FC) {
+                tx[k] = fma(kap, gx, fk * gy);
+                ty[k] = fma(kap, gy, -fk * gx);
+            } else {
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    const double p = Ps[(i * NP + k) * CC + c], q = Qs[(i * NP + k) * CC + c];
+                    tx[i] = fma(p, gx, fma(q, gy, tx[i]));
+                    ty[i] = fma(p, gy, fma(-q, gx, ty[i]));
+                }
+            }
+        }
+        const double tts = a.tau * a.ts;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            s[i] = i == j ? 1.0 : 0.0;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                const int pos = node_edge_pos(P, e, j);
+                if (pos >= 0) s[i] = fma(tts * geo[(6 + 3 * e) * CC + c], ref[O.lift + (e * NP + i) * PP + pos], s[i]);
+            }
+        }
+        add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, tx, ty, s);
+        // (T overwrites tau F, whose last readers are behind the barrier above)
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            Ts[(i * NP + j) * CC + c] = tx[i];
+            Ts[((NP + i) * NP + j) * CC + c] = ty[i];
+            Ss[(i * NP + j) * CC + c] = s[i];
+            So[(i * NP + j) * CC + c] = s[i];
+        }
+    }
+    block_inverse<NP, CC>(Ss, c, j, on, piv, &bad);
     if (bad) {
-        if (tid == 0) atomicOr(a.status, 1);
+        if (t == 0) atomicOr(a.status, 1);
         return;
     }
 
-    // ---- outputs
+    const double *x = a.X + size_t(cell ? K : 0) * 6;
+    const double det = (x[2] - x[0]) * (x[5] - x[1]) - (x[4] - x[0]) * (x[3] - x[1]);
+    double wn[3][3];                           // edge weights of C: (H t_y, -H t_x, tau_s |e|)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        wn[e][0] = a.H * det * geo[(4 + 3 * e) * CC + c];
+        wn[e][1] = a.H * det * geo[(5 + 3 * e) * CC + c];
+        wn[e][2] = a.ts * det * geo[(6 + 3 * e) * CC + c];
+    }
     const size_t N = a.N;
-    for (int idx = tid; idx < NK * M; idx += blockDim.x) {
-        const int rho = idx / M, t = idx % M;
-        a.Xb[size_t(idx) * N + K] = Aug[rho * LDA + NK + t];
+    // ---- X_B and S_K, column (edge e, trace node jj)
+    if (cell && j < M) {
+        const int e = j / PP, jj = j % PP;
+        const double bx = tg * geo[(4 + 3 * e) * CC + c], by = tg * geo[(5 + 3 * e) * CC + c];
+        const double bh = -a.tau * a.ts * geo[(6 + 3 * e) * CC + c];
+        double wx[NP], wy[NP], rh[NP], h[NP];
+        if constexpr (FC) {
+            const double rx = fma(kap, bx, fk * by), ry = fma(kap, by, -fk * bx);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                const double l = ref[O.lift + (e * NP + i) * PP + jj];
+                wx[i] = rx * l;
+                wy[i] = ry * l;
+                rh[i] = bh * l;
+            }
+        } else {
+            double pl[NP], ql[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) pl[i] = ql[i] = 0.0;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                row_fence();
+                const double l = ref[O.lift + (e * NP + k) * PP + jj];
+                rh[k] = bh * l;
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    pl[i] = fma(Ps[(i * NP + k) * CC + c], l, pl[i]);
+                    ql[i] = fma(Qs[(i * NP + k) * CC + c], l, ql[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                wx[i] = fma(bx, pl[i], by * ql[i]);
+                wy[i] = fma(by, pl[i], -bx * ql[i]);
+            }
+        }
+        add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
+        back_substitute<NP, CC>(Ss, So, Ts, c, rh, wx, wy, h);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            a.Xb[(size_t(i) * M + j) * N + K] = wx[i];
+            a.Xb[(size_t(NP + i) * M + j) * N + K] = wy[i];
+            a.Xb[(size_t(2 * NP + i) * M + j) * N + K] = h[i];
+        }
+        c_rows<P>(m1, wn, wx, wy, h, e, jj, a.ts * det * geo[(6 + 3 * e) * CC + c], a.Scell + size_t(K) * M * M + j, M);
     }
-    for (int idx = tid; idx < NK * NK; idx += blockDim.x) {
-        const int rho = idx / NK, kap = idx % NK;
-        a.Rm[size_t(idx) * N + K] = Aug[rho * LDA + NK + M + kap];
-    }
-    for (int idx = tid; idx < M * M; idx += blockDim.x) {
-        const int t = idx / M, t2 = idx % M;
-        double s = 0.0;
-        for (int kap = 0; kap < NK; ++kap) s += Cm[t * NK + kap] * Aug[kap * LDA + NK + t2];
-        if (t / PP == t2 / PP)
-            s += ts * geo[5 + t / PP] * ref[oM1 + (t % PP) * PP + (t2 % PP)];
-        a.Scell[size_t(K) * M * M + idx] = s;
-    }
-    for (int idx = tid; idx < M * NK; idx += blockDim.x) {
-        const int t = idx / NK, kap = idx % NK;
-        double s = 0.0;
-        for (int r = 0; r < NK; ++r) s += Cm[t * NK + r] * Aug[r * LDA + NK + M + kap];
-        a.W[size_t(idx) * N + K] = s;
+    // ---- R_M and W_K: the columns of the unit vectors in u_x, u_y and h
+    if (on) {
+#pragma unroll 1
+        for (int comp = 0; comp < 3; ++comp) {
+            double wx[NP], wy[NP], rh[NP], h[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                double p, q;
+                if constexpr (FC) {
+                    p = i == j ? kap : 0.0;
+                    q = i == j ? fk : 0.0;
+                } else {
+                    p = Ps[(i * NP + j) * CC + c];
+                    q = Qs[(i * NP + j) * CC + c];
+                }
+                wx[i] = comp == 0 ? p : comp == 1 ? q : 0.0;
+                wy[i] = comp == 0 ? -q : comp == 1 ? p : 0.0;
+                rh[i] = comp == 2 && i == j ? 1.0 : 0.0;
+            }
+            if (comp < 2) add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
+            back_substitute<NP, CC>(Ss, nullptr, Ts, c, rh, wx, wy, h);
+            const int kap_ = comp * NP + j;
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                a.Rm[(size_t(i) * NK + kap_) * N + K] = wx[i];
+                a.Rm[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
+                a.Rm[(size_t(2 * NP + i) * NK + kap_) * N + K] = h[i];
+            }
+            c_rows<P>(m1, wn, wx, wy, h, -1, 0, 0.0, a.W + size_t(kap_) * N + K, size_t(NK) * N);
+        }
     }
 }
 
@@ -626,18 +994,22 @@ __global__ void to_f32_kernel(const double *x, float *y, size_t n) {
     if (i < n) y[i] = float(x[i]);
 }
 
+template <int P, bool FC>
+cudaError_t condense_nodal_p(hdg_handle *h) {
+    constexpr size_t smem = sizeof(double) * CondSmem<P, FC>::total;
+    auto k = &condense_nodal_kernel<P, FC>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    NodalArgs a;
+    a.N = h->N; a.tau = h->prm.tau; a.g = h->prm.g; a.H = h->prm.H; a.ts = h->tau_s;
+    a.nref = h->d_nref; a.M1 = h->d_ref + ref_offsets(P).M1; a.X = h->d_X; a.fcell = h->d_fcell;
+    a.Xb = h->d_Xb; a.Rm = h->d_Rm; a.W = h->d_W; a.Scell = h->d_Scell; a.status = h->d_status;
+    k<<<(h->N + kCondCells<P> - 1) / kCondCells<P>, kCondThreads, smem, h->stream>>>(a);
+    return cudaGetLastError();
+}
 template <int P>
 cudaError_t condense_p(hdg_handle *h) {
-    using S = Sz<P>;
-    size_t smem = sizeof(double) * (S::NK * S::LDA + S::M * S::NK + S::LDA + S::NK);
-    cudaError_t e = cudaFuncSetAttribute(condense_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    CondenseArgs a;
-    a.N = h->N; a.tau = h->prm.tau; a.g = h->prm.g; a.H = h->prm.H; a.tau_s = h->tau_s;
-    a.ref = h->d_ref; a.X = h->d_X; a.fcell = h->d_fcell;
-    a.Xb = h->d_Xb; a.Rm = h->d_Rm; a.W = h->d_W; a.Scell = h->d_Scell; a.status = h->d_status;
-    condense_kernel<P><<<h->N, kCondenseThreads, smem, h->stream>>>(a);
-    return cudaGetLastError();
+    return h->f_const ? condense_nodal_p<P, true>(h) : condense_nodal_p<P, false>(h);
 }
 
 template <int P>

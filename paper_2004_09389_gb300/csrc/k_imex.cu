@@ -26,17 +26,6 @@ namespace {
 
 inline unsigned nblocks(size_t n, int bs) { return unsigned((n + bs - 1) / bs); }
 
-// index of the cell node at edge i, position j (edge from local vertex
-// (i+1)%3 to (i+2)%3); nodes (a/p, b/p) are numbered b outer, a inner
-template <int P>
-__device__ __forceinline__ int edge_node(int i, int j) {
-    int a, b;
-    if (i == 0) { a = P - j; b = j; }
-    else if (i == 1) { a = 0; b = P - j; }
-    else { a = j; b = 0; }
-    return b * (P + 1) - b * (b - 1) / 2 + a;
-}
-
 // tangent of edge i (from local vertex (i+1)%3 to (i+2)%3) of a cell with
 // local vertices x[6]; (ty, -tx) is its outward normal times its length
 __device__ __forceinline__ void edge_tangent(const double *x, int i, double &tx, double &ty) {
@@ -69,7 +58,7 @@ __global__ void upwind_trace_kernel(int NF, const int32_t *__restrict__ fcell, c
         const double w = c / sqrt(tx * tx + ty * ty), wx = w * ty, wy = -w * tx;
 #pragma unroll
         for (int r = 0; r < PP; ++r) {
-            const int node = edge_node<P>(i, fl ? P - r : r);
+            const int node = edge_cell_node(P, i, fl ? P - r : r);
             const double hv = h[size_t(K) * NP + node];
             v[r] = fma(wx, u[size_t(K) * 2 * NP + node], fma(wy, u[size_t(K) * 2 * NP + NP + node], fma(0.5, hv, v[r])));
         }
@@ -112,11 +101,11 @@ template <int P, bool L, bool N>
 __global__ void __launch_bounds__(kRateCells) imex_rates_kernel(RateArgs a) {
     constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, LD = NK | 1;
     constexpr NodalOffsets O = nodal_offsets(P);
-    __shared__ double ref[O.total];
+    __shared__ double ref[O.Wx];            // all but the weak derivatives
     __shared__ double sS[kRateCells * LD];
     const int t = threadIdx.x;
     const int K0 = blockIdx.x * kRateCells, nc = min(kRateCells, a.N - K0);
-    for (int k = t; k < O.total; k += kRateCells) ref[k] = a.nref[k];
+    for (int k = t; k < O.Wx; k += kRateCells) ref[k] = a.nref[k];
     for (int k = t; k < nc * 2 * NP; k += kRateCells) sS[(k / (2 * NP)) * LD + k % (2 * NP)] = a.u[size_t(K0) * 2 * NP + k];
     if (L)
         for (int k = t; k < nc * NP; k += kRateCells) sS[(k / NP) * LD + 2 * NP + k % NP] = a.h[size_t(K0) * NP + k];
@@ -154,7 +143,7 @@ __global__ void __launch_bounds__(kRateCells) imex_rates_kernel(RateArgs a) {
                 const int f = a.facet_of[3 * K + i], fl = a.flip[3 * K + i];
 #pragma unroll
                 for (int j = 0; j < PP; ++j)
-                    d[i][j] = s * (hh[edge_node<P>(i, j)] - a.lam[size_t(fl ? P - j : j) * a.NF + f]);
+                    d[i][j] = s * (hh[edge_cell_node(P, i, j)] - a.lam[size_t(fl ? P - j : j) * a.NF + f]);
             }
             const double g00 = -a.g * j00, g01 = -a.g * j01, g10 = -a.g * j10, g11 = -a.g * j11;
             // the contravariant velocity times -H

@@ -166,9 +166,9 @@ NodalRef build_nodal_ref(int p) {
                 r.Dy[size_t(k) * n + j] = dy[j];
             }
         }
-    // [lift | ML1 | ML2] = M^-1 [N_0 | N_1 | N_2 | ML_1 | ML_2]: Gauss-Jordan with
+    // [lift | ML1 | ML2 | -Wx | -Wy] = M^-1 [N_0 | N_1 | N_2 | ML_1 | ML_2 | Dxi^T | Deta^T]: Gauss-Jordan with
     // partial pivoting in extended precision, rounded once
-    const int w = 3 * pp + 2 * n;
+    const int w = 3 * pp + 4 * n;
     std::vector<long double> A(size_t(n) * n), B(size_t(n) * w);
     for (int i = 0; i < n; ++i) {
         for (int j = 0; j < n; ++j) A[size_t(i) * n + j] = re.M[size_t(i) * n + j];
@@ -178,6 +178,10 @@ NodalRef build_nodal_ref(int p) {
         for (int l = 0; l < 2; ++l)
             for (int j = 0; j < n; ++j)
                 B[size_t(i) * w + 3 * pp + l * n + j] = re.ML[(size_t(l + 1) * n + i) * n + j];
+        for (int j = 0; j < n; ++j) {
+            B[size_t(i) * w + 3 * pp + 2 * n + j] = re.Dxi[size_t(j) * n + i];
+            B[size_t(i) * w + 3 * pp + 3 * n + j] = re.Deta[size_t(j) * n + i];
+        }
     }
     for (int c = 0; c < n; ++c) {
         int piv = c;
@@ -198,12 +202,16 @@ NodalRef build_nodal_ref(int p) {
     r.lift.assign(size_t(3) * n * pp, 0.0);
     r.ML1.assign(size_t(n) * n, 0.0);
     r.ML2.assign(size_t(n) * n, 0.0);
+    r.Wx.assign(size_t(n) * n, 0.0);
+    r.Wy.assign(size_t(n) * n, 0.0);
     for (int i = 0; i < n; ++i) {
         for (int e = 0; e < 3; ++e)
             for (int j = 0; j < pp; ++j) r.lift[(size_t(e) * n + i) * pp + j] = double(B[size_t(i) * w + e * pp + j]);
         for (int j = 0; j < n; ++j) {
             r.ML1[size_t(i) * n + j] = double(B[size_t(i) * w + 3 * pp + j]);
             r.ML2[size_t(i) * n + j] = double(B[size_t(i) * w + 3 * pp + n + j]);
+            r.Wx[size_t(i) * n + j] = -double(B[size_t(i) * w + 3 * pp + 2 * n + j]);
+            r.Wy[size_t(i) * n + j] = -double(B[size_t(i) * w + 3 * pp + 3 * n + j]);
         }
     }
     return r;
@@ -211,7 +219,7 @@ NodalRef build_nodal_ref(int p) {
 
 std::vector<double> NodalRef::packed() const {
     std::vector<double> out;
-    for (const std::vector<double> *m : {&Dx, &Dy, &lift, &ML1, &ML2}) out.insert(out.end(), m->begin(), m->end());
+    for (const std::vector<double> *m : {&Dx, &Dy, &lift, &ML1, &ML2, &Wx, &Wy}) out.insert(out.end(), m->begin(), m->end());
     return out;
 }
 

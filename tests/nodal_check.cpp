@@ -1,6 +1,6 @@
 // Checks the nodal reference matrices (build_nodal_ref) against the weak ones
 // (build_ref_elem) they replace, p = 1..4: M Dx = Dxi, M Dy = Deta, M lift_i = N_i,
-// M ML_l = ML_l (weak), and that every entry the kernels leave out vanishes.
+// M ML_l = ML_l (weak), M W = -D^T, the edge node maps, and that every entry the kernels leave out vanishes.
 #include "../paper_2004_09389_gb300/csrc/common.h"
 
 #include <algorithm>
@@ -28,6 +28,19 @@ int main() {
         diff(q.Dy.data(), r.Deta.data(), n);
         diff(q.ML1.data(), r.ML.data() + n * n, n);
         diff(q.ML2.data(), r.ML.data() + 2 * n * n, n);
+        std::vector<double> t(size_t(2) * n * n);
+        for (int i = 0; i < n; ++i)
+            for (int j = 0; j < n; ++j) {
+                t[i * n + j] = -r.Dxi[j * n + i];
+                t[(n + i) * n + j] = -r.Deta[j * n + i];
+            }
+        diff(q.Wx.data(), t.data(), n);
+        diff(q.Wy.data(), t.data() + n * n, n);
+        for (int e = 0; e < 3; ++e)
+            for (int j = 0; j < pp; ++j) {
+                const int b = edge_cell_node(p, e, j);
+                if (node_edge_pos(p, e, b) != j) return 3;
+            }
         for (int e = 0; e < 3; ++e) diff(q.lift.data() + e * n * pp, r.N.data() + e * n * pp, pp);
         for (int i = 0; i < n; ++i)
             for (int j = 0; j < n; ++j) {
