@@ -451,6 +451,7 @@ def gpu_arm(args, rank: int, world: int):
                         condense_ms=condense_ms, n_p=s.n_p, prof_steps=nprof, tuned=tuned,
                         h2d=h2d, d2h=d2h, NF=NF, pp=pp, n_cells=s.n_cells,
                         keep_z=prec in (HDG_MIXED_FP32, HDG_MIXED_BF16),
+                        f_const=bool((np.asarray(f) == np.asarray(f).ravel()[0]).all()),
                         coarse=(f"P1 geometric V-cycle over {len(levels)} levels, {levels[0].n_vertices:,} -> "
                                 f"{levels[-1].n_vertices} vertices (dense coarsest solve)"),
                         data_gb=(8.0 * s.n_cells * (nK * nK + 2 * nK * m) + 8.0 * NF * 5 * pp * pp) / 1e9)
@@ -468,13 +469,15 @@ def gpu_arm(args, rank: int, world: int):
 def step13_bytes(arm: dict):
     """Algorithmic bytes of one condensed right-hand side (cell and gather
     kernels together) and of one recovery.  Two-float handles keep z_K = R_M r_K
-    in step 1: its cell kernel reads R_M, r and the cell geometry (9 float pairs)
+    in step 1: its cell kernel reads the h rows of R_M (and the inverse velocity
+    block where f varies over the cells), r and the cell weights (15 float pairs)
     and writes z and the cell rows; the recovery reads X_B, z and lambda and
     writes u, h.  FP64 handles read W_K, r in step 1 and R_M, X_B, r, lambda in
     step 3."""
-    N, nK, m = arm["n_cells"], 3 * arm["n_p"], 3 * arm["pp"]
+    N, n, nK, m = arm["n_cells"], arm["n_p"], 3 * arm["n_p"], 3 * arm["pp"]
     if arm.get("keep_z"):
-        return 8.0 * N * (nK * nK + 2 * nK + m) + 72.0 * N, 8.0 * N * (nK * m + 2 * nK + m)
+        mats = n * nK + (0 if arm.get("f_const", True) else 2 * n * n)
+        return 8.0 * N * (mats + 2 * nK + m + 15), 8.0 * N * (nK * m + 2 * nK + m)
     return 8.0 * N * (m * nK + nK + m), 8.0 * N * (nK * nK + nK * m + 3 * nK + m)
 
 
@@ -593,12 +596,15 @@ def roofline(arm: dict, peaks: dict, fma: dict | None = None, bf16_pre: bool = F
 
 def condense_rate(arm: dict, fma: dict) -> dict:
     """FP64 flop rate of the condensation against the measured FP64 FMA rate.
-    Per cell: Gauss-Jordan elimination of [A_K | B_K | Mass_K] (n_K x (2 n_K + m),
-    sum over pivots k of n_K (2 n_K + m - k - 1) FMAs), then S_K = Mt_K + C_K X_B
-    (m^2 n_K) and W_K = C_K R_M (m n_K^2)."""
-    nK, m, N = 3 * arm["n_p"], 3 * arm["pp"], arm["n_cells"]
-    lda = 2 * nK + m
-    fmas = sum(nK * (lda - k - 1) for k in range(nK)) + m * m * nK + m * nK * nK
+    Per cell, with f constant on every cell (an FP64 handle): the columns of T and
+    of the height system, its inverse, X_B with one refinement step, S_K, R_M and
+    W_K; div counts the non-zero nodal derivative entries."""
+    n, m, pp, N = arm["n_p"], 3 * arm["pp"], arm["pp"], arm["n_cells"]
+    nz = {3: 14, 6: 48, 10: 120, 15: 250}[n]
+    div, c_rows = 4 * n + nz, 9 * pp + 3 * pp * pp
+    fmas = (n * (8 * n + div + 2 * n + n * n)                    # T, the height system, its inverse
+            + m * (3 * n + div + 5 * n * n + c_rows)             # X_B (3 n^2 for h with refinement, 2 n^2 for u), S_K
+            + n * (2 * div + 9 * n * n + 3 * c_rows))            # R_M, W_K
     tf = 2.0 * fmas * N / (arm["condense_ms"] * 1e-3) / 1e12
     return {"flops_per_cell": 2 * fmas, "achieved_tflops": tf, "peak_tflops": fma["fp64_tflops"],
             "frac": tf / fma["fp64_tflops"], "timing": "host wall clock around hdg_condense (one call, synchronised)",

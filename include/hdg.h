@@ -160,10 +160,8 @@ typedef struct {
     int32_t       n_coarse;     /* flux 1: Chebyshev steps of the RT0 coarse solve (1..200) */
     int32_t       keep_rhs;     /* HDG_MIXED_FP32 / HDG_MIXED_BF16, upwind flux: 1 (default) =
                                    each solve's step 1 keeps z_K = A_K^-1 M_K r_K for a
-                                   recovery with NULL right-hand sides and forms C_K z_K
-                                   from the cell geometry (step 1 reads A_K^-1 M_K instead
-                                   of C_K A_K^-1 M_K: more bytes there, far fewer in step 3);
-                                   0 = step 1 reads C_K A_K^-1 M_K and keeps nothing (for
+                                   recovery with NULL right-hand sides;
+                                   0 = it keeps nothing and needs no memory for it (for
                                    solves that are not followed by a recovery)           */
 } hdg_params;
 
@@ -211,13 +209,11 @@ HDG_API int hdg_setup(const hdg_mesh_desc *mesh, const hdg_params *prm, void *st
  * C_K A_K^-1 M_K; then the facet-row trace operator (the S_K summed onto the
  * facets), the inverted facet diagonal blocks of the block-Jacobi smoother and
  * the P1 level operators (Eq. coarse_problem_upwind, divided by tau).
- * FP64 handles eliminate in FP64 (velocity first, then the n_p x n_p height
- * system).  Handles in HDG_MIXED_FP32 / HDG_MIXED_BF16,
- * which use these matrices only as two-float pairs, invert A_K in FP32 and
- * refine A_K^-1 [B_K | M_K] twice with two-float residuals (about 48-bit
- * results, written directly as the pairs); the environment variable
- * HDG_CONDENSE_FP64=1 (read once per process) gives them the FP64
- * elimination too.  A coarsest P1 level of more than 256 vertices is inverted
+ * The velocity is eliminated first, then the n_p x n_p height system, in FP64.
+ * Handles in HDG_MIXED_FP32 / HDG_MIXED_BF16 keep, as two-float pairs, A_K^-1 B_K,
+ * the height rows of A_K^-1 M_K and the inverse of the velocity block (two numbers
+ * per cell where f is constant on every cell) instead of A_K^-1 M_K and
+ * C_K A_K^-1 M_K. A coarsest P1 level of more than 256 vertices is inverted
  * by one pivot and one update launch per column.
  * HDG_ESINGULAR if a cell or facet block has a zero pivot. */
 HDG_API int hdg_condense(hdg_handle *h);

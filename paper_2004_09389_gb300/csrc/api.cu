@@ -1211,8 +1211,8 @@ void free_handle(hdg_handle *h) {
     dfree(h->d_ref); dfree(h->d_nref); dfree(h->d_X); dfree(h->d_fcell); dfree(h->d_facet_of); dfree(h->d_flip);
     dfree(h->d_facet_cell); dfree(h->d_facet_edge); dfree(h->d_facet_verts); dfree(h->d_v2f_ptr); dfree(h->d_v2f);
     dfree(h->d_nbr); dfree(h->d_Xb); dfree(h->d_Rm); dfree(h->d_W); dfree(h->d_Scell); dfree(h->d_Sval);
-    dfree(h->d_Xb2); dfree(h->d_Rm2); dfree(h->d_W2); dfree(h->d_Sval2);
-    dfree(h->d_cgeo); dfree(h->d_ctab_v); dfree(h->d_ctab_b);
+    dfree(h->d_Xb2); dfree(h->d_Sval2);
+    dfree(h->d_Hr2); dfree(h->d_PQ2); dfree(h->d_lgeo); dfree(h->d_fftab);
     dfree(h->d_Dinv); dfree(h->d_Sval32); dfree(h->d_Dinv32); dfree(h->d_Sval16); dfree(h->d_status); dfree(h->d_coarse_inv);
     dfree(h->tail_img[0].d); dfree(h->tail_img[1].d);
     dfree(h->d_coarse_work);
@@ -1350,54 +1350,25 @@ void drop_graphs(hdg_handle *h) {
             }
 }
 
-// The tables of C_K formed from geometry in the solves' step 1 (two-float
-// handles): per cell and edge the pairs of H t_y, -H t_x and tau_s |e| (t the
-// edge vector, as the condensation's C_K uses them), and per row (edge i, trace
-// node j) the cell nodes b with a nonzero reference facet entry N_ibj and its
-// pair.  Those are the p + 1 nodes on the edge; another pattern leaves cz_ok
-// false and the solves read the stored W_K instead.
+// The reference matrices of the two-float cell solve as float pairs (FFTabOffsets).
 float2 host_split(double v) {
     const float hi = static_cast<float>(v);
     return float2{hi, static_cast<float>(v - static_cast<double>(hi))};
 }
-int build_cz(hdg_handle *h, const RefElem &re) {
-    cudaStream_t s = h->stream;
-    const int np = h->np, pp = h->pp, N = h->N;
-    const HostMesh &hm = h->hm;
-    double nmax = 0.0;
-    for (double v : re.N) nmax = std::max(nmax, std::fabs(v));
-    std::vector<int32_t> tb(size_t(3) * pp * pp, 0);
-    std::vector<float2> tv(size_t(3) * pp * pp, float2{0.0f, 0.0f});
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < pp; ++j) {
-            int c = 0;
-            for (int b = 0; b < np; ++b) {
-                const double v = re.N[(size_t(i) * np + b) * pp + j];
-                if (!(std::fabs(v) > 1e-13 * nmax)) continue;
-                if (c == pp) return HDG_OK;
-                tb[(size_t(i) * pp + j) * pp + c] = b;
-                tv[(size_t(i) * pp + j) * pp + c] = host_split(v);
-                ++c;
-            }
-        }
-    const double H = h->prm.H, ts = h->tau_s;
-    std::vector<float2> cg(size_t(N) * 9);
-    for (int K = 0; K < N; ++K) {
-        const double *x = hm.X.data() + size_t(K) * 6;
-        for (int i = 0; i < 3; ++i) {
-            const int v1 = (i + 1) % 3, v2 = (i + 2) % 3;
-            const double tx = x[2 * v2] - x[2 * v1], ty = x[2 * v2 + 1] - x[2 * v1 + 1];
-            float2 *o = cg.data() + (size_t(K) * 3 + i) * 3;
-            o[0] = host_split(H * ty);
-            o[1] = host_split(-H * tx);
-            o[2] = host_split(ts * std::sqrt(tx * tx + ty * ty));
-        }
+int build_fftab(hdg_handle *h, const RefElem &re, const NodalRef &nr) {
+    const int n = h->np, pp = h->pp;
+    const FFTabOffsets o = ff_tab_offsets(h->p);
+    std::vector<float4> t(size_t(o.total), float4{0.0f, 0.0f, 0.0f, 0.0f});
+    for (int k = 0; k < n * n; ++k) {
+        const float2 x = host_split(nr.Wx[size_t(k)]), y = host_split(nr.Wy[size_t(k)]);
+        t[size_t(o.W + k)] = float4{x.x, x.y, y.x, y.y};
     }
-    TRY(upload(&h->d_ctab_b, tb, s));
-    TRY(upload(&h->d_ctab_v, tv, s));
-    TRY(upload(&h->d_cgeo, cg, s));
-    TRY(cudaStreamSynchronize(s));      // the host vectors go out of scope
-    h->cz_ok = true;
+    for (int k = 0; k < pp * pp; ++k) {
+        const float2 v = host_split(re.M1[size_t(k)]);
+        t[size_t(o.m1 + k)] = float4{v.x, v.y, 0.0f, 0.0f};
+    }
+    TRY(upload(&h->d_fftab, t, h->stream));
+    TRY(cudaStreamSynchronize(h->stream));      // the host vector goes out of scope
     return HDG_OK;
 }
 
@@ -1406,7 +1377,8 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     const HostMesh &hm = h->hm;
     RefElem re = build_ref_elem(h->p);
     TRY(upload(&h->d_ref, re.packed(), s));
-    TRY(upload(&h->d_nref, build_nodal_ref(h->p).packed(), s));
+    const NodalRef nr = build_nodal_ref(h->p);
+    TRY(upload(&h->d_nref, nr.packed(), s));
     TRY(upload(&h->d_X, hm.X, s));
     std::vector<double> fcell(size_t(h->N) * 3, 0.0);
     if (prm->f_vertex)
@@ -1426,9 +1398,11 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(upload(&h->d_v2f, hm.v2f, s));
     const size_t N = h->N, NF = h->NF, nK = h->nK, m = h->m, pp = h->pp;
     TRY(dalloc(&h->d_nbr, 4 * NF));
-    TRY(dalloc(&h->d_Xb, nK * m * N));
-    TRY(dalloc(&h->d_Rm, nK * nK * N));
-    TRY(dalloc(&h->d_W, m * nK * N));
+    if (!mode_ff(*prm)) {
+        TRY(dalloc(&h->d_Xb, nK * m * N));
+        TRY(dalloc(&h->d_Rm, nK * nK * N));
+        TRY(dalloc(&h->d_W, m * nK * N));
+    }
     TRY(dalloc(&h->d_Scell, N * m * m));
     auto packed = [&](size_t n, size_t G) { return (n + G - 1) / G * G * NF; };
     TRY(dalloc(&h->d_Sval, packed(5 * pp * pp, 2)));
@@ -1442,13 +1416,13 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
             // pairs of row entries (odd rows padded by one zero entry), tiles of 32 cells
             const size_t Nt = (N + 31) / 32 * 32;
             TRY(dalloc(&h->d_Xb2, nK * ((m + 1) / 2 * 2) * Nt));
-            TRY(dalloc(&h->d_Rm2, nK * ((nK + 1) / 2 * 2) * Nt));
-            TRY(dalloc(&h->d_W2, m * ((nK + 1) / 2 * 2) * Nt));
+            const size_t np = h->np, np2 = (np + 1) / 2 * 2;
+            TRY(dalloc(&h->d_Hr2, np * ((nK + 1) / 2 * 2) * Nt));
+            if (!h->f_const) TRY(dalloc(&h->d_PQ2, 2 * np * np2 * Nt));
+            TRY(dalloc(&h->d_lgeo, size_t(kLGeo) * Nt));
             TRY(dalloc(&h->d_Sval2, packed(5 * pp * pp, 2)));
-            if (prm->flux == 0) {
-                const int rc = build_cz(h, re);
-                if (rc) return rc;
-            }
+            const int rc = build_fftab(h, re, nr);
+            if (rc) return rc;
         }
         if (prm->precision == HDG_MIXED_BF16) TRY(dalloc(&h->d_Sval16, packed(5 * pp * pp, 8)));
     }
@@ -1592,7 +1566,7 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(dalloc(&W.lam_int, W.NT));
     TRY(dalloc(&W.ycell, N * m));
     if (mode_ff(h->prm)) TRY(dalloc(&W.x2, W.NT));
-    if (h->cz_ok && h->prm.keep_rhs) TRY(dalloc(&W.z2, size_t(h->nK) * N));
+    if (mode_ff(h->prm) && h->prm.keep_rhs) TRY(dalloc(&W.z2, size_t(h->nK) * N));
     const size_t mm = W.m;
     W.ld = (W.NT + 3) / 4 * 4;
     // one 16-byte group of w per thread (enough loads in flight for the few-vector
@@ -1834,12 +1808,10 @@ int solve_internal(hdg_handle *h, const double *r_u, const double *r_h, hdg_solv
     W.have_z = false;
     if (!mode_ff(h->prm)) {
         TRY(KL(HDG_PROF_RHS, 2, launch_rhs(h, r_u, r_h, W.g, W.ycell, nrm)));
-    } else if (W.z2) {
-        // keeping z_K = R_M r_K for the recovery of this solve
-        TRY(KL(HDG_PROF_RHS, 2, launch_rhs_z(h, r_u, r_h, W.g, W.ycell, W.z2, copy_u, copy_h, nrm)));
-        W.have_z = true;
     } else {
-        TRY(KL(HDG_PROF_RHS, 2, launch_rhs_ff(h, r_u, r_h, W.g, W.ycell, copy_u, copy_h, nrm)));
+        // keeping z_K = A_K^-1 M_K r_K for the recovery of this solve (keep_rhs)
+        TRY(KL(HDG_PROF_RHS, 2, launch_rhs_z(h, r_u, r_h, W.g, W.ycell, W.z2, copy_u, copy_h, nrm)));
+        W.have_z = W.z2 != nullptr;
     }
     int rc;
     if (mode_krylov64(h->prm)) {
@@ -2105,12 +2077,7 @@ int hdg_condense(hdg_handle *h) {
         }
         if (mode_ff(h->prm)) {
             // (hi, lo) float pairs for the two-float FP64 steps
-            const size_t N = h->N, nK = h->nK, m = h->m, pp = h->pp, NS = 5 * pp * pp;
-            if (!condense_writes_pairs(h)) {
-                TRY(KL(HDG_PROF_CONDENSE, 1, launch_split_pairs(h->d_Xb, h->d_Xb2, int(nK), int(m), N, s)));
-                TRY(KL(HDG_PROF_CONDENSE, 1, launch_split_pairs(h->d_Rm, h->d_Rm2, int(nK), int(nK), N, s)));
-                TRY(KL(HDG_PROF_CONDENSE, 1, launch_split_pairs(h->d_W, h->d_W2, int(m), int(nK), N, s)));
-            }
+            const size_t pp = h->pp, NS = 5 * pp * pp;
             TRY(KL(HDG_PROF_CONDENSE, 1, launch_split(h->d_Sval, h->d_Sval2, (NS + 1) / 2 * 2 * size_t(h->NF), s)));
         }
     }

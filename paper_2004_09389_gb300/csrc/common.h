@@ -415,6 +415,18 @@ __device__ __forceinline__ float2 split(double a) {
 // pc = row * CP + cp (CP = (cols + 1) / 2) of cell K at
 // ((K / kFFCells) * rows * CP + pc) * kFFCells + K % kFFCells.
 constexpr int kFFCells = 32;
+// Weights of a cell for the two-float cell solve: tau g J^-T (0..3), per edge H t_y,
+// -H t_x, tau_s |e| (4..12), P and Q where f is constant on the cell (13, 14)
+constexpr int kLGeo = 15;
+// The reference matrices of the two-float cell solve, float4 each: the weak derivatives
+// [NP][NP] as (Wx, Wy) pairs and the edge mass matrix [PP][PP] (one pair)
+struct FFTabOffsets {
+    int W, m1, total;
+};
+__host__ __device__ constexpr FFTabOffsets ff_tab_offsets(int p) {
+    const int n = (p + 1) * (p + 2) / 2, pp = p + 1;
+    return FFTabOffsets{0, n * n, n * n + pp * pp};
+}
 __host__ __device__ __forceinline__ size_t ff_pair_index(size_t K, size_t pc, size_t np) {
     return ((K / kFFCells) * np + pc) * kFFCells + K % kFFCells;
 }
@@ -628,15 +640,15 @@ struct hdg_handle {
     double *d_Xb = nullptr;         // A^-1 B        [nK*m][N]
     double *d_Rm = nullptr;         // A^-1 Mass     [nK*nK][N]
     double *d_W = nullptr;          // C A^-1 Mass   [m*nK][N]
-    // mixed modes: the same three matrices and the FP64 trace operator as
-    // (hi, lo) float pairs for the two-float FP64 steps (k_ff.cu)
-    float2 *d_Xb2 = nullptr, *d_Rm2 = nullptr, *d_W2 = nullptr, *d_Sval2 = nullptr;
-    // C_K from geometry (two-float handles): pairs of H t_y, -H t_x, tau_s |e| per
-    // cell and edge [N][3][3]; per row of C_K the cell nodes and pairs of the
-    // nonzero reference facet entries [3(p+1)][p+1]; cz_ok once they are built
-    float2 *d_cgeo = nullptr, *d_ctab_v = nullptr;
-    int32_t *d_ctab_b = nullptr;
-    bool cz_ok = false;
+    // mixed modes: A^-1 B and the FP64 trace operator as (hi, lo) float pairs
+    // for the two-float FP64 steps (k_ff.cu)
+    float2 *d_Xb2 = nullptr, *d_Sval2 = nullptr;
+    // two-float handles: what the cell solve takes (k_condense.cu, k_ff.cu) as float
+    // pairs in tiles of 32 cells: the h rows of R_M [NP][3 NP], P and Q [2 NP][NP] (null
+    // where f is constant on every cell), kLGeo weights per cell; and the reference
+    // matrices as pairs (FFTab)
+    float2 *d_Hr2 = nullptr, *d_PQ2 = nullptr, *d_lgeo = nullptr;
+    float4 *d_fftab = nullptr;
     double *d_Scell = nullptr;      // S_K           [N][m][m]
     // facet-row trace operator
     double *d_Sval = nullptr;       // 5(p+1)^2 values per facet, packed in 16-byte groups
@@ -765,9 +777,6 @@ cudaError_t launch_p1_assemble(hdg_handle *h, DevLevel &L, double tau, double gH
 // every P1 level operator as the Galerkin product of the trace operator (k_galerkin.cu)
 cudaError_t launch_p1_galerkin(hdg_handle *h);
 cudaError_t launch_dense_inverse(hdg_handle *h, const DevLevel &L, double *work, double *inv, int n);
-// true when launch_condense writes the mixed handles' float-pair matrices
-// (X_B, R_M, W_K) itself, so that no FP64 copy of them exists to split
-bool condense_writes_pairs(const hdg_handle *h);
 // a tail level's ELL arrays in the staged layout: values (tsz bytes each)
 // slot-major into A_dst, columns as 16-bit indices into col_dst
 cudaError_t launch_tail_pack(const int32_t *col, const void *A, size_t tsz, int nv, int W, void *col_dst, void *A_dst,
@@ -809,9 +818,6 @@ cudaError_t launch_rhs(hdg_handle *h, const double *r_u, const double *r_h, doub
 cudaError_t launch_rhs_gather(hdg_handle *h, const double *ycell, double *g, const NormOut &nrm = NormOut());
 // two-float versions of the FP64 steps (mixed modes, k_ff.cu)
 cudaError_t launch_split(const double *a, float2 *out, size_t n, cudaStream_t s);
-// a per-cell matrix [rows][cols][N] split into pairs of row entries, tiled by 32 cells:
-// [ceil(N/32)][rows][(cols+1)/2][32] (float4)
-cudaError_t launch_split_pairs(const double *a, float2 *out, int rows, int cols, size_t N, cudaStream_t s);
 // facets per block of the two-float residual (its grid: ceil(NF / kResFFFacets)
 // blocks, each writing one partial sum)
 constexpr int kResFFFacets = 64;
@@ -827,14 +833,11 @@ cudaError_t launch_ff_join(const float2 *x2, double *a, double *b, size_t n, cud
 cudaError_t launch_residual_ff(hdg_handle *h, const double *b, const float2 *x2, double *res,
                                double *partial = nullptr, unsigned int *counter = nullptr, double *out = nullptr,
                                HostValue *pub = nullptr, int32_t seq = 0, const F32Copy &c32 = F32Copy());
-// (r_u, r_h may be device aliases of page-locked host memory; copy_u / copy_h,
-// if non-null, receive a device copy of them)
-cudaError_t launch_rhs_ff(hdg_handle *h, const double *r_u, const double *r_h, double *g, double *ycell,
-                          double *copy_u, double *copy_h, const NormOut &nrm = NormOut());
 cudaError_t launch_recover_ff(hdg_handle *h, const double *r_u, const double *r_h, const double *lam, double *u,
                               double *hout);
-// step 1 of a solve keeping z_K = R_M r_K (pairs, [nK][N]) for step 3, C_K z_K
-// formed from the cell geometry (handles with cz_ok); step 3 from that z
+// step 1: the cell solve z_K = A_K^-1 M_K r_K and g from C_K z_K; z2 (pairs,
+// [nK][N]; may be null) receives z_K for step 3.  r_u, r_h may be device aliases of
+// page-locked host memory; copy_u / copy_h, if non-null, receive a device copy
 cudaError_t launch_rhs_z(hdg_handle *h, const double *r_u, const double *r_h, double *g, double *ycell, float2 *z2,
                          double *copy_u, double *copy_h, const NormOut &nrm = NormOut());
 cudaError_t launch_recover_z(hdg_handle *h, const float2 *z2, const double *lam, double *u, double *hout);

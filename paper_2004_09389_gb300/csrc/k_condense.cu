@@ -11,20 +11,14 @@
 //   S_K = Mt_K + C_K X_B      (the cell's part of Eq. schur_system)
 //   W_K = C_K R_M             (step 1: g = sum_K P_K^T W_K r_K)
 // R_M and X_B serve step 3 (Eq. reconstruct_solution): q = R_M r - X_B lambda_K.
-// FP64 handles eliminate the velocity first, in function space (condense_nodal_kernel);
-// the two-float handles invert A_K in FP32 and refine (condense_mp_kernel), the momentum
-// rows scaled by H/g: the scaled A_K has the positive-definite symmetric part
-// diag((H/g) M, M + tau tau_s E) (the Coriolis and the tau H div coupling are skew after
-// scaling), so every leading minor is non-zero and no pivoting is needed.
+// The velocity is eliminated first, in function space, in FP64 (condense_nodal_kernel).
+// The two-float handles keep S_K, X_B and, instead of R_M and W_K, what their cell solve
+// takes: the h rows of R_M and the inverse of the velocity block (P and Q).
 #include "common.h"
-
-#include <cstdlib>
 
 namespace hdg {
 
 namespace {
-
-constexpr int kCondenseThreads = 128;
 
 template <int P>
 struct Sz {
@@ -32,109 +26,7 @@ struct Sz {
     static constexpr int NP = (P + 1) * (P + 2) / 2;
     static constexpr int NK = 3 * NP;
     static constexpr int M = 3 * PP;
-    static constexpr int LDA = NK + M + NK;
 };
-
-struct CondenseArgs {
-    int N;
-    double tau, g, H, tau_s;
-    const double *ref;      // packed reference matrices
-    const double *X;        // [N][3][2]
-    const double *fcell;    // [N][3]
-    double *Xb, *Rm, *W, *Scell;
-    int32_t *status;
-    float4 *Xb2, *Rm2, *W2;   // mixed-precision kernel: the float-pair copies, written directly
-};
-
-// The cell's system in shared memory: geometry (geo: detJ, J^-T, edge
-// lengths, outward normals), the vertex Coriolis values fK, the augmented rows
-// [D A | D B | D Mass] (Aug, NK x LDA; D the momentum-row scaling) and C (Cm,
-// M x NK).  Ends with a barrier.
-template <int P>
-__device__ __forceinline__ void cell_system(const CondenseArgs &a, int K, double *Aug, double *Cm, double *geo,
-                                            double *fK) {
-    using S = Sz<P>;
-    constexpr int NP = S::NP, NK = S::NK, M = S::M, PP = S::PP, LDA = S::LDA;
-    constexpr int oM = 0, oML = oM + NP * NP, oDxi = oML + 3 * NP * NP, oDeta = oDxi + NP * NP,
-                  oE = oDeta + NP * NP, oN = oE + 3 * NP * NP;
-    const int tid = threadIdx.x;
-    const double *ref = a.ref;
-    if (tid == 0) {
-        const double *x = a.X + size_t(K) * 6;
-        double J00 = x[2] - x[0], J01 = x[4] - x[0], J10 = x[3] - x[1], J11 = x[5] - x[1];
-        double det = J00 * J11 - J01 * J10;
-        geo[0] = det;
-        // Jit = J^-T
-        geo[1] = J11 / det;  geo[2] = -J10 / det;
-        geo[3] = -J01 / det; geo[4] = J00 / det;
-        for (int i = 0; i < 3; ++i) {
-            int v1 = (i + 1) % 3, v2 = (i + 2) % 3;
-            double tx = x[2 * v2] - x[2 * v1], ty = x[2 * v2 + 1] - x[2 * v1 + 1];
-            double l = sqrt(tx * tx + ty * ty);
-            geo[5 + i] = l;
-            geo[8 + 2 * i] = ty / l;       // outward normal of a counter-clockwise cell
-            geo[9 + 2 * i] = -tx / l;
-        }
-        for (int i = 0; i < 3; ++i) fK[i] = a.fcell[size_t(K) * 3 + i];
-    }
-    __syncthreads();
-    const double det = geo[0], j00 = geo[1], j01 = geo[2], j10 = geo[3], j11 = geo[4];
-    const double tau = a.tau, g = a.g, H = a.H, ts = a.tau_s, sH = H / g;
-
-    // ---- assemble [D A | D B | D Mass] and C
-    for (int idx = tid; idx < NK * LDA; idx += blockDim.x) {
-        const int rho = idx / LDA, col = idx % LDA;
-        const int R = rho / NP, ia = rho % NP;
-        double v = 0.0;
-        if (col < NK) {
-            const int Cc = col / NP, ib = col % NP;
-            const double Mab = det * ref[oM + ia * NP + ib];
-            if (R < 2) {
-                if (Cc == R) v = Mab;
-                else if (Cc < 2) {
-                    double mf = det * (fK[0] * ref[oML + ia * NP + ib] + fK[1] * ref[oML + NP * NP + ia * NP + ib] +
-                                       fK[2] * ref[oML + 2 * NP * NP + ia * NP + ib]);
-                    v = (R == 0 ? -tau : tau) * mf;
-                } else {
-                    // -tau g (h, d_x phi_a): D_x[b][a] = int phi_b d_x phi_a
-                    double dxi = ref[oDxi + ib * NP + ia], deta = ref[oDeta + ib * NP + ia];
-                    double d = (R == 0) ? det * (j00 * dxi + j01 * deta) : det * (j10 * dxi + j11 * deta);
-                    v = -tau * g * d;
-                }
-                v *= sH;
-            } else {
-                if (Cc < 2) {
-                    // tau H (d_x u_x, psi_a): D_x[a][b]
-                    double dxi = ref[oDxi + ia * NP + ib], deta = ref[oDeta + ia * NP + ib];
-                    double d = (Cc == 0) ? det * (j00 * dxi + j01 * deta) : det * (j10 * dxi + j11 * deta);
-                    v = tau * H * d;
-                } else {
-                    double e = 0.0;
-                    for (int i = 0; i < 3; ++i) e += geo[5 + i] * ref[oE + (i * NP + ia) * NP + ib];
-                    v = Mab + tau * ts * e;
-                }
-            }
-        } else if (col < NK + M) {
-            const int t = col - NK, i = t / PP, j = t % PP;
-            const double nl = geo[5 + i] * ref[oN + (i * NP + ia) * PP + j];
-            if (R == 0) v = tau * H * geo[8 + 2 * i] * nl;        // (H/g) tau g n_x <lambda, phi_a>
-            else if (R == 1) v = tau * H * geo[9 + 2 * i] * nl;
-            else v = -tau * ts * nl;
-        } else {
-            const int kap = col - NK - M, Cc = kap / NP, ib = kap % NP;
-            if (Cc == R) v = det * ref[oM + ia * NP + ib] * (R < 2 ? sH : 1.0);
-        }
-        Aug[idx] = v;
-    }
-    for (int idx = tid; idx < M * NK; idx += blockDim.x) {
-        const int t = idx / NK, kap = idx % NK;
-        const int i = t / PP, j = t % PP, Cc = kap / NP, ib = kap % NP;
-        const double nl = geo[5 + i] * ref[oN + (i * NP + ib) * PP + j];
-        Cm[idx] = (Cc == 0) ? H * geo[8 + 2 * i] * nl : (Cc == 1) ? H * geo[9 + 2 * i] * nl : ts * nl;
-    }
-    __syncthreads();
-
-}
 
 // ---------------------------------------------------------------- condensation in function space
 // Every cell matrix multiplied by M_K^-1, so that the cell equations act on
@@ -169,7 +61,9 @@ struct NodalArgs {
     const double *M1;       // [PP][PP] edge mass matrix
     const double *X;        // [N][3][2]
     const double *fcell;    // [N][3]
-    double *Xb, *Rm, *W, *Scell;
+    double *Xb, *Rm, *W, *Scell;       // FP64 handles (Scell: both)
+    float2 *Xb2, *Hr2, *lgeo;          // two-float handles: X_B, the h rows of R_M, the cell
+    float4 *PQ2;                       // weights and (f varying over a cell) P, Q
     int32_t *status;
 };
 
@@ -268,7 +162,7 @@ __device__ __forceinline__ void add_div(const double *ref, double g00, double g0
     });
 }
 
-// h = S^-1 rh and (wx, wy) -= T h, cell c of the block's matrices.  So non-null: S
+// h = S^-1 rh and (wx, wy) -= T h (Ts null: h alone), cell c of the block's matrices.  So non-null: S
 // itself, for one step of iterative refinement of h.  The explicit inverse alone
 // leaves S_K about 20 times less exact than an elimination of the whole cell system
 // (p = 3, Courant 16: S_K applied to a nearly constant trace off by 1e-12 instead of
@@ -304,6 +198,7 @@ __device__ __forceinline__ void back_substitute(const double *Ss, const double *
             h[i] = v;
         }
     }
+    if (!Ts) return;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
         row_fence();
@@ -351,7 +246,7 @@ struct CondSmem {
     static constexpr int oQ = oP + (FC ? 0 : NN * CC), total = oQ + (FC ? 0 : NN * CC);
 };
 
-template <int P, bool FC>
+template <int P, bool FC, bool FF>
 __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs a) {
     using L = CondSmem<P, FC>;
     constexpr int PP = P + 1, NP = L::NP, NK = 3 * NP, M = 3 * PP, CC = L::CC;
@@ -533,15 +428,51 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
         }
         add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
         back_substitute<NP, CC>(Ss, So, Ts, c, rh, wx, wy, h);
+        if constexpr (FF) {
+            constexpr int CPb = (M + 1) / 2;
 #pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            a.Xb[(size_t(i) * M + j) * N + K] = wx[i];
-            a.Xb[(size_t(NP + i) * M + j) * N + K] = wy[i];
-            a.Xb[(size_t(2 * NP + i) * M + j) * N + K] = h[i];
+            for (int i = 0; i < NP; ++i) {
+                const double v[3] = {wx[i], wy[i], h[i]};
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    a.Xb2[2 * ff_pair_index(size_t(K), size_t(q * NP + i) * CPb + j / 2, size_t(NK) * CPb) + j % 2] =
+                        split(v[q]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                a.Xb[(size_t(i) * M + j) * N + K] = wx[i];
+                a.Xb[(size_t(NP + i) * M + j) * N + K] = wy[i];
+                a.Xb[(size_t(2 * NP + i) * M + j) * N + K] = h[i];
+            }
         }
         c_rows<P>(m1, wn, wx, wy, h, e, jj, a.ts * det * geo[(6 + 3 * e) * CC + c], a.Scell + size_t(K) * M * M + j, M);
     }
-    // ---- R_M and W_K: the columns of the unit vectors in u_x, u_y and h
+    if constexpr (FF) {
+        // P and Q (f varying over the cell) as float pairs in cell tiles, and the cell's weights (k_ff.cu)
+        if constexpr (!FC) {
+            constexpr int CP = (NP + 1) / 2;
+            for (int idx = t; idx < 2 * NP * CP * CC; idx += kCondThreads) {
+                const int cc = idx % CC, pc = idx / CC, i = pc / CP, k0 = 2 * (pc % CP), Kc = blockIdx.x * CC + cc;
+                if (Kc >= a.N) continue;
+                const double *A = i < NP ? Ps + i * NP * CC : Qs + (i - NP) * NP * CC;
+                const float2 v0 = split(A[k0 * CC + cc]);
+                const float2 v1 = k0 + 1 < NP ? split(A[(k0 + 1) * CC + cc]) : make_float2(0.f, 0.f);
+                a.PQ2[ff_pair_index(size_t(Kc), size_t(pc), size_t(2) * NP * CP)] = make_float4(v0.x, v0.y, v1.x, v1.y);
+            }
+        }
+        if (cell && j == 0) {
+            const double jit[4] = {j00, j01, j10, j11};
+            float2 *o = a.lgeo + ff_pair_index(size_t(K), 0, kLGeo);
+            for (int q = 0; q < 4; ++q) o[size_t(q) * kFFCells] = split(tg * jit[q]);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) o[size_t(4 + q) * kFFCells] = split(wn[q / 3][q % 3]);
+            o[size_t(13) * kFFCells] = split(kap);
+            o[size_t(14) * kFFCells] = split(fk);
+        }
+    }
+    // ---- R_M and W_K (two-float handles: the h rows of R_M): the columns of the unit
+    // vectors in u_x, u_y and h
     if (on) {
 #pragma unroll 1
         for (int comp = 0; comp < 3; ++comp) {
@@ -561,8 +492,17 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                 rh[i] = comp == 2 && i == j ? 1.0 : 0.0;
             }
             if (comp < 2) add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
-            back_substitute<NP, CC>(Ss, nullptr, Ts, c, rh, wx, wy, h);
             const int kap_ = comp * NP + j;
+            if constexpr (FF) {
+                constexpr int CPk = (NK + 1) / 2;
+                back_substitute<NP, CC>(Ss, So, nullptr, c, rh, wx, wy, h);
+#pragma unroll
+                for (int i = 0; i < NP; ++i)
+                    a.Hr2[2 * ff_pair_index(size_t(K), size_t(i) * CPk + kap_ / 2, size_t(NP) * CPk) + kap_ % 2] =
+                        split(h[i]);
+                continue;
+            }
+            back_substitute<NP, CC>(Ss, nullptr, Ts, c, rh, wx, wy, h);
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
                 a.Rm[(size_t(i) * NK + kap_) * N + K] = wx[i];
@@ -571,176 +511,6 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
             }
             c_rows<P>(m1, wn, wx, wy, h, -1, 0, 0.0, a.W + size_t(kap_) * N + K, size_t(NK) * N);
         }
-    }
-}
-
-// ---------------------------------------------------------------- mixed-precision condensation
-// The same outputs for the mixed-precision handles, which use X_B, R_M, S_K
-// and W_K only as two-float pairs (and FP32 / BF16 copies): A_K is inverted in
-// FP32 (Gauss-Jordan in place, no pivoting, as above), X = A^-1 [B | Mass]
-// formed in FP32 and refined twice, each time with the residual
-// [B | Mass] - A X formed in two-float arithmetic (FFAcc) from the FP64 system
-// and the two-float X, and the correction A^-1 R added to X, kept as a
-// two-float pair.  S_K = Mt_K + C X_B and W_K = C R_M are formed in two-float
-// arithmetic too.  Each refinement step gains the factor ||I - Ainv A|| (about
-// cond(A_K) 2^-24) up to the two-float resolution (about 2^-48 relative):
-// two steps reach it for cells with a condition number well below 2^12.  No
-// FP64 product or elimination is left (GB300's FP32 rate is about 70 times its
-// FP64 rate), and with an explicit FP32 inverse every solve is a product, free
-// of the barrier per elimination step that triangular solves would take.
-// refinement steps (each costs about 60 % of the kernel's instructions)
-constexpr int kMpRefine = 2;
-
-template <int P>
-struct SzMp {
-    using S = Sz<P>;
-    static constexpr int NR = S::M + S::NK;                        // right-hand sides: B, Mass
-    static constexpr int oAi = S::NK * S::LDA + S::M * S::NK;      // in doubles: after Aug and Cm
-    static constexpr int nAi = (S::NK * S::NK + 1) / 2;            // FP32 inverse
-    static constexpr int oAp = oAi + nAi;                          // split A (float2 = one double each)
-    static constexpr int oXp = oAp + S::NK * S::NK;                // two-float X
-    static constexpr int oBp = oXp + S::NK * NR;                   // split right-hand sides
-    static constexpr int oRf = oBp + S::NK * NR;                   // FP32 residual
-    static constexpr int oFac = oRf + (S::NK * NR + 1) / 2;        // FP32 column factors
-    static constexpr int total = oFac + (S::NK + 1) / 2;           // doubles of dynamic shared memory
-};
-
-template <int P>
-__global__ void __launch_bounds__(kCondenseThreads) condense_mp_kernel(CondenseArgs a) {
-    using S = Sz<P>;
-    using Z = SzMp<P>;
-    constexpr int NP = S::NP, NK = S::NK, M = S::M, PP = S::PP, LDA = S::LDA, NR = Z::NR;
-    constexpr int oM1 = NP * NP + 3 * NP * NP + NP * NP + NP * NP + 3 * NP * NP + 3 * NP * PP;
-    extern __shared__ double smem[];
-    double *Aug = smem;                                            // [NK][LDA]
-    double *Cm = Aug + NK * LDA;                                   // [M][NK]
-    float *Ai = reinterpret_cast<float *>(smem + Z::oAi);          // [NK][NK] FP32 inverse
-    float2 *Ap = reinterpret_cast<float2 *>(smem + Z::oAp);        // [NK][NK] split A; later split C
-    float2 *Xp = reinterpret_cast<float2 *>(smem + Z::oXp);        // [NK][NR] two-float X
-    float2 *Bp = reinterpret_cast<float2 *>(smem + Z::oBp);        // [NK][NR] split [B | Mass]
-    float *Rf = reinterpret_cast<float *>(smem + Z::oRf);          // [NK][NR]
-    float *fac = reinterpret_cast<float *>(smem + Z::oFac);        // [NK]
-    __shared__ double geo[16];
-    __shared__ double fK[3];
-    __shared__ int bad;
-
-    const int K = blockIdx.x;
-    const int tid = threadIdx.x;
-    const double *ref = a.ref;
-    const double ts = a.tau_s;
-    if (tid == 0) bad = 0;
-    cell_system<P>(a, K, Aug, Cm, geo, fK);
-
-    for (int idx = tid; idx < NK * NK; idx += blockDim.x) {
-        const float2 v = split(Aug[(idx / NK) * LDA + idx % NK]);
-        Ap[idx] = v;
-        Ai[idx] = v.x;
-    }
-    __syncthreads();
-    // ---- FP32 inverse in place: step k scales row k (its pivot entry becomes
-    // 1 / pivot) and records column k, then eliminates column k from the other
-    // rows (their column-k entries become -a_ik / pivot)
-    for (int k = 0; k < NK; ++k) {
-        const float piv = Ai[k * NK + k];
-        if (tid == 0 && !(fabsf(piv) > 1e-30f)) bad = 1;
-        const float pinv = 1.0f / piv;
-        for (int i = tid; i < NK; i += blockDim.x) fac[i] = Ai[i * NK + k];
-        __syncthreads();
-        for (int c = tid; c < NK; c += blockDim.x) Ai[k * NK + c] = (c == k) ? pinv : Ai[k * NK + c] * pinv;
-        __syncthreads();
-        for (int idx = tid; idx < NK * NK; idx += blockDim.x) {
-            const int i = idx / NK, c = idx % NK;
-            if (i == k) continue;
-            Ai[idx] = (c == k) ? -fac[i] * pinv : fmaf(-fac[i], Ai[k * NK + c], Ai[idx]);
-        }
-        __syncthreads();
-    }
-    if (bad) {
-        if (tid == 0) atomicOr(a.status, 1);
-        return;
-    }
-    // ---- X_0 = Ainv [B | Mass] in FP32, then the refinement steps
-    for (int idx = tid; idx < NK * NR; idx += blockDim.x) {
-        const float2 v = split(Aug[(idx / NR) * LDA + NK + idx % NR]);
-        Bp[idx] = v;
-        Rf[idx] = v.x;
-    }
-    __syncthreads();
-    for (int idx = tid; idx < NK * NR; idx += blockDim.x) {
-        const int i = idx / NR, c = idx % NR;
-        float x = 0.0f;
-#pragma unroll 6
-        for (int j = 0; j < NK; ++j) x = fmaf(Ai[i * NK + j], Rf[j * NR + c], x);
-        Xp[idx] = make_float2(x, 0.0f);
-    }
-    __syncthreads();
-    for (int it = 0; it < kMpRefine; ++it) {
-        for (int idx = tid; idx < NK * NR; idx += blockDim.x) {
-            const int r = idx / NR, c = idx % NR;
-            FFAcc acc;
-#pragma unroll 5
-            for (int j = 0; j < NK; ++j) acc.add(Ap[r * NK + j], Xp[j * NR + c]);
-            // r = b - A X to FP32 accuracy: the leading parts nearly cancel exactly
-            const float2 bv = Bp[idx];
-            Rf[idx] = __fadd_rn(__fsub_rn(bv.x, acc.s), __fsub_rn(bv.y, acc.c));
-        }
-        __syncthreads();
-        for (int idx = tid; idx < NK * NR; idx += blockDim.x) {
-            const int i = idx / NR, c = idx % NR;
-            float d = 0.0f;
-#pragma unroll 6
-            for (int j = 0; j < NK; ++j) d = fmaf(Ai[i * NK + j], Rf[j * NR + c], d);
-            // (hi, lo) + d: TwoSum of the leading parts, then renormalise
-            const float2 x = Xp[idx];
-            const float s1 = __fadd_rn(x.x, d);
-            const float bp = __fsub_rn(s1, x.x);
-            const float e = __fadd_rn(__fsub_rn(x.x, __fsub_rn(s1, bp)), __fsub_rn(d, bp));
-            const float lo = __fadd_rn(x.y, e);
-            const float hi = __fadd_rn(s1, lo);
-            Xp[idx] = make_float2(hi, __fsub_rn(lo, __fsub_rn(hi, s1)));
-        }
-        __syncthreads();
-    }
-    // ---- outputs: X_B, R_M and W_K as float pairs in the cell tiles of the
-    // two-float kernels, S_K in FP64 (C split into the space of the split A)
-    float2 *Cp = Ap;
-    for (int idx = tid; idx < M * NK; idx += blockDim.x) Cp[idx] = split(Cm[idx]);
-    __syncthreads();
-    {
-        constexpr int CPb = (M + 1) / 2, CPr = (NK + 1) / 2;
-        for (int idx = tid; idx < NK * CPb; idx += blockDim.x) {
-            const int rho = idx / CPb, c0 = 2 * (idx % CPb);
-            const float2 x0 = Xp[rho * NR + c0];
-            const float2 x1 = c0 + 1 < M ? Xp[rho * NR + c0 + 1] : make_float2(0.f, 0.f);
-            a.Xb2[ff_pair_index(size_t(K), size_t(idx), size_t(NK) * CPb)] = make_float4(x0.x, x0.y, x1.x, x1.y);
-        }
-        for (int idx = tid; idx < NK * CPr; idx += blockDim.x) {
-            const int rho = idx / CPr, c0 = 2 * (idx % CPr);
-            const float2 x0 = Xp[rho * NR + M + c0];
-            const float2 x1 = c0 + 1 < NK ? Xp[rho * NR + M + c0 + 1] : make_float2(0.f, 0.f);
-            a.Rm2[ff_pair_index(size_t(K), size_t(idx), size_t(NK) * CPr)] = make_float4(x0.x, x0.y, x1.x, x1.y);
-        }
-        // W_K = C R_M: each pair of columns from two two-float sums, renormalised
-        for (int idx = tid; idx < M * CPr; idx += blockDim.x) {
-            const int t = idx / CPr, c0 = 2 * (idx % CPr);
-            float v[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int q = 0; q < 2 && c0 + q < NK; ++q) {
-                FFAcc acc;
-                for (int r = 0; r < NK; ++r) acc.add(Cp[t * NK + r], Xp[r * NR + M + c0 + q]);
-                const float hi = __fadd_rn(acc.s, acc.c);
-                v[2 * q] = hi;
-                v[2 * q + 1] = __fsub_rn(acc.c, __fsub_rn(hi, acc.s));
-            }
-            a.W2[ff_pair_index(size_t(K), size_t(idx), size_t(M) * CPr)] = make_float4(v[0], v[1], v[2], v[3]);
-        }
-    }
-    for (int idx = tid; idx < M * M; idx += blockDim.x) {
-        const int t = idx / M, t2 = idx % M;
-        FFAcc acc;
-        for (int kap = 0; kap < NK; ++kap) acc.add(Cp[t * NK + kap], Xp[kap * NR + t2]);
-        double v = acc.value();
-        if (t / PP == t2 / PP) v += ts * geo[5 + t / PP] * ref[oM1 + (t % PP) * PP + (t2 % PP)];
-        a.Scell[size_t(K) * M * M + idx] = v;
     }
 }
 
@@ -994,39 +764,24 @@ __global__ void to_f32_kernel(const double *x, float *y, size_t n) {
     if (i < n) y[i] = float(x[i]);
 }
 
-template <int P, bool FC>
+template <int P, bool FC, bool FF>
 cudaError_t condense_nodal_p(hdg_handle *h) {
     constexpr size_t smem = sizeof(double) * CondSmem<P, FC>::total;
-    auto k = &condense_nodal_kernel<P, FC>;
+    auto k = &condense_nodal_kernel<P, FC, FF>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     NodalArgs a;
     a.N = h->N; a.tau = h->prm.tau; a.g = h->prm.g; a.H = h->prm.H; a.ts = h->tau_s;
     a.nref = h->d_nref; a.M1 = h->d_ref + ref_offsets(P).M1; a.X = h->d_X; a.fcell = h->d_fcell;
     a.Xb = h->d_Xb; a.Rm = h->d_Rm; a.W = h->d_W; a.Scell = h->d_Scell; a.status = h->d_status;
+    a.Xb2 = h->d_Xb2; a.Hr2 = h->d_Hr2; a.lgeo = h->d_lgeo; a.PQ2 = reinterpret_cast<float4 *>(h->d_PQ2);
     k<<<(h->N + kCondCells<P> - 1) / kCondCells<P>, kCondThreads, smem, h->stream>>>(a);
     return cudaGetLastError();
 }
 template <int P>
 cudaError_t condense_p(hdg_handle *h) {
-    return h->f_const ? condense_nodal_p<P, true>(h) : condense_nodal_p<P, false>(h);
-}
-
-template <int P>
-cudaError_t condense_mp_p(hdg_handle *h) {
-    const size_t smem = sizeof(double) * SzMp<P>::total;
-    cudaError_t e = cudaFuncSetAttribute(condense_mp_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    CondenseArgs a;
-    a.N = h->N; a.tau = h->prm.tau; a.g = h->prm.g; a.H = h->prm.H; a.tau_s = h->tau_s;
-    a.ref = h->d_ref; a.X = h->d_X; a.fcell = h->d_fcell;
-    a.Xb = h->d_Xb; a.Rm = h->d_Rm; a.W = h->d_W; a.Scell = h->d_Scell; a.status = h->d_status;
-    a.Xb2 = reinterpret_cast<float4 *>(h->d_Xb2);
-    a.Rm2 = reinterpret_cast<float4 *>(h->d_Rm2);
-    a.W2 = reinterpret_cast<float4 *>(h->d_W2);
-    if (!a.Xb2 || !a.Rm2 || !a.W2) return cudaErrorInvalidValue;
-    condense_mp_kernel<P><<<h->N, kCondenseThreads, smem, h->stream>>>(a);
-    return cudaGetLastError();
+    if (mode_ff(h->prm)) return h->f_const ? condense_nodal_p<P, true, true>(h) : condense_nodal_p<P, false, true>(h);
+    return h->f_const ? condense_nodal_p<P, true, false>(h) : condense_nodal_p<P, false, false>(h);
 }
 
 template <int P>
@@ -1041,31 +796,7 @@ cudaError_t assemble_p(hdg_handle *h) {
 
 }  // namespace
 
-namespace {
-// HDG_CONDENSE_FP64=1: the FP64 elimination for the mixed handles too (read once)
-bool force_fp64_condense() {
-    static const bool on = [] {
-        const char *e = std::getenv("HDG_CONDENSE_FP64");
-        return e && e[0] == '1';
-    }();
-    return on;
-}
-}  // namespace
-
-bool condense_writes_pairs(const hdg_handle *h) { return mode_ff(h->prm) && !force_fp64_condense(); }
-
 cudaError_t launch_condense(hdg_handle *h) {
-    // mixed-precision handles: FP32 inverse with two-float refinement, writing
-    // the float-pair matrices directly
-    if (condense_writes_pairs(h)) {
-        switch (h->p) {
-            case 1: return condense_mp_p<1>(h);
-            case 2: return condense_mp_p<2>(h);
-            case 3: return condense_mp_p<3>(h);
-            case 4: return condense_mp_p<4>(h);
-        }
-        return cudaErrorInvalidValue;
-    }
     switch (h->p) {
         case 1: return condense_p<1>(h);
         case 2: return condense_p<2>(h);

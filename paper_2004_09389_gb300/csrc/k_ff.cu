@@ -41,26 +41,6 @@ __global__ void split_kernel(const double *__restrict__ a, float2 *__restrict__ 
     if (i < n) out[i] = split(a[i]);
 }
 
-// A per-cell matrix a[(row * cols + col) * N + K] split into pairs of
-// consecutive row entries, in tiles of kCells cells: the pair (col 2cp, col
-// 2cp + 1, or zeros past the row's end) of plane pc = row * CP + cp, CP =
-// (cols + 1) / 2, for cell K sits at out[((K / kCells) * rows * CP + pc) *
-// kCells + K % kCells].  One 16-byte load per lane brings two entries of a row,
-// a warp's loads are coalesced, and a block of kCells cells streams one
-// contiguous tile.
-__global__ void split_pairs_kernel(const double *__restrict__ a, float4 *__restrict__ out, int rows, int cols,
-                                   size_t N) {
-    const int CP = (cols + 1) / 2;
-    const size_t np = size_t(rows) * CP;
-    const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= np * N) return;
-    const size_t K = i % N, pc = i / N;
-    const int row = int(pc / CP), c0 = 2 * int(pc % CP);
-    const float2 lo = split(a[(size_t(row) * cols + c0) * N + K]);
-    const float2 hi = c0 + 1 < cols ? split(a[(size_t(row) * cols + c0 + 1) * N + K]) : make_float2(0.f, 0.f);
-    out[ff_pair_index(K, pc, np)] = make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-
 // acc += sum over the NCOL entries of one row (pairs p[cp * kCells], cp <
 // (NCOL + 1) / 2, within the cell's tile) times x[col][lane], in column order
 template <int NCOL>
@@ -510,98 +490,208 @@ __device__ __forceinline__ float2 ff_mul(const float2 a, const float2 b) {
     return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, p)));
 }
 
-// Step 1 of a solve, keeping what step 3 needs: z_K = R_M r_K (= A_K^-1
-// Mass_K r_K, the cell solution for lambda = 0) in two-float arithmetic, stored
-// as normalised pairs (z2 [NK][N], when given), and the cell rows ycell =
-// C_K z_K (= W_K r_K) formed from the cell's geometry instead of a stored
-// W_K.  Row (i, j) of C_K (edge i, trace node j) is sum_b N_ibj (H t_y z_u[b]
-// - H t_x z_v[b] + tau_s |e_i| z_h[b]) with t the edge vector and N_ibj =
-// int_e phi_b mu_j, nonzero only for the cell nodes b on the edge: cgeo holds
-// the pairs of H t_y, -H t_x, tau_s |e_i| per cell and edge ([N][3][3]), ctab_b
-// / ctab_v the nodes and pairs of N per row ([3(p+1)][p+1]).  The block's 32
-// cells are the lanes; the eight warps take the rows of R_M in turn, then the
-// rows of C_K.
+// ---------------------------------------------------------------- the cell solve
+// q = A_K^-1 M_K v for 32 cells per block (lane = cell), v in function space: the h rows
+// of the stored R_M = A_K^-1 M_K, then the velocity from the momentum equations,
+//   h = (R_M v)_h,   u = R (v_u - tau g G h),
+// with the weak gradient G by reference matrices shared by all cells in the cell's J^-T,
+// and R two n_p x n_p matrices (P, Q) or, where f is constant on every cell (FC), two
+// numbers.  A cell reads 3 n_p^2 pairs (FC) or 5 n_p^2 instead of the 9 n_p^2 of R_M,
+// with about as many products.  Only h is taken from a stored inverse on purpose:
+// eliminating the velocity in two-float arithmetic as well (S^-1 (v_h - tau H div R v_u),
+// n_p^2 pairs) reads less still, but the cancellation in that sum is amplified twice by
+// the derivatives: 1.8e-12 instead of 1e-14 relative at p = 3, Courant 8.
+// The warps take the rows in turn (kSolveWarps divides n_p).  sV holds v as pairs on
+// entry and q on return (rows u_x, u_y, h; [33]: no bank conflicts); ends with a barrier.
+template <int P> constexpr int kSolveWarps = P == 1 ? 3 : P == 2 ? 6 : 5;
+
+__device__ __forceinline__ float2 ff_pair(const FFAcc &a) {
+    const float hi = __fadd_rn(a.s, a.c);
+    return make_float2(hi, __fsub_rn(a.c, __fsub_rn(hi, a.s)));
+}
+__device__ __forceinline__ float2 ff_neg(const float2 a) { return make_float2(-a.x, -a.y); }
+
+struct SolveMat {
+    const float4 *Hr2, *PQ2;    // tiles of the condensation
+    const float2 *lgeo;
+    const float4 *tab;          // FFTabOffsets
+};
+
+template <int P, bool FC>
+__device__ __forceinline__ void cell_solve(const SolveMat &m, int tile, bool on, const float4 *tab,
+                                           float2 (*sV)[kCellsPad]) {
+    constexpr int NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, CP = (NP + 1) / 2, KP = (NK + 1) / 2;
+    constexpr int NW = kSolveWarps<P>, RW = NP / NW;
+    constexpr FFTabOffsets O = ff_tab_offsets(P);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float2 *geo = m.lgeo + size_t(tile) * kLGeo * kCells + lane;
+    const float4 *Hr = m.Hr2 + size_t(tile) * NP * KP * kCells + lane;
+    const float4 *PQ = FC ? nullptr : m.PQ2 + size_t(tile) * 2 * NP * CP * kCells + lane;
+    // padding cells of the last tile have no matrices: their lanes keep zeros
+    float2 hv[RW];
+#pragma unroll
+    for (int u = 0; u < RW; ++u) {
+        FFAcc acc;
+        if (on) row_pairs<NK>(acc, Hr + size_t(w + u * NW) * KP * kCells, sV, lane);
+        hv[u] = ff_pair(acc);
+    }
+    __syncthreads();                            // every warp has read v
+#pragma unroll
+    for (int u = 0; u < RW; ++u) sV[2 * NP + w + u * NW][lane] = hv[u];
+    __syncthreads();
+    // v_u - tau g G h
+    if (on) {
+        const float2 j00 = __ldg(geo), j01 = __ldg(geo + kCells), j10 = __ldg(geo + 2 * kCells),
+                     j11 = __ldg(geo + 3 * kCells);
+#pragma unroll
+        for (int u = 0; u < RW; ++u) {
+            const int i = w + u * NW;
+            FFAcc g1, g2;
+#pragma unroll 5
+            for (int k = 0; k < NP; ++k) {
+                const float4 d = tab[O.W + i * NP + k];
+                const float2 h = sV[2 * NP + k][lane];
+                g1.add(make_float2(d.x, d.y), h);
+                g2.add(make_float2(d.z, d.w), h);
+            }
+            const float2 a1 = ff_neg(ff_pair(g1)), a2 = ff_neg(ff_pair(g2));
+            const float2 vx = sV[i][lane], vy = sV[NP + i][lane];
+            FFAcc x, y;
+            x.s = vx.x;
+            x.c = vx.y;
+            x.add(j00, a1);
+            x.add(j01, a2);
+            y.s = vy.x;
+            y.c = vy.y;
+            y.add(j10, a1);
+            y.add(j11, a2);
+            float2 px = ff_pair(x), py = ff_pair(y);
+            if constexpr (FC) {
+                const float2 kap = __ldg(geo + 13 * kCells), fk = __ldg(geo + 14 * kCells);
+                FFAcc ax, ay;
+                ax.add(kap, px);
+                ax.add(fk, py);
+                ay.add(kap, py);
+                ay.add(ff_neg(fk), px);
+                px = ff_pair(ax);
+                py = ff_pair(ay);
+            }
+            sV[i][lane] = px;
+            sV[NP + i][lane] = py;
+        }
+    }
+    __syncthreads();
+    if constexpr (!FC) {
+        // u = R (...): rows P x + Q y and P y - Q x
+        float2 ux[RW], uy[RW];
+#pragma unroll
+        for (int u = 0; u < RW; ++u) {
+            const int i = w + u * NW;
+            FFAcc ax, ay;
+            if (on) {
+#pragma unroll 2
+                for (int cp = 0; cp < CP; ++cp) {
+                    const float4 p = __ldg(PQ + size_t(i * CP + cp) * kCells);
+                    const float4 q = __ldg(PQ + size_t((NP + i) * CP + cp) * kCells);
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) {
+                        const int k = 2 * cp + g;
+                        if (k >= NP) break;
+                        const float2 pk = g ? make_float2(p.z, p.w) : make_float2(p.x, p.y);
+                        const float2 qk = g ? make_float2(q.z, q.w) : make_float2(q.x, q.y);
+                        const float2 x = sV[k][lane], y = sV[NP + k][lane];
+                        ax.add(pk, x);
+                        ax.add(qk, y);
+                        ay.add(pk, y);
+                        ay.add(ff_neg(qk), x);
+                    }
+                }
+            }
+            ux[u] = ff_pair(ax);
+            uy[u] = ff_pair(ay);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < RW; ++u) {
+            sV[w + u * NW][lane] = ux[u];
+            sV[NP + w + u * NW][lane] = uy[u];
+        }
+        __syncthreads();
+    }
+}
+
+// the cell solve's tables into shared memory (no barrier)
 template <int P>
-__device__ __forceinline__ void rhs_cell_z_kernel_impl(int bid_, int nb_, int N, const float4 *__restrict__ Rm2,
-                                                       const float2 *__restrict__ cgeo,
-                                                       const int32_t *__restrict__ ctab_b,
-                                                       const float2 *__restrict__ ctab_v,
+__device__ __forceinline__ void stage_tab(float4 *tab, const float4 *src) {
+    for (int k = threadIdx.x; k < ff_tab_offsets(P).total; k += blockDim.x) tab[k] = __ldg(src + k);
+}
+
+// Step 1: z_K = A_K^-1 M_K r_K by the cell solve, stored as normalised pairs (z2
+// [NK][N], when given) for step 3, and the cell rows ycell = C_K z_K: on edge i the
+// flux H t_y u_x - H t_x u_y + tau_s |e| h at its p + 1 cell nodes, times the edge mass
+// matrix.  Bound by HBM and FP32 issue together: 98 us on 131,072 cells at p = 3 with f
+// constant per cell (430 MB, 4.4 TB/s), 118 us on 327,680 at p = 2 with f varying,
+// against 188 and 178 us with the rows of the stored A_K^-1 M_K (1,029 MB, HBM-bound).
+template <int P, bool FC>
+__device__ __forceinline__ void rhs_cell_z_kernel_impl(int bid_, int nb_, int N, const SolveMat &m,
                                                        const double *__restrict__ r_u,
                                                        const double *__restrict__ r_h, double *__restrict__ ycell,
                                                        float2 *__restrict__ z2, double *__restrict__ cu,
                                                        double *__restrict__ ch) {
-    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP, NW = 8;
-    constexpr int KP = (NK + 1) / 2, RW = (NK + NW - 1) / NW;
-    __shared__ float2 sIn[NK][kCellsPad];      // r_K, then z_K
-    __shared__ int32_t tb[M][PP];
-    __shared__ float2 tv[M][PP];
-    for (int t = threadIdx.x; t < M * PP; t += blockDim.x) {
-        tb[t / PP][t % PP] = ctab_b[t];
-        tv[t / PP][t % PP] = ctab_v[t];
-    }
+    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP, NW = kSolveWarps<P>;
+    constexpr FFTabOffsets O = ff_tab_offsets(P);
+    __shared__ float2 sV[NK][kCellsPad];
+    __shared__ float2 sC[M][kCellsPad];        // edge fluxes
+    __shared__ float4 tab[O.total];
     const int K0 = bid_ * kCells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    stage_cell_rhs<NP>(N, K0, r_u, r_h, sIn, cu, ch);
-    __syncthreads();
+    stage_tab<P>(tab, m.tab);
+    stage_cell_rhs<NP>(N, K0, r_u, r_h, sV, cu, ch);
     const int K = K0 + lane;
     const bool on = K < N;
-    float2 zr[RW];
-#pragma unroll
-    for (int u = 0; u < RW; ++u) {
-        const int rho = w + u * NW;
-        zr[u] = make_float2(0.0f, 0.0f);
-        if (on && rho < NK) {
-            FFAcc acc;
-            row_pairs<NK>(acc, Rm2 + (size_t(bid_) * NK * KP + size_t(rho) * KP) * kCells + lane, sIn, lane);
-            const float hi = __fadd_rn(acc.s, acc.c);
-            zr[u] = make_float2(hi, __fsub_rn(acc.c, __fsub_rn(hi, acc.s)));
+    if (!on)
+        for (int q = w; q < NK; q += NW) sV[q][lane] = make_float2(0.f, 0.f);
+    __syncthreads();
+    cell_solve<P, FC>(m, bid_, on, tab, sV);
+    if (z2 && on)
+        for (int q = w; q < NK; q += NW) z2[size_t(q) * N + K] = sV[q][lane];
+    const float2 *geo = m.lgeo + size_t(bid_) * kLGeo * kCells + lane;
+    for (int t = w; t < M; t += NW) {
+        const int i = t / PP, b = edge_cell_node(P, i, t % PP);
+        FFAcc acc;
+        if (on) {
+            acc.add(__ldg(geo + (4 + 3 * i) * kCells), sV[b][lane]);
+            acc.add(__ldg(geo + (5 + 3 * i) * kCells), sV[NP + b][lane]);
+            acc.add(__ldg(geo + (6 + 3 * i) * kCells), sV[2 * NP + b][lane]);
         }
-    }
-    __syncthreads();                            // every warp has read r_K
-#pragma unroll
-    for (int u = 0; u < RW; ++u) {
-        const int rho = w + u * NW;
-        if (rho < NK) {
-            sIn[rho][lane] = zr[u];
-            if (z2 && on) z2[size_t(rho) * N + K] = zr[u];
-        }
+        sC[t][lane] = ff_pair(acc);
     }
     __syncthreads();
     if (!on) return;
     for (int t = w; t < M; t += NW) {
-        const float2 *gc = cgeo + (size_t(K) * 3 + t / PP) * 3;
-        const float2 g0 = gc[0], g1 = gc[1], g2 = gc[2];
+        const int i = t / PP, jj = t % PP;
         FFAcc acc;
 #pragma unroll
-        for (int q = 0; q < PP; ++q) {
-            const int b = tb[t][q];
-            const float2 v = tv[t][q];
-            acc.add(ff_mul(v, g0), sIn[b][lane]);
-            acc.add(ff_mul(v, g1), sIn[NP + b][lane]);
-            acc.add(ff_mul(v, g2), sIn[2 * NP + b][lane]);
+        for (int jb = 0; jb < PP; ++jb) {
+            const float4 v = tab[O.m1 + jb * PP + jj];
+            acc.add(make_float2(v.x, v.y), sC[i * PP + jb][lane]);
         }
         ycell[size_t(t) * N + K] = acc.value();
     }
 }
-template <int P>
-__global__ void __launch_bounds__(256) rhs_cell_z_kernel(int N, const float4 *__restrict__ Rm2,
-                                                         const float2 *__restrict__ cgeo,
-                                                         const int32_t *__restrict__ ctab_b,
-                                                         const float2 *__restrict__ ctab_v,
+template <int P, bool FC>
+__global__ void __launch_bounds__(32 * kSolveWarps<P>) rhs_cell_z_kernel(int N, const SolveMat m,
                                                          const double *__restrict__ r_u,
                                                          const double *__restrict__ r_h, double *__restrict__ ycell,
                                                          float2 *__restrict__ z2, double *__restrict__ cu,
                                                          double *__restrict__ ch) {
     pdl_wait();
-    rhs_cell_z_kernel_impl<P>(blockIdx.x, gridDim.x, N, Rm2, cgeo, ctab_b, ctab_v, r_u, r_h, ycell, z2, cu, ch);
+    rhs_cell_z_kernel_impl<P, FC>(blockIdx.x, gridDim.x, N, m, r_u, r_h, ycell, z2, cu, ch);
 }
-template <int P>
+template <int P, bool FC>
 struct rhs_cell_z_kernel_args {
     int nb_;
     int N;
-    const float4 *Rm2;
-    const float2 *cgeo;
-    const int32_t *ctab_b;
-    const float2 *ctab_v;
+    SolveMat m;
     const double *r_u;
     const double *r_h;
     double *ycell;
@@ -609,144 +699,93 @@ struct rhs_cell_z_kernel_args {
     double *cu;
     double *ch;
 };
-template <int P>
-__global__ void __launch_bounds__(256) rhs_cell_z_kernel_multi(const __grid_constant__ MultiP<rhs_cell_z_kernel_args<P>> M) {
+template <int P, bool FC>
+__global__ void __launch_bounds__(32 * kSolveWarps<P>) rhs_cell_z_kernel_multi(const __grid_constant__ MultiP<rhs_cell_z_kernel_args<P, FC>> M) {
     pdl_wait();
     int b_;
-    const rhs_cell_z_kernel_args<P> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    rhs_cell_z_kernel_impl<P>(b_, q_.nb_, q_.N, q_.Rm2, q_.cgeo, q_.ctab_b, q_.ctab_v, q_.r_u, q_.r_h, q_.ycell, q_.z2,
-                              q_.cu, q_.ch);
+    const rhs_cell_z_kernel_args<P, FC> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    rhs_cell_z_kernel_impl<P, FC>(b_, q_.nb_, q_.N, q_.m, q_.r_u, q_.r_h, q_.ycell, q_.z2, q_.cu, q_.ch);
 }
-template <int P>
-void rhs_cell_z_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int N, const float4 *Rm2,
-                          const float2 *cgeo, const int32_t *ctab_b, const float2 *ctab_v, const double *r_u,
-                          const double *r_h, double *ycell, float2 *z2, double *cu, double *ch) {
+template <int P, bool FC>
+void rhs_cell_z_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int N, const SolveMat &m,
+                          const double *r_u, const double *r_h, double *ycell, float2 *z2, double *cu, double *ch) {
     if (Recorder *r_ = batch_recorder()) {
-        rhs_cell_z_kernel_args<P> q_;
+        rhs_cell_z_kernel_args<P, FC> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
         q_.N = N;
-        q_.Rm2 = Rm2;
-        q_.cgeo = cgeo;
-        q_.ctab_b = ctab_b;
-        q_.ctab_v = ctab_v;
+        q_.m = m;
         q_.r_u = r_u;
         q_.r_h = r_h;
         q_.ycell = ycell;
         q_.z2 = z2;
         q_.cu = cu;
         q_.ch = ch;
-        batch_record(r_, reinterpret_cast<const void *>(&rhs_cell_z_kernel_multi<P>), q_, grid_, block_, smem_,
+        batch_record(r_, reinterpret_cast<const void *>(&rhs_cell_z_kernel_multi<P, FC>), q_, grid_, block_, smem_,
                      kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &rhs_cell_z_kernel<P>, grid_, block_, smem_, s_, N, Rm2, cgeo, ctab_b, ctab_v, r_u, r_h,
-               ycell, z2, cu, ch);
+    pdl_launch(kPdlFamily, &rhs_cell_z_kernel<P, FC>, grid_, block_, smem_, s_, N, m, r_u, r_h, ycell, z2, cu, ch);
 }
 
-// step 1, cell part: ycell[t][K] = sum_kappa W[t*NK + kappa][K] r_K[kappa]
+// lambda on the block's cells (the pairs of its three facets' nodes in the cell's order)
 template <int P>
-__device__ __forceinline__ void rhs_cell_ff_kernel_impl(int bid_, int nb_, int N, const float4 *__restrict__ W2,
-                                                        const double *__restrict__ r_u,
-                                                        const double *__restrict__ r_h, double *__restrict__ ycell,
-                                                        double *__restrict__ cu, double *__restrict__ ch) {
-    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP, NW = 4;
-    constexpr int KP = (NK + 1) / 2;
-    __shared__ float2 sIn[NK][kCellsPad];
-    const int K0 = bid_ * kCells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    stage_cell_rhs<NP>(N, K0, r_u, r_h, sIn, cu, ch);
-    __syncthreads();
-    const int K = K0 + lane;
-    if (K >= N) return;
-    for (int t = w; t < M; t += NW) {
-        FFAcc acc;
-        row_pairs<NK>(acc, W2 + (size_t(bid_) * M * KP + size_t(t) * KP) * kCells + lane, sIn, lane);
-        ycell[size_t(t) * N + K] = acc.value();
+__device__ __forceinline__ void stage_cell_trace(int N, int NF, int K0, const double *__restrict__ lam,
+                                                 const int32_t *__restrict__ facet_of,
+                                                 const int32_t *__restrict__ flip, float2 (*sL)[kCellsPad]) {
+    constexpr int PP = P + 1, M = 3 * PP;
+    const int nc = min(kCells, N - K0);
+    for (int j = threadIdx.x; j < nc * M; j += blockDim.x) {
+        const int cell = j / M, q = j % M, i = q / PP, jj = q % PP, K = K0 + cell;
+        const int f = facet_of[3 * K + i], fl = flip[3 * K + i];
+        sL[q][cell] = split(lam[size_t(fl ? P - jj : jj) * NF + f]);
     }
 }
-template <int P>
-__global__ void __launch_bounds__(128, 8) rhs_cell_ff_kernel(int N, const float4 *__restrict__ W2,
-                                                             const double *__restrict__ r_u,
-                                                             const double *__restrict__ r_h,
-                                                             double *__restrict__ ycell, double *__restrict__ cu,
-                                                             double *__restrict__ ch) {
-    pdl_wait();
-    rhs_cell_ff_kernel_impl<P>(blockIdx.x, gridDim.x, N, W2, r_u, r_h, ycell, cu, ch);
-}
-template <int P>
-struct rhs_cell_ff_kernel_args {
-    int nb_;
-    int N;
-    const float4 *W2;
-    const double *r_u;
-    const double *r_h;
-    double *ycell;
-    double *cu;
-    double *ch;
-};
-template <int P>
-__global__ void __launch_bounds__(128, 8) rhs_cell_ff_kernel_multi(const __grid_constant__ MultiP<rhs_cell_ff_kernel_args<P>> M) {
-    pdl_wait();
-    int b_;
-    const rhs_cell_ff_kernel_args<P> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    rhs_cell_ff_kernel_impl<P>(b_, q_.nb_, q_.N, q_.W2, q_.r_u, q_.r_h, q_.ycell, q_.cu, q_.ch);
-}
-template <int P>
-void rhs_cell_ff_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int N, const float4 *W2,
-                           const double *r_u, const double *r_h, double *ycell, double *cu, double *ch) {
-    if (Recorder *r_ = batch_recorder()) {
-        rhs_cell_ff_kernel_args<P> q_;
-        std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
-        q_.nb_ = int(grid_);
-        q_.N = N;
-        q_.W2 = W2;
-        q_.r_u = r_u;
-        q_.r_h = r_h;
-        q_.ycell = ycell;
-        q_.cu = cu;
-        q_.ch = ch;
-        batch_record(r_, reinterpret_cast<const void *>(&rhs_cell_ff_kernel_multi<P>), q_, grid_, block_, smem_, kPdlFamily);
-        return;
-    }
-    pdl_launch(kPdlFamily, &rhs_cell_ff_kernel<P>, grid_, block_, smem_, s_, N, W2, r_u, r_h, ycell, cu, ch);
-}
 
-
-// step 3: q_K = R_M r_K - X_B lambda_K, written in the caller's u / h layout
-template <int P>
-__global__ void __launch_bounds__(256) recover_ff_kernel(int N, int NF, const float4 *__restrict__ Rm2,
+// Step 3 from explicit right-hand sides: q_K = A_K^-1 M_K r_K - X_B lambda_K, the cell
+// solve of r and the stored X_B, written in the caller's u / h layout
+template <int P, bool FC>
+__global__ void __launch_bounds__(32 * kSolveWarps<P>) recover_ff_kernel(int N, int NF, const SolveMat m,
                                                          const float4 *__restrict__ Xb2, const double *__restrict__ r_u,
                                                          const double *__restrict__ r_h, const double *__restrict__ lam,
                                                          const int32_t *__restrict__ facet_of,
                                                          const int32_t *__restrict__ flip, double *__restrict__ u,
                                                          double *__restrict__ hout) {
-    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP, NW = 8;
-    constexpr int KP = (NK + 1) / 2, MP = (M + 1) / 2;
-    __shared__ float2 sIn[NK + M][kCellsPad];   // r_K, then lambda on the cell's three facets
-    __shared__ double sOut[NK][kCellsPad];
+    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP, NW = kSolveWarps<P>;
+    constexpr int MP = (M + 1) / 2;
+    constexpr FFTabOffsets O = ff_tab_offsets(P);
+    __shared__ float2 sV[NK][kCellsPad];
+    __shared__ float2 sL[M][kCellsPad];         // lambda on the cell's three facets
+    __shared__ float4 tab[O.total];
     const int K0 = blockIdx.x * kCells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nc = min(kCells, N - K0);
-    stage_cell_rhs<NP>(N, K0, r_u, r_h, sIn);
-    for (int j = threadIdx.x; j < nc * M; j += blockDim.x) {
-        const int cell = j / M, q = j % M, i = q / PP, jj = q % PP, K = K0 + cell;
-        const int f = facet_of[3 * K + i], fl = flip[3 * K + i];
-        sIn[NK + q][cell] = split(lam[size_t(fl ? P - jj : jj) * NF + f]);
-    }
+    stage_tab<P>(tab, m.tab);
+    stage_cell_rhs<NP>(N, K0, r_u, r_h, sV);
+    stage_cell_trace<P>(N, NF, K0, lam, facet_of, flip, sL);
+    const bool on = K0 + lane < N;
+    if (!on)
+        for (int q = w; q < NK; q += NW) sV[q][lane] = make_float2(0.f, 0.f);
     __syncthreads();
-    const int K = K0 + lane;
-    if (K < N) {
+    cell_solve<P, FC>(m, blockIdx.x, on, tab, sV);
+    if (on) {
         for (int rho = w; rho < NK; rho += NW) {
             FFAcc acc;
-            row_pairs<NK>(acc, Rm2 + (size_t(blockIdx.x) * NK * KP + size_t(rho) * KP) * kCells + lane, sIn, lane);
-            row_pairs<M>(acc, Xb2 + (size_t(blockIdx.x) * NK * MP + size_t(rho) * MP) * kCells + lane, sIn + NK,
-                         lane, true);
-            sOut[rho][lane] = acc.value();
+            const float2 z = sV[rho][lane];
+            acc.s = z.x;
+            acc.c = z.y;
+            row_pairs<M>(acc, Xb2 + (size_t(blockIdx.x) * NK * MP + size_t(rho) * MP) * kCells + lane, sL, lane, true);
+            sV[rho][lane] = ff_pair(acc);
         }
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < nc * 2 * NP; j += blockDim.x)
-        u[size_t(K0) * 2 * NP + j] = sOut[j % (2 * NP)][j / (2 * NP)];
-    for (int j = threadIdx.x; j < nc * NP; j += blockDim.x) hout[size_t(K0) * NP + j] = sOut[2 * NP + j % NP][j / NP];
+    for (int j = threadIdx.x; j < nc * 2 * NP; j += blockDim.x) {
+        const float2 v = sV[j % (2 * NP)][j / (2 * NP)];
+        u[size_t(K0) * 2 * NP + j] = double(v.x) + double(v.y);
+    }
+    for (int j = threadIdx.x; j < nc * NP; j += blockDim.x) {
+        const float2 v = sV[2 * NP + j % NP][j / NP];
+        hout[size_t(K0) * NP + j] = double(v.x) + double(v.y);
+    }
 }
 
 // step 3 from the kept z_K: q_K = z_K - X_B lambda_K (two-float, z as the
@@ -764,11 +803,7 @@ __global__ void __launch_bounds__(256) recover_z_kernel(int N, int NF, const flo
     __shared__ double sOut[NK][kCellsPad];
     const int K0 = blockIdx.x * kCells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nc = min(kCells, N - K0);
-    for (int j = threadIdx.x; j < nc * M; j += blockDim.x) {
-        const int cell = j / M, q = j % M, i = q / PP, jj = q % PP, K = K0 + cell;
-        const int f = facet_of[3 * K + i], fl = flip[3 * K + i];
-        sIn[q][cell] = split(lam[size_t(fl ? P - jj : jj) * NF + f]);
-    }
+    stage_cell_trace<P>(N, NF, K0, lam, facet_of, flip, sIn);
     __syncthreads();
     const int K = K0 + lane;
     if (K < N) {
@@ -793,13 +828,6 @@ __global__ void __launch_bounds__(256) recover_z_kernel(int N, int NF, const flo
 cudaError_t launch_split(const double *a, float2 *out, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     split_kernel<<<blocks(n, 256), 256, 0, s>>>(a, out, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_split_pairs(const double *a, float2 *out, int rows, int cols, size_t N, cudaStream_t s) {
-    const size_t n = size_t(rows) * ((cols + 1) / 2) * N;
-    if (n == 0) return cudaSuccess;
-    split_pairs_kernel<<<blocks(n, 256), 256, 0, s>>>(a, reinterpret_cast<float4 *>(out), rows, cols, N);
     return cudaGetLastError();
 }
 
@@ -833,20 +861,24 @@ cudaError_t launch_residual_ff(hdg_handle *h, const double *b, const float2 *x2,
     return cudaGetLastError();
 }
 
-cudaError_t launch_rhs_ff(hdg_handle *h, const double *r_u, const double *r_h, double *g, double *ycell,
-                          double *copy_u, double *copy_h, const NormOut &nrm) {
-    HDG_DISPATCH_P(h->p, (rhs_cell_ff_kernel_go<P>(blocks(h->N, kCells), 128, 0, h->stream, h->N, reinterpret_cast<const float4 *>(h->d_W2), r_u, r_h,
-                                                                                               ycell, copy_u, copy_h)));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_rhs_gather(h, ycell, g, nrm);
+namespace {
+SolveMat solve_mat(const hdg_handle *h) {
+    return SolveMat{reinterpret_cast<const float4 *>(h->d_Hr2), reinterpret_cast<const float4 *>(h->d_PQ2), h->d_lgeo,
+                    h->d_fftab};
 }
+}  // namespace
 
 cudaError_t launch_rhs_z(hdg_handle *h, const double *r_u, const double *r_h, double *g, double *ycell, float2 *z2,
                          double *copy_u, double *copy_h, const NormOut &nrm) {
-    HDG_DISPATCH_P(h->p, (rhs_cell_z_kernel_go<P>(blocks(h->N, kCells), 256, 0, h->stream, h->N,
-                                                  reinterpret_cast<const float4 *>(h->d_Rm2), h->d_cgeo, h->d_ctab_b,
-                                                  h->d_ctab_v, r_u, r_h, ycell, z2, copy_u, copy_h)));
+    const SolveMat m = solve_mat(h);
+    const unsigned nb = blocks(h->N, kCells);
+    if (h->f_const) {
+        HDG_DISPATCH_P(h->p, (rhs_cell_z_kernel_go<P, true>(nb, 32 * kSolveWarps<P>, 0, h->stream, h->N, m, r_u, r_h,
+                                                            ycell, z2, copy_u, copy_h)));
+    } else {
+        HDG_DISPATCH_P(h->p, (rhs_cell_z_kernel_go<P, false>(nb, 32 * kSolveWarps<P>, 0, h->stream, h->N, m, r_u, r_h,
+                                                             ycell, z2, copy_u, copy_h)));
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_rhs_gather(h, ycell, g, nrm);
@@ -861,10 +893,17 @@ cudaError_t launch_recover_z(hdg_handle *h, const float2 *z2, const double *lam,
 
 cudaError_t launch_recover_ff(hdg_handle *h, const double *r_u, const double *r_h, const double *lam, double *u,
                               double *hout) {
-    HDG_DISPATCH_P(h->p, (recover_ff_kernel<P><<<blocks(h->N, kCells), 256, 0, h->stream>>>(
-                             h->N, h->NF, reinterpret_cast<const float4 *>(h->d_Rm2),
-                             reinterpret_cast<const float4 *>(h->d_Xb2), r_u, r_h, lam, h->d_facet_of, h->d_flip, u,
-                             hout)));
+    const SolveMat m = solve_mat(h);
+    const unsigned nb = blocks(h->N, kCells);
+    if (h->f_const) {
+        HDG_DISPATCH_P(h->p, (recover_ff_kernel<P, true><<<nb, 32 * kSolveWarps<P>, 0, h->stream>>>(
+                                 h->N, h->NF, m, reinterpret_cast<const float4 *>(h->d_Xb2), r_u, r_h, lam,
+                                 h->d_facet_of, h->d_flip, u, hout)));
+    } else {
+        HDG_DISPATCH_P(h->p, (recover_ff_kernel<P, false><<<nb, 32 * kSolveWarps<P>, 0, h->stream>>>(
+                                 h->N, h->NF, m, reinterpret_cast<const float4 *>(h->d_Xb2), r_u, r_h, lam,
+                                 h->d_facet_of, h->d_flip, u, hout)));
+    }
     return cudaGetLastError();
 }
 

@@ -1102,6 +1102,7 @@ cudaError_t launch_rhs_gather(hdg_handle *h, const double *ycell, double *g, con
 cudaError_t launch_rhs(hdg_handle *h, const double *r_u, const double *r_h, double *g, double *ycell,
                        const NormOut &nrm) {
     if (h->prm.flux == 1) return nrm.partial ? cudaErrorInvalidValue : launch_rhs_lf(h, r_u, r_h, g, ycell);
+    if (mode_ff(h->prm)) return launch_rhs_z(h, r_u, r_h, g, ycell, nullptr, nullptr, nullptr, nrm);
     size_t n = size_t(h->N) * h->m;
     HDG_DISPATCH_P(h->p, (rhs_cell_kernel<P><<<blocks(n, 256), 256, 0, h->stream>>>(h->N, h->d_W, r_u, r_h, ycell)));
     cudaError_t e = cudaGetLastError();
