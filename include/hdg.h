@@ -187,9 +187,11 @@ HDG_API void hdg_default_params(hdg_params *prm);
  * error text is available from hdg_last_error(NULL).
  * Two environment variables, read here, select equivalent launch structures
  * (for timing comparisons; results agree up to summation order):
- * HDG_TAIL_MAX_VERTICES (16..4096; default 1024 for the FP32 levels, 256 for
- * the FP64 levels) bounds the P1 levels run by the single-block coarse cycle; HDG_P1_FUSED=0 replaces the patch-fused P1
- * kernels by one launch per smoothing / transfer step; HDG_FACET_BLOCK
+ * HDG_TAIL_MAX_VERTICES (16..4096; default 1024, 256 for the FP64 levels of handles
+ * with an FP32 preconditioner) bounds the first P1 level of the coarse cycle's tail,
+ * which runs as one product with the dense FP64 operator of the tail's V-cycle (formed
+ * by hdg_condense; small tails) or in a single block; HDG_P1_FUSED=0 replaces the
+ * patch-fused P1 kernels by one launch per smoothing / transfer step; HDG_FACET_BLOCK
  * (64, 128 or 256; default 128 for HDG_FP64 handles, 256 otherwise) sets the
  * threads per block of the facet-row kernels.  HDG_PDL (a bit mask, read once
  * per process; default 6) selects the kernel families launched with
@@ -332,8 +334,8 @@ HDG_API int hdg_batch_destroy(hdg_batch *b);
 /* Pick launch shapes for this handle by timing one Arnoldi step (preconditioner,
  * operator application, Gram-Schmidt) for each candidate: threads per block of
  * the facet-row kernels (64 / 128 / 256), blocks of the fused Gram-Schmidt
- * kernels (152 / 304 / 608 / 1216) and the largest level of the single-CTA coarse
- * cycle (256 / 1024 / 4096 vertices), one parameter at a time.  Needs
+ * kernels (152 / 304 / 608 / 1216) and the largest first level of the coarse
+ * cycle's tail (256 / 1024 / 4096 vertices), one parameter at a time.  Needs
  * hdg_condense.  choice[0..2] (may be NULL) receives the three picks.  Results
  * do not depend on the choice beyond floating-point summation order. */
 HDG_API int hdg_autotune(hdg_handle *h, int32_t *choice);

@@ -343,6 +343,26 @@ template <typename T>
 cudaError_t dots(hdg_handle *h, const T *V, int k, const T *w, double *out, HostValue *pub = nullptr,
                  int32_t seq = 0, double *root_a = nullptr, double *root_b = nullptr);
 
+// arguments of the single-CTA cycle on levels ts and coarser (image im, the inverse
+// diagonal of level ts in the image's precision)
+TailArgs tail_args(hdg_handle *h, const TailImage &im, int ts, const void *dinv0) {
+    TailArgs a{};
+    a.nlev = int(h->lev.size()) - ts;
+    a.nu1 = h->prm.p1_nu_pre;
+    a.nu2 = h->prm.p1_nu_post;
+    a.omega = h->prm.p1_omega;
+    a.img = im.d;
+    a.img_bytes = im.img_bytes;
+    a.inv_off = im.inv_off;
+    a.nv0 = h->lev[size_t(ts)].nv;
+    a.ob0 = im.ob0;
+    a.ox0 = im.ox0;
+    a.dinv0 = dinv0;
+    a.inv = h->d_coarse_inv;          // the coarsest solve stays FP64 in every precision
+    a.status = h->d_status;
+    return a;
+}
+
 // P1 V-cycle for the coarse problem (Eq. coarse_problem_upwind) with
 // right-hand side levB(level 0).  Levels above the tail: the first
 // pre-smoothing sweep of each level rides on the restriction that produced
@@ -350,8 +370,8 @@ cudaError_t dots(hdg_handle *h, const T *V, int k, const T *w, double *out, Host
 // last pre-sweep, the residual and the restriction share one patch kernel, and
 // so do the prolongation and the first two post-sweeps; elsewhere one kernel
 // per sweep, with the residual inside the restriction and the prolongation
-// inside the first post-sweep.  Levels from tail_start down: one single-CTA
-// kernel.  Returns the device vector that holds the level-0 result.  The first
+// inside the first post-sweep.  Levels from tail_start down: one dense product
+// (kTailOpMax) or one single-CTA kernel.  Returns the device vector that holds the level-0 result.  The first
 // pre-smoothing sweep of level 0 (when it is above the tail) was done by the
 // trace-to-P1 restriction.
 template <typename T>
@@ -385,30 +405,16 @@ cudaError_t p1_cycle(hdg_handle *h, T **result) {
         }
         cur[l] = x; oth[l] = x2;
     }
-    if (nlev - ts == 1 && h->lev[ts].nv > kTailDenseMax) {
-        // the coarsest level alone, too large for one CTA's dense product: the
-        // exact solve as a product with its FP64 inverse over many CTAs
-        if ((e = KL(HDG_PROF_P1, 1, launch_p1_coarse_dense<T>(h->d_coarse_inv, h->lev[ts].nv, levB<T>(h->lev[ts]),
-                                                               levX<T>(h->lev[ts]), s))) != cudaSuccess)
+    if (const double *op = h->tail_op[sizeof(T) == 8 ? 0 : 1]) {
+        // the tail as one dense product (kTailOpMax)
+        if ((e = KL(HDG_PROF_P1, 1, launch_p1_dense<T>(op, h->lev[ts].nv, levB<T>(h->lev[ts]), levX<T>(h->lev[ts]), s))) !=
+            cudaSuccess)
             return e;
         res[ts] = levX<T>(h->lev[ts]);
     } else {
         const TailImage &im = h->tail_img[sizeof(T) == 8 ? 0 : 1];
         if (im.ts != ts || !im.d) return cudaErrorInvalidValue;   // image not built for this tail start
-        TailArgs a{};
-        a.nlev = nlev - ts;
-        a.nu1 = nu1;
-        a.nu2 = nu2;
-        a.omega = h->prm.p1_omega;
-        a.img = im.d;
-        a.img_bytes = im.img_bytes;
-        a.inv_off = im.inv_off;
-        a.nv0 = h->lev[ts].nv;
-        a.ob0 = im.ob0;
-        a.ox0 = im.ox0;
-        a.dinv0 = levD<T>(h->lev[ts]);
-        a.inv = h->d_coarse_inv;          // the coarsest solve stays FP64 in every precision
-        a.status = h->d_status;
+        TailArgs a = tail_args(h, im, ts, levD<T>(h->lev[ts]));
         a.b_top = levB<T>(h->lev[ts]);
         a.x_top = levX<T>(h->lev[ts]);
         const size_t smem = im.smem_bytes;
@@ -1214,7 +1220,8 @@ void free_handle(hdg_handle *h) {
     dfree(h->d_Xb2); dfree(h->d_Sval2);
     dfree(h->d_Hr2); dfree(h->d_PQ2); dfree(h->d_lgeo); dfree(h->d_fftab);
     dfree(h->d_Dinv); dfree(h->d_Sval32); dfree(h->d_Dinv32); dfree(h->d_Sval16); dfree(h->d_status); dfree(h->d_coarse_inv);
-    dfree(h->tail_img[0].d); dfree(h->tail_img[1].d);
+    for (auto &im : h->tail_img) dfree(im.d);
+    dfree(h->d_tail_op);
     dfree(h->d_coarse_work);
     dfree(h->d_coarse_fac);
     for (auto &L : h->lev) {
@@ -1258,14 +1265,13 @@ void free_handle(hdg_handle *h) {
 
 void drop_graphs(hdg_handle *h);
 
-// The tail image of precision pi (0: FP64, 1: FP32) for the current tail
-// start: header table, every level's staged arrays and, when it fits, the
-// coarsest FP64 inverse, copied device to device into one buffer.  Needs the
-// assembled level operators (hdg_condense).
-int build_tail_image(hdg_handle *h, int pi) {
-    if (pi == 1 && !h->lev[0].A32) return HDG_OK;          // no FP32 levels on this handle
+// The tail image im of precision pi (0: FP64, 1: FP32) for levels ts and coarser: header
+// table, every level's staged arrays and, when it fits, the coarsest FP64 inverse, copied
+// device to device into one buffer.  Needs the assembled level operators (hdg_condense);
+// the table and the transfers do not change between condensations and are copied once.
+int build_tail_image(hdg_handle *h, int pi, int ts, TailImage &im) {
     const size_t tsz = pi == 0 ? sizeof(double) : sizeof(float);
-    const int ts = h->tail_start[pi], n = int(h->lev.size()) - ts;
+    const int n = int(h->lev.size()) - ts;
     TailLayout lay;
     if (!tail_layout(tail_sizes(h->lev, ts), tsz, size_t(h->lev.back().nv), lay))
         return fail(h, HDG_EINVAL, "coarsest P1 levels too large for the single-CTA coarse cycle");
@@ -1286,16 +1292,21 @@ int build_tail_image(hdg_handle *h, int pi) {
         default: return h->d_coarse_inv;
         }
     };
-    TailImage &im = h->tail_img[pi];
+    bool fresh = im.ts != ts || im.img_bytes != img_bytes;
     if (im.cap < img_bytes) {
         dfree(im.d);
         im.cap = 0;
         TRY(dalloc(&im.d, img_bytes));
         im.cap = img_bytes;
-        if (h->ws) drop_graphs(h);                         // captured launches hold the old address
+        fresh = true;
     }
+    if (fresh && h->ws) drop_graphs(h);                    // captured launches hold the old address or shape
+    im.ts = -1;
     cudaStream_t s = h->stream;
-    TRY(cudaMemcpyAsync(im.d, hdr.data(), sizeof(TailHdr) * n, cudaMemcpyHostToDevice, s));
+    if (fresh) {
+        TRY(cudaMemcpyAsync(im.d, hdr.data(), sizeof(TailHdr) * n, cudaMemcpyHostToDevice, s));
+        TRY(cudaStreamSynchronize(s));                     // hdr is host memory on this stack
+    }
     for (const TailPiece &q : lay.pieces) {
         if (q.kind == kTailCol) continue;                  // packed together with the values
         if (q.kind == kTailA) {
@@ -1303,11 +1314,8 @@ int build_tail_image(hdg_handle *h, int pi) {
             TRY(launch_tail_pack(L.col, source(q), tsz, L.nv, L.width, im.d + hdr[size_t(q.level)].ocol, im.d + q.off, s));
             continue;
         }
+        if (!fresh && (q.kind == kTailCw || q.kind == kTailCp || q.kind == kTailCi || q.kind == kTailPar)) continue;
         TRY(cudaMemcpyAsync(im.d + q.off, source(q), q.bytes, cudaMemcpyDeviceToDevice, s));
-    }
-    TRY(cudaStreamSynchronize(s));                         // hdr is host memory on this stack
-    if (im.ts != ts || im.img_bytes != img_bytes) {
-        if (h->ws) drop_graphs(h);
     }
     im.ts = ts;
     im.img_bytes = uint32_t(img_bytes);
@@ -1318,25 +1326,81 @@ int build_tail_image(hdg_handle *h, int pi) {
     return HDG_OK;
 }
 
-// First level of the single-CTA coarse cycle, per precision: the largest
-// suffix of P1 levels whose levels have at most tail_max vertices and whose
-// operators, transfers and vectors fit in one CTA's shared memory.
-int set_tail_start(hdg_handle *h, int tail_max64, int tail_max32) {
-    const int nlev = int(h->lev.size());
-    for (int pi = 0; pi < 2; ++pi) {
-        const size_t tsz = pi == 0 ? sizeof(double) : sizeof(float);
-        const int tail_max = pi == 0 ? tail_max64 : tail_max32;
-        int ts = nlev - 1;
-        while (ts > 0 && h->lev[ts - 1].nv <= tail_max && nlev - (ts - 1) <= kTailMaxLevels &&
-               tail_smem_bytes(h->lev, ts - 1, tsz) <= size_t(220) * 1024)
-            --ts;
-        if (tail_smem_bytes(h->lev, ts, tsz) > kTailSmemMax)
-            return fail(h, HDG_EINVAL, "coarsest P1 level too large for the single-CTA coarse cycle");
-        h->tail_start[pi] = ts;
-        if (h->condensed) {
-            int rc = build_tail_image(h, pi);
+// largest first tail level that runs as a dense product on this handle (kTailOpMax)
+int tail_op_max(const hdg_handle *h) {
+    if (h->prm.precision == HDG_FP64) return kTailOpMax;
+    if (h->prm.precision == HDG_MIXED_FGMRES64 || h->lev.back().nv > kTailOpCoarse) return kTailOpMax32;
+    return kTailOpMaxBatch;
+}
+bool tail_is_op(const hdg_handle *h, int ts) {
+    return ts == int(h->lev.size()) - 1 || h->lev[size_t(ts)].nv <= tail_op_max(h);
+}
+
+// What the coarse cycle runs from its tail start: the dense operator of the tail's
+// V-cycle (the coarsest inverse itself when the tail is the coarsest level alone, else
+// formed from the FP64 levels), or the image of the single-CTA kernel.  The levels that
+// precondition the solves (FP32 ones where the handle has them) come first; the others
+// share the operator when their tail starts at the same level and take the image else.
+int build_tail(hdg_handle *h) {
+    const bool f32 = h->lev[0].A32 != nullptr;
+    const int pm = f32 ? 1 : 0;
+    for (int k = 0; k < (f32 ? 2 : 1); ++k) {
+        const int pi = k == 0 ? pm : 0;
+        const int ts = h->tail_start[pi], nv = h->lev[size_t(ts)].nv;
+        const double *old = h->tail_op[pi], *op = nullptr;
+        if (ts == int(h->lev.size()) - 1) {
+            op = h->d_coarse_inv;
+        } else if (k == 1 && h->tail_op[pm] && h->tail_start[pm] == ts) {
+            op = h->tail_op[pm];
+        } else if (k == 0 && tail_is_op(h, ts)) {
+            TailImage &im = h->tail_img[0];
+            int rc = build_tail_image(h, 0, ts, im);
+            if (rc) return rc;
+            const size_t need = size_t(nv) * size_t(nv);
+            if (h->tail_op_cap < need) {
+                dfree(h->d_tail_op);
+                h->tail_op_cap = 0;
+                TRY(dalloc(&h->d_tail_op, need));
+                h->tail_op_cap = need;
+            }
+            TRY(KL(HDG_PROF_CONDENSE, 1,
+                   launch_p1_tail_columns(tail_args(h, im, ts, h->lev[size_t(ts)].dinv), im.smem_bytes, h->d_tail_op,
+                                          h->stream)));
+            op = h->d_tail_op;
+        } else {
+            int rc = build_tail_image(h, pi, ts, h->tail_img[pi]);
             if (rc) return rc;
         }
+        h->tail_op[pi] = op;
+        if (op != old && h->ws) drop_graphs(h);            // captured launches hold the old operator
+    }
+    return HDG_OK;
+}
+
+// First level of the coarse cycle's tail, per precision: the largest suffix of P1 levels
+// whose levels have at most tail_max vertices and whose operators, transfers and vectors
+// fit in one CTA's shared memory (in FP64 where the tail's dense operator is formed).
+int set_tail_start(hdg_handle *h, int tail_max64, int tail_max32) {
+    const int nlev = int(h->lev.size());
+    bool moved = false;
+    for (int pi = 1; pi >= 0; --pi) {
+        const int tail_max = pi == 0 ? tail_max64 : tail_max32;
+        auto tsz = [&](int l) { return pi == 0 || tail_is_op(h, l) ? sizeof(double) : sizeof(float); };
+        int ts = nlev - 1;
+        while (ts > 0 && h->lev[ts - 1].nv <= tail_max && nlev - (ts - 1) <= kTailMaxLevels &&
+               tail_smem_bytes(h->lev, ts - 1, tsz(ts - 1)) <= size_t(220) * 1024)
+            --ts;
+        // FP64 levels beside an FP32 preconditioner share its operator
+        if (pi == 0 && h->prm.precision != HDG_FP64 && tail_is_op(h, h->tail_start[1])) ts = h->tail_start[1];
+        if (!tail_is_op(h, ts) && tail_smem_bytes(h->lev, ts, tsz(ts)) > kTailSmemMax)
+            return fail(h, HDG_EINVAL, "coarsest P1 level too large for the single-CTA coarse cycle");
+        moved |= h->tail_start[pi] != ts;
+        h->tail_start[pi] = ts;
+    }
+    if (h->condensed) {
+        int rc = build_tail(h);
+        if (rc) return rc;
+        if (moved) drop_graphs(h);                         // other levels above the tail
     }
     return HDG_OK;
 }
@@ -1502,9 +1566,9 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
         }
     }
     {
-        // largest level of the single-CTA coarse cycle per precision (FP64 levels:
-        // 256, FP32 levels: 1,024, as measured fastest); HDG_TAIL_MAX_VERTICES sets both
-        int tail_max64 = kTailMaxVertices64, tail_max32 = kTailMaxVertices;
+        // largest level of the coarse cycle's tail; HDG_TAIL_MAX_VERTICES sets it
+        int tail_max64 = prm->precision == HDG_FP64 ? kTailMaxVertices : kTailMaxVertices64;
+        int tail_max32 = kTailMaxVertices;
         if (const char *ev = std::getenv("HDG_TAIL_MAX_VERTICES"))
             tail_max64 = tail_max32 = std::max(16, std::min(4096, std::atoi(ev)));
         // HDG_P1_FUSED=0 selects the unfused P1 kernels (same arithmetic; for timing comparisons)
@@ -2081,11 +2145,9 @@ int hdg_condense(hdg_handle *h) {
             TRY(KL(HDG_PROF_CONDENSE, 1, launch_split(h->d_Sval, h->d_Sval2, (NS + 1) / 2 * 2 * size_t(h->NF), s)));
         }
     }
-    for (int pi = 0; pi < 2; ++pi) {
-        int rc = build_tail_image(h, pi);
-        if (rc) return rc;
-    }
-    int rc = check_status(h);
+    int rc = build_tail(h);
+    if (rc) return rc;
+    rc = check_status(h);
     if (rc) return rc;
     if (h->prm.smoother == 1 && (rc = chebyshev_setup(h)) != HDG_OK) return rc;
     h->condensed = true;
@@ -2461,7 +2523,7 @@ int hdg_autotune(hdg_handle *h, int32_t *choice) {
     }
     W.nblk_gs = best_nb;
     // first level of the single-CTA coarse cycle
-    int best_tm = f32 ? kTailMaxVertices : kTailMaxVertices64;
+    int best_tm = kTailMaxVertices;
     best_t = 1e30f;
     int last_ts = -1;
     for (int tm : {256, 1024, 4096}) {

@@ -326,8 +326,21 @@ __device__ __forceinline__ void finish_partials(const double *partial, int nb, i
 // levels of the single-CTA V-cycle tail (k_p1.cu)
 constexpr int kMaxGsBlocks = 1216;     // largest grid of the fused Gram-Schmidt kernels (8 x 152 SMs)
 constexpr int kTailMaxLevels = 8;
-constexpr int kTailMaxVertices = 1024;     // default largest level run inside the tail kernel
-constexpr int kTailMaxVertices64 = 256;    // the same for the FP64 levels (measured faster there)
+constexpr int kTailMaxVertices = 1024;     // default largest level of the coarse cycle's tail
+constexpr int kTailMaxVertices64 = 256;    // the same for FP64 levels under an FP32 preconditioner
+// The tail's V-cycle from its first right-hand side is a fixed linear map; formed column
+// by column in FP64 at condensation (h->tail_op) it runs as one dense product over all
+// SMs instead of the single-CTA cycle's 25 or so barrier-separated steps.  Per cycle,
+// first tail level of n vertices: n = 256 3.1 us instead of 11.5 (FP64), n = 642 5.6 instead
+// of 9.3, or of 22.4 where the coarsest level has 162 vertices (its FP64 product alone
+// takes 8 us on one SM), n = 1,024 7.4 instead of 10.7 (FP32 levels) or 26 (FP64 levels,
+// with the 1,024-vertex level's own two launches).  It reads 8 n^2 bytes, which is what
+// draws the lines (tail_op_max): at n = 1,024 under FP32 sweeps the 8 MB displace the
+// facet operators from L2 (flat 256 x 256 x 2 mixed step 1,592 instead of 1,566 us), and in
+// a merged batch every problem reads its own (16 problems: 3,420 instead of 3,330 us).
+// So: FP64 preconditioners up to 1,024; FP32 ones up to 724 (4 MB) in the mode that no
+// merged batch takes, or where the coarsest level is large, otherwise up to 256.
+constexpr int kTailOpMax = 1024, kTailOpMax32 = 724, kTailOpMaxBatch = 256, kTailOpCoarse = 96;
 constexpr size_t kTailSmemMax = 226 * 1024; // dynamic shared memory limit of the tail kernel
 constexpr size_t kTailInvSmemMax = 64 * 1024; // largest coarsest-level inverse staged in shared memory
 constexpr int kPatchMaxVertices = 32768;      // largest P1 level smoothed by the fused patch kernels
@@ -347,7 +360,7 @@ static_assert(sizeof(TailHdr) == 64, "tail header entries are 64 bytes");
 struct TailImage {
     unsigned char *d = nullptr;
     size_t cap = 0;
-    int ts = -1;                        // first level the image was built for
+    int ts = -1;                        // first level the image was built for (its static parts too)
     uint32_t img_bytes = 0;             // bytes staged by the bulk copies
     uint32_t smem_bytes = 0;            // image plus scratch vectors
     int32_t inv_off = -1;               // offset of the staged inverse, -1: read from global memory
@@ -667,6 +680,10 @@ struct hdg_handle {
     int bs_facet = 256;               // threads per block of the facet-row kernels (autotuned)
     double *d_coarse_inv = nullptr;   // dense inverse of the coarsest P1 operator
     hdg::TailImage tail_img[2];       // shared-memory images of the tail levels (FP64, FP32)
+    double *d_tail_op = nullptr;      // the tail's dense operator (kTailOpMax)
+    size_t tail_op_cap = 0;
+    const double *tail_op[2] = {nullptr, nullptr};   // operator in use per precision (that, the coarsest
+                                      // inverse; null: the single-CTA kernel and its image)
     double *d_coarse_work = nullptr;
     double *d_coarse_fac = nullptr;   // row factors of one elimination step (coarsest levels above 256 vertices)
     hdg::Workspace *ws = nullptr;
@@ -871,11 +888,12 @@ cudaError_t launch_p1_up_fused(const DevLevel &fine, const DevLevel &coarse, con
                                const T *b_f, const T *x_f, const T *ec, T *xout, T omega, cudaStream_t s);
 template <typename T>
 cudaError_t launch_p1_tail(const TailArgs &a, size_t smem, cudaStream_t s);
-// x = inv b on the coarsest level (n vertices, FP64 inverse) over many CTAs
+// op[i * n + j]: entry i of the tail's FP64 V-cycle of the unit vector e_j (a.b_top and
+// a.x_top are not used)
+cudaError_t launch_p1_tail_columns(const TailArgs &a, size_t smem, double *op, cudaStream_t s);
+// x = op b (n x n, row-major, FP64 sums in every precision) over many CTAs
 template <typename T>
-cudaError_t launch_p1_coarse_dense(const double *inv, int n, const T *b, T *x, cudaStream_t s);
-// coarsest levels above this size alone in the tail take the multi-CTA product
-constexpr int kTailDenseMax = 256;
+cudaError_t launch_p1_dense(const double *op, int n, const T *b, T *x, cudaStream_t s);
 
 // Krylov kernels (k_krylov.cu)
 template <typename T>

@@ -871,77 +871,117 @@ __device__ __forceinline__ void coarse_product(const double *inv, int n, const T
 }
 
 
-// x = inv b on a coarsest level too large for the single-CTA cycle (FP64
-// inverse, FP64 sums in every precision): one block of four warps per row,
-// each thread summing pairs of columns 256 apart (16-byte loads, all of a
-// thread's loads independent), then a fixed shuffle tree per warp and the
-// four warp sums in order.
-template <typename T>
-__device__ __forceinline__ void coarse_dense_kernel_impl(int bid_, int nb_, const double *__restrict__ inv, int n,
-                                                         const T *__restrict__ b, T *__restrict__ x) {
-    __shared__ double part[4];
-    const int row = bid_, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const double *a = inv + size_t(row) * n;
-    double acc = 0.0;
-    if ((n & 1) == 0) {
-        // rows start on 16-byte boundaries when n is even
-#pragma unroll 4
-        for (int j = 2 * tid; j < n; j += 256) {
-            const double2 av = *reinterpret_cast<const double2 *>(a + j);
-            acc = fma(av.x, double(b[j]), acc);
-            acc = fma(av.y, double(b[j + 1]), acc);
-        }
-    } else {
-#pragma unroll 4
-        for (int j = tid; j < n; j += 128) acc = fma(a[j], double(b[j]), acc);
+// x = op b for a dense n x n FP64 operator, FP64 sums in every precision: R rows per
+// block of eight warps, warp q taking columns [q C, (q + 1) C), C = n / 8 rounded up to
+// 32.  The FP64 pipe bounds it (n^2 FMAs over 152 SMs: 2 us at n = 1,024), so the rows
+// go evenly over the SMs (R: about n / 152), each value of b is widened once per warp
+// for R rows, and the lanes' R sums are added by halving exchanges (R adds instead of
+// 5 R) before the eight warps' sums.  The operator is static during a solve: the first
+// kDensePre columns' entries per lane are loaded before the wait for the previous kernel.
+constexpr int kDenseWarps = 8, kDensePre = 4;
+template <int R>
+__device__ __forceinline__ void dense_loads(const double *op, int n, int row0, int j, int jend, double (&a)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) a[r] = (j < jend && row0 + r < n) ? __ldg(op + size_t(row0 + r) * n + j) : 0.0;
+}
+template <typename T, int R>
+__device__ __forceinline__ void dense_kernel_impl(int bid_, int nb_, const double *__restrict__ op, int n,
+                                                  const T *__restrict__ b, T *__restrict__ x) {
+    __shared__ double part[kDenseWarps][R];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row0 = bid_ * R;
+    const int C = ((n + kDenseWarps - 1) / kDenseWarps + 31) / 32 * 32;
+    const int j0 = warp * C + lane, jend = min(n, warp * C + C);
+    double a[kDensePre][R], acc[R];
+#pragma unroll
+    for (int u = 0; u < kDensePre; ++u) dense_loads<R>(op, n, row0, j0 + 32 * u, jend, a[u]);
+    pdl_wait();
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = 0.0;
+    T bv[kDensePre];
+#pragma unroll
+    for (int u = 0; u < kDensePre; ++u) bv[u] = j0 + 32 * u < jend ? b[j0 + 32 * u] : T(0);
+#pragma unroll
+    for (int u = 0; u < kDensePre; ++u) {
+        if (warp * C + 32 * u >= jend) break;
+        const double bd = double(bv[u]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = fma(a[u][r], bd, acc[r]);
     }
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) part[warp] = acc;
+    for (int j = j0 + 32 * kDensePre; j - lane < jend; j += 32) {   // n above 1,024
+        double v[R];
+        dense_loads<R>(op, n, row0, j, jend, v);
+        const double bd = j < jend ? double(b[j]) : 0.0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = fma(v[r], bd, acc[r]);
+    }
+    // halving exchange: lane groups keep half of the rows each time, then the rest of
+    // the tree; row (lane's kept index) ends complete in every lane of its group
+    int keep = 0;
+#pragma unroll
+    for (int h = R / 2, off = 16; h > 0; h /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int r = 0; r < h; ++r) {
+            const double send = up ? acc[r] : acc[r + h], mine = up ? acc[r + h] : acc[r];
+            acc[r] = mine + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+        keep = 2 * keep + (up ? 1 : 0);
+    }
+    double t = acc[0];
+#pragma unroll
+    for (int off = 16 / R; off > 0; off /= 2) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (lane % (32 / R) == 0) part[warp][keep] = t;
     __syncthreads();
-    if (tid == 0) x[row] = T(((part[0] + part[1]) + part[2]) + part[3]);
+    // R groups of eight lanes add the warps' sums
+    if (threadIdx.x < 8 * R || threadIdx.x < 32) {
+        const int r = threadIdx.x >> 3;
+        double v = r < R ? part[threadIdx.x & 7][r] : 0.0;
+#pragma unroll
+        for (int off = 4; off > 0; off /= 2) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if ((threadIdx.x & 7) == 0 && r < R && row0 + r < n) x[row0 + r] = T(v);
+    }
     (void)nb_;
 }
-template <typename T>
-__global__ void __launch_bounds__(128) coarse_dense_kernel(const double *inv, int n, const T *b, T *x) {
-    pdl_wait();
-    coarse_dense_kernel_impl<T>(blockIdx.x, gridDim.x, inv, n, b, x);
+template <typename T, int R>
+__global__ void __launch_bounds__(32 * kDenseWarps) dense_kernel(const double *op, int n, const T *b, T *x) {
+    dense_kernel_impl<T, R>(blockIdx.x, gridDim.x, op, n, b, x);
 }
 template <typename T>
-struct coarse_dense_kernel_args {
+struct dense_kernel_args {
     int nb_;
-    const double *inv;
+    const double *op;
     int n;
     const T *b;
     T *x;
 };
-template <typename T>
-__global__ void __launch_bounds__(128) coarse_dense_kernel_multi(const __grid_constant__ MultiP<coarse_dense_kernel_args<T>> M) {
-    pdl_wait();
+template <typename T, int R>
+__global__ void __launch_bounds__(32 * kDenseWarps) dense_kernel_multi(const __grid_constant__ MultiP<dense_kernel_args<T>> M) {
     int b_;
-    const coarse_dense_kernel_args<T> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    coarse_dense_kernel_impl<T>(b_, q_.nb_, q_.inv, q_.n, q_.b, q_.x);
+    const dense_kernel_args<T> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    dense_kernel_impl<T, R>(b_, q_.nb_, q_.op, q_.n, q_.b, q_.x);
 }
-template <typename T>
-void coarse_dense_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, const double *inv, int n,
-                            const T *b, T *x) {
+template <typename T, int R>
+void dense_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, const double *op, int n, const T *b,
+                     T *x) {
     if (Recorder *r_ = batch_recorder()) {
-        coarse_dense_kernel_args<T> q_;
+        dense_kernel_args<T> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
-        q_.inv = inv;
+        q_.op = op;
         q_.n = n;
         q_.b = b;
         q_.x = x;
-        batch_record(r_, reinterpret_cast<const void *>(&coarse_dense_kernel_multi<T>), q_, grid_, block_, smem_, kPdlFamily);
+        batch_record(r_, reinterpret_cast<const void *>(&dense_kernel_multi<T, R>), q_, grid_, block_, smem_,
+                     kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &coarse_dense_kernel<T>, grid_, block_, smem_, s_, inv, n, b, x);
+    pdl_launch(kPdlFamily, &dense_kernel<T, R>, grid_, block_, smem_, s_, op, n, b, x);
 }
 
 // Every array pointer below is the shared-memory base plus an offset from the
 // level table, so that the compiler addresses shared memory directly.
 template <typename T>
-__device__ __forceinline__ void tail_kernel_impl(int bid_, int nb_, TailArgs a) {
+__device__ __forceinline__ void tail_kernel_impl(int bid_, int nb_, TailArgs a, double *op = nullptr) {
     extern __shared__ __align__(16) unsigned char tail_smem[];
     __shared__ __align__(8) uint64_t bar;
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -976,7 +1016,7 @@ __device__ __forceinline__ void tail_kernel_impl(int bid_, int nb_, TailArgs a) 
         const T *d0 = static_cast<const T *>(a.dinv0);
         T *b0 = PT(a.ob0), *x0 = PT(a.ox0);
         for (int i = tid; i < a.nv0; i += nt) {
-            const T bi = btop[i];
+            const T bi = op ? T(i == bid_ ? 1 : 0) : btop[i];
             b0[i] = bi;
             x0[i] = a.nu1 == 0 ? T(0) : om * d0[i] * bi;
         }
@@ -1057,9 +1097,18 @@ __device__ __forceinline__ void tail_kernel_impl(int bid_, int nb_, TailArgs a) 
         }
         oec = ox;
     }
-    T *xtop = static_cast<T *>(a.x_top);
     const T *ec = PT(oec);
+    if (op) {
+        for (int i = tid; i < a.nv0; i += nt) op[size_t(i) * a.nv0 + bid_] = double(ec[i]);
+        return;
+    }
+    T *xtop = static_cast<T *>(a.x_top);
     for (int i = tid; i < a.nv0; i += nt) xtop[i] = ec[i];
+}
+// the tail's V-cycle of every unit vector, one block each: column blockIdx.x of its
+// dense operator
+__global__ void __launch_bounds__(1024, 1) tail_columns_kernel(TailArgs a, double *op) {
+    tail_kernel_impl<double>(blockIdx.x, gridDim.x, a, op);
 }
 template <typename T>
 __global__ void __launch_bounds__(1024, 1) tail_kernel(TailArgs a) {
@@ -1155,8 +1204,21 @@ cudaError_t launch_p1_up_fused(const DevLevel &fine, const DevLevel &coarse, con
     return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_p1_coarse_dense(const double *inv, int n, const T *b, T *x, cudaStream_t s) {
-    coarse_dense_kernel_go<T>(unsigned(n), 128, 0, s, inv, n, b, x);
+cudaError_t launch_p1_dense(const double *op, int n, const T *b, T *x, cudaStream_t s) {
+    // rows per block: about one block per SM
+    constexpr unsigned bs = 32 * kDenseWarps;
+    if (n <= 152) dense_kernel_go<T, 1>(blocks(n, 1), bs, 0, s, op, n, b, x);
+    else if (n <= 304) dense_kernel_go<T, 2>(blocks(n, 2), bs, 0, s, op, n, b, x);
+    else if (n <= 608) dense_kernel_go<T, 4>(blocks(n, 4), bs, 0, s, op, n, b, x);
+    else dense_kernel_go<T, 8>(blocks(n, 8), bs, 0, s, op, n, b, x);
+    return cudaGetLastError();
+}
+cudaError_t launch_p1_tail_columns(const TailArgs &a, size_t smem, double *op, cudaStream_t s) {
+    if (smem > kTailSmemMax) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(tail_columns_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(kTailSmemMax));
+    if (e != cudaSuccess) return e;
+    tail_columns_kernel<<<a.nv0, 1024, smem, s>>>(a, op);
     return cudaGetLastError();
 }
 template <typename T>
@@ -1213,7 +1275,7 @@ cudaError_t launch_tail_pack(const int32_t *col, const void *A, size_t tsz, int 
                                                const T *, const T *, T *, T, cudaStream_t);                        \
     template bool p1_patch_ok<T>(const DevLevel &);                                                          \
     template cudaError_t launch_p1_tail<T>(const TailArgs &, size_t, cudaStream_t);                           \
-    template cudaError_t launch_p1_coarse_dense<T>(const double *, int, const T *, T *, cudaStream_t);
+    template cudaError_t launch_p1_dense<T>(const double *, int, const T *, T *, cudaStream_t);
 HDG_P1_INST(double)
 HDG_P1_INST(float)
 
