@@ -121,8 +121,8 @@ def trace_bytes(cat: str, NF: int, pp: int, s_width: int | None = None) -> float
     base = cat[:-2]
     if base == "apply":
         per = S + 2 * vec
-    elif base == "residual":
-        per = S + 3 * vec
+    elif base == "residual":      # with the first post-smoothing sweep's part before the correction
+        per = S + pp * pp * w + 4 * vec
     elif base == "smooth":
         per = S + pp * pp * w + 3 * vec
     elif base == "smooth_first":
@@ -507,7 +507,7 @@ def whole_solve(arm: dict, peaks: dict, steps: int) -> dict:
 def fp64_fmas_per_facet(cat: str, pp: int) -> int:
     """FMAs per facet of an FP64 facet-row kernel (operator blocks, inverse block)."""
     base = cat[:-2]
-    return {"apply": 5 * pp * pp, "residual": 5 * pp * pp, "smooth": 6 * pp * pp, "smooth_first": pp * pp}[base]
+    return {"apply": 5 * pp * pp, "residual": 6 * pp * pp, "smooth": 6 * pp * pp, "smooth_first": pp * pp}[base]
 
 
 def p1_cycle_bytes(levels_nv: list, w: int, width: int = 8) -> float:

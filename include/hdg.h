@@ -416,7 +416,7 @@ HDG_API int hdg_get_rt0_chebyshev(const hdg_handle *h, double *ellipse, double *
 #define HDG_PROF_RESIDUAL32     5
 #define HDG_PROF_SMOOTH32       6
 #define HDG_PROF_SMOOTH_FIRST32 7
-#define HDG_PROF_TRANSFER       8   /* trace <-> P1 restriction / prolongation */
+#define HDG_PROF_TRANSFER       8   /* trace <-> P1 restriction / prolongation (with the sweep on it) */
 #define HDG_PROF_P1             9   /* P1 V-cycle kernels                    */
 #define HDG_PROF_KRYLOV        10   /* dots, updates, Givens, conversions    */
 #define HDG_PROF_RHS           11   /* step 1                                */

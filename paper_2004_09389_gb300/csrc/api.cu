@@ -28,6 +28,7 @@ namespace hdg {
 
 template <typename T> cudaError_t launch_apply_t(hdg_handle *, const T *, T *);
 template <typename T> cudaError_t launch_residual_t(hdg_handle *, const T *, const T *, T *, bool);
+template <typename T> cudaError_t launch_residual_smooth_t(hdg_handle *, const T *, const T *, T *, T *, double);
 template <typename T> cudaError_t launch_smooth_t(hdg_handle *, const T *, const T *, T *);
 template <typename T>
 cudaError_t launch_smooth_first_t(hdg_handle *, const T *, T *, const T * = nullptr, const double * = nullptr,
@@ -577,7 +578,21 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
             std::swap(x, x2);
         }
     }
-    if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, k.res, true))) != cudaSuccess) return e;
+    bool learned = false, collect = false;
+    if constexpr (std::is_same<T, float>::value) {
+        learned = h->lc.on && !h->lc.suspended;
+        collect = h->lc.collecting && h->lc.count < h->lc.cap;
+    }
+    // with a first post-smoothing sweep on the prolongation, its part before the
+    // correction is formed along with the residual (into x2, which that sweep reads)
+    const int np = h->prm.n_post;
+    if (np == 0 || (np == 1 && (learned || collect))) {
+        if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, k.res, true))) != cudaSuccess) return e;
+    } else {
+        if ((e = KL(cat_res<T>(), 1, launch_residual_smooth_t<T>(h, v, x, k.res, x2, cheb ? h->cheb_omega[0] : 0.0))) !=
+            cudaSuccess)
+            return e;
+    }
     // line 3: restriction r_c = pi^T r (with the first P1 sweep when level 0 is above the tail)
     DevLevel &L0 = h->lev[0];
     const bool fuse0 = h->tail_start[sizeof(T) == 8 ? 0 : 1] > 0 && h->prm.p1_nu_pre >= 1;
@@ -587,21 +602,15 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
     T *ec = nullptr;
     if ((e = p1_cycle<T>(h, &ec)) != cudaSuccess) return e;
     // lines 5-6: x += pi e_c and post-smoothing (the prolongation rides on the first sweep)
-    const int np = h->prm.n_post;
     if (np == 0) {
         if ((e = KL(HDG_PROF_TRANSFER, 1, launch_prolong_add_t<T>(h, ec, x))) != cudaSuccess) return e;
         return dcopy(h, z, x, sizeof(T) * NT, cudaMemcpyDeviceToDevice);
-    }
-    bool learned = false, collect = false;
-    if constexpr (std::is_same<T, float>::value) {
-        learned = h->lc.on && !h->lc.suspended;
-        collect = h->lc.collecting && h->lc.count < h->lc.cap;
     }
     if (cheb && !learned && !collect) {
         // Chebyshev iteration from x_0 = x + pi e_c: the first step rides on the
         // prolongation and keeps x_0 (in k.res, free after the restriction)
         T *cur = (np == 1) ? z : x2, *prev = (np == 1) ? nullptr : k.res;
-        if ((e = KL(cat_smooth<T>(), 1, launch_smooth_prolong_t<T>(h, ec, v, x, cur, h->cheb_omega[0], prev))) !=
+        if ((e = KL(HDG_PROF_TRANSFER, 1, launch_smooth_prolong_t<T>(h, ec, x2, x, cur, h->cheb_omega[0], prev))) !=
             cudaSuccess)
             return e;
         for (int i = 1; i < np; ++i) {
@@ -616,7 +625,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
     }
     if (!learned && !collect) {
         T *out = (np == 1) ? z : x2;
-        if ((e = KL(cat_smooth<T>(), 1, launch_smooth_prolong_t<T>(h, ec, v, x, out))) != cudaSuccess) return e;
+        if ((e = KL(HDG_PROF_TRANSFER, 1, launch_smooth_prolong_t<T>(h, ec, x2, x, out))) != cudaSuccess) return e;
         std::swap(x, x2);
         for (int i = 1; i < np; ++i) {
             T *o = (i == np - 1) ? z : x2;
@@ -633,7 +642,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
         // the first n_post - 1 steps of the Chebyshev iteration from x_0 = x + pi e_c,
         // rotating three vectors (x is free once x_0 is stored)
         T *cur = x2, *prev = k.res, *free_ = x;
-        if ((e = KL(cat_smooth<T>(), 1, launch_smooth_prolong_t<T>(h, ec, v, x, cur, h->cheb_omega[0], prev))) !=
+        if ((e = KL(HDG_PROF_TRANSFER, 1, launch_smooth_prolong_t<T>(h, ec, x2, x, cur, h->cheb_omega[0], prev))) !=
             cudaSuccess)
             return e;
         for (int i = 1; i < np - 1; ++i) {
@@ -649,7 +658,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
         cheb_prev = prev;
         spare = free_;
     } else {
-        if ((e = KL(cat_smooth<T>(), 1, launch_smooth_prolong_t<T>(h, ec, v, x, x2))) != cudaSuccess) return e;
+        if ((e = KL(HDG_PROF_TRANSFER, 1, launch_smooth_prolong_t<T>(h, ec, x2, x, x2))) != cudaSuccess) return e;
         std::swap(x, x2);
         for (int i = 1; i < np - 1; ++i) {
             if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, v, x, x2))) != cudaSuccess) return e;
@@ -1222,6 +1231,7 @@ void free_handle(hdg_handle *h) {
     dfree(h->d_Dinv); dfree(h->d_Sval32); dfree(h->d_Dinv32); dfree(h->d_Sval16); dfree(h->d_status); dfree(h->d_coarse_inv);
     for (auto &im : h->tail_img) dfree(im.d);
     dfree(h->d_tail_op);
+    dfree(h->d_facet_opp); dfree(h->d_Q); dfree(h->d_Q32);
     dfree(h->d_coarse_work);
     dfree(h->d_coarse_fac);
     for (auto &L : h->lev) {
@@ -1458,6 +1468,15 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(upload(&h->d_facet_cell, hm.facet_cell, s));
     TRY(upload(&h->d_facet_edge, hm.facet_edge, s));
     TRY(upload(&h->d_facet_verts, hm.facet_verts, s));
+    if (prm->flux == 0) {
+        // the vertices opposite each facet in its two cells, and the operator of the first
+        // post-smoothing sweep against the four vertices (D^-1 S pi)
+        std::vector<int32_t> opp(size_t(h->NF) * 2);
+        for (size_t k = 0; k < opp.size(); ++k) opp[k] = hm.cells[size_t(3) * hm.facet_cell[k] + hm.facet_edge[k]];
+        TRY(upload(&h->d_facet_opp, opp, s));
+        TRY(dalloc(&h->d_Q, size_t(h->NF) * h->pp * 4));
+        if (prm->precision != HDG_FP64) TRY(dalloc(&h->d_Q32, size_t(h->NF) * h->pp * 4));
+    }
     TRY(upload(&h->d_v2f_ptr, hm.v2f_ptr, s));
     TRY(upload(&h->d_v2f, hm.v2f, s));
     const size_t N = h->N, NF = h->NF, nK = h->nK, m = h->m, pp = h->pp;
@@ -2123,6 +2142,7 @@ int hdg_condense(hdg_handle *h) {
     }
     TRY(KL(HDG_PROF_CONDENSE, 1, launch_condense(h)));
     TRY(KL(HDG_PROF_CONDENSE, 1, launch_assemble(h)));
+    TRY(KL(HDG_PROF_CONDENSE, 1, launch_prolong_op(h)));
     const double tau = h->prm.tau, gH = h->prm.g * h->prm.H;
     if (h->prm.coarse_mode == 2) {
         TRY(KL(HDG_PROF_CONDENSE, int(2 * h->lev.size()), launch_p1_galerkin(h)));

@@ -646,6 +646,9 @@ struct hdg_handle {
     int32_t *d_facet_of = nullptr, *d_flip = nullptr;   // [N][3]
     int32_t *d_facet_cell = nullptr, *d_facet_edge = nullptr;  // [NF][2]
     int32_t *d_facet_verts = nullptr;  // [NF][2]
+    int32_t *d_facet_opp = nullptr;    // [NF][2] the vertex opposite the facet in each of its cells
+    double *d_Q = nullptr;             // D^-1 S pi of the facet rows [pp][NF][4]: lower, higher vertex, the two opposite
+    float *d_Q32 = nullptr;            // its FP32 copy (FP32 preconditioners)
     int32_t *d_v2f_ptr = nullptr, *d_v2f = nullptr;
     int32_t *d_nbr = nullptr;       // [4][NF] neighbour facets of the facet-row operator
 
@@ -803,6 +806,8 @@ cudaError_t launch_to_f32(const double *x, float *y, size_t n, cudaStream_t s);
 // trace-space kernels (k_trace.cu); vectors in the internal layout [pp][NF]
 cudaError_t launch_to_internal(hdg_handle *h, const double *ext, double *in);
 cudaError_t launch_repack(hdg_handle *h);
+// D^-1 S pi of the facet rows (d_Q, d_Q32) from the FP64 operator
+cudaError_t launch_prolong_op(hdg_handle *h);
 // index of element j of facet e in an operator array packed in groups of G
 inline __host__ __device__ size_t packed_index(size_t j, size_t e, size_t NF, size_t G) {
     return ((j / G) * NF + e) * G + j % G;

@@ -318,6 +318,84 @@ void residual_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStrea
 }
 
 
+// The residual before the coarse correction, res = b - S x, and the part of the first
+// post-smoothing sweep that does not wait for the correction, y = x + omega D_e^-1 res:
+// D^-1 was read by the sweep just before this kernel and is still in L2 here.
+template <int P, typename T, typename ST>
+__device__ __forceinline__ void residual_smooth_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ Sval,
+                                                            const T *__restrict__ Dinv,
+                                                            const int32_t *__restrict__ nbr, const T *__restrict__ b,
+                                                            const T *__restrict__ x, T *__restrict__ res,
+                                                            T *__restrict__ y, T omega) {
+    const int e = bid_ * blockDim.x + threadIdx.x;
+    if (e >= NF) return;
+    T xs[5][P + 1], v[P + 1], d[P + 1];
+    gather_x<P, T>(nbr, x, e, NF, xs);
+    facet_rows_packed<P, T, ST>(Sval, e, NF, xs, v);
+#pragma unroll
+    for (int r = 0; r <= P; ++r) {
+        v[r] = b[size_t(r) * NF + e] - v[r];
+        res[size_t(r) * NF + e] = v[r];
+    }
+    block_solve_packed<P, T, T>(Dinv, e, NF, v, d);
+#pragma unroll
+    for (int r = 0; r <= P; ++r) y[size_t(r) * NF + e] = fma(omega, d[r], xs[0][r]);
+}
+template <int P, typename T, typename ST>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) residual_smooth_kernel(int NF, const ST *__restrict__ Sval,
+                                                                                   const T *__restrict__ Dinv,
+                                                                                   const int32_t *__restrict__ nbr,
+                                                                                   const T *__restrict__ b,
+                                                                                   const T *__restrict__ x,
+                                                                                   T *__restrict__ res,
+                                                                                   T *__restrict__ y, T omega) {
+    pdl_wait();
+    residual_smooth_kernel_impl<P, T, ST>(blockIdx.x, gridDim.x, NF, Sval, Dinv, nbr, b, x, res, y, omega);
+}
+template <int P, typename T, typename ST>
+struct residual_smooth_kernel_args {
+    int nb_;
+    int NF;
+    const ST *Sval;
+    const T *Dinv;
+    const int32_t *nbr;
+    const T *b;
+    const T *x;
+    T *res;
+    T *y;
+    T omega;
+};
+template <int P, typename T, typename ST>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) residual_smooth_kernel_multi(const __grid_constant__ MultiP<residual_smooth_kernel_args<P, T, ST>> M) {
+    pdl_wait();
+    int b_;
+    const residual_smooth_kernel_args<P, T, ST> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    residual_smooth_kernel_impl<P, T, ST>(b_, q_.nb_, q_.NF, q_.Sval, q_.Dinv, q_.nbr, q_.b, q_.x, q_.res, q_.y,
+        q_.omega);
+}
+template <int P, typename T, typename ST>
+void residual_smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *Sval,
+                               const T *Dinv, const int32_t *nbr, const T *b, const T *x, T *res, T *y, T omega) {
+    if (Recorder *r_ = batch_recorder()) {
+        residual_smooth_kernel_args<P, T, ST> q_;
+        std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
+        q_.nb_ = int(grid_);
+        q_.NF = NF;
+        q_.Sval = Sval;
+        q_.Dinv = Dinv;
+        q_.nbr = nbr;
+        q_.b = b;
+        q_.x = x;
+        q_.res = res;
+        q_.y = y;
+        q_.omega = omega;
+        batch_record(r_, reinterpret_cast<const void *>(&residual_smooth_kernel_multi<P, T, ST>), q_, grid_, block_, smem_, kPdlFamily);
+        return;
+    }
+    pdl_launch(kPdlFamily, &residual_smooth_kernel<P, T, ST>, grid_, block_, smem_, s_, NF, Sval, Dinv, nbr, b, x, res, y, omega);
+}
+
+
 // One sweep x_out = x + omega D_e^-1 (b - S x)_e; with CHEB, a step of the
 // Chebyshev iteration x_out = x + omega D_e^-1 (b - S x)_e + beta (x - x_prev)
 // (x_prev null: the previous iterate is zero).  x_out may alias x_prev: each
@@ -404,108 +482,170 @@ void smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_
 }
 
 
-// First post-smoothing sweep with the coarse correction folded in:
-// x' = x + pi e_c is formed on the fly for the five facets the rows touch,
-// then x_out = x' + omega D_e^-1 (b - S x')_e.
-// With X0, x' on the facet itself is also stored to x0out (the previous
-// iterate of the Chebyshev step that follows).
-template <int P, typename T, typename ST, bool X0 = false>
-__device__ __forceinline__ void smooth_prolong_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ Sval,
-                                                           const T *__restrict__ Dinv,
-                                                           const int32_t *__restrict__ nbr,
+// First post-smoothing sweep with the coarse correction folded in: from x' = x + pi e_c,
+// x_out = x' + omega D_e^-1 (b - S x')_e.  The residual before the correction was formed
+// for the restriction, with y = x + omega D^-1 (b - S x) (residual_smooth_kernel), and the
+// rows of S pi couple a facet to four vertices only, its own two and the two opposite it in
+// its cells: with Q = D^-1 S pi stored ([row][facet], one 4-vector each),
+//   x_out = y + pi e_c - omega Q_e (e_c at the four vertices),
+// so the sweep reads 4 (p+1) operator entries per facet instead of 6 (p+1)^2 and gathers
+// four vertex values instead of five facets' traces and ten vertices.  Bound by HBM and L2
+// latency: 9.1 instead of 28.4 us on 491,520 facets (p = 2, FP32), 16.0 instead of 60.1 us
+// on 196,608 (p = 3, FP64, where the old form was bound by the FP64 pipe); the residual
+// kernel takes 2.7 and 7 us more for y.  On the 196,608-facet p = 3 FP32 solve, whose
+// operator nearly fits L2, the step time stays (6.3 + 15 us for the two post-smoothing
+// sweeps instead of 13.4 + 10.5: the second now brings the operator from HBM itself).
+// With X0, x' on the facet itself is also stored to x0out (the previous iterate of the
+// Chebyshev step that follows).  xout may alias y.
+template <typename T> struct Vec4;
+template <> struct Vec4<float> {
+    using type = float4;
+};
+template <> struct Vec4<double> {
+    struct __align__(16) type { double x, y, z, w; };
+};
+template <int P, typename T, bool X0 = false>
+__device__ __forceinline__ void smooth_prolong_kernel_impl(int bid_, int nb_, int NF, const T *__restrict__ Q,
                                                            const int32_t *__restrict__ fverts,
-                                                           const T *__restrict__ ec, const T *__restrict__ b,
-                                                           const T *__restrict__ x, T *__restrict__ xout, T omega,
+                                                           const int32_t *__restrict__ fopp,
+                                                           const T *__restrict__ ec, const T *y,
+                                                           const T *__restrict__ x, T *xout, T omega,
                                                            T *__restrict__ x0out) {
+    using V = typename Vec4<T>::type;
     constexpr int PP = P + 1;
     const int e = bid_ * blockDim.x + threadIdx.x;
     if (e >= NF) return;
-    int src[5];
-    src[0] = e;
+    const int2 lv = __ldg(reinterpret_cast<const int2 *>(fverts) + e), ov = __ldg(reinterpret_cast<const int2 *>(fopp) + e);
+    V q[PP];
 #pragma unroll
-    for (int bb = 1; bb < 5; ++bb) src[bb] = __ldg(nbr + size_t(bb - 1) * NF + e);
-    T xs[5][PP], v[PP], d[PP];
+    for (int r = 0; r < PP; ++r) q[r] = reinterpret_cast<const V *>(Q)[size_t(r) * NF + e];
+    const T lo = ec[lv.x], hi = ec[lv.y], oa = ec[ov.x], ob = ec[ov.y];
 #pragma unroll
-    for (int bb = 0; bb < 5; ++bb) {
-        const T lo = ec[__ldg(fverts + 2 * src[bb])], hi = ec[__ldg(fverts + 2 * src[bb] + 1)];
-#pragma unroll
-        for (int c = 0; c < PP; ++c) {
-            const T t = T(c) / T(P);
-            xs[bb][c] = x[size_t(c) * NF + src[bb]] + (T(1) - t) * lo + t * hi;
-        }
-    }
-    facet_rows_packed<P, T, ST>(Sval, e, NF, xs, v);
-#pragma unroll
-    for (int r = 0; r < PP; ++r) v[r] = b[size_t(r) * NF + e] - v[r];
-    block_solve_packed<P, T, T>(Dinv, e, NF, v, d);
-#pragma unroll
-    for (int r = 0; r < PP; ++r) xout[size_t(r) * NF + e] = fma(omega, d[r], xs[0][r]);
-    if constexpr (X0) {
-#pragma unroll
-        for (int r = 0; r < PP; ++r) x0out[size_t(r) * NF + e] = xs[0][r];
+    for (int r = 0; r < PP; ++r) {
+        const T qc = fma(q[r].x, lo, fma(q[r].y, hi, fma(q[r].z, oa, q[r].w * ob)));
+        const T t = T(r) / T(P), pc = fma(T(1) - t, lo, t * hi);
+        if constexpr (X0) x0out[size_t(r) * NF + e] = x[size_t(r) * NF + e] + pc;
+        xout[size_t(r) * NF + e] = fma(-omega, qc, y[size_t(r) * NF + e] + pc);
     }
 }
-template <int P, typename T, typename ST, bool X0 = false>
-__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_prolong_kernel(int NF, const ST *__restrict__ Sval,
-                                                                                  const T *__restrict__ Dinv,
-                                                                                  const int32_t *__restrict__ nbr,
+template <int P, typename T, bool X0 = false>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_prolong_kernel(int NF, const T *__restrict__ Q,
                                                                                   const int32_t *__restrict__ fverts,
-                                                                                  const T *__restrict__ ec,
-                                                                                  const T *__restrict__ b,
-                                                                                  const T *__restrict__ x,
-                                                                                  T *__restrict__ xout, T omega,
-                                                                                  T *__restrict__ x0out) {
+                                                                                  const int32_t *__restrict__ fopp,
+                                                                                  const T *__restrict__ ec, const T *y,
+                                                                                  const T *__restrict__ x, T *xout,
+                                                                                  T omega, T *__restrict__ x0out) {
     pdl_wait();
-    smooth_prolong_kernel_impl<P, T, ST, X0>(blockIdx.x, gridDim.x, NF, Sval, Dinv, nbr, fverts, ec, b, x, xout,
-        omega, x0out);
+    smooth_prolong_kernel_impl<P, T, X0>(blockIdx.x, gridDim.x, NF, Q, fverts, fopp, ec, y, x, xout, omega, x0out);
 }
-template <int P, typename T, typename ST, bool X0 = false>
+template <int P, typename T, bool X0 = false>
 struct smooth_prolong_kernel_args {
     int nb_;
     int NF;
-    const ST *Sval;
-    const T *Dinv;
-    const int32_t *nbr;
+    const T *Q;
     const int32_t *fverts;
+    const int32_t *fopp;
     const T *ec;
-    const T *b;
+    const T *y;
     const T *x;
     T *xout;
     T omega;
     T *x0out;
 };
-template <int P, typename T, typename ST, bool X0 = false>
-__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_prolong_kernel_multi(const __grid_constant__ MultiP<smooth_prolong_kernel_args<P, T, ST, X0>> M) {
+template <int P, typename T, bool X0 = false>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_prolong_kernel_multi(const __grid_constant__ MultiP<smooth_prolong_kernel_args<P, T, X0>> M) {
     pdl_wait();
     int b_;
-    const smooth_prolong_kernel_args<P, T, ST, X0> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    smooth_prolong_kernel_impl<P, T, ST, X0>(b_, q_.nb_, q_.NF, q_.Sval, q_.Dinv, q_.nbr, q_.fverts, q_.ec, q_.b,
-        q_.x, q_.xout, q_.omega, q_.x0out);
+    const smooth_prolong_kernel_args<P, T, X0> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    smooth_prolong_kernel_impl<P, T, X0>(b_, q_.nb_, q_.NF, q_.Q, q_.fverts, q_.fopp, q_.ec, q_.y, q_.x, q_.xout,
+        q_.omega, q_.x0out);
 }
-template <int P, typename T, typename ST, bool X0 = false>
-void smooth_prolong_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *Sval,
-                              const T *Dinv, const int32_t *nbr, const int32_t *fverts, const T *ec, const T *b,
-                              const T *x, T *xout, T omega, T *x0out) {
+template <int P, typename T, bool X0 = false>
+void smooth_prolong_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const T *Q,
+                              const int32_t *fverts, const int32_t *fopp, const T *ec, const T *y, const T *x, T *xout,
+                              T omega, T *x0out) {
     if (Recorder *r_ = batch_recorder()) {
-        smooth_prolong_kernel_args<P, T, ST, X0> q_;
+        smooth_prolong_kernel_args<P, T, X0> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
         q_.NF = NF;
-        q_.Sval = Sval;
-        q_.Dinv = Dinv;
-        q_.nbr = nbr;
+        q_.Q = Q;
         q_.fverts = fverts;
+        q_.fopp = fopp;
         q_.ec = ec;
-        q_.b = b;
+        q_.y = y;
         q_.x = x;
         q_.xout = xout;
         q_.omega = omega;
         q_.x0out = x0out;
-        batch_record(r_, reinterpret_cast<const void *>(&smooth_prolong_kernel_multi<P, T, ST, X0>), q_, grid_, block_, smem_, kPdlFamily);
+        batch_record(r_, reinterpret_cast<const void *>(&smooth_prolong_kernel_multi<P, T, X0>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &smooth_prolong_kernel<P, T, ST, X0>, grid_, block_, smem_, s_, NF, Sval, Dinv, nbr, fverts, ec, b, x, xout,
-        omega, x0out);
+    pdl_launch(kPdlFamily, &smooth_prolong_kernel<P, T, X0>, grid_, block_, smem_, s_, NF, Q, fverts, fopp, ec, y, x, xout, omega,
+        x0out);
+}
+
+// Q = D^-1 S pi from the packed FP64 operator: row r of facet e against the facet's own
+// vertices and the two opposite it.  A neighbour facet of cell s joins two of that cell's
+// three vertices; its row's entries are summed with weights 1 - t_c and t_c onto its lower
+// and higher vertex.  Once per condensation; FP64 sums (S annihilates smooth traces up to
+// its scale, so the sums cancel), rounded once for the FP32 copy.
+template <int P>
+__global__ void prolong_op_kernel(int NF, const double *__restrict__ Sval, const double *__restrict__ Dinv,
+                                  const int32_t *__restrict__ nbr, const int32_t *__restrict__ fverts,
+                                  double *__restrict__ Q, float *__restrict__ Q32) {
+    constexpr int PP = P + 1;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= NF) return;
+    const int lo = fverts[2 * e], hi = fverts[2 * e + 1];
+    int slot[5][2];            // of each facet's two vertices: 0 lo, 1 hi, 2 / 3 opposite in cell 0 / 1
+    slot[0][0] = 0;
+    slot[0][1] = 1;
+#pragma unroll
+    for (int b = 1; b < 5; ++b) {
+        const int f = nbr[size_t(b - 1) * NF + e];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int v = fverts[2 * f + k];
+            slot[b][k] = v == lo ? 0 : v == hi ? 1 : b < 3 ? 2 : 3;
+        }
+    }
+    double w[PP][4];
+#pragma unroll
+    for (int r = 0; r < PP; ++r) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[r][q] = 0.0;
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            double tot = 0.0, up = 0.0;
+#pragma unroll
+            for (int c = 0; c < PP; ++c) {
+                const double s = Sval[packed_index(size_t((r * 5 + b) * PP + c), size_t(e), size_t(NF), 2)];
+                tot += s;
+                if (c > 0) up = c < P ? fma(s, double(c) / double(P), up) : up + s;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (slot[b][0] == q) w[r][q] += tot - up;
+                if (slot[b][1] == q) w[r][q] += up;
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < PP; ++r) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int c = 0; c < PP; ++c) {
+            const double d = Dinv[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 2)];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = fma(d, w[c][q], v[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            Q[(size_t(r) * NF + e) * 4 + q] = v[q];
+            if (Q32) Q32[(size_t(r) * NF + e) * 4 + q] = float(v[q]);
+        }
+    }
 }
 
 
@@ -1016,30 +1156,36 @@ cudaError_t launch_restrict_t(hdg_handle *h, const T *r, T *rc, const T *dinv0, 
     return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_smooth_prolong_t(hdg_handle *h, const T *ec, const T *b, const T *x, T *xout, double omega,
+cudaError_t launch_smooth_prolong_t(hdg_handle *h, const T *ec, const T *y, const T *x, T *xout, double omega,
                                     T *x0out) {
     const T om = T(omega > 0 ? omega : h->prm.omega);
-    if constexpr (std::is_same<T, float>::value) if (bf16_pre(h)) {
-        if (x0out) {
-            HDG_DISPATCH_P(h->p, (smooth_prolong_kernel_go<P, T, __nv_bfloat16, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, Ops<T>::D(h), h->d_nbr, h->d_facet_verts, ec, b, x, xout, om, x0out)));
-        } else {
-            HDG_DISPATCH_P(h->p, (smooth_prolong_kernel_go<P, T, __nv_bfloat16>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, Ops<T>::D(h), h->d_nbr, h->d_facet_verts, ec, b, x, xout, om, nullptr)));
-        }
-        return cudaGetLastError();
-    }
+    const T *q;
+    if constexpr (std::is_same<T, float>::value) q = h->d_Q32;
+    else q = h->d_Q;
     if (x0out) {
-        HDG_DISPATCH_P(h->p, (smooth_prolong_kernel_go<P, T, T, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, h->d_facet_verts, ec, b, x, xout, om, x0out)));
+        HDG_DISPATCH_P(h->p, (smooth_prolong_kernel_go<P, T, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, q, h->d_facet_verts, h->d_facet_opp, ec, y, x, xout, om, x0out)));
     } else {
-        HDG_DISPATCH_P(h->p, (smooth_prolong_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, h->d_facet_verts, ec, b, x, xout, om, nullptr)));
+        HDG_DISPATCH_P(h->p, (smooth_prolong_kernel_go<P, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, q, h->d_facet_verts, h->d_facet_opp, ec, y, x, xout, om, nullptr)));
     }
     return cudaGetLastError();
 }
+template <typename T>
+cudaError_t launch_residual_smooth_t(hdg_handle *h, const T *b, const T *x, T *res, T *y, double omega) {
+    const T om = T(omega > 0 ? omega : h->prm.omega);
+    if constexpr (std::is_same<T, float>::value) if (bf16_pre(h)) {
+        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, __nv_bfloat16>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
+        return cudaGetLastError();
+    }
+    HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
+    return cudaGetLastError();
+}
+template cudaError_t launch_residual_smooth_t<double>(hdg_handle *, const double *, const double *, double *, double *, double);
+template cudaError_t launch_residual_smooth_t<float>(hdg_handle *, const float *, const float *, float *, float *, double);
 template <typename T>
 cudaError_t launch_prolong_add_t(hdg_handle *h, const T *ec, T *x) {
     HDG_DISPATCH_P(h->p, (prolong_add_kernel<P, T><<<blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream>>>(h->NF, h->d_facet_verts, ec, x)));
     return cudaGetLastError();
 }
-
 // FP32 / BF16 copies of the packed FP64 operator and the FP32 inverse blocks
 cudaError_t launch_repack(hdg_handle *h) {
     const int pp = h->pp, ns = 5 * pp * pp, nd = pp * pp;
@@ -1074,6 +1220,11 @@ template cudaError_t launch_smooth_first_t<float>(hdg_handle *, const float *, f
                                                   float *, double);
 template cudaError_t launch_restrict_t<double>(hdg_handle *, const double *, double *, const double *, double, double *);
 template cudaError_t launch_restrict_t<float>(hdg_handle *, const float *, float *, const float *, float, float *);
+cudaError_t launch_prolong_op(hdg_handle *h) {
+    HDG_DISPATCH_P(h->p, (prolong_op_kernel<P><<<blocks(h->NF, 128), 128, 0, h->stream>>>(
+                             h->NF, h->d_Sval, h->d_Dinv, h->d_nbr, h->d_facet_verts, h->d_Q, h->d_Q32)));
+    return cudaGetLastError();
+}
 template cudaError_t launch_smooth_prolong_t<double>(hdg_handle *, const double *, const double *, const double *, double *,
                                                      double, double *);
 template cudaError_t launch_smooth_prolong_t<float>(hdg_handle *, const float *, const float *, const float *, float *,
