@@ -37,7 +37,7 @@ template <typename T>
 cudaError_t launch_smooth_cheb_t(hdg_handle *, const T *, const T *, T *, double, double, const T *);
 template <typename T>
 cudaError_t launch_apply_dots_t(hdg_handle *, const T *, T *, const T *, size_t, int, double *, unsigned int *,
-                                double *);
+                                double *, T *);
 template <typename T> cudaError_t launch_restrict_t(hdg_handle *, const T *, T *, const T *, T, T *);
 template <typename T>
 cudaError_t launch_smooth_prolong_t(hdg_handle *, const T *, const T *, const T *, T *, double = 0.0, T * = nullptr);
@@ -73,6 +73,7 @@ struct Workspace {
     KSpace<float> k32;
     // small device arrays
     double *Hm = nullptr, *cs = nullptr, *sn = nullptr, *sv = nullptr, *h1 = nullptr, *h2 = nullptr;
+    double *hneg = nullptr, *rot = nullptr;    // -h1 in the vector type; the rotated entry h_jj and 1 / ||b|| of a step
     double *nrm2 = nullptr, *est = nullptr, *y = nullptr, *partial = nullptr;
     double *scal = nullptr;   // restart normalisation of a Krylov cycle
     double *bnorm = nullptr;  // ||b|| of the current Krylov solve
@@ -793,12 +794,14 @@ cudaError_t arnoldi_step(hdg_handle *h, int j, const T *src0 = nullptr) {
         if (e != cudaSuccess) return e;
     }
     // w = S z_j with the first Gram-Schmidt pass h1 = V^T w in the same kernel
-    if ((e = KL(cat_apply<T>(), 1, launch_apply_dots_t<T>(h, zj, k.w, k.V, ld, j + 1, W.partial, W.counter, W.h1))) !=
+    if ((e = KL(cat_apply<T>(), 1, launch_apply_dots_t<T>(h, zj, k.w, k.V, ld, j + 1, W.partial, W.counter, W.h1,
+                                                                reinterpret_cast<T *>(W.hneg)))) !=
         cudaSuccess)
         return e;
     const bool reorth = h->prm.reorth != 0;
     if ((e = KL(HDG_PROF_KRYLOV, 1 + (reorth ? 1 : 0) + (fuse_scale ? 0 : 1),
-                launch_gs_step<T>(k.V, ld, j, k.w, W.partial, W.counter, W.nblk_gs, W.h1, W.h2, W.nrm2, W.Hm, ldh,
+                launch_gs_step<T>(k.V, ld, j, k.w, W.partial, W.counter, W.nblk_gs, W.h1, W.h2,
+                                  reinterpret_cast<const T *>(W.hneg), W.rot, W.nrm2, W.Hm, ldh,
                                   W.cs, W.sn, W.sv, W.bnorm, W.rb, W.host_rb_dev + j, k.V + size_t(j + 1) * ld, reorth,
                                   !fuse_scale, s))) != cudaSuccess)
         return e;
@@ -1249,7 +1252,7 @@ void free_handle(hdg_handle *h) {
         dfree(W.k64.V); dfree(W.k64.Z); dfree(W.k64.w); dfree(W.k64.t0); dfree(W.k64.t1); dfree(W.k64.res);
         dfree(W.k32.V); dfree(W.k32.Z); dfree(W.k32.w); dfree(W.k32.t0); dfree(W.k32.t1); dfree(W.k32.res);
         dfree(W.k32.b); dfree(W.k32.x);
-        dfree(W.Hm); dfree(W.cs); dfree(W.sn); dfree(W.sv); dfree(W.h1); dfree(W.h2); dfree(W.nrm2);
+        dfree(W.Hm); dfree(W.cs); dfree(W.sn); dfree(W.sv); dfree(W.h1); dfree(W.h2); dfree(W.hneg); dfree(W.rot); dfree(W.nrm2);
         dfree(W.est); dfree(W.counter); dfree(W.rb);
         if (W.host_rb) cudaFreeHost(W.host_rb);
         if (W.host_val) cudaFreeHost(W.host_val);
@@ -1693,6 +1696,8 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(dalloc(&W.sv, mm + 1));
     TRY(dalloc(&W.h1, mm + 1));
     TRY(dalloc(&W.h2, mm + 1));
+    TRY(dalloc(&W.hneg, mm + 1));
+    TRY(dalloc(&W.rot, 2));
     TRY(dalloc(&W.nrm2, 1));
     TRY(dalloc(&W.est, 1));
     TRY(dalloc(&W.scal, 1));

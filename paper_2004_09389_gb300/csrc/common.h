@@ -284,6 +284,50 @@ struct ReadBack {
 };
 
 #ifdef __CUDACC__
+// Sums over a warp of V values per lane (V a power of two <= 32): lane groups exchange
+// halves, keeping half of the values each time (V - 1 adds), then the tree over the
+// lanes left (log2(32 / V) adds), instead of 5 V: an FP64 add takes a scheduler's pipe
+// about 77 cycles here.  Returns the sum of value `which`, complete in every lane of its
+// group of 32 / V lanes.
+template <int V, typename A>
+__device__ __forceinline__ A warp_sums(A (&a)[V], int &which) {
+    const int lane = threadIdx.x & 31;
+    which = 0;
+#pragma unroll
+    for (int h = V / 2, off = 16; h > 0; h /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int r = 0; r < h; ++r) {
+            const A send = up ? a[r] : a[r + h], mine = up ? a[r + h] : a[r];
+            a[r] = mine + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+        which = 2 * which + (up ? 1 : 0);
+    }
+    A t = a[0];
+#pragma unroll
+    for (int off = 16 / V; off > 0; off /= 2) t += __shfl_xor_sync(0xffffffffu, t, off);
+    return t;
+}
+
+// y = R^-1 s for the k x k upper triangle R (row-major, leading dimension k, k <= 64) in
+// shared memory, by one whole warp: the diagonal's reciprocals at once, then column by
+// column, every row's update of a step in parallel (one product and two FMAs deep per
+// step; a single thread's substitution took k^2 / 2 dependent FMAs and k divisions:
+// 10.3 us at k = 12)
+__device__ __forceinline__ void hess_back_substitute(const double *R, const double *s, double *y, int k) {
+    const int lane = threadIdx.x & 31, i1 = lane + 32;
+    double t0 = lane < k ? s[lane] : 0.0, t1 = i1 < k ? s[i1] : 0.0;
+    const double r0 = lane < k ? 1.0 / R[lane * k + lane] : 0.0;
+    const double r1 = i1 < k ? 1.0 / R[i1 * k + i1] : 0.0;
+    for (int l = k - 1; l >= 0; --l) {
+        const double yl = __shfl_sync(0xffffffffu, l < 32 ? t0 * r0 : t1 * r1, l & 31);
+        if (lane == (l & 31)) y[l] = yl;
+        if (lane < l) t0 = fma(-R[lane * k + l], yl, t0);
+        if (i1 < l) t1 = fma(-R[i1 * k + l], yl, t1);
+    }
+    __syncwarp();
+}
+
 // f(integral_constant<int, 0>) ... f(integral_constant<int, N - 1>): a loop whose
 // index is a constant expression in the body (zero entries left out at compile time)
 template <class F, int... I>
@@ -923,9 +967,9 @@ template <typename T>
 cudaError_t launch_fill(T *x, T v, size_t n, cudaStream_t s);
 template <typename T>
 cudaError_t launch_gs_step(const T *V, size_t ld, int j, T *w, double *partial, unsigned int *counter, int nblk,
-                           double *h1, double *h2, double *nrm2, double *Hm, int ldh, double *cs, double *sn,
-                           double *sv, const double *bnorm, ReadBack *rb, ReadBack *host_rb, T *vnext, bool reorth, bool scale,
-                           cudaStream_t s);
+                           double *h1, double *h2, const T *hneg, double *rot, double *nrm2, double *Hm, int ldh,
+                           double *cs, double *sn, double *sv, const double *bnorm, ReadBack *rb, ReadBack *host_rb,
+                           T *vnext, bool reorth, bool scale, cudaStream_t s);
 int learned_n_params(int p, int hid);
 cudaError_t launch_learned_infer(hdg_handle *h, const float *r, const float *x, float *xout);
 cudaError_t launch_learned_infer_tc(hdg_handle *h, const float *r, const float *x, float *xout);

@@ -133,7 +133,7 @@ void ff_axpy_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream
 
 // The end of the last cycle of an inner solve of the mixed refinement, in one
 // pass: y = R^-1 s for the leading k x k triangle of the rotated Hessenberg
-// matrix (column-major, leading dimension ldh), solved by one thread of every
+// matrix (column-major, leading dimension ldh), solved by one warp of every
 // block with the substitution of the separate triangular-solve kernel; d = x +
 // sum_c y_c Z_c with the FP32 sums of the separate basis update (x null: the
 // inner iterate is still zero); then the refinement iterate's pairs +=
@@ -166,14 +166,8 @@ __device__ __forceinline__ void ff_finish_kernel_impl(int bid_, int nb_, const d
     }
     for (int i = threadIdx.x; i < k; i += blockDim.x) sS[i] = sv[i];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = k - 1; i >= 0; --i) {
-            double t = sS[i];
-            for (int l = i + 1; l < k; ++l) t -= R[i * k + l] * yS[l];
-            yS[i] = t / R[i * k + i];
-        }
-        sc = split(scl);
-    }
+    if (threadIdx.x < 32) hess_back_substitute(R, sS, yS, k);
+    else if (threadIdx.x == 32) sc = split(scl);
     __syncthreads();
     for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = float(1.0 * yS[i]);
     __syncthreads();

@@ -311,24 +311,20 @@ void scale_copy_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStr
 
 // y = R^-1 s for the leading k x k upper triangle R of the rotated Hessenberg
 // matrix (column-major, leading dimension ldh): the triangle and s are first
-// loaded into shared memory by the whole block, then one thread substitutes
-// backwards (k <= 64)
+// loaded into shared memory by the whole block, then one warp substitutes
+// backwards (hess_back_substitute; k <= 64)
 __device__ __forceinline__ void hessenberg_solve_kernel_impl(int bid_, int nb_, const double *Hm, int ldh,
                                                              const double *sv, int k, double *y) {
-    __shared__ double R[64][65], sS[64], yS[64];
+    __shared__ double R[64 * 64], sS[64], yS[64];
     for (int t = threadIdx.x; t < k * k; t += blockDim.x) {
         const int l = t / k, i = t % k;            // column l, row i
-        if (i <= l) R[i][l] = Hm[size_t(l) * ldh + i];
+        if (i <= l) R[i * k + l] = Hm[size_t(l) * ldh + i];
     }
     for (int i = threadIdx.x; i < k; i += blockDim.x) sS[i] = sv[i];
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    for (int i = k - 1; i >= 0; --i) {
-        double s = sS[i];
-        for (int l = i + 1; l < k; ++l) s -= R[i][l] * yS[l];
-        yS[i] = s / R[i][i];
-        y[i] = yS[i];
-    }
+    if (threadIdx.x >= 32) return;
+    hess_back_substitute(R, sS, yS, k);
+    for (int i = threadIdx.x; i < k; i += 32) y[i] = yS[i];
 }
 __global__ void hessenberg_solve_kernel(const double *Hm, int ldh, const double *sv, int k, double *y) {
     pdl_wait();
@@ -661,16 +657,25 @@ __global__ void __launch_bounds__(256) gs_update_dots_kernel(const T *V, size_t 
     dots_and_finish<T>(V4p, ld4, k, w4, n4, partial, counter, h2, &last);
 }
 
-// w -= V h2 (h2 null: w -= V h1, one classical Gram-Schmidt pass) and
+// w -= V h2 (h2 null: w -= V h1, one classical Gram-Schmidt pass, whose coefficients
+// -h1 in the vector type come with w from the operator kernel: hneg) and
 // ||w||^2 in the same pass; the last block adds the per-block partials and
 // forms Hessenberg column j (h1 + h2, or h1 alone;
 // h_{j+1,j} = ||w||), applies the previous Givens rotations, forms rotation j,
 // updates the least-squares right-hand side and writes the residual
 // estimate |s_{j+1}| / ||b|| and the flags (2: breakdown, 4: NaN/Inf) to rb.
+// Latency bounds it: scalar FP64 operations take about 80 cycles each here and a division,
+// square root or hypot hundreds.  So what does not wait for the norm (the previous
+// rotations on h, 1 / ||b||) is done by a ninth warp of block 0 while the others update,
+// and only one square root, one reciprocal square root and a few products follow the last
+// partial.  FP64 on 768 facets 12.7 -> 11.3 us (25.1 -> 23.6 on 196,608 at p = 3);
+// what is left is the chain of grid-wide steps: partial, fence, count, sum, publication.
+constexpr int kGsThreads = 256;               // threads that update; block 0 takes 32 more
 template <typename T>
 __device__ __forceinline__ void gs_update_norm_givens_kernel_impl(int bid_, int nb_, const T *V, size_t ld, int k,
                                                                   T *w, size_t n, const double *h1, const double *h2,
-                                                                  double *partial, unsigned int *counter,
+                                                                  const T *hneg, double *partial,
+                                                                  unsigned int *counter, double *rot,
                                                                   double *nrm2, double *Hm, int ldh, double *cs,
                                                                   double *sn, double *sv, int j, const double *bnorm,
                                                                   ReadBack *rb, ReadBack *host_rb) {
@@ -679,107 +684,143 @@ __device__ __forceinline__ void gs_update_norm_givens_kernel_impl(int bid_, int 
     const size_t ld4 = ld / (16 / sizeof(T)), n4 = n / (16 / sizeof(T));
     const V4 *V4p = reinterpret_cast<const V4 *>(V);
     V4 *w4 = reinterpret_cast<V4 *>(w);
-    const double *c = h2 ? h2 : h1;
+    constexpr int nwarp = kGsThreads / 32;
     __shared__ T cs_[66];
-    __shared__ A red[32];
-    __shared__ double redd[32];
+    __shared__ A red[nwarp];
+    __shared__ double redd[nwarp];
     __shared__ bool last;
-    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, nwarp = blockDim.x / 32;
-    for (int i = threadIdx.x; i < k; i += blockDim.x) cs_[i] = T(-c[i]);
-    __syncthreads();
-    // the update and ||w||^2 in one pass: each updated value is squared from registers
-    A nrm = A(0);
-    for (size_t idx = size_t(bid_) * blockDim.x + threadIdx.x; idx < n4; idx += size_t(nb_) * blockDim.x) {
-        V4 acc = w4[idx];
-        for (int i = 0; i < k; ++i) acc = V16<T>::axpy(cs_[i], V4p[size_t(i) * ld4 + idx], acc);
-        w4[idx] = acc;
-        nrm += V16<T>::dot(acc, acc);
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    double *col = Hm + size_t(j) * ldh;
+    if (h2) {
+        for (int i = threadIdx.x; i < k; i += blockDim.x) cs_[i] = T(-h2[i]);
+        __syncthreads();
     }
-    for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
-    if (lane == 0) red[warp] = nrm;
+    const T *c = h2 ? cs_ : hneg;
+    if (warp == nwarp) {
+        // the previous rotations on the column (its entries and the rotations one load
+        // each), the rotated entries into Hm, the last one and 1 / ||b|| into rot
+        if (bid_ == 0) {
+            __shared__ double colS[66], csS[66], snS[66];
+            for (int i = lane; i <= j; i += 32) colS[i] = h2 ? h1[i] + h2[i] : h1[i];
+            for (int i = lane; i < j; i += 32) {
+                csS[i] = cs[i];
+                snS[i] = sn[i];
+            }
+            const double ib = lane == 1 ? 1.0 / bnorm[0] : 0.0;
+            __syncwarp();
+            if (lane == 0) {
+                double a = colS[0];
+                for (int i = 0; i < j; ++i) {
+                    const double ci = csS[i], si = snS[i], nx = colS[i + 1];
+                    colS[i] = ci * a + si * nx;
+                    a = -si * a + ci * nx;
+                }
+                rot[0] = a;
+            }
+            if (lane == 1) rot[1] = ib;
+            __syncwarp();
+            for (int i = lane; i < j; i += 32) col[i] = colS[i];
+            __threadfence();                   // visible before this block's count
+        }
+    } else {
+        // the update and ||w||^2 in one pass: each updated value is squared from registers
+        A nrm = A(0);
+        for (size_t idx = size_t(bid_) * kGsThreads + threadIdx.x; idx < n4; idx += size_t(nb_) * kGsThreads) {
+            V4 acc = w4[idx];
+#pragma unroll 4
+            for (int i = 0; i < k; ++i) acc = V16<T>::axpy(c[i], V4p[size_t(i) * ld4 + idx], acc);
+            w4[idx] = acc;
+            nrm += V16<T>::dot(acc, acc);
+        }
+        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+        if (lane == 0) red[warp] = nrm;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        A t = A(0);
-        for (int q = 0; q < nwarp; ++q) t += red[q];
-        partial[bid_] = double(t);
-        __threadfence();                       // the partial is visible before the count
-        last = atomicAdd(counter, 1u) == nb_ - 1;
+    if (warp == 0) {
+        A t = lane < nwarp ? red[lane] : A(0);
+        for (int off = nwarp / 2; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        if (lane == 0) {
+            partial[bid_] = double(t);
+            __threadfence();                   // the partial is visible before the count
+            last = atomicAdd(counter, 1u) == nb_ - 1;
+        }
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // the Hessenberg column and the previous rotations into shared memory (one
-    // load per thread, alongside the partials), so that the sequential
-    // rotations below touch no global memory
-    __shared__ double colS[66], csS[66], snS[66];
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) colS[i] = h2 ? h1[i] + h2[i] : h1[i];
-    for (int i = threadIdx.x; i < j; i += blockDim.x) {
-        csS[i] = cs[i];
-        snS[i] = sn[i];
+    // the last block adds the partials with its updating threads, in a fixed order
+    // (thread t: partials t, t + 256, ...; then the warp tree; then the warps' tree)
+    double svj = 0.0, a = 0.0, ib = 0.0;
+    if (threadIdx.x == 0) {
+        svj = sv[j];
+        a = __ldcg(rot);
+        ib = __ldcg(rot + 1);
     }
-    // the last block adds the partials with all its threads, in a fixed order
-    // (thread t: partials t, t + blockDim, ...; then the warp tree; then the warps)
-    double v = 0.0;
-    for (unsigned b = threadIdx.x; b < nb_; b += blockDim.x) v += partial[b];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) redd[warp] = v;
+    if (warp < nwarp) {
+        double v = 0.0;
+        for (unsigned b = threadIdx.x; b < unsigned(nb_); b += kGsThreads) v += __ldcg(partial + b);
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0) redd[warp] = v;
+    }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    const double svj = sv[j], bn = bnorm[0];
-    double ww = 0.0;
-    for (int q = 0; q < nwarp; ++q) ww += redd[q];
+    if (warp != 0) return;
+    double ww = lane < nwarp ? redd[lane] : 0.0;
+    for (int off = nwarp / 2; off > 0; off >>= 1) ww += __shfl_xor_sync(0xffffffffu, ww, off);
+    if (lane != 0) return;
     *counter = 0u;
     nrm2[0] = ww;
-    colS[j + 1] = sqrt(ww);
-    for (int i = 0; i < j; ++i) {
-        const double t = csS[i] * colS[i] + snS[i] * colS[i + 1];
-        colS[i + 1] = -snS[i] * colS[i] + csS[i] * colS[i + 1];
-        colS[i] = t;
-    }
-    double *col = Hm + size_t(j) * ldh;
-    for (int i = 0; i < j; ++i) col[i] = colS[i];
-    const double a = colS[j], b = colS[j + 1];
-    const double den = hypot(a, b);
+    const double b = sqrt(ww), d2 = fma(a, a, ww);
     int32_t fl = 0;
-    double cj = 1.0, sj = 0.0;
-    if (!(den > 0.0)) {
-        fl |= 2;
+    double cj = 1.0, sj = 0.0, den;
+    if (d2 > 1e-280 && d2 < 1e280) {
+        const double r = rsqrt(d2);
+        den = d2 * r;
+        cj = a * r;
+        sj = b * r;
     } else {
-        cj = a / den;
-        sj = b / den;
+        den = hypot(a, b);                     // zero, NaN, or squares near the range's ends
+        if (!(den > 0.0)) {
+            fl |= 2;
+        } else {
+            cj = a / den;
+            sj = b / den;
+        }
     }
-    cs[j] = cj;
-    sn[j] = sj;
+    const double sj1 = -sj * svj, est = fabs(sj1) * ib;
     if (!(fabs(b) > 1e-300 * (fabs(a) + 1e-300))) fl |= 2;
-    col[j] = (den > 0.0) ? den : a;
-    col[j + 1] = 0.0;
-    sv[j + 1] = -sj * svj;
-    sv[j] = cj * svj;
-    const double est = fabs(-sj * svj) / bn;
     if (!isfinite(est) || !isfinite(den)) fl |= 4;
-    rb->est = est;
-    rb->flags = fl;
-    rb->hnext = b;
     if (host_rb) {
         // the page-locked copy the host polls: the fields, a system-scope fence,
         // then the step number, so that the host may read the fields once it sees it
         host_rb->est = est;
         host_rb->flags = fl;
         host_rb->hnext = b;
+    }
+    cs[j] = cj;
+    sn[j] = sj;
+    col[j] = (den > 0.0) ? den : a;
+    col[j + 1] = 0.0;
+    sv[j + 1] = sj1;
+    sv[j] = cj * svj;
+    rb->est = est;
+    rb->flags = fl;
+    rb->hnext = b;
+    if (host_rb) {
         __threadfence_system();
         *reinterpret_cast<volatile int32_t *>(&host_rb->seq) = j + 1;
     }
 }
 template <typename T>
-__global__ void __launch_bounds__(256) gs_update_norm_givens_kernel(const T *V, size_t ld, int k, T *w, size_t n,
+__global__ void __launch_bounds__(kGsThreads + 32) gs_update_norm_givens_kernel(const T *V, size_t ld, int k, T *w, size_t n,
                                                                     const double *h1, const double *h2,
-                                                                    double *partial, unsigned int *counter,
+                                                                    const T *hneg, double *partial,
+                                                                    unsigned int *counter, double *rot,
                                                                     double *nrm2, double *Hm, int ldh, double *cs,
                                                                     double *sn, double *sv, int j,
                                                                     const double *bnorm, ReadBack *rb,
                                                                     ReadBack *host_rb) {
     pdl_wait();
-    gs_update_norm_givens_kernel_impl<T>(blockIdx.x, gridDim.x, V, ld, k, w, n, h1, h2, partial, counter, nrm2, Hm,
+    gs_update_norm_givens_kernel_impl<T>(blockIdx.x, gridDim.x, V, ld, k, w, n, h1, h2, hneg, partial, counter, rot, nrm2, Hm,
         ldh, cs, sn, sv, j, bnorm, rb, host_rb);
 }
 template <typename T>
@@ -792,8 +833,10 @@ struct gs_update_norm_givens_kernel_args {
     size_t n;
     const double *h1;
     const double *h2;
+    const T *hneg;
     double *partial;
     unsigned int *counter;
+    double *rot;
     double *nrm2;
     double *Hm;
     int ldh;
@@ -806,18 +849,18 @@ struct gs_update_norm_givens_kernel_args {
     ReadBack *host_rb;
 };
 template <typename T>
-__global__ void __launch_bounds__(256) gs_update_norm_givens_kernel_multi(const __grid_constant__ MultiP<gs_update_norm_givens_kernel_args<T>> M) {
+__global__ void __launch_bounds__(kGsThreads + 32) gs_update_norm_givens_kernel_multi(const __grid_constant__ MultiP<gs_update_norm_givens_kernel_args<T>> M) {
     pdl_wait();
     int b_;
     const gs_update_norm_givens_kernel_args<T> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    gs_update_norm_givens_kernel_impl<T>(b_, q_.nb_, q_.V, q_.ld, q_.k, q_.w, q_.n, q_.h1, q_.h2, q_.partial,
-        q_.counter, q_.nrm2, q_.Hm, q_.ldh, q_.cs, q_.sn, q_.sv, q_.j, q_.bnorm, q_.rb, q_.host_rb);
+    gs_update_norm_givens_kernel_impl<T>(b_, q_.nb_, q_.V, q_.ld, q_.k, q_.w, q_.n, q_.h1, q_.h2, q_.hneg, q_.partial,
+        q_.counter, q_.rot, q_.nrm2, q_.Hm, q_.ldh, q_.cs, q_.sn, q_.sv, q_.j, q_.bnorm, q_.rb, q_.host_rb);
 }
 template <typename T>
 void gs_update_norm_givens_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, const T *V,
                                      size_t ld, int k, T *w, size_t n, const double *h1, const double *h2,
-                                     double *partial, unsigned int *counter, double *nrm2, double *Hm, int ldh,
-                                     double *cs, double *sn, double *sv, int j, const double *bnorm, ReadBack *rb,
+                                     const T *hneg, double *partial, unsigned int *counter, double *rot, double *nrm2,
+                                     double *Hm, int ldh, double *cs, double *sn, double *sv, int j, const double *bnorm, ReadBack *rb,
                                      ReadBack *host_rb) {
     if (Recorder *r_ = batch_recorder()) {
         gs_update_norm_givens_kernel_args<T> q_;
@@ -830,8 +873,10 @@ void gs_update_norm_givens_kernel_go(unsigned grid_, unsigned block_, size_t sme
         q_.n = n;
         q_.h1 = h1;
         q_.h2 = h2;
+        q_.hneg = hneg;
         q_.partial = partial;
         q_.counter = counter;
+        q_.rot = rot;
         q_.nrm2 = nrm2;
         q_.Hm = Hm;
         q_.ldh = ldh;
@@ -845,7 +890,7 @@ void gs_update_norm_givens_kernel_go(unsigned grid_, unsigned block_, size_t sme
         batch_record(r_, reinterpret_cast<const void *>(&gs_update_norm_givens_kernel_multi<T>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &gs_update_norm_givens_kernel<T>, grid_, block_, smem_, s_, V, ld, k, w, n, h1, h2, partial, counter, nrm2, Hm,
+    pdl_launch(kPdlFamily, &gs_update_norm_givens_kernel<T>, grid_, block_, smem_, s_, V, ld, k, w, n, h1, h2, hneg, partial, counter, rot, nrm2, Hm,
         ldh, cs, sn, sv, j, bnorm, rb, host_rb);
 }
 
@@ -967,14 +1012,14 @@ cudaError_t launch_d2f_scaled(const double *x, float *y, const double *scale, si
 
 template <typename T>
 cudaError_t launch_gs_step(const T *V, size_t ld, int j, T *w, double *partial, unsigned int *counter, int nblk,
-                           double *h1, double *h2, double *nrm2, double *Hm, int ldh, double *cs, double *sn,
-                           double *sv, const double *bnorm, ReadBack *rb, ReadBack *host_rb, T *vnext, bool reorth, bool scale,
-                           cudaStream_t s) {
+                           double *h1, double *h2, const T *hneg, double *rot, double *nrm2, double *Hm, int ldh,
+                           double *cs, double *sn, double *sv, const double *bnorm, ReadBack *rb, ReadBack *host_rb,
+                           T *vnext, bool reorth, bool scale, cudaStream_t s) {
     // h1 = V^T w comes with w from the operator kernel (apply_dots_kernel)
     const int k = j + 1;
     if (reorth) gs_update_dots_kernel<T><<<nblk, 256, 0, s>>>(V, ld, k, w, ld, h1, partial, counter, h2);
-    gs_update_norm_givens_kernel_go<T>(nblk, 256, 0, s, V, ld, k, w, ld, h1, reorth ? h2 : nullptr, partial, counter,
-                                                        nrm2, Hm, ldh, cs, sn, sv, j, bnorm, rb, host_rb);
+    gs_update_norm_givens_kernel_go<T>(nblk, kGsThreads + 32, 0, s, V, ld, k, w, ld, h1, reorth ? h2 : nullptr, hneg,
+                                                        partial, counter, rot, nrm2, Hm, ldh, cs, sn, sv, j, bnorm, rb, host_rb);
     if (scale) {   // otherwise the next step's first smoothing sweep forms v_{j+1}
         const size_t n4 = ld / (16 / sizeof(T));
         gs_scale_kernel_go<T>(blocks(n4, 256), 256, 0, s, w, vnext, ld, rb);
@@ -982,11 +1027,13 @@ cudaError_t launch_gs_step(const T *V, size_t ld, int j, T *w, double *partial, 
     return cudaGetLastError();
 }
 template cudaError_t launch_gs_step<float>(const float *, size_t, int, float *, double *, unsigned int *, int, double *,
-                                           double *, double *, double *, int, double *, double *, double *,
-                                           const double *, ReadBack *, ReadBack *, float *, bool, bool, cudaStream_t);
+                                           double *, const float *, double *, double *, double *, int, double *,
+                                           double *, double *, const double *, ReadBack *, ReadBack *, float *, bool,
+                                           bool, cudaStream_t);
 template cudaError_t launch_gs_step<double>(const double *, size_t, int, double *, double *, unsigned int *, int,
-                                            double *, double *, double *, double *, int, double *, double *, double *,
-                                            const double *, ReadBack *, ReadBack *, double *, bool, bool, cudaStream_t);
+                                            double *, double *, const double *, double *, double *, double *, int,
+                                            double *, double *, double *, const double *, ReadBack *, ReadBack *,
+                                            double *, bool, bool, cudaStream_t);
 
 #define HDG_KRYLOV_INST(T)                                                                                      \
     template cudaError_t launch_multidot<T>(const T *, size_t, int, const T *, size_t, double *, int,           \

@@ -914,22 +914,8 @@ __device__ __forceinline__ void dense_kernel_impl(int bid_, int nb_, const doubl
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[r] = fma(v[r], bd, acc[r]);
     }
-    // halving exchange: lane groups keep half of the rows each time, then the rest of
-    // the tree; row (lane's kept index) ends complete in every lane of its group
-    int keep = 0;
-#pragma unroll
-    for (int h = R / 2, off = 16; h > 0; h /= 2, off /= 2) {
-        const bool up = lane & off;
-#pragma unroll
-        for (int r = 0; r < h; ++r) {
-            const double send = up ? acc[r] : acc[r + h], mine = up ? acc[r + h] : acc[r];
-            acc[r] = mine + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-        keep = 2 * keep + (up ? 1 : 0);
-    }
-    double t = acc[0];
-#pragma unroll
-    for (int off = 16 / R; off > 0; off /= 2) t += __shfl_xor_sync(0xffffffffu, t, off);
+    int keep;
+    const double t = warp_sums<R>(acc, keep);
     if (lane % (32 / R) == 0) part[warp][keep] = t;
     __syncthreads();
     // R groups of eight lanes add the warps' sums
