@@ -111,22 +111,23 @@ def make_workload(kind: str, full: bool, p: int, courant: float, seed: int) -> d
 
 # ---------------------------------------------------------------- algorithmic bytes per launch
 def trace_bytes(cat: str, NF: int, pp: int, s_width: int | None = None) -> float:
-    """Minimum bytes a facet-row kernel must move: the operator values (5 blocks
-    of (p+1)^2 per facet), the neighbour ids, the inverted facet blocks where
-    used, and each trace vector it touches read or written once.  s_width
-    overrides the bytes per operator value (2 for the BF16 preconditioner copy)."""
+    """Minimum bytes a facet-row kernel must move: the operator values (apply: the 5
+    blocks of (p+1)^2 per facet of S; sweeps: the 4 neighbour blocks of D^-1 S; the
+    residual of the V-cycle: those and the diagonal block; the sizes of FP32 solves whose
+    sweeps take S and the inverse blocks move half as much again), the neighbour ids, and
+    each trace vector it touches read or written once.  s_width overrides the bytes per value
+    of the smoother's operator (2 for the BF16 copy)."""
     w = 8 if cat.endswith("64") else 4
-    S = 5 * pp * pp * (s_width or w) + 16
-    vec = pp * w
+    blk, vec = pp * pp, pp * w
     base = cat[:-2]
     if base == "apply":
-        per = S + 2 * vec
+        per = 5 * blk * w + 16 + 2 * vec
     elif base == "residual":      # with the first post-smoothing sweep's part before the correction
-        per = S + pp * pp * w + 4 * vec
+        per = 4 * blk * (s_width or w) + 16 + blk * w + 4 * vec
     elif base == "smooth":
-        per = S + pp * pp * w + 3 * vec
+        per = 4 * blk * (s_width or w) + 16 + 3 * vec
     elif base == "smooth_first":
-        per = pp * pp * w + 2 * vec
+        per = blk * w + 2 * vec
     else:
         raise KeyError(cat)
     return float(NF) * per
@@ -505,9 +506,9 @@ def whole_solve(arm: dict, peaks: dict, steps: int) -> dict:
 
 
 def fp64_fmas_per_facet(cat: str, pp: int) -> int:
-    """FMAs per facet of an FP64 facet-row kernel (operator blocks, inverse block)."""
+    """FMAs per facet of an FP64 facet-row kernel (operator blocks, diagonal or inverse block)."""
     base = cat[:-2]
-    return {"apply": 5 * pp * pp, "residual": 6 * pp * pp, "smooth": 6 * pp * pp, "smooth_first": pp * pp}[base]
+    return {"apply": 5 * pp * pp, "residual": 5 * pp * pp, "smooth": 4 * pp * pp, "smooth_first": pp * pp}[base]
 
 
 def p1_cycle_bytes(levels_nv: list, w: int, width: int = 8) -> float:

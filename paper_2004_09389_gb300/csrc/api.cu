@@ -31,7 +31,7 @@ template <typename T> cudaError_t launch_residual_t(hdg_handle *, const T *, con
 template <typename T> cudaError_t launch_residual_smooth_t(hdg_handle *, const T *, const T *, T *, T *, double);
 template <typename T> cudaError_t launch_smooth_t(hdg_handle *, const T *, const T *, T *);
 template <typename T>
-cudaError_t launch_smooth_first_t(hdg_handle *, const T *, T *, const T * = nullptr, const double * = nullptr,
+cudaError_t launch_smooth_first_t(hdg_handle *, const T *, T *, T *, const T * = nullptr, const double * = nullptr,
                                   T * = nullptr, double = 0.0);
 template <typename T>
 cudaError_t launch_smooth_cheb_t(hdg_handle *, const T *, const T *, T *, double, double, const T *);
@@ -48,6 +48,7 @@ template <typename T>
 struct KSpace {
     T *V = nullptr, *Z = nullptr, *w = nullptr;      // (m+1) x NT, m x NT, NT
     T *t0 = nullptr, *t1 = nullptr, *res = nullptr;  // preconditioner work
+    T *bh = nullptr;                                 // D^-1 v of the current application (smoothing sweeps)
     T *b = nullptr, *x = nullptr;                    // right-hand side / solution (FP32 inner solve)
 };
 
@@ -465,19 +466,22 @@ cudaError_t precond_lf(hdg_handle *h, const double *v, double *z, const double *
     cudaError_t e;
     // pre-smoothing from zero
     if (h->prm.n_pre == 0) {
+        if (h->prm.n_post > 0 &&
+            (e = KL(HDG_PROF_SMOOTH_FIRST64, 1, launch_smooth_first_t<double>(h, v, x, k.bh))) != cudaSuccess)
+            return e;
         if ((e = KL(HDG_PROF_KRYLOV, 1, launch_fill<double>(x, 0.0, NT, s))) != cudaSuccess) return e;
     } else {
         if ((e = KL(HDG_PROF_SMOOTH_FIRST64, 1,
-                    launch_smooth_first_t<double>(h, v, x, w_src, w_src ? &h->ws->rb->hnext : nullptr,
+                    launch_smooth_first_t<double>(h, v, x, k.bh, w_src, w_src ? &h->ws->rb->hnext : nullptr,
                                                   const_cast<double *>(v), cheb ? h->cheb_omega[0] : 0.0))) !=
             cudaSuccess)
             return e;
         double *prev = nullptr;
         for (int i = 1; i < h->prm.n_pre; ++i) {
             double *o = cheb ? (prev ? prev : x2) : x2;
-            e = cheb ? KL(HDG_PROF_SMOOTH64, 1, launch_smooth_cheb_t<double>(h, v, x, o, h->cheb_omega[i],
+            e = cheb ? KL(HDG_PROF_SMOOTH64, 1, launch_smooth_cheb_t<double>(h, k.bh, x, o, h->cheb_omega[i],
                                                                              h->cheb_beta[i], prev))
-                     : KL(HDG_PROF_SMOOTH64, 1, launch_smooth_t<double>(h, v, x, o));
+                     : KL(HDG_PROF_SMOOTH64, 1, launch_smooth_t<double>(h, k.bh, x, o));
             if (e != cudaSuccess) return e;
             if (cheb) {
                 prev = x;
@@ -512,7 +516,7 @@ cudaError_t precond_lf(hdg_handle *h, const double *v, double *z, const double *
     if (!cheb) {
         for (int i = 0; i < np; ++i) {
             double *o = (i == np - 1) ? z : x2;
-            if ((e = KL(HDG_PROF_SMOOTH64, 1, launch_smooth_t<double>(h, v, x, o))) != cudaSuccess) return e;
+            if ((e = KL(HDG_PROF_SMOOTH64, 1, launch_smooth_t<double>(h, k.bh, x, o))) != cudaSuccess) return e;
             if (i < np - 1) std::swap(x, x2);
         }
         return cudaSuccess;
@@ -524,7 +528,7 @@ cudaError_t precond_lf(hdg_handle *h, const double *v, double *z, const double *
         int out_i = 0;
         while (out_i == cur_i || out_i == prev_i) ++out_i;
         double *o = (i == np - 1) ? z : buf[out_i];
-        if ((e = KL(HDG_PROF_SMOOTH64, 1, launch_smooth_cheb_t<double>(h, v, buf[cur_i], o, h->cheb_omega[size_t(i)],
+        if ((e = KL(HDG_PROF_SMOOTH64, 1, launch_smooth_cheb_t<double>(h, k.bh, buf[cur_i], o, h->cheb_omega[size_t(i)],
                                                                          i ? h->cheb_beta[size_t(i)] : 0.0,
                                                                          i ? buf[prev_i] : nullptr))) != cudaSuccess)
             return e;
@@ -532,6 +536,13 @@ cudaError_t precond_lf(hdg_handle *h, const double *v, double *z, const double *
         cur_i = out_i;
     }
     return cudaSuccess;
+}
+
+// Do the sweeps of this type work on the rows of D^-1 S (H and bh, k_trace.cu)?
+template <typename T>
+bool hat_form(const hdg_handle *h) {
+    if constexpr (sizeof(T) == 8) return h->d_H != nullptr;
+    else return h->d_H32 != nullptr || h->d_H16 != nullptr;
 }
 
 // With w_src (Arnoldi steps j >= 1, n_pre >= 1), v is first formed as
@@ -548,19 +559,22 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
     const size_t NT = h->NT;
     T *x = k.t0, *x2 = k.t1;
     cudaError_t e;
+    // sweeps on D^-1 S (hat_form) take bh = D^-1 v, which the first one forms
+    T *const bh = hat_form<T>(h) ? k.bh : nullptr;
+    const T *const rhs = bh ? bh : v;
     const bool cheb = h->prm.smoother == 1;
     // lines 1-2: pre-smoothing and residual
     if (cheb && h->prm.n_pre > 0) {
         // Chebyshev iteration from zero: x_1 = s_0 D^-1 v, then x_{k+1} = x_k +
         // 2 s_k D^-1 (v - S x_k) + delta^2 s_k s_{k-1} (x_k - x_{k-1})
         if ((e = KL(cat_first<T>(), 1,
-                    launch_smooth_first_t<T>(h, v, x, w_src, w_src ? (hsrc ? hsrc : &h->ws->rb->hnext) : nullptr,
+                    launch_smooth_first_t<T>(h, v, x, bh, w_src, w_src ? (hsrc ? hsrc : &h->ws->rb->hnext) : nullptr,
                                              const_cast<T *>(v), h->cheb_omega[0]))) != cudaSuccess)
             return e;
         T *prev = nullptr;
         for (int i = 1; i < h->prm.n_pre; ++i) {
             T *o = prev ? prev : x2;
-            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, v, x, o, h->cheb_omega[i], h->cheb_beta[i],
+            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, rhs, x, o, h->cheb_omega[i], h->cheb_beta[i],
                                                                      prev))) != cudaSuccess)
                 return e;
             prev = x;
@@ -568,14 +582,17 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
         }
         x2 = (x == k.t0) ? k.t1 : k.t0;
     } else if (h->prm.n_pre == 0) {
+        if (bh && h->prm.n_post > 0 &&
+            (e = KL(cat_first<T>(), 1, launch_smooth_first_t<T>(h, v, x, bh))) != cudaSuccess)
+            return e;
         if ((e = KL(HDG_PROF_KRYLOV, 1, launch_fill<T>(x, T(0), NT, s))) != cudaSuccess) return e;
     } else {
         if ((e = KL(cat_first<T>(), 1,
-                    launch_smooth_first_t<T>(h, v, x, w_src, w_src ? (hsrc ? hsrc : &h->ws->rb->hnext) : nullptr,
+                    launch_smooth_first_t<T>(h, v, x, bh, w_src, w_src ? (hsrc ? hsrc : &h->ws->rb->hnext) : nullptr,
                                              const_cast<T *>(v)))) != cudaSuccess)
             return e;
         for (int i = 1; i < h->prm.n_pre; ++i) {
-            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, v, x, x2))) != cudaSuccess) return e;
+            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, rhs, x, x2))) != cudaSuccess) return e;
             std::swap(x, x2);
         }
     }
@@ -590,7 +607,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
     if (np == 0 || (np == 1 && (learned || collect))) {
         if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, k.res, true))) != cudaSuccess) return e;
     } else {
-        if ((e = KL(cat_res<T>(), 1, launch_residual_smooth_t<T>(h, v, x, k.res, x2, cheb ? h->cheb_omega[0] : 0.0))) !=
+        if ((e = KL(cat_res<T>(), 1, launch_residual_smooth_t<T>(h, rhs, x, k.res, x2, cheb ? h->cheb_omega[0] : 0.0))) !=
             cudaSuccess)
             return e;
     }
@@ -616,7 +633,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
             return e;
         for (int i = 1; i < np; ++i) {
             T *o = (i == np - 1) ? z : prev;
-            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, v, cur, o, h->cheb_omega[i], h->cheb_beta[i],
+            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, rhs, cur, o, h->cheb_omega[i], h->cheb_beta[i],
                                                                      prev))) != cudaSuccess)
                 return e;
             prev = cur;
@@ -630,7 +647,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
         std::swap(x, x2);
         for (int i = 1; i < np; ++i) {
             T *o = (i == np - 1) ? z : x2;
-            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, v, x, o))) != cudaSuccess) return e;
+            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, rhs, x, o))) != cudaSuccess) return e;
             if (i < np - 1) std::swap(x, x2);
         }
         return cudaSuccess;
@@ -647,7 +664,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
             cudaSuccess)
             return e;
         for (int i = 1; i < np - 1; ++i) {
-            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, v, cur, free_, h->cheb_omega[i],
+            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, rhs, cur, free_, h->cheb_omega[i],
                                                                      h->cheb_beta[i], prev))) != cudaSuccess)
                 return e;
             T *t = free_;
@@ -662,7 +679,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
         if ((e = KL(HDG_PROF_TRANSFER, 1, launch_smooth_prolong_t<T>(h, ec, x2, x, x2))) != cudaSuccess) return e;
         std::swap(x, x2);
         for (int i = 1; i < np - 1; ++i) {
-            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, v, x, x2))) != cudaSuccess) return e;
+            if ((e = KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, rhs, x, x2))) != cudaSuccess) return e;
             std::swap(x, x2);
         }
     }
@@ -682,9 +699,9 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
         h->lc.count += 1;
     }
     if (cheb_prev)
-        return KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, v, x, z, h->cheb_omega[size_t(np - 1)],
+        return KL(cat_smooth<T>(), 1, launch_smooth_cheb_t<T>(h, rhs, x, z, h->cheb_omega[size_t(np - 1)],
                                                               h->cheb_beta[size_t(np - 1)], cheb_prev));
-    return KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, v, x, z));
+    return KL(cat_smooth<T>(), 1, launch_smooth_t<T>(h, rhs, x, z));
 }
 
 // ---------------------------------------------------------------- Krylov helpers
@@ -1231,7 +1248,8 @@ void free_handle(hdg_handle *h) {
     dfree(h->d_nbr); dfree(h->d_Xb); dfree(h->d_Rm); dfree(h->d_W); dfree(h->d_Scell); dfree(h->d_Sval);
     dfree(h->d_Xb2); dfree(h->d_Sval2);
     dfree(h->d_Hr2); dfree(h->d_PQ2); dfree(h->d_lgeo); dfree(h->d_fftab);
-    dfree(h->d_Dinv); dfree(h->d_Sval32); dfree(h->d_Dinv32); dfree(h->d_Sval16); dfree(h->d_status); dfree(h->d_coarse_inv);
+    dfree(h->d_Dinv); dfree(h->d_Sval32); dfree(h->d_Dinv32); dfree(h->d_H); dfree(h->d_D);
+    dfree(h->d_H32); dfree(h->d_D32); dfree(h->d_H16); dfree(h->d_status); dfree(h->d_coarse_inv);
     for (auto &im : h->tail_img) dfree(im.d);
     dfree(h->d_tail_op);
     dfree(h->d_facet_opp); dfree(h->d_Q); dfree(h->d_Q32);
@@ -1249,8 +1267,8 @@ void free_handle(hdg_handle *h) {
     if (h->ws) {
         Workspace &W = *h->ws;
         dfree(W.g); dfree(W.x); dfree(W.r); dfree(W.ycell); dfree(W.x2); dfree(W.z2);
-        dfree(W.k64.V); dfree(W.k64.Z); dfree(W.k64.w); dfree(W.k64.t0); dfree(W.k64.t1); dfree(W.k64.res);
-        dfree(W.k32.V); dfree(W.k32.Z); dfree(W.k32.w); dfree(W.k32.t0); dfree(W.k32.t1); dfree(W.k32.res);
+        dfree(W.k64.V); dfree(W.k64.Z); dfree(W.k64.w); dfree(W.k64.t0); dfree(W.k64.t1); dfree(W.k64.res); dfree(W.k64.bh);
+        dfree(W.k32.V); dfree(W.k32.Z); dfree(W.k32.w); dfree(W.k32.t0); dfree(W.k32.t1); dfree(W.k32.res); dfree(W.k32.bh);
         dfree(W.k32.b); dfree(W.k32.x);
         dfree(W.Hm); dfree(W.cs); dfree(W.sn); dfree(W.sv); dfree(W.h1); dfree(W.h2); dfree(W.hneg); dfree(W.rot); dfree(W.nrm2);
         dfree(W.est); dfree(W.counter); dfree(W.rb);
@@ -1449,6 +1467,21 @@ int build_fftab(hdg_handle *h, const RefElem &re, const NodalRef &nr) {
     return HDG_OK;
 }
 
+// FP32 sweeps on D^-1 S read 16 (p+1)^2 bytes of operator per facet instead of 24 (p+1)^2,
+// but an FP32 Krylov space applies S itself, so a cycle then touches 56 (p+1)^2 bytes per
+// facet.  With S alone (24 (p+1)^2 with its inverse blocks) in L2 from one kernel to the
+// next, that costs more than it saves; it pays where both sets lie in L2 or neither does.
+// One step with / without H, in us, at the two sets' sizes in MB (L2: 126 MB): flat p = 3,
+// n = 64 887 / 903 (11; 5), r = 5 p = 3 1024 / 1045 (28; 12), n = 128 1102 / 1100 (44; 19),
+// 160 1318 / 1248 (69; 29), 256 1996 / 1960 (176; 75), 320 2824 / 3124 (275; 118); p = 2,
+// n = 256 1500 / 1427 (99; 42), 384 2466 / 2736 (223; 96), r = 7 2431 / 2700 (248; 106);
+// p = 1, n = 256 1199 / 1161 (44; 19).  Under an FP64 Krylov space S is not read in FP32 and
+// H always pays: n = 192 1977 / 2013, n = 256 2884 / 2991.
+bool hat_pays32(const hdg_params &prm, size_t NF, size_t pp, size_t l2) {
+    const size_t blk = 4 * pp * pp * NF;
+    return mode_pre32(prm) || 14 * blk <= l2 / 3 || 6 * blk > l2 / 3 * 2;
+}
+
 int setup_device(hdg_handle *h, const hdg_params *prm) {
     cudaStream_t s = h->stream;
     const HostMesh &hm = h->hm;
@@ -1495,6 +1528,10 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(dalloc(&h->d_Dinv, packed(pp * pp, 2)));
     TRY(dalloc(&h->d_status, 1));
     const bool mixed = prm->precision != HDG_FP64;
+    if (!mixed) {
+        TRY(dalloc(&h->d_H, packed(4 * pp * pp, 2)));
+        TRY(dalloc(&h->d_D, packed(pp * pp, 2)));
+    }
     if (mixed) {
         TRY(dalloc(&h->d_Sval32, packed(5 * pp * pp, 4)));
         TRY(dalloc(&h->d_Dinv32, packed(pp * pp, 4)));
@@ -1510,7 +1547,13 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
             const int rc = build_fftab(h, re, nr);
             if (rc) return rc;
         }
-        if (prm->precision == HDG_MIXED_BF16) TRY(dalloc(&h->d_Sval16, packed(5 * pp * pp, 8)));
+        int dev = 0, l2 = 0;
+        TRY(cudaGetDevice(&dev));
+        TRY(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+        const bool bf16 = prm->precision == HDG_MIXED_BF16;
+        if (bf16) TRY(dalloc(&h->d_H16, packed(4 * pp * pp, 8)));
+        else if (hat_pays32(*prm, NF, pp, size_t(l2))) TRY(dalloc(&h->d_H32, packed(4 * pp * pp, 4)));
+        if (h->d_H16 || h->d_H32) TRY(dalloc(&h->d_D32, packed(pp * pp, 4)));
     }
     // Coriolis parameter per cell (mean of its vertices) on every P1 level; on a
     // coarser level a vertex takes the value of the finer-level vertex that
@@ -1667,6 +1710,7 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
         if (mode_pre32(h->prm)) {
             // the FP32 preconditioner's work vectors, its input and its output
             TRY(dalloc(&W.k32.t0, W.NT));
+            if (hat_form<float>(h)) TRY(dalloc(&W.k32.bh, W.NT));
             TRY(dalloc(&W.k32.t1, W.NT));
             TRY(dalloc(&W.k32.res, W.NT));
             TRY(dalloc(&W.k32.b, W.NT));
@@ -1682,12 +1726,14 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
         TRY(cudaMemsetAsync(W.k32.V, 0, sizeof(float) * (mm + 1) * W.ld, s));
         TRY(cudaMemsetAsync(W.k32.w, 0, sizeof(float) * W.ld, s));
         TRY(dalloc(&W.k32.t0, W.NT));
+        if (hat_form<float>(h)) TRY(dalloc(&W.k32.bh, W.NT));
         TRY(dalloc(&W.k32.t1, W.NT));
         TRY(dalloc(&W.k32.res, W.NT));
         TRY(dalloc(&W.k32.b, W.NT));
         TRY(dalloc(&W.k32.x, W.NT));
     }
     TRY(dalloc(&W.k64.t0, W.NT));
+    if (hat_form<double>(h)) TRY(dalloc(&W.k64.bh, W.NT));
     TRY(dalloc(&W.k64.t1, W.NT));
     TRY(dalloc(&W.k64.res, W.NT));
     TRY(dalloc(&W.Hm, (mm + 1) * mm));
@@ -1838,7 +1884,7 @@ int chebyshev_setup(hdg_handle *h) {
             for (size_t r = 0; r < pp; ++r) v0[r * NF + e_] = cheb_start(e_ * pp + r);
         int rc = arnoldi_ritz_dev(h, v0, h->prm.cheb_steps, [&](const double *x, double *y, double *tmp) {
             cudaError_t e = launch_apply_t<double>(h, x, tmp);
-            return e == cudaSuccess ? launch_smooth_first_t<double>(h, tmp, y, nullptr, nullptr, nullptr, 1.0) : e;
+            return e == cudaSuccess ? launch_smooth_first_t<double>(h, tmp, y, nullptr, nullptr, nullptr, nullptr, 1.0) : e;
         }, h->cheb_ritz, "Chebyshev estimate");
         if (rc) return rc;
         chebyshev_ellipse(h->cheb_ritz, 0.1, 1.1, h->cheb_theta, h->cheb_delta2);
@@ -2137,6 +2183,7 @@ int hdg_condense(hdg_handle *h) {
         // Lax-Friedrichs: cell operators and the facet-row operator on 2(p+1) blocks,
         // the RT0 coarse operator and its Chebyshev coarse solve
         TRY(KL(HDG_PROF_CONDENSE, 2, launch_condense_lf(h)));
+        TRY(KL(HDG_PROF_CONDENSE, 1, launch_hat_op(h)));
         TRY(KL(HDG_PROF_CONDENSE, 2, launch_rt0_assemble(h)));
         int rc = check_status(h);
         if (rc) return rc;
@@ -2147,7 +2194,7 @@ int hdg_condense(hdg_handle *h) {
     }
     TRY(KL(HDG_PROF_CONDENSE, 1, launch_condense(h)));
     TRY(KL(HDG_PROF_CONDENSE, 1, launch_assemble(h)));
-    TRY(KL(HDG_PROF_CONDENSE, 1, launch_prolong_op(h)));
+    TRY(KL(HDG_PROF_CONDENSE, 1, launch_hat_op(h)));
     const double tau = h->prm.tau, gH = h->prm.g * h->prm.H;
     if (h->prm.coarse_mode == 2) {
         TRY(KL(HDG_PROF_CONDENSE, int(2 * h->lev.size()), launch_p1_galerkin(h)));
@@ -2159,7 +2206,7 @@ int hdg_condense(hdg_handle *h) {
     TRY(KL(HDG_PROF_CONDENSE, Lc.nv <= 256 ? 2 : 2 + 2 * Lc.nv,
            launch_dense_inverse(h, Lc, h->d_coarse_work, h->d_coarse_inv, Lc.nv)));
     if (h->prm.precision != HDG_FP64) {
-        TRY(KL(HDG_PROF_CONDENSE, h->d_Sval16 ? 3 : 2, launch_repack(h)));
+        TRY(KL(HDG_PROF_CONDENSE, 2, launch_repack(h)));
         for (auto &L : h->lev) {
             TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.A, L.A32, size_t(L.nnz), s)));
             TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.dinv, L.dinv32, size_t(L.nv), s)));

@@ -714,7 +714,12 @@ struct hdg_handle {
     double *d_Sval = nullptr;       // 5(p+1)^2 values per facet, packed in 16-byte groups
     double *d_Dinv = nullptr;       // (p+1)^2 values per facet, packed likewise
     float *d_Sval32 = nullptr, *d_Dinv32 = nullptr;
-    __nv_bfloat16 *d_Sval16 = nullptr;   // preconditioner copy (HDG_MIXED_BF16)
+    // the smoother's operator (k_trace.cu): the neighbour blocks H of D^-1 S, 4(p+1)^2 values
+    // per facet, and the diagonal block D, (p+1)^2, packed likewise; BF16: HDG_MIXED_BF16;
+    // null where the sweeps of that type take S and the inverse blocks
+    double *d_H = nullptr, *d_D = nullptr;
+    float *d_H32 = nullptr, *d_D32 = nullptr;
+    __nv_bfloat16 *d_H16 = nullptr;
     int32_t *d_status = nullptr;    // device error flags: 1 zero pivot in A_K, 2 singular facet block,
                                     // 4 singular coarsest P1 operator, 8 coarse-cycle staging wait ran
                                     // out, 16 learned-sweep MMA wait ran out
@@ -850,8 +855,8 @@ cudaError_t launch_to_f32(const double *x, float *y, size_t n, cudaStream_t s);
 // trace-space kernels (k_trace.cu); vectors in the internal layout [pp][NF]
 cudaError_t launch_to_internal(hdg_handle *h, const double *ext, double *in);
 cudaError_t launch_repack(hdg_handle *h);
-// D^-1 S pi of the facet rows (d_Q, d_Q32) from the FP64 operator
-cudaError_t launch_prolong_op(hdg_handle *h);
+// the smoother's operators (H, D and, for the upwind solver, Q) from the FP64 operator
+cudaError_t launch_hat_op(hdg_handle *h);
 // index of element j of facet e in an operator array packed in groups of G
 inline __host__ __device__ size_t packed_index(size_t j, size_t e, size_t NF, size_t G) {
     return ((j / G) * NF + e) * G + j % G;

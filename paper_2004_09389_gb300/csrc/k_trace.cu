@@ -27,7 +27,6 @@ namespace {
 template <typename TO> __device__ __forceinline__ TO convert_to(double v);
 template <> __device__ __forceinline__ double convert_to<double>(double v) { return v; }
 template <> __device__ __forceinline__ float convert_to<float>(double v) { return float(v); }
-template <> __device__ __forceinline__ __nv_bfloat16 convert_to<__nv_bfloat16>(double v) { return __double2bfloat16(v); }
 
 // Operator values are packed in 16-byte groups: element j of facet e lives at
 // group (j / G, e), lane j % G, with G = 16 / sizeof(storage); every thread
@@ -92,6 +91,31 @@ __device__ __forceinline__ void facet_rows_packed(const ST *__restrict__ Sval, i
             if (j < NS) {
                 const int r = j / (5 * PP), rem = j % (5 * PP), b = rem / PP, c = rem % PP;
                 y[r] = fma(T(o[g]), xs[b][c], y[r]);
+            }
+        }
+    }
+}
+
+// y_r = sum over the four neighbour blocks of H[(r*4+b)*PP+c] xs[1+b][c] with packed loads
+template <int P, typename T, typename ST>
+__device__ __forceinline__ void hat_rows_packed(const ST *__restrict__ H, int e, size_t NF, const T (&xs)[5][P + 1],
+                                                T (&y)[P + 1]) {
+    constexpr int PP = P + 1, NS = 4 * PP * PP, G = Pack<ST>::G, NQ = (NS + G - 1) / G;
+    using V = typename Pack<ST>::V;
+    const V *Hp = reinterpret_cast<const V *>(H);
+#pragma unroll
+    for (int r = 0; r < PP; ++r) y[r] = T(0);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const V v = __ldg(Hp + size_t(q) * NF + e);
+        unpacked_t<ST> o[G];
+        Pack<ST>::unpack(v, o);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int j = q * G + g;
+            if (j < NS) {
+                const int r = j / (4 * PP), rem = j % (4 * PP), b = rem / PP, c = rem % PP;
+                y[r] = fma(T(o[g]), xs[1 + b][c], y[r]);
             }
         }
     }
@@ -329,12 +353,24 @@ void residual_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStrea
 }
 
 
-// The residual before the coarse correction, res = b - S x, and the part of the first
-// post-smoothing sweep that does not wait for the correction, y = x + omega D_e^-1 res:
-// D^-1 was read by the sweep just before this kernel and is still in L2 here.
-template <int P, typename T, typename ST>
-__device__ __forceinline__ void residual_smooth_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ Sval,
-                                                            const T *__restrict__ Dinv,
+// The smoothing sweeps, on one of two sets of operators.  With HAT, on the rows of D^-1 S:
+// with b standing for bh = D^-1 b (formed once per preconditioner application by the first
+// sweep), op for H, the four neighbour blocks of D^-1 S (the diagonal block is the identity),
+//   D_e^-1 (b - S x)_e = bh_e - x_e - sum_b H_b x_nbr(b),
+// so a sweep reads 4 (p+1)^2 operator values per facet instead of 6 (p+1)^2 (S and the
+// inverse block).  Without, op is S, blk the inverse block: kept for FP32 handles of the
+// sizes where S, which the Krylov space applies too, stays in L2 from one kernel to the
+// next (hat_pays32 in api.cu).  What bounds a sweep is the operator's stream (HBM and L2);
+// in FP64 the FP64 pipe, 64 instead of 96 FMAs per facet at p = 3: the step with 196,608
+// facets takes 3440 instead of 3650 us in FP64, the one with 491,520 (p = 2, FP32) 2435
+// instead of 2683, with 30,000 (p = 4, BF16) 1175 instead of 1258.
+//
+// The residual before the coarse correction, res = b - S x (with HAT as D (D^-1 (b - S x)),
+// blk the diagonal block D), and the part of the first post-smoothing sweep that does not
+// wait for the correction, y = x + omega D^-1 (b - S x).
+template <int P, typename T, typename ST, bool HAT>
+__device__ __forceinline__ void residual_smooth_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ op,
+                                                            const T *__restrict__ blk,
                                                             const int32_t *__restrict__ nbr, const T *__restrict__ b,
                                                             const T *__restrict__ x, T *__restrict__ res,
                                                             T *__restrict__ y, T omega) {
@@ -342,33 +378,35 @@ __device__ __forceinline__ void residual_smooth_kernel_impl(int bid_, int nb_, i
     if (e >= NF) return;
     T xs[5][P + 1], v[P + 1], d[P + 1];
     gather_x<P, T>(nbr, x, e, NF, xs);
-    facet_rows_packed<P, T, ST>(Sval, e, NF, xs, v);
+    if constexpr (HAT) hat_rows_packed<P, T, ST>(op, e, NF, xs, v);
+    else facet_rows_packed<P, T, ST>(op, e, NF, xs, v);
 #pragma unroll
     for (int r = 0; r <= P; ++r) {
-        v[r] = b[size_t(r) * NF + e] - v[r];
-        res[size_t(r) * NF + e] = v[r];
+        if constexpr (HAT) v[r] = (b[size_t(r) * NF + e] - xs[0][r]) - v[r];
+        else v[r] = b[size_t(r) * NF + e] - v[r];
+        (HAT ? y : res)[size_t(r) * NF + e] = HAT ? fma(omega, v[r], xs[0][r]) : v[r];
     }
-    block_solve_packed<P, T, T>(Dinv, e, NF, v, d);
+    block_solve_packed<P, T, T>(blk, e, NF, v, d);
 #pragma unroll
-    for (int r = 0; r <= P; ++r) y[size_t(r) * NF + e] = fma(omega, d[r], xs[0][r]);
+    for (int r = 0; r <= P; ++r) (HAT ? res : y)[size_t(r) * NF + e] = HAT ? d[r] : fma(omega, d[r], xs[0][r]);
 }
-template <int P, typename T, typename ST>
-__global__ void __launch_bounds__(256, MinBlocks<T>::value) residual_smooth_kernel(int NF, const ST *__restrict__ Sval,
-                                                                                   const T *__restrict__ Dinv,
+template <int P, typename T, typename ST, bool HAT>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) residual_smooth_kernel(int NF, const ST *__restrict__ op,
+                                                                                   const T *__restrict__ blk,
                                                                                    const int32_t *__restrict__ nbr,
                                                                                    const T *__restrict__ b,
                                                                                    const T *__restrict__ x,
                                                                                    T *__restrict__ res,
                                                                                    T *__restrict__ y, T omega) {
     pdl_wait();
-    residual_smooth_kernel_impl<P, T, ST>(blockIdx.x, gridDim.x, NF, Sval, Dinv, nbr, b, x, res, y, omega);
+    residual_smooth_kernel_impl<P, T, ST, HAT>(blockIdx.x, gridDim.x, NF, op, blk, nbr, b, x, res, y, omega);
 }
-template <int P, typename T, typename ST>
+template <int P, typename T, typename ST, bool HAT>
 struct residual_smooth_kernel_args {
     int nb_;
     int NF;
-    const ST *Sval;
-    const T *Dinv;
+    const ST *op;
+    const T *blk;
     const int32_t *nbr;
     const T *b;
     const T *x;
@@ -376,34 +414,34 @@ struct residual_smooth_kernel_args {
     T *y;
     T omega;
 };
-template <int P, typename T, typename ST>
-__global__ void __launch_bounds__(256, MinBlocks<T>::value) residual_smooth_kernel_multi(const __grid_constant__ MultiP<residual_smooth_kernel_args<P, T, ST>> M) {
+template <int P, typename T, typename ST, bool HAT>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) residual_smooth_kernel_multi(const __grid_constant__ MultiP<residual_smooth_kernel_args<P, T, ST, HAT>> M) {
     pdl_wait();
     int b_;
-    const residual_smooth_kernel_args<P, T, ST> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    residual_smooth_kernel_impl<P, T, ST>(b_, q_.nb_, q_.NF, q_.Sval, q_.Dinv, q_.nbr, q_.b, q_.x, q_.res, q_.y,
+    const residual_smooth_kernel_args<P, T, ST, HAT> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    residual_smooth_kernel_impl<P, T, ST, HAT>(b_, q_.nb_, q_.NF, q_.op, q_.blk, q_.nbr, q_.b, q_.x, q_.res, q_.y,
         q_.omega);
 }
-template <int P, typename T, typename ST>
-void residual_smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *Sval,
-                               const T *Dinv, const int32_t *nbr, const T *b, const T *x, T *res, T *y, T omega) {
+template <int P, typename T, typename ST, bool HAT>
+void residual_smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *op,
+                               const T *blk, const int32_t *nbr, const T *b, const T *x, T *res, T *y, T omega) {
     if (Recorder *r_ = batch_recorder()) {
-        residual_smooth_kernel_args<P, T, ST> q_;
+        residual_smooth_kernel_args<P, T, ST, HAT> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
         q_.NF = NF;
-        q_.Sval = Sval;
-        q_.Dinv = Dinv;
+        q_.op = op;
+        q_.blk = blk;
         q_.nbr = nbr;
         q_.b = b;
         q_.x = x;
         q_.res = res;
         q_.y = y;
         q_.omega = omega;
-        batch_record(r_, reinterpret_cast<const void *>(&residual_smooth_kernel_multi<P, T, ST>), q_, grid_, block_, smem_, kPdlFamily);
+        batch_record(r_, reinterpret_cast<const void *>(&residual_smooth_kernel_multi<P, T, ST, HAT>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &residual_smooth_kernel<P, T, ST>, grid_, block_, smem_, s_, NF, Sval, Dinv, nbr, b, x, res, y, omega);
+    pdl_launch(kPdlFamily, &residual_smooth_kernel<P, T, ST, HAT>, grid_, block_, smem_, s_, NF, op, blk, nbr, b, x, res, y, omega);
 }
 
 
@@ -411,47 +449,51 @@ void residual_smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cu
 // Chebyshev iteration x_out = x + omega D_e^-1 (b - S x)_e + beta (x - x_prev)
 // (x_prev null: the previous iterate is zero).  x_out may alias x_prev: each
 // thread reads x_prev only at its own facet before writing it.
-template <int P, typename T, typename ST, bool CHEB = false>
-__device__ __forceinline__ void smooth_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ Sval,
-                                                   const T *__restrict__ Dinv, const int32_t *__restrict__ nbr,
-                                                   const T *__restrict__ b, const T *__restrict__ x, T *xout, T omega,
-                                                   T beta, const T *xprev) {
+template <int P, typename T, typename ST, bool HAT, bool CHEB>
+__device__ __forceinline__ void smooth_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ op, const T *__restrict__ blk,
+                                                   const int32_t *__restrict__ nbr, const T *__restrict__ b,
+                                                   const T *__restrict__ x, T *xout, T omega, T beta,
+                                                   const T *xprev) {
     constexpr int PP = P + 1;
     const int e = bid_ * blockDim.x + threadIdx.x;
     if (e >= NF) return;
     T xs[5][PP], v[PP], d[PP];
     gather_x<P, T>(nbr, x, e, NF, xs);
-    facet_rows_packed<P, T, ST>(Sval, e, NF, xs, v);
+    if constexpr (HAT) {
+        hat_rows_packed<P, T, ST>(op, e, NF, xs, v);
 #pragma unroll
-    for (int r = 0; r < PP; ++r) v[r] = b[size_t(r) * NF + e] - v[r];
-    block_solve_packed<P, T, T>(Dinv, e, NF, v, d);
-    if constexpr (CHEB) {
-#pragma unroll
-        for (int r = 0; r < PP; ++r) {
-            const T xp = xprev ? xprev[size_t(r) * NF + e] : T(0);
-            xout[size_t(r) * NF + e] = fma(beta, xs[0][r] - xp, fma(omega, d[r], xs[0][r]));
-        }
+        for (int r = 0; r < PP; ++r) d[r] = (b[size_t(r) * NF + e] - xs[0][r]) - v[r];
     } else {
+        facet_rows_packed<P, T, ST>(op, e, NF, xs, v);
 #pragma unroll
-        for (int r = 0; r < PP; ++r) xout[size_t(r) * NF + e] = fma(omega, d[r], xs[0][r]);
+        for (int r = 0; r < PP; ++r) v[r] = b[size_t(r) * NF + e] - v[r];
+        block_solve_packed<P, T, T>(blk, e, NF, v, d);
+    }
+#pragma unroll
+    for (int r = 0; r < PP; ++r) {
+        T o = fma(omega, d[r], xs[0][r]);
+        if constexpr (CHEB) {
+            const T xp = xprev ? xprev[size_t(r) * NF + e] : T(0);
+            o = fma(beta, xs[0][r] - xp, o);
+        }
+        xout[size_t(r) * NF + e] = o;
     }
 }
-template <int P, typename T, typename ST, bool CHEB = false>
-__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_kernel(int NF, const ST *__restrict__ Sval,
-                                                                          const T *__restrict__ Dinv,
+template <int P, typename T, typename ST, bool HAT, bool CHEB>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_kernel(int NF, const ST *__restrict__ op, const T *__restrict__ blk,
                                                                           const int32_t *__restrict__ nbr,
                                                                           const T *__restrict__ b,
                                                                           const T *__restrict__ x, T *xout, T omega,
                                                                           T beta, const T *xprev) {
     pdl_wait();
-    smooth_kernel_impl<P, T, ST, CHEB>(blockIdx.x, gridDim.x, NF, Sval, Dinv, nbr, b, x, xout, omega, beta, xprev);
+    smooth_kernel_impl<P, T, ST, HAT, CHEB>(blockIdx.x, gridDim.x, NF, op, blk, nbr, b, x, xout, omega, beta, xprev);
 }
-template <int P, typename T, typename ST, bool CHEB = false>
+template <int P, typename T, typename ST, bool HAT, bool CHEB>
 struct smooth_kernel_args {
     int nb_;
     int NF;
-    const ST *Sval;
-    const T *Dinv;
+    const ST *op;
+    const T *blk;
     const int32_t *nbr;
     const T *b;
     const T *x;
@@ -460,25 +502,25 @@ struct smooth_kernel_args {
     T beta;
     const T *xprev;
 };
-template <int P, typename T, typename ST, bool CHEB = false>
-__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_kernel_multi(const __grid_constant__ MultiP<smooth_kernel_args<P, T, ST, CHEB>> M) {
+template <int P, typename T, typename ST, bool HAT, bool CHEB>
+__global__ void __launch_bounds__(256, MinBlocks<T>::value) smooth_kernel_multi(const __grid_constant__ MultiP<smooth_kernel_args<P, T, ST, HAT, CHEB>> M) {
     pdl_wait();
     int b_;
-    const smooth_kernel_args<P, T, ST, CHEB> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    smooth_kernel_impl<P, T, ST, CHEB>(b_, q_.nb_, q_.NF, q_.Sval, q_.Dinv, q_.nbr, q_.b, q_.x, q_.xout, q_.omega,
+    const smooth_kernel_args<P, T, ST, HAT, CHEB> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    smooth_kernel_impl<P, T, ST, HAT, CHEB>(b_, q_.nb_, q_.NF, q_.op, q_.blk, q_.nbr, q_.b, q_.x, q_.xout, q_.omega,
         q_.beta, q_.xprev);
 }
-template <int P, typename T, typename ST, bool CHEB = false>
-void smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *Sval,
-                      const T *Dinv, const int32_t *nbr, const T *b, const T *x, T *xout, T omega, T beta,
+template <int P, typename T, typename ST, bool HAT, bool CHEB>
+void smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *op, const T *blk,
+                      const int32_t *nbr, const T *b, const T *x, T *xout, T omega, T beta,
                       const T *xprev) {
     if (Recorder *r_ = batch_recorder()) {
-        smooth_kernel_args<P, T, ST, CHEB> q_;
+        smooth_kernel_args<P, T, ST, HAT, CHEB> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
         q_.NF = NF;
-        q_.Sval = Sval;
-        q_.Dinv = Dinv;
+        q_.op = op;
+        q_.blk = blk;
         q_.nbr = nbr;
         q_.b = b;
         q_.x = x;
@@ -486,10 +528,10 @@ void smooth_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_
         q_.omega = omega;
         q_.beta = beta;
         q_.xprev = xprev;
-        batch_record(r_, reinterpret_cast<const void *>(&smooth_kernel_multi<P, T, ST, CHEB>), q_, grid_, block_, smem_, kPdlFamily);
+        batch_record(r_, reinterpret_cast<const void *>(&smooth_kernel_multi<P, T, ST, HAT, CHEB>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &smooth_kernel<P, T, ST, CHEB>, grid_, block_, smem_, s_, NF, Sval, Dinv, nbr, b, x, xout, omega, beta, xprev);
+    pdl_launch(kPdlFamily, &smooth_kernel<P, T, ST, HAT, CHEB>, grid_, block_, smem_, s_, NF, op, blk, nbr, b, x, xout, omega, beta, xprev);
 }
 
 
@@ -596,74 +638,105 @@ void smooth_prolong_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cud
         x0out);
 }
 
-// Q = D^-1 S pi from the packed FP64 operator: row r of facet e against the facet's own
-// vertices and the two opposite it.  A neighbour facet of cell s joins two of that cell's
-// three vertices; its row's entries are summed with weights 1 - t_c and t_c onto its lower
-// and higher vertex.  Once per condensation; FP64 sums (S annihilates smooth traces up to
-// its scale, so the sums cancel), rounded once for the FP32 copy.
-template <int P>
-__global__ void prolong_op_kernel(int NF, const double *__restrict__ Sval, const double *__restrict__ Dinv,
-                                  const int32_t *__restrict__ nbr, const int32_t *__restrict__ fverts,
-                                  double *__restrict__ Q, float *__restrict__ Q32) {
+// The smoother's operators from the packed FP64 operator, once per condensation, in FP64
+// and rounded once for the FP32 and BF16 copies: H, the four neighbour blocks of D^-1 S
+// (element (r*4+b)*PP+c, packed), the diagonal block D (packed), and, with PROL, Q = D^-1 S
+// pi: row r of facet e against the facet's own vertices and the two opposite it.  A
+// neighbour facet of cell s joins two of that cell's three vertices; its row's entries are
+// summed with weights 1 - t_c and t_c onto its lower and higher vertex.
+struct HatOut {
+    double *H, *D, *Q;
+    float *H32, *D32, *Q32;
+    __nv_bfloat16 *H16;
+};
+template <int P, bool PROL>
+__global__ void hat_op_kernel(int NF, const double *__restrict__ Sval, const double *__restrict__ Dinv,
+                              const int32_t *__restrict__ nbr, const int32_t *__restrict__ fverts, HatOut o) {
     constexpr int PP = P + 1;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= NF) return;
-    const int lo = fverts[2 * e], hi = fverts[2 * e + 1];
-    int slot[5][2];            // of each facet's two vertices: 0 lo, 1 hi, 2 / 3 opposite in cell 0 / 1
-    slot[0][0] = 0;
-    slot[0][1] = 1;
+    double d[PP][PP], w[PP][4];
 #pragma unroll
-    for (int b = 1; b < 5; ++b) {
-        const int f = nbr[size_t(b - 1) * NF + e];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int v = fverts[2 * f + k];
-            slot[b][k] = v == lo ? 0 : v == hi ? 1 : b < 3 ? 2 : 3;
-        }
-    }
-    double w[PP][4];
-#pragma unroll
-    for (int r = 0; r < PP; ++r) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[r][q] = 0.0;
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-            double tot = 0.0, up = 0.0;
-#pragma unroll
-            for (int c = 0; c < PP; ++c) {
-                const double s = Sval[packed_index(size_t((r * 5 + b) * PP + c), size_t(e), size_t(NF), 2)];
-                tot += s;
-                if (c > 0) up = c < P ? fma(s, double(c) / double(P), up) : up + s;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (slot[b][0] == q) w[r][q] += tot - up;
-                if (slot[b][1] == q) w[r][q] += up;
-            }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < PP; ++r) {
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int r = 0; r < PP; ++r)
 #pragma unroll
         for (int c = 0; c < PP; ++c) {
-            const double d = Dinv[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 2)];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = fma(d, w[c][q], v[q]);
+            d[r][c] = Dinv[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 2)];
+            const double s = Sval[packed_index(size_t(r * 5 * PP + c), size_t(e), size_t(NF), 2)];
+            if (o.D) o.D[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 2)] = s;
+            if (o.D32) o.D32[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 4)] = float(s);
         }
+    int lo = 0, hi = 0;
+    if constexpr (PROL) {
+        lo = fverts[2 * e];
+        hi = fverts[2 * e + 1];
+        // the facet's own block (the identity)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            Q[(size_t(r) * NF + e) * 4 + q] = v[q];
-            if (Q32) Q32[(size_t(r) * NF + e) * 4 + q] = float(v[q]);
+        for (int r = 0; r < PP; ++r) {
+            w[r][1] = double(r) / double(P);
+            w[r][0] = 1.0 - w[r][1];
+            w[r][2] = w[r][3] = 0.0;
         }
     }
+#pragma unroll 1
+    for (int b = 0; b < 4; ++b) {
+        int s0 = 0, s1 = 0;                    // slots of the neighbour's vertices: 0 lo, 1 hi, 2 / 3 opposite in cell 0 / 1
+        if constexpr (PROL) {
+            const int f = nbr[size_t(b) * NF + e], v0 = fverts[2 * f], v1 = fverts[2 * f + 1], op = b < 2 ? 2 : 3;
+            s0 = v0 == lo ? 0 : v0 == hi ? 1 : op;
+            s1 = v1 == lo ? 0 : v1 == hi ? 1 : op;
+        }
+        double tot[PP], up[PP];
+#pragma unroll
+        for (int r = 0; r < PP; ++r) tot[r] = up[r] = 0.0;
+#pragma unroll
+        for (int c = 0; c < PP; ++c) {
+            double s[PP];
+#pragma unroll
+            for (int q = 0; q < PP; ++q)
+                s[q] = Sval[packed_index(size_t((q * 5 + 1 + b) * PP + c), size_t(e), size_t(NF), 2)];
+#pragma unroll
+            for (int r = 0; r < PP; ++r) {
+                double v = 0.0;
+#pragma unroll
+                for (int q = 0; q < PP; ++q) v = fma(d[r][q], s[q], v);
+                const size_t j = size_t((r * 4 + b) * PP + c);
+                if (o.H) o.H[packed_index(j, size_t(e), size_t(NF), 2)] = v;
+                if (o.H32) o.H32[packed_index(j, size_t(e), size_t(NF), 4)] = float(v);
+                if (o.H16) o.H16[packed_index(j, size_t(e), size_t(NF), 8)] = __double2bfloat16(v);
+                if constexpr (PROL) {
+                    tot[r] += v;
+                    if (c > 0) up[r] = c < P ? fma(v, double(c) / double(P), up[r]) : up[r] + v;
+                }
+            }
+        }
+        if constexpr (PROL) {
+#pragma unroll
+            for (int r = 0; r < PP; ++r)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (s0 == q) w[r][q] += tot[r] - up[r];
+                    if (s1 == q) w[r][q] += up[r];
+                }
+        }
+    }
+    if constexpr (PROL) {
+#pragma unroll
+        for (int r = 0; r < PP; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                o.Q[(size_t(r) * NF + e) * 4 + q] = w[r][q];
+                if (o.Q32) o.Q32[(size_t(r) * NF + e) * 4 + q] = float(w[r][q]);
+            }
+    }
+    // (padding lanes of the last groups are never multiplied)
 }
 
 
-// first sweep from a zero initial guess: x = omega D^-1 b
+// first sweep from a zero initial guess: bh = D^-1 b (kept for the sweeps that follow;
+// null: not wanted), x = omega bh
 template <int P, typename T>
 __device__ __forceinline__ void smooth_first_kernel_impl(int bid_, int nb_, int NF, const T *__restrict__ Dinv,
-                                                         const T *__restrict__ b, T *__restrict__ xout, T omega,
+                                                         const T *__restrict__ b, T *__restrict__ xout, T *__restrict__ bh, T omega,
                                                          const T *__restrict__ w, const double *__restrict__ hnext,
                                                          T *__restrict__ bout) {
     // with w: the right-hand side is the next Arnoldi vector b = w / h_{j+1,j}
@@ -691,14 +764,17 @@ __device__ __forceinline__ void smooth_first_kernel_impl(int bid_, int nb_, int 
     }
     block_solve_packed<P, T, T>(Dinv, e, NF, v, d);
 #pragma unroll
-    for (int r = 0; r < PP; ++r) xout[size_t(r) * NF + e] = omega * d[r];
+    for (int r = 0; r < PP; ++r) {
+        if (bh) bh[size_t(r) * NF + e] = d[r];
+        xout[size_t(r) * NF + e] = omega * d[r];
+    }
 }
 template <int P, typename T>
-__global__ void smooth_first_kernel(int NF, const T *__restrict__ Dinv, const T *__restrict__ b, T *__restrict__ xout,
+__global__ void smooth_first_kernel(int NF, const T *__restrict__ Dinv, const T *__restrict__ b, T *__restrict__ xout, T *__restrict__ bh,
                                     T omega, const T *__restrict__ w, const double *__restrict__ hnext,
                                     T *__restrict__ bout) {
     pdl_wait();
-    smooth_first_kernel_impl<P, T>(blockIdx.x, gridDim.x, NF, Dinv, b, xout, omega, w, hnext, bout);
+    smooth_first_kernel_impl<P, T>(blockIdx.x, gridDim.x, NF, Dinv, b, xout, bh, omega, w, hnext, bout);
 }
 template <int P, typename T>
 struct smooth_first_kernel_args {
@@ -707,6 +783,7 @@ struct smooth_first_kernel_args {
     const T *Dinv;
     const T *b;
     T *xout;
+    T *bh;
     T omega;
     const T *w;
     const double *hnext;
@@ -717,11 +794,11 @@ __global__ void smooth_first_kernel_multi(const __grid_constant__ MultiP<smooth_
     pdl_wait();
     int b_;
     const smooth_first_kernel_args<P, T> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    smooth_first_kernel_impl<P, T>(b_, q_.nb_, q_.NF, q_.Dinv, q_.b, q_.xout, q_.omega, q_.w, q_.hnext, q_.bout);
+    smooth_first_kernel_impl<P, T>(b_, q_.nb_, q_.NF, q_.Dinv, q_.b, q_.xout, q_.bh, q_.omega, q_.w, q_.hnext, q_.bout);
 }
 template <int P, typename T>
 void smooth_first_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const T *Dinv,
-                            const T *b, T *xout, T omega, const T *w, const double *hnext, T *bout) {
+                            const T *b, T *xout, T *bh, T omega, const T *w, const double *hnext, T *bout) {
     if (Recorder *r_ = batch_recorder()) {
         smooth_first_kernel_args<P, T> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
@@ -730,6 +807,7 @@ void smooth_first_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaS
         q_.Dinv = Dinv;
         q_.b = b;
         q_.xout = xout;
+        q_.bh = bh;
         q_.omega = omega;
         q_.w = w;
         q_.hnext = hnext;
@@ -737,7 +815,7 @@ void smooth_first_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaS
         batch_record(r_, reinterpret_cast<const void *>(&smooth_first_kernel_multi<P, T>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &smooth_first_kernel<P, T>, grid_, block_, smem_, s_, NF, Dinv, b, xout, omega, w, hnext, bout);
+    pdl_launch(kPdlFamily, &smooth_first_kernel<P, T>, grid_, block_, smem_, s_, NF, Dinv, b, xout, bh, omega, w, hnext, bout);
 }
 
 
@@ -1097,12 +1175,16 @@ template <typename T> struct Ops;
 template <> struct Ops<double> {
     static const double *S(hdg_handle *h, bool) { return h->d_Sval; }
     static const double *D(hdg_handle *h) { return h->d_Dinv; }
+    static const double *H(hdg_handle *h) { return h->d_H; }
+    static const double *Dg(hdg_handle *h) { return h->d_D; }
 };
 template <> struct Ops<float> {
     static const float *S(hdg_handle *h, bool) { return h->d_Sval32; }
     static const float *D(hdg_handle *h) { return h->d_Dinv32; }
+    static const float *H(hdg_handle *h) { return h->d_H32; }
+    static const float *Dg(hdg_handle *h) { return h->d_D32; }
 };
-inline bool bf16_pre(hdg_handle *h) { return h->prm.precision == HDG_MIXED_BF16 && h->d_Sval16; }
+inline bool bf16_pre(hdg_handle *h) { return h->prm.precision == HDG_MIXED_BF16 && h->d_H16; }
 
 template <typename T>
 cudaError_t launch_apply_dots_t(hdg_handle *h, const T *x, T *y, const T *V, size_t ld, int k, double *partial,
@@ -1120,45 +1202,39 @@ cudaError_t launch_apply_t(hdg_handle *h, const T *x, T *y) {
 // Krylov residual (pre = false)
 template <typename T>
 cudaError_t launch_residual_t(hdg_handle *h, const T *b, const T *x, T *r, bool pre) {
-    if constexpr (std::is_same<T, float>::value) if (pre && bf16_pre(h)) {
-        HDG_DISPATCH_PF(h->pf, T, (residual_kernel_go<P, T, __nv_bfloat16>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, h->d_nbr, b, x, r)));
+    HDG_DISPATCH_PF(h->pf, T, (residual_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, pre), h->d_nbr, b, x, r)));
+    return cudaGetLastError();
+}
+// A sweep with b = D^-1 times the right-hand side where the handle's sweeps of this type
+// work on D^-1 S (hat_form), else the right-hand side itself; with cheb, a step of the
+// Chebyshev iteration xout = x + omega D^-1 (b - S x) + beta (x - xprev)
+template <typename T, bool CHEB>
+cudaError_t smooth_any(hdg_handle *h, const T *b, const T *x, T *xout, T om, T beta, const T *xprev) {
+    if constexpr (std::is_same<T, float>::value) if (bf16_pre(h)) {
+        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, __nv_bfloat16, true, CHEB>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_H16, nullptr, h->d_nbr, b, x, xout, om, beta, xprev)));
         return cudaGetLastError();
     }
-    {
-        HDG_DISPATCH_PF(h->pf, T, (residual_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, pre), h->d_nbr, b, x, r)));
+    if (Ops<T>::H(h)) {
+        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T, true, CHEB>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::H(h), nullptr, h->d_nbr, b, x, xout, om, beta, xprev)));
+    } else {
+        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T, false, CHEB>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, xout, om, beta, xprev)));
     }
     return cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_smooth_t(hdg_handle *h, const T *b, const T *x, T *xout) {
-    const T om = T(h->prm.omega);
-    if constexpr (std::is_same<T, float>::value) if (bf16_pre(h)) {
-        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, __nv_bfloat16>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, Ops<T>::D(h), h->d_nbr, b, x, xout, om, T(0), nullptr)));
-        return cudaGetLastError();
-    }
-    {
-        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, xout, om, T(0), nullptr)));
-    }
-    return cudaGetLastError();
+    return smooth_any<T, false>(h, b, x, xout, T(h->prm.omega), T(0), nullptr);
 }
-// a step of the Chebyshev iteration: xout = x + omega D^-1 (b - S x) + beta (x - xprev)
 template <typename T>
 cudaError_t launch_smooth_cheb_t(hdg_handle *h, const T *b, const T *x, T *xout, double omega, double beta,
                                  const T *xprev) {
-    if constexpr (std::is_same<T, float>::value) if (bf16_pre(h)) {
-        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, __nv_bfloat16, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, Ops<T>::D(h), h->d_nbr, b, x, xout, T(omega), T(beta), xprev)));
-        return cudaGetLastError();
-    }
-    {
-        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, xout, T(omega), T(beta), xprev)));
-    }
-    return cudaGetLastError();
+    return smooth_any<T, true>(h, b, x, xout, T(omega), T(beta), xprev);
 }
 template <typename T>
-cudaError_t launch_smooth_first_t(hdg_handle *h, const T *b, T *x, const T *w, const double *hnext, T *bout,
+cudaError_t launch_smooth_first_t(hdg_handle *h, const T *b, T *x, T *bh, const T *w, const double *hnext, T *bout,
                                   double omega) {
     const T om = T(omega > 0 ? omega : h->prm.omega);
-    HDG_DISPATCH_PF(h->pf, T, (smooth_first_kernel_go<P, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::D(h), b, x, om, w, hnext, bout)));
+    HDG_DISPATCH_PF(h->pf, T, (smooth_first_kernel_go<P, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::D(h), b, x, bh, om, w, hnext, bout)));
     return cudaGetLastError();
 }
 template <typename T>
@@ -1184,10 +1260,14 @@ template <typename T>
 cudaError_t launch_residual_smooth_t(hdg_handle *h, const T *b, const T *x, T *res, T *y, double omega) {
     const T om = T(omega > 0 ? omega : h->prm.omega);
     if constexpr (std::is_same<T, float>::value) if (bf16_pre(h)) {
-        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, __nv_bfloat16>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_Sval16, Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
+        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, __nv_bfloat16, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, h->d_H16, Ops<T>::Dg(h), h->d_nbr, b, x, res, y, om)));
         return cudaGetLastError();
     }
-    HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
+    if (Ops<T>::H(h)) {
+        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::H(h), Ops<T>::Dg(h), h->d_nbr, b, x, res, y, om)));
+    } else {
+        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T, false>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
+    }
     return cudaGetLastError();
 }
 template cudaError_t launch_residual_smooth_t<double>(hdg_handle *, const double *, const double *, double *, double *, double);
@@ -1197,7 +1277,7 @@ cudaError_t launch_prolong_add_t(hdg_handle *h, const T *ec, T *x) {
     HDG_DISPATCH_P(h->p, (prolong_add_kernel<P, T><<<blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream>>>(h->NF, h->d_facet_verts, ec, x)));
     return cudaGetLastError();
 }
-// FP32 / BF16 copies of the packed FP64 operator and the FP32 inverse blocks
+// FP32 copies of the packed FP64 operator and the inverse blocks
 cudaError_t launch_repack(hdg_handle *h) {
     const int pp = h->pp, ns = 5 * pp * pp, nd = pp * pp;
     const size_t NF = h->NF;
@@ -1206,8 +1286,6 @@ cudaError_t launch_repack(hdg_handle *h) {
         repack_kernel<float><<<blocks(nq(ns, 4), 256), 256, 0, h->stream>>>(h->d_Sval, ns, NF, h->d_Sval32);
         repack_kernel<float><<<blocks(nq(nd, 4), 256), 256, 0, h->stream>>>(h->d_Dinv, nd, NF, h->d_Dinv32);
     }
-    if (h->d_Sval16)
-        repack_kernel<__nv_bfloat16><<<blocks(nq(ns, 8), 256), 256, 0, h->stream>>>(h->d_Sval, ns, NF, h->d_Sval16);
     return cudaGetLastError();
 }
 
@@ -1225,15 +1303,22 @@ template cudaError_t launch_smooth_cheb_t<double>(hdg_handle *, const double *, 
                                                   double, const double *);
 template cudaError_t launch_smooth_cheb_t<float>(hdg_handle *, const float *, const float *, float *, double, double,
                                                  const float *);
-template cudaError_t launch_smooth_first_t<double>(hdg_handle *, const double *, double *, const double *,
+template cudaError_t launch_smooth_first_t<double>(hdg_handle *, const double *, double *, double *, const double *,
                                                    const double *, double *, double);
-template cudaError_t launch_smooth_first_t<float>(hdg_handle *, const float *, float *, const float *, const double *,
+template cudaError_t launch_smooth_first_t<float>(hdg_handle *, const float *, float *, float *, const float *, const double *,
                                                   float *, double);
 template cudaError_t launch_restrict_t<double>(hdg_handle *, const double *, double *, const double *, double, double *);
 template cudaError_t launch_restrict_t<float>(hdg_handle *, const float *, float *, const float *, float, float *);
-cudaError_t launch_prolong_op(hdg_handle *h) {
-    HDG_DISPATCH_P(h->p, (prolong_op_kernel<P><<<blocks(h->NF, 128), 128, 0, h->stream>>>(
-                             h->NF, h->d_Sval, h->d_Dinv, h->d_nbr, h->d_facet_verts, h->d_Q, h->d_Q32)));
+cudaError_t launch_hat_op(hdg_handle *h) {
+    const HatOut o{h->d_H, h->d_D, h->d_Q, h->d_H32, h->d_D32, h->d_Q32, h->d_H16};
+    const unsigned nb = blocks(h->NF, 128);
+    if (h->d_Q) {
+        HDG_DISPATCH_P(h->p, (hat_op_kernel<P, true><<<nb, 128, 0, h->stream>>>(h->NF, h->d_Sval, h->d_Dinv, h->d_nbr,
+                                                                              h->d_facet_verts, o)));
+    } else {
+        HDG_DISPATCH_PF(h->pf, double, (hat_op_kernel<P, false><<<nb, 128, 0, h->stream>>>(h->NF, h->d_Sval, h->d_Dinv,
+                                                                                         h->d_nbr, h->d_facet_verts, o)));
+    }
     return cudaGetLastError();
 }
 template cudaError_t launch_smooth_prolong_t<double>(hdg_handle *, const double *, const double *, const double *, double *,
