@@ -761,7 +761,7 @@ __global__ void identity_kernel(int n, double *inv) {
 
 __global__ void to_f32_kernel(const double *x, float *y, size_t n) {
     size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = float(x[i]);
+    if (i < n) y[i] = to_float(x[i]);
 }
 
 template <int P, bool FC, bool FF>

@@ -250,7 +250,7 @@ __device__ __forceinline__ void ff_join_kernel_impl(int bid_, int nb_, const flo
     const size_t i = size_t(bid_) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float2 v = x2[i];
-    const double r = double(v.x) + double(v.y);
+    const double r = join(v);
     a[i] = r;
     if (b) b[i] = r;
 }
@@ -291,22 +291,6 @@ void ff_join_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream
 
 // r = b - S x with x given split; S split in the packed FP64 layout (element
 // j of facet e in 16-byte group (j / 2, e), lane j % 2, here two float pairs)
-// sum of a double over the block (fixed tree: warp shuffles, then warp 0 over
-// the warp sums); every thread gets the block's sum in warp 0, the others
-// their warp's
-__device__ __forceinline__ double ff_block_sum(double v) {
-    __shared__ double red[32];
-    __syncthreads();
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    const int nw = blockDim.x / 32;
-    v = (threadIdx.x < nw) ? red[threadIdx.x] : 0.0;
-    if (warp == 0)
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
 
 // res = b - S x in two-float arithmetic (x as split pairs), one thread per
 // facet row: a block takes kResFacets facets, thread (r, f) of it row r of
@@ -358,14 +342,14 @@ __device__ __forceinline__ void residual_ff_kernel_impl(int bid_, int nb_, int N
         const double rv = b[size_t(r) * NF + e] - acc.value();
         if (res) res[size_t(r) * NF + e] = rv;
         if (c32.b32) {
-            c32.b32[size_t(r) * NF + e] = float(rv * c32.scale);
+            c32.b32[size_t(r) * NF + e] = to_float(rv * c32.scale);
             c32.z32[size_t(r) * NF + e] = 0.0f;
         }
         sq = rv * rv;
     }
     if (!partial) return;
     __shared__ bool last;
-    const double tot = ff_block_sum(sq);
+    const double tot = block_sum_warp0(sq);
     if (threadIdx.x == 0) {
         partial[bid_] = tot;
         __threadfence();                       // the partial is visible before the count
@@ -376,7 +360,7 @@ __device__ __forceinline__ void residual_ff_kernel_impl(int bid_, int nb_, int N
     __threadfence();
     double a = 0.0;
     for (int i = threadIdx.x; i < nb_; i += blockDim.x) a += partial[i];
-    a = ff_block_sum(a);
+    a = block_sum_warp0(a);
     if (threadIdx.x == 0) {
         *counter = 0u;
         out[0] = a;
@@ -774,11 +758,11 @@ __global__ void __launch_bounds__(32 * kSolveWarps<P>) recover_ff_kernel(int N, 
     __syncthreads();
     for (int j = threadIdx.x; j < nc * 2 * NP; j += blockDim.x) {
         const float2 v = sV[j % (2 * NP)][j / (2 * NP)];
-        u[size_t(K0) * 2 * NP + j] = double(v.x) + double(v.y);
+        u[size_t(K0) * 2 * NP + j] = join(v);
     }
     for (int j = threadIdx.x; j < nc * NP; j += blockDim.x) {
         const float2 v = sV[2 * NP + j % NP][j / NP];
-        hout[size_t(K0) * NP + j] = double(v.x) + double(v.y);
+        hout[size_t(K0) * NP + j] = join(v);
     }
 }
 

@@ -253,7 +253,7 @@ __global__ void scale_round_kernel(const double *__restrict__ w, const double *_
         v = v * inv_h;
         v64[i] = v;
     }
-    v32[i] = float(v);
+    v32[i] = to_float(v);
 }
 
 // the FP32 preconditioner's output widened to the FP64 basis Z
@@ -432,7 +432,7 @@ __device__ __forceinline__ void d2f_norm_kernel_impl(int bid_, int nb_, const do
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
             if (i + u * stride < n) {
-                const float v = float(a[u] * inv);
+                const float v = to_float(a[u] * inv);
                 y[i + u * stride] = v;
                 z[i + u * stride] = 0.0f;
                 acc = fmaf(v, v, acc);

@@ -26,7 +26,7 @@ namespace {
 
 template <typename TO> __device__ __forceinline__ TO convert_to(double v);
 template <> __device__ __forceinline__ double convert_to<double>(double v) { return v; }
-template <> __device__ __forceinline__ float convert_to<float>(double v) { return float(v); }
+template <> __device__ __forceinline__ float convert_to<float>(double v) { return to_float(v); }
 
 // Operator values are packed in 16-byte groups: element j of facet e lives at
 // group (j / G, e), lane j % G, with G = 16 / sizeof(storage); every thread
@@ -663,7 +663,7 @@ __global__ void hat_op_kernel(int NF, const double *__restrict__ Sval, const dou
             d[r][c] = Dinv[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 2)];
             const double s = Sval[packed_index(size_t(r * 5 * PP + c), size_t(e), size_t(NF), 2)];
             if (o.D) o.D[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 2)] = s;
-            if (o.D32) o.D32[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 4)] = float(s);
+            if (o.D32) o.D32[packed_index(size_t(r * PP + c), size_t(e), size_t(NF), 4)] = to_float(s);
         }
     int lo = 0, hi = 0;
     if constexpr (PROL) {
@@ -701,7 +701,7 @@ __global__ void hat_op_kernel(int NF, const double *__restrict__ Sval, const dou
                 for (int q = 0; q < PP; ++q) v = fma(d[r][q], s[q], v);
                 const size_t j = size_t((r * 4 + b) * PP + c);
                 if (o.H) o.H[packed_index(j, size_t(e), size_t(NF), 2)] = v;
-                if (o.H32) o.H32[packed_index(j, size_t(e), size_t(NF), 4)] = float(v);
+                if (o.H32) o.H32[packed_index(j, size_t(e), size_t(NF), 4)] = to_float(v);
                 if (o.H16) o.H16[packed_index(j, size_t(e), size_t(NF), 8)] = __double2bfloat16(v);
                 if constexpr (PROL) {
                     tot[r] += v;
@@ -725,7 +725,7 @@ __global__ void hat_op_kernel(int NF, const double *__restrict__ Sval, const dou
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 o.Q[(size_t(r) * NF + e) * 4 + q] = w[r][q];
-                if (o.Q32) o.Q32[(size_t(r) * NF + e) * 4 + q] = float(w[r][q]);
+                if (o.Q32) o.Q32[(size_t(r) * NF + e) * 4 + q] = to_float(w[r][q]);
             }
     }
     // (padding lanes of the last groups are never multiplied)
@@ -906,23 +906,6 @@ __global__ void rhs_cell_kernel(int N, const double *__restrict__ W, const doubl
     ycell[idx] = acc;
 }
 
-// step 1, facet part: g_{e,r} = sum over the two cells of their row of edge i_s
-// sum of a double over the block (fixed tree: warp shuffles, then warp 0 over
-// the warp sums); thread 0 holds the block's sum
-__device__ __forceinline__ double gather_block_sum(double v) {
-    __shared__ double red[32];
-    __syncthreads();
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    const int nw = blockDim.x / 32;
-    v = (threadIdx.x < nw) ? red[threadIdx.x] : 0.0;
-    if (warp == 0)
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-
 // g on facet e = the two cells' contributions (step 1 of Sec. 4.2); with
 // partial non-null also ||g||^2 (block sums, the last block adding them in
 // block order into out[0] and handing the value to the host through pub)
@@ -940,12 +923,13 @@ __device__ __forceinline__ void rhs_gather_kernel_impl(int bid_, int nb_, int N,
     if (e < NF) {
         double v[PP];
 #pragma unroll
-        for (int r = 0; r < PP; ++r) v[r] = 0.0;
-#pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int K = fcell[2 * e + s], i = fedge[2 * e + s], f = flip[3 * K + i];
 #pragma unroll
-            for (int r = 0; r < PP; ++r) v[r] += ycell[size_t(i * PP + (f ? P - r : r)) * N + K];
+            for (int r = 0; r < PP; ++r) {
+                const double y = ycell[size_t(i * PP + (f ? P - r : r)) * N + K];
+                v[r] = s == 0 ? y : v[r] + y;
+            }
         }
 #pragma unroll
         for (int r = 0; r < PP; ++r) {
@@ -955,14 +939,14 @@ __device__ __forceinline__ void rhs_gather_kernel_impl(int bid_, int nb_, int N,
         if (c32.b32) {
 #pragma unroll
             for (int r = 0; r < PP; ++r) {
-                c32.b32[size_t(r) * NF + e] = float(v[r] * c32.scale);
+                c32.b32[size_t(r) * NF + e] = to_float(v[r] * c32.scale);
                 c32.z32[size_t(r) * NF + e] = 0.0f;
             }
         }
     }
     if (!partial) return;
     __shared__ bool last;
-    const double tot = gather_block_sum(sq);
+    const double tot = block_sum_warp0(sq);
     if (threadIdx.x == 0) {
         partial[bid_] = tot;
         __threadfence();                       // the partial is visible before the count
@@ -973,7 +957,7 @@ __device__ __forceinline__ void rhs_gather_kernel_impl(int bid_, int nb_, int N,
     __threadfence();
     double a = 0.0;
     for (int i = threadIdx.x; i < nb_; i += blockDim.x) a += partial[i];
-    a = gather_block_sum(a);
+    a = block_sum_warp0(a);
     if (threadIdx.x == 0) {
         *counter = 0u;
         out[0] = a;
