@@ -465,8 +465,8 @@ struct TailArgs {
 //
 // Conversions between FP64 and FP32 run at the FP64 pipe's rate (a warp instruction in
 // about 77 cycles of a scheduler, measured), four instructions for split and three for
-// join, so the three below work on the bits instead: a dozen integer instructions, the
-// same rounding to nearest even, bit for bit.  Values whose parts leave the normal range
+// join, so the functions below work on the bits instead: a dozen integer instructions, the
+// same rounding to nearest even, bit for bit.  Values that leave the normal range
 // (zeros, infinities and NaN among them) take the plain conversions.  At p = 3 the
 // condensation of 20,480 cells takes 1773 instead of 1885 us, step 1 on 81,920 cells 62
 // instead of 70 us.
@@ -517,6 +517,13 @@ __host__ __device__ __forceinline__ float to_float(double a) {
     const uint64_t u = bits_of(a);
     if ((uint32_t(u >> 52) & 0x7ffu) - 898u > 251u) return float(a);
     return round_bits(u);
+}
+// a * p2 for a power of two p2: the exponents added where both values are normal
+__host__ __device__ __forceinline__ double mul_pow2(double a, double p2) {
+    const uint64_t u = bits_of(a);
+    const int ex = int(uint32_t(u >> 52) & 0x7ffu), k = int(uint32_t(bits_of(p2) >> 52)) - 1023;
+    if (unsigned(ex - 1) > 2045u || unsigned(ex + k - 1) > 2045u) return a * p2;
+    return double_of(uint32_t(u >> 32) + (uint32_t(k) << 20), uint32_t(u));
 }
 // (rn(a), rn(a - hi)): a - hi is the signed count of the last mantissa units rounded off
 __host__ __device__ __forceinline__ float2 split(double a) {
@@ -991,7 +998,7 @@ cudaError_t launch_rhs(hdg_handle *h, const double *r_u, const double *r_h, doub
 cudaError_t launch_rhs_gather(hdg_handle *h, const double *ycell, double *g, const NormOut &nrm = NormOut());
 // two-float versions of the FP64 steps (mixed modes, k_ff.cu)
 cudaError_t launch_split(const double *a, float2 *out, size_t n, cudaStream_t s);
-// facets per block of the two-float residual (its grid: ceil(NF / kResFFFacets)
+// facets per tile of the two-float residual (its grid: at most ceil(NF / kResFFFacets)
 // blocks, each writing one partial sum)
 constexpr int kResFFFacets = 64;
 // x2 += scale[0] * d in two-float arithmetic (first: x2 = scale[0] * d)

@@ -939,7 +939,7 @@ __device__ __forceinline__ void rhs_gather_kernel_impl(int bid_, int nb_, int N,
         if (c32.b32) {
 #pragma unroll
             for (int r = 0; r < PP; ++r) {
-                c32.b32[size_t(r) * NF + e] = to_float(v[r] * c32.scale);
+                c32.b32[size_t(r) * NF + e] = to_float(mul_pow2(v[r], c32.scale));
                 c32.z32[size_t(r) * NF + e] = 0.0f;
             }
         }

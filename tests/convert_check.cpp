@@ -1,4 +1,4 @@
-// Checks the bitwise FP64 / FP32 conversions (common.h: to_float, split, join) against the
+// Checks the bitwise FP64 / FP32 conversions (common.h: to_float, split, join, mul_pow2) against the
 // plain ones, bit for bit: random mantissas at every exponent, ties and carries of the
 // rounding, zeros, infinities and NaN.  Prints the number of cases that differ (a zero
 // trailing part may have either sign).
@@ -21,6 +21,8 @@ int main() {
         const float2 v = split(a);
         if (!same(to_float(a), hi) || !same(v.x, hi) || !(same(v.y, lo) || (v.y == 0.f && lo == 0.f))) ++wrong;
         if (!same(join(make_float2(hi, lo)), double(hi) + double(lo))) ++wrong;
+        for (double p2 : {0x1p-1000, 0x1p-30, 1.0, 0x1p60, 0x1p900})
+            if (!same(mul_pow2(a, p2), a * p2)) ++wrong;
     };
     const uint64_t low[] = {0, 1, 0x0fffffff, 0x10000000, 0x10000001, 0x1fffffff, 0x20000000, 0x2fffffff, 0x30000000,
                             0xfffffffffffffull, 0xfffffe0000000ull, 0xffffff0000000ull, 0xfffffefffffffull};
