@@ -46,11 +46,16 @@ struct Sz {
 // the fastest thread index (shared-memory reads without bank conflicts, global
 // writes in runs of neighbouring cells).  The FP64 pipe is the bound (1.05 TFLOP/s
 // measured, one warp instruction in about 77 cycles per scheduler), so the split is
-// the one that keeps the warps full: at p = 3 8 x 10 columns in the first phase and
-// 8 x 12 in the second, of 96 threads.  The elimination of the whole augmented cell
-// system [A | B | Mass], one cell per block with two barriers per pivot, took 1,466 us
-// on 18,432 cells at p = 2; a change of the time step followed by a solve and recovery
-// there went from 3,014 to 1,965 us.
+// the one that keeps the warps full (at p = 3 8 x 10 columns up to S, 8 x 12 for X_B
+// and all 8 x 30 of R_M dealt to the 96 threads) and what need not be FP64 is not: the
+// conversions to float pairs, the correction of the refinement, pivot tests.  The h
+// columns of R_M are S^-1 as it stands, and R_M's h rows are not refined (step 1 and
+// the recovery of the two-float handles are as exact either way, 1e-14 to 7e-14 of the
+// oracle at p = 1 .. 4, Courant 8 and 16).  20,480 cells at p = 3, two-float, f varying:
+// 1,345 us instead of 1,773 (one pass of 10 of 12 columns per component of R_M, all of
+// them refined in FP64, a full division per pivot and column, two products where column
+// k meets the pivot's); 18,432 cells at p = 2 in FP64: 384 instead of 419, against 1,466
+// by elimination of the whole augmented cell system [A | B | Mass], one cell per block.
 template <int P> constexpr int kCondCells = P == 1 ? 16 : P == 2 ? 10 : P == 3 ? 8 : 6;
 constexpr int kCondThreads = 96;
 
@@ -66,6 +71,16 @@ struct NodalArgs {
     float4 *PQ2;                       // weights and (f varying over a cell) P, Q
     int32_t *status;
 };
+
+// 1 / d by Newton's iteration from a single-precision reciprocal: two steps from 2^-23
+// (four FMAs; the division takes about twice as many FP64 instructions)
+__device__ __forceinline__ double reciprocal(double d) {
+    const unsigned ex = (unsigned(__double2hiint(d)) >> 20) & 0x7ffu;
+    if (ex - 923u > 200u) return 1.0 / d;                      // outside 2^-100 .. 2^100
+    double r = join(make_float2(__frcp_rn(to_float(d)), 0.0f));
+    r = fma(r, fma(-d, r, 1.0), r);
+    return fma(r, fma(-d, r, 1.0), r);
+}
 
 // In-place inverse of the n x n matrices A[(i * n + j) * CC + c] of the block's cells
 // by Gauss-Jordan elimination with partial pivoting; thread (c, j) owns column j.
@@ -98,8 +113,10 @@ __device__ __forceinline__ void block_inverse(double *A, int c, int j, bool on, 
                 if (i == p) d = f[i];
                 if (i == k) fk = f[i];
             }
-            if (!(fabs(d) > 1e-300)) *bad = 1;
-            const double r = 1.0 / d;
+            // (the exponent first: comparisons take the FP64 pipe)
+            const unsigned ex = (unsigned(__double2hiint(d)) >> 20) & 0x7ffu;
+            if (ex - 27u > 2019u && !(fabs(d) > 1e-300)) *bad = 1;
+            const double r = reciprocal(d);
             double *a = A + j * CC + c;
             const double akj = a[k * n * CC], apj = a[p * n * CC];
             if (p != k) a[p * n * CC] = akj;   // the rows swapped
@@ -108,7 +125,7 @@ __device__ __forceinline__ void block_inverse(double *A, int c, int j, bool on, 
             for (int i = 0; i < n; ++i) {
                 const double fi = i == p ? fk : f[i];   // column k after the swap
                 const double aij = a[i * n * CC];
-                a[i * n * CC] = i == k ? row : j == k ? -fi * r : fma(-fi, row, aij);
+                a[i * n * CC] = i == k ? row : fma(-fi, row, j == k ? 0.0 : aij);   // (j == k: row = r)
             }
             if (j == 0) piv[k * CC + c] = p;
         }
@@ -162,14 +179,15 @@ __device__ __forceinline__ void add_div(const double *ref, double g00, double g0
     });
 }
 
-// h = S^-1 rh and (wx, wy) -= T h (Ts null: h alone), cell c of the block's matrices.  So non-null: S
-// itself, for one step of iterative refinement of h.  The explicit inverse alone
+// h = S^-1 rh and (wx, wy) -= T h (Ts null: h alone), cell c of the block's matrices.  So
+// non-null: S itself, for one step of iterative refinement of h, the residual in FP64 and
+// its correction, 1e-14 of h, with the inverse rounded to FP32 (Sf).  The explicit inverse alone
 // leaves S_K about 20 times less exact than an elimination of the whole cell system
 // (p = 3, Courant 16: S_K applied to a nearly constant trace off by 1e-12 instead of
 // 7e-14); one step brings it to 2e-14.
 template <int NP, int CC>
-__device__ __forceinline__ void back_substitute(const double *Ss, const double *So, const double *Ts, int c,
-                                                const double (&rh)[NP], double (&wx)[NP], double (&wy)[NP],
+__device__ __forceinline__ void back_substitute(const double *Ss, const double *So, const float *Sf, const double *Ts,
+                                                int c, const double (&rh)[NP], double (&wx)[NP], double (&wy)[NP],
                                                 double (&h)[NP]) {
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
@@ -180,22 +198,22 @@ __device__ __forceinline__ void back_substitute(const double *Ss, const double *
         h[i] = v;
     }
     if (So) {
-        double res[NP];
+        float res[NP];
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             row_fence();
             double v = rh[i];
 #pragma unroll
             for (int k = 0; k < NP; ++k) v = fma(-So[(i * NP + k) * CC + c], h[k], v);
-            res[i] = v;
+            res[i] = to_float(v);
         }
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             row_fence();
-            double v = h[i];
+            float v = 0.0f;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) v = fma(Ss[(i * NP + k) * CC + c], res[k], v);
-            h[i] = v;
+            for (int k = 0; k < NP; ++k) v = fmaf(Sf[(i * NP + k) * CC + c], res[k], v);
+            h[i] += join(make_float2(v, 0.0f));
         }
     }
     if (!Ts) return;
@@ -208,6 +226,16 @@ __device__ __forceinline__ void back_substitute(const double *Ss, const double *
             wy[i] = fma(-Ts[((NP + i) * NP + k) * CC + c], h[k], wy[i]);
         }
     }
+}
+
+// edge weights of C: (H t_y, -H t_x, tau_s |e|) of edge e of cell K
+__device__ __forceinline__ void edge_weights(const NodalArgs &a, const double *geo, int CC, int c, int K, int e,
+                                             double (&w)[3]) {
+    const double *x = a.X + size_t(K) * 6;
+    const double det = (x[2] - x[0]) * (x[5] - x[1]) - (x[4] - x[0]) * (x[3] - x[1]);
+    w[0] = a.H * det * geo[(4 + 3 * e) * CC + c];
+    w[1] = a.H * det * geo[(5 + 3 * e) * CC + c];
+    w[2] = a.ts * det * geo[(6 + 3 * e) * CC + c];
 }
 
 // row (edge e, node jj) of C q into out[row * ld]; diag is added to the rows of edge e0
@@ -243,7 +271,8 @@ struct CondSmem {
     static constexpr int oRef = 0, oM1 = nodal_offsets(P).total, oGeo = oM1 + PP * PP;
     static constexpr int nGeo = 4 + 9 + 2 + 3;                     // j, edge weights, R (FC), f
     static constexpr int oS = oGeo + nGeo * CC, oT = oS + NN * CC, oSo = oT + 2 * NN * CC, oP = oSo + NN * CC;
-    static constexpr int oQ = oP + (FC ? 0 : NN * CC), total = oQ + (FC ? 0 : NN * CC);
+    static constexpr int oQ = oP + (FC ? 0 : NN * CC);
+    static constexpr int oSf = oQ + (FC ? 0 : NN * CC), total = oSf + (NN * CC + 1) / 2;   // (oSf: floats)
 };
 
 template <int P, bool FC, bool FF>
@@ -254,6 +283,7 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
     extern __shared__ double sm[];
     double *ref = sm + L::oRef, *m1 = sm + L::oM1, *geo = sm + L::oGeo;
     double *Ss = sm + L::oS, *Ts = sm + L::oT, *So = sm + L::oSo, *Ps = sm + L::oP, *Qs = sm + L::oQ;
+    float *Sf = reinterpret_cast<float *>(sm + L::oSf);
     __shared__ int piv[NP * CC];
     __shared__ int bad;
     const int t = threadIdx.x, c = t % CC, j = t / CC;
@@ -379,16 +409,15 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
         if (t == 0) atomicOr(a.status, 1);
         return;
     }
-
-    const double *x = a.X + size_t(cell ? K : 0) * 6;
-    const double det = (x[2] - x[0]) * (x[5] - x[1]) - (x[4] - x[0]) * (x[3] - x[1]);
-    double wn[3][3];                           // edge weights of C: (H t_y, -H t_x, tau_s |e|)
+    if (on) {
 #pragma unroll
-    for (int e = 0; e < 3; ++e) {
-        wn[e][0] = a.H * det * geo[(4 + 3 * e) * CC + c];
-        wn[e][1] = a.H * det * geo[(5 + 3 * e) * CC + c];
-        wn[e][2] = a.ts * det * geo[(6 + 3 * e) * CC + c];
+        for (int i = 0; i < NP; ++i) Sf[(i * NP + j) * CC + c] = to_float(Ss[(i * NP + j) * CC + c]);
     }
+    __syncthreads();
+
+    double wn[3][3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, cell ? K : 0, e, wn[e]);
     const size_t N = a.N;
     // ---- X_B and S_K, column (edge e, trace node jj)
     if (cell && j < M) {
@@ -427,7 +456,7 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
             }
         }
         add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
-        back_substitute<NP, CC>(Ss, So, Ts, c, rh, wx, wy, h);
+        back_substitute<NP, CC>(Ss, So, Sf, Ts, c, rh, wx, wy, h);
         if constexpr (FF) {
             constexpr int CPb = (M + 1) / 2;
 #pragma unroll
@@ -446,7 +475,7 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                 a.Xb[(size_t(2 * NP + i) * M + j) * N + K] = h[i];
             }
         }
-        c_rows<P>(m1, wn, wx, wy, h, e, jj, a.ts * det * geo[(6 + 3 * e) * CC + c], a.Scell + size_t(K) * M * M + j, M);
+        c_rows<P>(m1, wn, wx, wy, h, e, jj, e == 0 ? wn[0][2] : e == 1 ? wn[1][2] : wn[2][2], a.Scell + size_t(K) * M * M + j, M);
     }
     if constexpr (FF) {
         // P and Q (f varying over the cell) as float pairs in cell tiles, and the cell's weights (k_ff.cu)
@@ -472,11 +501,16 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
         }
     }
     // ---- R_M and W_K (two-float handles: the h rows of R_M): the columns of the unit
-    // vectors in u_x, u_y and h
-    if (on) {
-#pragma unroll 1
-        for (int comp = 0; comp < 3; ++comp) {
-            double wx[NP], wy[NP], rh[NP], h[NP];
+    // vectors in u_x, u_y and h, spread over all the block's threads.  The h columns' h is
+    // a column of S^-1 itself.
+    for (int it = t; it < 3 * NP * CC; it += kCondThreads) {
+        const int c = it % CC, kap_ = it / CC, comp = kap_ / NP, j = kap_ % NP, K = blockIdx.x * CC + c;
+        if (K >= a.N) continue;
+        const double j00 = geo[0 * CC + c], j01 = geo[1 * CC + c], j10 = geo[2 * CC + c], j11 = geo[3 * CC + c];
+        double wx[NP], wy[NP], h[NP];
+        if (comp < 2) {
+            const double kap = geo[13 * CC + c], fk = geo[14 * CC + c];
+            double rh[NP];
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
                 double p, q;
@@ -487,28 +521,45 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                     p = Ps[(i * NP + j) * CC + c];
                     q = Qs[(i * NP + j) * CC + c];
                 }
-                wx[i] = comp == 0 ? p : comp == 1 ? q : 0.0;
-                wy[i] = comp == 0 ? -q : comp == 1 ? p : 0.0;
-                rh[i] = comp == 2 && i == j ? 1.0 : 0.0;
+                wx[i] = comp == 0 ? p : q;
+                wy[i] = comp == 0 ? -q : p;
+                rh[i] = 0.0;
             }
-            if (comp < 2) add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
-            const int kap_ = comp * NP + j;
-            if constexpr (FF) {
-                constexpr int CPk = (NK + 1) / 2;
-                back_substitute<NP, CC>(Ss, So, nullptr, c, rh, wx, wy, h);
+            add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
+            back_substitute<NP, CC>(Ss, nullptr, nullptr, FF ? nullptr : Ts, c, rh, wx, wy, h);
+        } else {
 #pragma unroll
-                for (int i = 0; i < NP; ++i)
-                    a.Hr2[2 * ff_pair_index(size_t(K), size_t(i) * CPk + kap_ / 2, size_t(NP) * CPk) + kap_ % 2] =
-                        split(h[i]);
-                continue;
+            for (int i = 0; i < NP; ++i) h[i] = Ss[(i * NP + j) * CC + c];
+            if constexpr (!FF) {
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    row_fence();
+                    double vx = 0.0, vy = 0.0;
+#pragma unroll
+                    for (int k = 0; k < NP; ++k) {
+                        vx = fma(-Ts[(i * NP + k) * CC + c], h[k], vx);
+                        vy = fma(-Ts[((NP + i) * NP + k) * CC + c], h[k], vy);
+                    }
+                    wx[i] = vx;
+                    wy[i] = vy;
+                }
             }
-            back_substitute<NP, CC>(Ss, nullptr, Ts, c, rh, wx, wy, h);
+        }
+        if constexpr (FF) {
+            constexpr int CPk = (NK + 1) / 2;
+#pragma unroll
+            for (int i = 0; i < NP; ++i)
+                a.Hr2[2 * ff_pair_index(size_t(K), size_t(i) * CPk + kap_ / 2, size_t(NP) * CPk) + kap_ % 2] = split(h[i]);
+        } else {
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
                 a.Rm[(size_t(i) * NK + kap_) * N + K] = wx[i];
                 a.Rm[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
                 a.Rm[(size_t(2 * NP + i) * NK + kap_) * N + K] = h[i];
             }
+            double wn[3][3];
+#pragma unroll
+            for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, K, e, wn[e]);
             c_rows<P>(m1, wn, wx, wy, h, -1, 0, 0.0, a.W + size_t(kap_) * N + K, size_t(NK) * N);
         }
     }
