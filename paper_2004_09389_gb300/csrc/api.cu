@@ -2199,15 +2199,14 @@ int hdg_condense(hdg_handle *h) {
     if (h->prm.coarse_mode == 2) {
         TRY(KL(HDG_PROF_CONDENSE, int(2 * h->lev.size()), launch_p1_galerkin(h)));
     } else {
-        for (auto &L : h->lev)
-            TRY(KL(HDG_PROF_CONDENSE, 2, launch_p1_assemble(h, L, tau, gH, h->prm.coarse_mode == 0 ? 1 : 0)));
+        TRY(KL(HDG_PROF_CONDENSE, 1, launch_p1_levels(h, tau, gH, h->prm.coarse_mode == 0 ? 1 : 0)));
     }
     const DevLevel &Lc = h->lev.back();
-    TRY(KL(HDG_PROF_CONDENSE, Lc.nv <= 256 ? 2 : 2 + 2 * Lc.nv,
+    TRY(KL(HDG_PROF_CONDENSE, Lc.nv <= 160 ? 1 : Lc.nv <= 256 ? 2 : 2 + 2 * Lc.nv,
            launch_dense_inverse(h, Lc, h->d_coarse_work, h->d_coarse_inv, Lc.nv)));
     if (h->prm.precision != HDG_FP64) {
         TRY(KL(HDG_PROF_CONDENSE, 2, launch_repack(h)));
-        for (auto &L : h->lev) {
+        if (h->prm.coarse_mode == 2) for (auto &L : h->lev) {
             TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.A, L.A32, size_t(L.nnz), s)));
             TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.dinv, L.dinv32, size_t(L.nv), s)));
         }

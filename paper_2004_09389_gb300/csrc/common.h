@@ -951,7 +951,8 @@ cudaError_t launch_rt0_prolong_add(hdg_handle *h, const double *ec, double *x);
 
 cudaError_t launch_condense(hdg_handle *h);
 cudaError_t launch_assemble(hdg_handle *h);
-cudaError_t launch_p1_assemble(hdg_handle *h, DevLevel &L, double tau, double gH, int rotating);
+// every P1 level's operator, inverse diagonal and FP32 copies
+cudaError_t launch_p1_levels(hdg_handle *h, double tau, double gH, int rotating);
 // every P1 level operator as the Galerkin product of the trace operator (k_galerkin.cu)
 cudaError_t launch_p1_galerkin(hdg_handle *h);
 cudaError_t launch_dense_inverse(hdg_handle *h, const DevLevel &L, double *work, double *inv, int n);

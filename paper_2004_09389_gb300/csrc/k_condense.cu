@@ -661,36 +661,136 @@ __global__ void assemble_kernel(AssembleArgs a) {
 // divided by tau to match the scale of the trace operator on smooth traces.
 // rotating = 0 drops f (the form printed in the paper).  Every CSR entry sums
 // its contributions in a fixed (cell) order.
-__global__ void p1_assemble_kernel(int nnz, const int32_t *__restrict__ cptr, const int32_t *__restrict__ contrib,
-                                   const double *__restrict__ elem, const double *__restrict__ fK, double tau,
-                                   double gH, int rotating, double *__restrict__ A) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nnz) return;
+//
+// One launch forms every level's values, inverse diagonal and their FP32 copies, a thread
+// per ELL slot.  What it takes is the latency of one slot's chain (contribution list,
+// element entries, sum), so the levels run side by side and the division by tau is left to
+// the end: r = 5, five levels, 28 us for all of it instead of 120 in twenty launches.
+constexpr int kP1Levels = 12;
+struct P1Levels {
+    int n;
+    int start[kP1Levels + 1];               // first thread of each level
+    struct Level {
+        int width;
+        const int32_t *cptr, *contrib, *diag;
+        const double *elem, *fK;
+        double *A, *dinv;
+        float *A32, *dinv32;                // null in FP64
+    } l[kP1Levels];
+};
+__global__ void __launch_bounds__(256) p1_levels_kernel(const __grid_constant__ P1Levels m, double tau, double gH,
+                                                        int rotating) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= m.start[m.n]) return;
+    int i = 0;
+    while (t >= m.start[i + 1]) ++i;
+    const P1Levels::Level &L = m.l[i];
+    const int q = t - m.start[i], k1 = L.cptr[q + 1];
+    const double t2 = tau * tau, t2g = t2 * gH;
     double acc = 0.0;
-    for (int k = cptr[q]; k < cptr[q + 1]; ++k) {
-        const int code = contrib[k], K = code / 9, ab = code % 9;
-        const double *el = elem + size_t(K) * 27;
-        const double f = rotating ? fK[K] : 0.0;
-        const double kap = 1.0 / (1.0 + tau * tau * f * f);
-        acc += (el[ab] + tau * tau * gH * kap * (el[9 + ab] - tau * f * el[18 + ab])) / tau;
+    for (int k = L.cptr[q]; k < k1; ++k) {
+        const int code = L.contrib[k], K = code / 9, ab = code % 9;
+        const double *el = L.elem + size_t(K) * 27;
+        const double e0 = el[ab], e1 = el[9 + ab];
+        if (rotating) {
+            const double f = L.fK[K];
+            acc += e0 + t2g * reciprocal(fma(t2 * f, f, 1.0)) * (e1 - tau * f * el[18 + ab]);
+        } else {
+            acc += e0 + t2g * e1;
+        }
     }
-    A[q] = acc;
+    acc /= tau;
+    L.A[q] = acc;
+    if (L.A32) L.A32[q] = to_float(acc);
+    const int v = q / L.width;
+    if (L.diag[v] == q) {
+        const double r = 1.0 / acc;
+        L.dinv[v] = r;
+        if (L.dinv32) L.dinv32[v] = to_float(r);
+    }
 }
 
-__global__ void p1_dinv_kernel(int nv, const int32_t *__restrict__ diag, const double *__restrict__ A,
-                               double *__restrict__ dinv) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nv) dinv[i] = 1.0 / A[diag[i]];
-}
-
-// dense copy of a padded ELL matrix (n <= 1024; unused slots add 0 to the
-// diagonal), then in-place Gauss-Jordan inverse with partial pivoting by one CTA.
+// dense copy of a padded ELL matrix (kInvSmem < n <= 1024; unused slots add 0 to the
+// diagonal), then Gauss-Jordan inverse with partial pivoting, by one CTA up to n = 256.
 __global__ void ell_to_dense_kernel(int n, int width, const int32_t *col, const double *A, double *D) {
     const int r = blockIdx.x;
     for (int c = threadIdx.x; c < n; c += blockDim.x) D[size_t(r) * n + c] = 0.0;
     __syncthreads();
     if (threadIdx.x == 0)
         for (int q = 0; q < width; ++q) D[size_t(r) * n + col[size_t(r) * width + q]] += A[size_t(r) * width + q];
+}
+
+// The inverse of a small ELL matrix (n <= kInvSmem) by in-place Gauss-Jordan elimination
+// with partial pivoting in the shared memory of one CTA, each element with the arithmetic
+// of the kernels below, so that all give the same inverse bit for bit.  Bound by the chain
+// of n steps, three barriers each: 80 us for 42 vertices, 52 for 36, instead of 160 and 127
+// with matrix and inverse in global memory and a tree of 1024 threads per pivot.
+constexpr int kInvSmem = 160;
+constexpr int kInvThreads = 512;
+__global__ void __launch_bounds__(kInvThreads) ell_inverse_kernel(int n, int width, const int32_t *__restrict__ col,
+                                                                  const double *__restrict__ Ae,
+                                                                  double *__restrict__ inv, int32_t *status) {
+    extern __shared__ double A[];              // [n][n], the pivot row, the pivot column
+    double *row = A + size_t(n) * n, *fac = row + n;
+    __shared__ int piv[kInvSmem];
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int k = tid; k < n * n; k += kInvThreads) A[k] = 0.0;
+    __syncthreads();
+    if (tid < n)
+        for (int q = 0; q < width; ++q) A[tid * n + col[size_t(tid) * width + q]] += Ae[size_t(tid) * width + q];
+    __syncthreads();
+    for (int k = 0; k < n; ++k) {
+        if (tid < 32) {
+            // largest magnitude (as bits, which order alike), then the lowest row; a NaN never wins
+            long long best = -1;
+            int p = k;
+            for (int r = k + lane; r < n; r += 32) {
+                const long long v = __double_as_longlong(A[r * n + k]) & 0x7fffffffffffffffll;
+                if (v <= 0x7ff0000000000000ll && v > best) {
+                    best = v;
+                    p = r;
+                }
+            }
+            for (int off = 16; off > 0; off >>= 1) {
+                const long long v = __shfl_xor_sync(0xffffffffu, best, off);
+                const int r = __shfl_xor_sync(0xffffffffu, p, off);
+                if (v > best || (v == best && r < p)) {
+                    best = v;
+                    p = r;
+                }
+            }
+            if (lane == 0) {
+                piv[k] = p;
+                if (best < 0 || !(__longlong_as_double(best) > 1e-300)) atomicOr(status, 4);
+            }
+        }
+        __syncthreads();
+        const int p = piv[k];
+        if (tid < n) {
+            // the pivot row scaled, row k in its place; the factors of the other rows
+            const int c = tid;
+            const double pinv = 1.0 / A[p * n + k], akc = A[k * n + c], apc = A[p * n + c];
+            row[c] = c == k ? pinv : apc * pinv;
+            fac[c] = c == p ? A[k * n + k] : A[c * n + k];
+            if (p != k && c != k) A[p * n + c] = akc;      // (column k is not read again)
+        }
+        __syncthreads();
+        for (int idx = tid; idx < n * n; idx += kInvThreads) {
+            const int r = idx / n, c = idx - r * n;
+            A[idx] = r == k ? row[c] : fma(-fac[r], row[c], c == k ? 0.0 : A[idx]);
+        }
+        __syncthreads();
+    }
+    // the row swaps, undone on the columns in reverse order: column j goes to place q
+    for (int idx = tid; idx < n * n; idx += kInvThreads) {
+        const int r = idx / n, j = idx - r * n;
+        int q = j;
+        for (int k = n - 1; k >= 0; --k) {
+            const int p = piv[k];
+            q = q == k ? p : q == p ? k : q;
+        }
+        inv[r * n + q] = A[idx];
+    }
 }
 
 __global__ void dense_inverse_kernel(int n, double *Aw, double *inv, int32_t *status) {
@@ -867,16 +967,29 @@ cudaError_t launch_assemble(hdg_handle *h) {
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_p1_assemble(hdg_handle *h, DevLevel &L, double tau, double gH, int rotating) {
-    p1_assemble_kernel<<<(L.nnz + 255) / 256, 256, 0, h->stream>>>(L.nnz, L.contrib_ptr, L.contrib, L.elem, L.fK, tau,
-                                                                    gH, rotating, L.A);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    p1_dinv_kernel<<<(L.nv + 255) / 256, 256, 0, h->stream>>>(L.nv, L.diag, L.A, L.dinv);
+cudaError_t launch_p1_levels(hdg_handle *h, double tau, double gH, int rotating) {
+    for (size_t l0 = 0; l0 < h->lev.size(); l0 += kP1Levels) {
+        P1Levels m = {};
+        m.n = int(std::min(h->lev.size() - l0, size_t(kP1Levels)));
+        for (int i = 0; i < m.n; ++i) {
+            const DevLevel &L = h->lev[l0 + size_t(i)];
+            m.start[i + 1] = m.start[i] + L.nnz;
+            m.l[i] = {L.width, L.contrib_ptr, L.contrib, L.diag, L.elem, L.fK, L.A, L.dinv, L.A32, L.dinv32};
+        }
+        p1_levels_kernel<<<unsigned(m.start[m.n] + 255) / 256, 256, 0, h->stream>>>(m, tau, gH, rotating);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_dense_inverse(hdg_handle *h, const DevLevel &L, double *work, double *inv, int n) {
+    if (n <= kInvSmem) {
+        const size_t smem = sizeof(double) * size_t(n) * size_t(n + 2);
+        cudaError_t e = cudaFuncSetAttribute(ell_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             int(sizeof(double) * kInvSmem * (kInvSmem + 2)));
+        if (e != cudaSuccess) return e;
+        ell_inverse_kernel<<<1, kInvThreads, smem, h->stream>>>(n, L.width, L.col, L.A, inv, h->d_status);
+        return cudaGetLastError();
+    }
     ell_to_dense_kernel<<<n, 128, 0, h->stream>>>(n, L.width, L.col, L.A, work);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
