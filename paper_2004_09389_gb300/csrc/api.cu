@@ -1290,6 +1290,9 @@ void free_handle(hdg_handle *h) {
         dfree(L.wimg); dfree(L.gpart);
         dfree(L.buf); dfree(L.c); dfree(L.rn); dfree(L.gc); dfree(L.tmp); dfree(L.coef); dfree(L.nrm);
     }
+    if (h->forked) cudaEventDestroy(h->forked);
+    if (h->joined) cudaEventDestroy(h->joined);
+    if (h->side) cudaStreamDestroy(h->side);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
 }
@@ -2157,6 +2160,13 @@ int hdg_setup(const hdg_mesh_desc *mesh, const hdg_params *prm, void *stream, hd
         h->own_stream = true;
     }
     int rc = setup_device(h, prm);
+    if (!rc && prm->flux == 0 && prm->coarse_mode != 2) {
+        // the coarse operators' stream (hdg_condense)
+        cudaError_t ce = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
+        if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->forked, cudaEventDisableTiming);
+        if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->joined, cudaEventDisableTiming);
+        if (ce != cudaSuccess) rc = fail(h, HDG_ECUDA, std::string("side stream: ") + cudaGetErrorString(ce));
+    }
     if (!rc) {
         // the device this handle lives on, and the no-allocation scratch array
         // loaded onto it now rather than inside a later call
@@ -2172,6 +2182,59 @@ int hdg_setup(const hdg_mesh_desc *mesh, const hdg_params *prm, void *stream, hd
     *out = h;
     return HDG_OK;
 }
+
+namespace {
+
+// The facet-row operator from the cells' S_K, the smoother's operators and their copies
+int facet_operators(hdg_handle *h) {
+    TRY(KL(HDG_PROF_CONDENSE, 1, launch_assemble(h)));
+    TRY(KL(HDG_PROF_CONDENSE, 1, launch_hat_op(h)));
+    if (h->prm.precision != HDG_FP64) TRY(KL(HDG_PROF_CONDENSE, 2, launch_repack(h)));
+    if (mode_ff(h->prm)) {
+        // (hi, lo) float pairs for the two-float FP64 steps
+        const size_t pp = h->pp, NS = 5 * pp * pp;
+        TRY(KL(HDG_PROF_CONDENSE, 1, launch_split(h->d_Sval, h->d_Sval2, (NS + 1) / 2 * 2 * size_t(h->NF), h->stream)));
+    }
+    return HDG_OK;
+}
+
+// The operators of the P1 levels, the coarsest inverse and the tail
+int coarse_operators(hdg_handle *h) {
+    if (h->prm.coarse_mode == 2) {
+        TRY(KL(HDG_PROF_CONDENSE, int(2 * h->lev.size()), launch_p1_galerkin(h)));
+        if (h->prm.precision != HDG_FP64)
+            for (auto &L : h->lev) {
+                TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.A, L.A32, size_t(L.nnz), h->stream)));
+                TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.dinv, L.dinv32, size_t(L.nv), h->stream)));
+            }
+    } else {
+        TRY(KL(HDG_PROF_CONDENSE, 1,
+               launch_p1_levels(h, h->prm.tau, h->prm.g * h->prm.H, h->prm.coarse_mode == 0 ? 1 : 0)));
+    }
+    const DevLevel &Lc = h->lev.back();
+    TRY(KL(HDG_PROF_CONDENSE, Lc.nv <= 160 ? 1 : Lc.nv <= 256 ? 2 : 2 + 2 * Lc.nv,
+           launch_dense_inverse(h, Lc, h->d_coarse_work, h->d_coarse_inv, Lc.nv)));
+    return build_tail(h);
+}
+
+// Runs f with the handle's launches on its side stream, behind what its stream held when
+// h->forked was recorded; h->joined then marks the end of that work.
+int on_side_stream(hdg_handle *h, int (*f)(hdg_handle *)) {
+    struct Restore {
+        hdg_handle *h;
+        cudaStream_t s;
+        ~Restore() { h->stream = s; }
+    } restore{h, h->stream};
+    TRY(cudaStreamWaitEvent(h->side, h->forked, 0));
+    h->stream = h->side;
+    const int rc = f(h);
+    const cudaError_t e = cudaEventRecord(h->joined, h->side);
+    if (rc) return rc;
+    TRY(e);
+    return HDG_OK;
+}
+
+}  // namespace
 
 int hdg_condense(hdg_handle *h) {
     if (!h) return HDG_EINVAL;
@@ -2192,32 +2255,19 @@ int hdg_condense(hdg_handle *h) {
         h->condensed = true;
         return HDG_OK;
     }
+    // The cells are condensed and the facet operators follow from them; the P1 operators
+    // come from the geometry alone (coarse_mode 2: from the facet operators), a chain of
+    // small kernels that runs beside the condensation on the side stream (with event timing
+    // on, one after the other): r = 5, p = 3 set_tau + step 2537 us instead of 2687, flat
+    // n = 96, p = 2 in FP64 1530 instead of 1621.
+    const bool beside = h->side && !h->prof.on;
+    if (beside) TRY(cudaEventRecord(h->forked, s));
     TRY(KL(HDG_PROF_CONDENSE, 1, launch_condense(h)));
-    TRY(KL(HDG_PROF_CONDENSE, 1, launch_assemble(h)));
-    TRY(KL(HDG_PROF_CONDENSE, 1, launch_hat_op(h)));
-    const double tau = h->prm.tau, gH = h->prm.g * h->prm.H;
-    if (h->prm.coarse_mode == 2) {
-        TRY(KL(HDG_PROF_CONDENSE, int(2 * h->lev.size()), launch_p1_galerkin(h)));
-    } else {
-        TRY(KL(HDG_PROF_CONDENSE, 1, launch_p1_levels(h, tau, gH, h->prm.coarse_mode == 0 ? 1 : 0)));
-    }
-    const DevLevel &Lc = h->lev.back();
-    TRY(KL(HDG_PROF_CONDENSE, Lc.nv <= 160 ? 1 : Lc.nv <= 256 ? 2 : 2 + 2 * Lc.nv,
-           launch_dense_inverse(h, Lc, h->d_coarse_work, h->d_coarse_inv, Lc.nv)));
-    if (h->prm.precision != HDG_FP64) {
-        TRY(KL(HDG_PROF_CONDENSE, 2, launch_repack(h)));
-        if (h->prm.coarse_mode == 2) for (auto &L : h->lev) {
-            TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.A, L.A32, size_t(L.nnz), s)));
-            TRY(KL(HDG_PROF_CONDENSE, 1, launch_to_f32(L.dinv, L.dinv32, size_t(L.nv), s)));
-        }
-        if (mode_ff(h->prm)) {
-            // (hi, lo) float pairs for the two-float FP64 steps
-            const size_t pp = h->pp, NS = 5 * pp * pp;
-            TRY(KL(HDG_PROF_CONDENSE, 1, launch_split(h->d_Sval, h->d_Sval2, (NS + 1) / 2 * 2 * size_t(h->NF), s)));
-        }
-    }
-    int rc = build_tail(h);
-    if (rc) return rc;
+    int rc = beside ? on_side_stream(h, coarse_operators) : HDG_OK;
+    const int rc2 = rc ? rc : facet_operators(h);
+    if (beside) TRY(cudaStreamWaitEvent(s, h->joined, 0));
+    if (rc2) return rc2;
+    if (!beside && (rc = coarse_operators(h)) != HDG_OK) return rc;
     rc = check_status(h);
     if (rc) return rc;
     if (h->prm.smoother == 1 && (rc = chebyshev_setup(h)) != HDG_OK) return rc;

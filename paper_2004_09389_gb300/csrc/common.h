@@ -788,6 +788,8 @@ struct hdg_handle {
     double tau_s = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    cudaStream_t side = nullptr;    // the coarse operators' stream during a condensation
+    cudaEvent_t forked = nullptr, joined = nullptr;
     bool condensed = false;
     hdg::HostMesh hm;
 

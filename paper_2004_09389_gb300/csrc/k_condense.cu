@@ -726,7 +726,7 @@ __global__ void ell_to_dense_kernel(int n, int width, const int32_t *col, const 
 // of n steps, three barriers each: 80 us for 42 vertices, 52 for 36, instead of 160 and 127
 // with matrix and inverse in global memory and a tree of 1024 threads per pivot.
 constexpr int kInvSmem = 160;
-constexpr int kInvThreads = 512;
+constexpr int kInvThreads = 256;             // fits an SM beside the condensation's blocks
 __global__ void __launch_bounds__(kInvThreads) ell_inverse_kernel(int n, int width, const int32_t *__restrict__ col,
                                                                   const double *__restrict__ Ae,
                                                                   double *__restrict__ inv, int32_t *status) {
