@@ -147,10 +147,6 @@ __device__ __forceinline__ void block_solve_packed(const DT *__restrict__ Dinv, 
 // 256-thread blocks fit per SM (one wave over the facets of large meshes);
 // FP64 ones are bound by the FP64 pipe and keep their registers.
 template <typename T> struct MinBlocks { static constexpr int value = sizeof(T) == 4 ? 6 : 1; };
-// the operator kernel with the Gram-Schmidt dots: as above for FP32 (one wave),
-// four blocks per SM for FP64
-template <typename T> struct DotsMinBlocks { static constexpr int value = sizeof(T) == 4 ? 6 : 4; };
-
 template <int P, typename T, typename ST>
 __global__ void __launch_bounds__(256, MinBlocks<T>::value) apply_kernel(int NF, const ST *__restrict__ Sval, const int32_t *__restrict__ nbr,
                                                     const T *__restrict__ x, T *__restrict__ y) {
@@ -171,8 +167,10 @@ __global__ void __launch_bounds__(256, MinBlocks<T>::value) apply_kernel(int NF,
 // The sums over a warp by halving exchanges (warp_sums) and the warps' sums for all
 // vectors after one barrier: 63.1 instead of 70.4 us on 196,608 facets at p = 3 in FP64
 // (bound by the FP64 pipe: 80 + 4 k FMAs per facet, and k adds per block by the last one),
-// 9.6 instead of 11.5 us on 768 facets (latency); FP32 unchanged (14.9 us).
-template <int P, typename T, typename ST>
+// 9.6 instead of 11.5 us on 768 facets (latency).  In FP32 what bounds it is the latency
+// of the loads: B blocks per SM (launch_apply_dots_t) decide how many a thread
+// has in flight.
+template <int P, typename T, typename ST, int B>
 __device__ __forceinline__ void apply_dots_kernel_impl(int bid_, int nb_, int NF, const ST *__restrict__ Sval,
                                                        const int32_t *__restrict__ nbr, const T *__restrict__ x,
                                                        T *__restrict__ y, const T *__restrict__ V, size_t ld, int k,
@@ -180,7 +178,7 @@ __device__ __forceinline__ void apply_dots_kernel_impl(int bid_, int nb_, int NF
                                                        unsigned int *__restrict__ counter, double *__restrict__ h,
                                                        T *__restrict__ hneg) {
     using A = typename std::conditional<std::is_same<T, double>::value, double, float>::type;
-    constexpr int PP = P + 1, G = sizeof(T) == 8 ? 8 : 4, KM = 72;   // (FP32: 40 registers, see DotsMinBlocks)
+    constexpr int PP = P + 1, G = sizeof(T) == 8 ? 8 : B > 4 ? 4 : 8, KM = 72;   // (FP32, B = 6: 40 registers)
     __shared__ A red[8][KM];                   // the warps' sums of every vector (k <= 65)
     __shared__ bool last;
     const int e = bid_ * blockDim.x + threadIdx.x;
@@ -234,17 +232,17 @@ __device__ __forceinline__ void apply_dots_kernel_impl(int bid_, int nb_, int NF
         for (int i = threadIdx.x; i < k; i += blockDim.x) hneg[i] = T(-h[i]);
     if (threadIdx.x == 0) *counter = 0u;
 }
-template <int P, typename T, typename ST>
-__global__ void __launch_bounds__(256, DotsMinBlocks<T>::value) apply_dots_kernel(int NF, const ST *__restrict__ Sval,
+template <int P, typename T, typename ST, int B>
+__global__ void __launch_bounds__(256, B) apply_dots_kernel(int NF, const ST *__restrict__ Sval,
                                                             const int32_t *__restrict__ nbr, const T *__restrict__ x,
                                                             T *__restrict__ y, const T *__restrict__ V, size_t ld,
                                                             int k, double *__restrict__ partial,
                                                             unsigned int *__restrict__ counter,
                                                             double *__restrict__ h, T *__restrict__ hneg) {
     pdl_wait();
-    apply_dots_kernel_impl<P, T, ST>(blockIdx.x, gridDim.x, NF, Sval, nbr, x, y, V, ld, k, partial, counter, h, hneg);
+    apply_dots_kernel_impl<P, T, ST, B>(blockIdx.x, gridDim.x, NF, Sval, nbr, x, y, V, ld, k, partial, counter, h, hneg);
 }
-template <int P, typename T, typename ST>
+template <int P, typename T, typename ST, int B>
 struct apply_dots_kernel_args {
     int nb_;
     int NF;
@@ -260,20 +258,20 @@ struct apply_dots_kernel_args {
     double *h;
     T *hneg;
 };
-template <int P, typename T, typename ST>
-__global__ void __launch_bounds__(256, DotsMinBlocks<T>::value) apply_dots_kernel_multi(const __grid_constant__ MultiP<apply_dots_kernel_args<P, T, ST>> M) {
+template <int P, typename T, typename ST, int B>
+__global__ void __launch_bounds__(256, B) apply_dots_kernel_multi(const __grid_constant__ MultiP<apply_dots_kernel_args<P, T, ST, B>> M) {
     pdl_wait();
     int b_;
-    const apply_dots_kernel_args<P, T, ST> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    apply_dots_kernel_impl<P, T, ST>(b_, q_.nb_, q_.NF, q_.Sval, q_.nbr, q_.x, q_.y, q_.V, q_.ld, q_.k, q_.partial,
+    const apply_dots_kernel_args<P, T, ST, B> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    apply_dots_kernel_impl<P, T, ST, B>(b_, q_.nb_, q_.NF, q_.Sval, q_.nbr, q_.x, q_.y, q_.V, q_.ld, q_.k, q_.partial,
         q_.counter, q_.h, q_.hneg);
 }
-template <int P, typename T, typename ST>
+template <int P, typename T, typename ST, int B>
 void apply_dots_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int NF, const ST *Sval,
                           const int32_t *nbr, const T *x, T *y, const T *V, size_t ld, int k, double *partial,
                           unsigned int *counter, double *h, T *hneg) {
     if (Recorder *r_ = batch_recorder()) {
-        apply_dots_kernel_args<P, T, ST> q_;
+        apply_dots_kernel_args<P, T, ST, B> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
         q_.NF = NF;
@@ -288,10 +286,10 @@ void apply_dots_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStr
         q_.counter = counter;
         q_.h = h;
         q_.hneg = hneg;
-        batch_record(r_, reinterpret_cast<const void *>(&apply_dots_kernel_multi<P, T, ST>), q_, grid_, block_, smem_, kPdlFamily);
+        batch_record(r_, reinterpret_cast<const void *>(&apply_dots_kernel_multi<P, T, ST, B>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &apply_dots_kernel<P, T, ST>, grid_, block_, smem_, s_, NF, Sval, nbr, x, y, V, ld, k, partial, counter, h, hneg);
+    pdl_launch(kPdlFamily, &apply_dots_kernel<P, T, ST, B>, grid_, block_, smem_, s_, NF, Sval, nbr, x, y, V, ld, k, partial, counter, h, hneg);
 }
 
 
@@ -1170,12 +1168,35 @@ template <> struct Ops<float> {
 };
 inline bool bf16_pre(hdg_handle *h) { return h->prm.precision == HDG_MIXED_BF16 && h->d_H16; }
 
+template <typename T, int B>
+cudaError_t apply_dots_b(hdg_handle *h, unsigned nb, const T *x, T *y, const T *V, size_t ld, int k, double *partial,
+                         unsigned int *counter, double *hdots, T *hneg) {
+    constexpr int BB = sizeof(T) == 8 ? 4 : B;
+    HDG_DISPATCH_PF(h->pf, T, (apply_dots_kernel_go<P, T, T, BB>(nb, 256, 0, h->stream, 
+                             h->NF, Ops<T>::S(h, false), h->d_nbr, x, y, V, ld, k, partial, counter, hdots, hneg)));
+    return cudaGetLastError();
+}
 template <typename T>
 cudaError_t launch_apply_dots_t(hdg_handle *h, const T *x, T *y, const T *V, size_t ld, int k, double *partial,
                                 unsigned int *counter, double *hdots, T *hneg) {
-    HDG_DISPATCH_PF(h->pf, T, (apply_dots_kernel_go<P, T, T>(blocks(h->NF, 256), 256, 0, h->stream, 
-                             h->NF, Ops<T>::S(h, false), h->d_nbr, x, y, V, ld, k, partial, counter, hdots, hneg)));
-    return cudaGetLastError();
+    // Blocks per SM that the kernel is compiled for: fewer leave a thread the registers for
+    // more loads in flight (FP32, 4: eight vectors at a time instead of four), more finish
+    // the grid in fewer rounds.  A round of 4, 5 and 6 blocks per SM takes about 8, 9.5 and
+    // 10.5 us (p = 2, 491,520 facets: 4, 3 and 3 rounds, 31.3, 28.9 and 31.5 us; p = 3,
+    // 196,608: 2, 2 and 1 round, 16.5, 18.3 and 14.9; p = 4, 30,000: one, 8.7, 10.9 and
+    // 11.7).  FP64: bound by its pipe, four.
+    const unsigned nb = blocks(h->NF, 256);
+    auto rounds = [&](unsigned b) { return (nb + 152 * b - 1) / (152 * b); };
+    int B = 4;
+    if (sizeof(T) == 4) {
+        const unsigned c4 = 16 * rounds(4), c5 = 19 * rounds(5), c6 = 21 * rounds(6);
+        B = c4 <= c5 && c4 <= c6 ? 4 : c5 <= c6 ? 5 : 6;
+    }
+    switch (B) {
+        case 4: return apply_dots_b<T, 4>(h, nb, x, y, V, ld, k, partial, counter, hdots, hneg);
+        case 5: return apply_dots_b<T, 5>(h, nb, x, y, V, ld, k, partial, counter, hdots, hneg);
+        default: return apply_dots_b<T, 6>(h, nb, x, y, V, ld, k, partial, counter, hdots, hneg);
+    }
 }
 template <typename T>
 cudaError_t launch_apply_t(hdg_handle *h, const T *x, T *y) {
