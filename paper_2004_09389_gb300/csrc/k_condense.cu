@@ -553,8 +553,10 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
         } else {
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
-                a.Rm[(size_t(i) * NK + kap_) * N + K] = wx[i];
-                a.Rm[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
+                if constexpr (!FC) {            // (f constant: step 3 takes the h rows only)
+                    a.Rm[(size_t(i) * NK + kap_) * N + K] = wx[i];
+                    a.Rm[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
+                }
                 a.Rm[(size_t(2 * NP + i) * NK + kap_) * N + K] = h[i];
             }
             double wn[3][3];
