@@ -1169,36 +1169,48 @@ __global__ void __launch_bounds__(32 * kRecWarps<P>) recover_const_f_kernel(int 
 }
 
 // P1 restriction rho = pi^T: r_c[v] = sum over facet ends at v of the nodal
-// weights of the linear interpolant (1 - t_r at the lower vertex, t_r at the higher)
-template <int P, typename T>
+// weights of the linear interpolant (1 - t_r at the lower vertex, t_r at the higher).
+// Latency bounds it (list, facet id, p + 1 values, one after the other), so in FP32 eight
+// lanes (L) share a vertex's facet ends where that still is about one wave of threads: 5.4
+// instead of 6.5 us for 40,962 vertices at p = 3, 3.4 instead of 3.7 for 20,736 at p = 2, but
+// 6.5 instead of 5.3 for 65,536 and 12.0 instead of 7.8 for 163,842 (kRestrictShared).  In
+// FP64, where the lanes' additions would take the pipe longer than the loads, and on the
+// larger meshes one thread takes them all.
+constexpr int kRestrictShared = 49152;
+template <int P, typename T, int L>
 __device__ __forceinline__ void restrict_kernel_impl(int bid_, int nb_, int nv, int NF,
                                                      const int32_t *__restrict__ v2f_ptr,
                                                      const int32_t *__restrict__ v2f, const T *__restrict__ r,
                                                      T *__restrict__ rc, const T *__restrict__ dinv0, T omega,
                                                      T *__restrict__ x0) {
-    const int v = bid_ * blockDim.x + threadIdx.x;
-    if (v >= nv) return;
+    const int t = bid_ * blockDim.x + threadIdx.x, v = t / L, q = t % L;
     T acc = T(0);
-    for (int k = v2f_ptr[v]; k < v2f_ptr[v + 1]; ++k) {
-        const int code = v2f[k], e = code >> 1, hi = code & 1;
+    if (v < nv) {
+        const int k1 = v2f_ptr[v + 1];
+        for (int k = v2f_ptr[v] + q; k < k1; k += L) {
+            const int code = v2f[k], e = code >> 1, hi = code & 1;
 #pragma unroll
-        for (int j = 0; j <= P; ++j) {
-            const T t = T(j) / T(P);
-            acc = fma(hi ? t : T(1) - t, r[size_t(j) * NF + e], acc);
+            for (int j = 0; j <= P; ++j) {
+                const T w = T(j) / T(P);
+                acc = fma(hi ? w : T(1) - w, r[size_t(j) * NF + e], acc);
+            }
         }
     }
+#pragma unroll
+    for (int off = L / 2; off > 0; off /= 2) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (v >= nv || q != 0) return;
     rc[v] = acc;
     // first damped Jacobi sweep of the P1 level from zero, fused (x0 may be null)
     if (x0) x0[v] = omega * dinv0[v] * acc;
 }
-template <int P, typename T>
+template <int P, typename T, int L>
 __global__ void restrict_kernel(int nv, int NF, const int32_t *__restrict__ v2f_ptr, const int32_t *__restrict__ v2f,
                                 const T *__restrict__ r, T *__restrict__ rc, const T *__restrict__ dinv0, T omega,
                                 T *__restrict__ x0) {
     pdl_wait();
-    restrict_kernel_impl<P, T>(blockIdx.x, gridDim.x, nv, NF, v2f_ptr, v2f, r, rc, dinv0, omega, x0);
+    restrict_kernel_impl<P, T, L>(blockIdx.x, gridDim.x, nv, NF, v2f_ptr, v2f, r, rc, dinv0, omega, x0);
 }
-template <int P, typename T>
+template <int P, typename T, int L>
 struct restrict_kernel_args {
     int nb_;
     int nv;
@@ -1211,19 +1223,19 @@ struct restrict_kernel_args {
     T omega;
     T *x0;
 };
-template <int P, typename T>
-__global__ void restrict_kernel_multi(const __grid_constant__ MultiP<restrict_kernel_args<P, T>> M) {
+template <int P, typename T, int L>
+__global__ void restrict_kernel_multi(const __grid_constant__ MultiP<restrict_kernel_args<P, T, L>> M) {
     pdl_wait();
     int b_;
-    const restrict_kernel_args<P, T> &q_ = M.a[merge_find(M.start, M.n, b_)];
-    restrict_kernel_impl<P, T>(b_, q_.nb_, q_.nv, q_.NF, q_.v2f_ptr, q_.v2f, q_.r, q_.rc, q_.dinv0, q_.omega, q_.x0);
+    const restrict_kernel_args<P, T, L> &q_ = M.a[merge_find(M.start, M.n, b_)];
+    restrict_kernel_impl<P, T, L>(b_, q_.nb_, q_.nv, q_.NF, q_.v2f_ptr, q_.v2f, q_.r, q_.rc, q_.dinv0, q_.omega, q_.x0);
 }
-template <int P, typename T>
+template <int P, typename T, int L>
 void restrict_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStream_t s_, int nv, int NF,
                         const int32_t *v2f_ptr, const int32_t *v2f, const T *r, T *rc, const T *dinv0, T omega,
                         T *x0) {
     if (Recorder *r_ = batch_recorder()) {
-        restrict_kernel_args<P, T> q_;
+        restrict_kernel_args<P, T, L> q_;
         std::memset(static_cast<void *>(&q_), 0, sizeof(q_));
         q_.nb_ = int(grid_);
         q_.nv = nv;
@@ -1235,10 +1247,10 @@ void restrict_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStrea
         q_.dinv0 = dinv0;
         q_.omega = omega;
         q_.x0 = x0;
-        batch_record(r_, reinterpret_cast<const void *>(&restrict_kernel_multi<P, T>), q_, grid_, block_, smem_, kPdlFamily);
+        batch_record(r_, reinterpret_cast<const void *>(&restrict_kernel_multi<P, T, L>), q_, grid_, block_, smem_, kPdlFamily);
         return;
     }
-    pdl_launch(kPdlFamily, &restrict_kernel<P, T>, grid_, block_, smem_, s_, nv, NF, v2f_ptr, v2f, r, rc, dinv0, omega, x0);
+    pdl_launch(kPdlFamily, &restrict_kernel<P, T, L>, grid_, block_, smem_, s_, nv, NF, v2f_ptr, v2f, r, rc, dinv0, omega, x0);
 }
 
 
@@ -1354,7 +1366,11 @@ cudaError_t launch_smooth_first_t(hdg_handle *h, const T *b, T *x, T *bh, const 
 }
 template <typename T>
 cudaError_t launch_restrict_t(hdg_handle *h, const T *r, T *rc, const T *dinv0, T omega, T *x0) {
-    HDG_DISPATCH_P(h->p, (restrict_kernel_go<P, T>(blocks(h->nv, 256), 256, 0, h->stream, h->nv, h->NF, h->d_v2f_ptr, h->d_v2f, r, rc, dinv0, omega, x0)));
+    if (sizeof(T) == 4 && h->nv <= kRestrictShared) {
+        HDG_DISPATCH_P(h->p, (restrict_kernel_go<P, T, sizeof(T) == 4 ? 8 : 1>(blocks(size_t(h->nv) * 8, 256), 256, 0, h->stream, h->nv, h->NF, h->d_v2f_ptr, h->d_v2f, r, rc, dinv0, omega, x0)));
+        return cudaGetLastError();
+    }
+    HDG_DISPATCH_P(h->p, (restrict_kernel_go<P, T, 1>(blocks(h->nv, 256), 256, 0, h->stream, h->nv, h->NF, h->d_v2f_ptr, h->d_v2f, r, rc, dinv0, omega, x0)));
     return cudaGetLastError();
 }
 template <typename T>
