@@ -110,15 +110,24 @@ def make_workload(kind: str, full: bool, p: int, courant: float, seed: int) -> d
 
 
 # ---------------------------------------------------------------- algorithmic bytes per launch
-def trace_bytes(cat: str, NF: int, pp: int, s_width: int | None = None) -> float:
+L2_BYTES = 126 << 20     # GB300
+
+
+def trace_bytes(cat: str, NF: int, pp: int, s_width: int | None = None, krylov64: bool = False) -> float:
     """Minimum bytes a facet-row kernel must move: the operator values (apply: the 5
     blocks of (p+1)^2 per facet of S; sweeps: the 4 neighbour blocks of D^-1 S; the
-    residual of the V-cycle: those and the diagonal block; the sizes of FP32 solves whose
-    sweeps take S and the inverse blocks move half as much again), the neighbour ids, and
-    each trace vector it touches read or written once.  s_width overrides the bytes per value
-    of the smoother's operator (2 for the BF16 copy)."""
+    residual of the V-cycle: those and the diagonal block), the neighbour ids, and
+    each trace vector it touches read or written once.  FP32 sweeps beside an FP32 Krylov
+    space (krylov64 false) take S and the inverse block at the sizes where S stays in L2
+    (the library's hat_pays32).  s_width overrides the bytes per value of the smoother's
+    operator (2 for the BF16 copy)."""
     w = 8 if cat.endswith("64") else 4
     blk, vec = pp * pp, pp * w
+    set_bytes = 4 * blk * NF
+    if w == 4 and not s_width and not krylov64 and 14 * set_bytes > L2_BYTES / 3 and 6 * set_bytes <= L2_BYTES * 2 / 3:
+        swept = {"residual": 6 * blk * w + 16 + 4 * vec, "smooth": 6 * blk * w + 16 + 3 * vec}
+        if cat[:-2] in swept:
+            return float(NF) * swept[cat[:-2]]
     base = cat[:-2]
     if base == "apply":
         per = 5 * blk * w + 16 + 2 * vec
@@ -473,13 +482,14 @@ def step13_bytes(arm: dict):
     in step 1: its cell kernel reads the h rows of R_M (and the inverse velocity
     block where f varies over the cells), r and the cell weights (15 float pairs)
     and writes z and the cell rows; the recovery reads X_B, z and lambda and
-    writes u, h.  FP64 handles read W_K, r in step 1 and R_M, X_B, r, lambda in
-    step 3."""
+    writes u, h.  FP64 handles read W_K, r in step 1 and R_M, X_B (where f is
+    constant on every cell: their h rows), r, lambda in step 3."""
     N, n, nK, m = arm["n_cells"], arm["n_p"], 3 * arm["n_p"], 3 * arm["pp"]
     if arm.get("keep_z"):
         mats = n * nK + (0 if arm.get("f_const", True) else 2 * n * n)
         return 8.0 * N * (mats + 2 * nK + m + 15), 8.0 * N * (nK * m + 2 * nK + m)
-    return 8.0 * N * (m * nK + nK + m), 8.0 * N * (nK * nK + nK * m + 3 * nK + m)
+    rows = n if arm.get("f_const", True) else nK
+    return 8.0 * N * (m * nK + nK + m), 8.0 * N * (rows * (nK + m) + 3 * nK + m)
 
 
 def whole_solve(arm: dict, peaks: dict, steps: int) -> dict:
@@ -493,7 +503,7 @@ def whole_solve(arm: dict, peaks: dict, steps: int) -> dict:
     total = 0.0
     for cat, (_, n) in prof.items():
         if n and cat.startswith(("apply", "residual", "smooth")):
-            total += trace_bytes(cat, NF, pp) * n / ps
+            total += trace_bytes(cat, NF, pp, krylov64=bool(prof["apply64"][1])) * n / ps
     # step 1 (two launches per call) and step 3
     rhs_b, rec_b = step13_bytes(arm)
     total += rhs_b * (prof["rhs"][1] / 2) / ps
@@ -555,7 +565,7 @@ def roofline(arm: dict, peaks: dict, fma: dict | None = None, bf16_pre: bool = F
     total = sum(ms for ms, _ in prof.values())
     best = max(cats, key=lambda c: prof[c][0])
     bf16_op = bf16_pre and best.startswith("smooth") and best.endswith("32") and not best.startswith("smooth_first")
-    per_launch = trace_bytes(best, NF, pp, 2 if bf16_op else None)
+    per_launch = trace_bytes(best, NF, pp, 2 if bf16_op else None, bool(prof["apply64"][1]))
     ms_c, n_c = cold[best]
     ms_w, n_w = prof[best]
     achieved = per_launch * n_c / (ms_c * 1e-3) / 1e9 if ms_c > 0 else 0.0
@@ -604,8 +614,8 @@ def condense_rate(arm: dict, fma: dict) -> dict:
     nz = {3: 14, 6: 48, 10: 120, 15: 250}[n]
     div, c_rows = 4 * n + nz, 9 * pp + 3 * pp * pp
     fmas = (n * (8 * n + div + 2 * n + n * n)                    # T, the height system, its inverse
-            + m * (3 * n + div + 5 * n * n + c_rows)             # X_B (3 n^2 for h with refinement, 2 n^2 for u), S_K
-            + n * (2 * div + 9 * n * n + 3 * c_rows))            # R_M, W_K
+            + m * (3 * n + div + 4 * n * n + c_rows)             # X_B (2 n^2 for h and its residual, 2 n^2 for u), S_K
+            + n * (2 * div + 8 * n * n + 3 * c_rows))            # R_M (its h columns are S^-1), W_K
     tf = 2.0 * fmas * N / (arm["condense_ms"] * 1e-3) / 1e12
     return {"flops_per_cell": 2 * fmas, "achieved_tflops": tf, "peak_tflops": fma["fp64_tflops"],
             "frac": tf / fma["fp64_tflops"], "timing": "host wall clock around hdg_condense (one call, synchronised)",

@@ -78,8 +78,8 @@ extern "C" {
 #define HDG_MIXED_FP32  1   /* FP32 inner FGMRES + V-cycle, iterative refinement with the
                                residual, right-hand side, iterate and recovery in two-float
                                arithmetic (about 48 bits); lambda returned in FP64         */
-#define HDG_MIXED_BF16  2   /* as HDG_MIXED_FP32, with a BF16 copy of the trace operator for the
-                               smoother and V-cycle residual (FP32 accumulation)              */
+#define HDG_MIXED_BF16  2   /* as HDG_MIXED_FP32, with the smoother's and V-cycle residual's operator
+                               (the neighbour blocks of D^-1 S) in BF16 (FP32 accumulation)   */
 #define HDG_MIXED_FGMRES64 3 /* FP64 FGMRES (basis, orthogonalisation, residual, update, RHS and
                                recovery in FP64) preconditioned by the two-level V-cycle in FP32
                                (FP32 operator copies; the coarsest P1 solve stays FP64)       */

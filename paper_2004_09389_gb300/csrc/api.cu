@@ -27,7 +27,7 @@
 namespace hdg {
 
 template <typename T> cudaError_t launch_apply_t(hdg_handle *, const T *, T *);
-template <typename T> cudaError_t launch_residual_t(hdg_handle *, const T *, const T *, T *, bool);
+template <typename T> cudaError_t launch_residual_t(hdg_handle *, const T *, const T *, T *);
 template <typename T> cudaError_t launch_residual_smooth_t(hdg_handle *, const T *, const T *, T *, T *, double);
 template <typename T> cudaError_t launch_smooth_t(hdg_handle *, const T *, const T *, T *);
 template <typename T>
@@ -493,7 +493,7 @@ cudaError_t precond_lf(hdg_handle *h, const double *v, double *z, const double *
         x2 = (x == k.t0) ? k.t1 : k.t0;
     }
     // residual, restriction to RT0, coarse Chebyshev steps, prolongation
-    if ((e = KL(HDG_PROF_RESIDUAL64, 1, launch_residual_t<double>(h, v, x, k.res, true))) != cudaSuccess) return e;
+    if ((e = KL(HDG_PROF_RESIDUAL64, 1, launch_residual_t<double>(h, v, x, k.res))) != cudaSuccess) return e;
     Rt0Dev &R = h->rt0;
     if ((e = KL(HDG_PROF_TRANSFER, 1, launch_rt0_restrict(h, k.res, R.rc))) != cudaSuccess) return e;
     double *cur = R.e0, *prev = nullptr, *spare[2] = {R.e1, R.e2};
@@ -605,7 +605,7 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
     // correction is formed along with the residual (into x2, which that sweep reads)
     const int np = h->prm.n_post;
     if (np == 0 || (np == 1 && (learned || collect))) {
-        if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, k.res, true))) != cudaSuccess) return e;
+        if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, k.res))) != cudaSuccess) return e;
     } else {
         if ((e = KL(cat_res<T>(), 1, launch_residual_smooth_t<T>(h, rhs, x, k.res, x2, cheb ? h->cheb_omega[0] : 0.0))) !=
             cudaSuccess)
@@ -686,13 +686,13 @@ cudaError_t precond(hdg_handle *h, const T *v, T *z, const T *w_src = nullptr, c
     if constexpr (std::is_same<T, float>::value) {
         if (learned) {
             // the learned sweep replaces the last smoothing step
-            if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, spare, true))) != cudaSuccess) return e;
+            if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, spare))) != cudaSuccess) return e;
             return KL(HDG_PROF_KRYLOV, 1, h->lc.tc ? launch_learned_infer_tc(h, spare, x, z)
                                                    : launch_learned_infer(h, spare, x, z));
         }
         // collecting: store the residual (normalised), then the plain last step
         T *slot = h->lc.buf + size_t(h->lc.count) * NT;
-        if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, slot, true))) != cudaSuccess) return e;
+        if ((e = KL(cat_res<T>(), 1, launch_residual_t<T>(h, v, x, slot))) != cudaSuccess) return e;
         Workspace &W = *h->ws;
         if ((e = dots<T>(h, slot, 1, slot, W.nrm2)) != cudaSuccess) return e;
         if ((e = launch_normalize32(slot, slot, W.nrm2, NT, s)) != cudaSuccess) return e;
@@ -1075,7 +1075,7 @@ int fgmres(hdg_handle *h, const T *b, T *x, double rtol, int max_it, bool true_r
         if (first && x_zero) {
             r0 = b;
         } else {
-            TRY(KL(cat_res<T>(), 1, launch_residual_t<T>(h, b, x, k.V, false)));
+            TRY(KL(cat_res<T>(), 1, launch_residual_t<T>(h, b, x, k.V)));
             rc = norm_host<T>(h, k.V, beta);
             if (rc) return rc;
         }
@@ -1112,7 +1112,7 @@ int fgmres(hdg_handle *h, const T *b, T *x, double rtol, int max_it, bool true_r
         }
         if ((flag & 2) && est > rtol) {
             // breakdown without convergence: check the true residual once more
-            TRY(KL(cat_res<T>(), 1, launch_residual_t<T>(h, b, x, k.V, false)));
+            TRY(KL(cat_res<T>(), 1, launch_residual_t<T>(h, b, x, k.V)));
             double beta2;
             rc = norm_host<T>(h, k.V, beta2);
             if (rc) return rc;
@@ -3166,7 +3166,7 @@ int hdg_learned_train(hdg_handle *h, int steps, int batch, double lr, double *lo
         for (int b = 0; b < batch; ++b) {
             const float *r = L.buf + size_t(splitmix64(L.rng) % uint64_t(L.count)) * NT;
             TRY(launch_learned_forward(h, r, L.c));
-            TRY(launch_residual_t<float>(h, r, L.c, L.rn, false));
+            TRY(launch_residual_t<float>(h, r, L.c, L.rn));
             double nrn;
             rc = norm_host<float>(h, L.rn, nrn);
             if (rc) return rc;
@@ -3230,7 +3230,7 @@ int hdg_learned_loss_grad_dev(hdg_handle *h, const float *R, int n, float *grad,
         W.host_buf[6] = -2.0 / (double(n) * nr * nr);
         TRY(cudaMemcpyAsync(L.coef, W.host_buf + 6, sizeof(double), cudaMemcpyHostToDevice, s));
         TRY(launch_learned_forward(h, L.tmp, L.c));
-        TRY(launch_residual_t<float>(h, L.tmp, L.c, L.rn, false));
+        TRY(launch_residual_t<float>(h, L.tmp, L.c, L.rn));
         double nrn;
         rc = norm_host<float>(h, L.rn, nrn);
         if (rc) return rc;

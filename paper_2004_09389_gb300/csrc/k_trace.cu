@@ -1273,17 +1273,17 @@ inline unsigned blocks(size_t n, int bs) { return unsigned((n + bs - 1) / bs); }
 
 }  // namespace
 
-// operator storage per use: FP64 path, FP32 Krylov operator, and the
-// preconditioner's copy (BF16 in HDG_MIXED_BF16, else the FP32 one)
+// operators by type: S, the inverse diagonal blocks, and the sweeps' H and D (null where the
+// sweeps of that type take S; HDG_MIXED_BF16 keeps H in BF16)
 template <typename T> struct Ops;
 template <> struct Ops<double> {
-    static const double *S(hdg_handle *h, bool) { return h->d_Sval; }
+    static const double *S(hdg_handle *h) { return h->d_Sval; }
     static const double *D(hdg_handle *h) { return h->d_Dinv; }
     static const double *H(hdg_handle *h) { return h->d_H; }
     static const double *Dg(hdg_handle *h) { return h->d_D; }
 };
 template <> struct Ops<float> {
-    static const float *S(hdg_handle *h, bool) { return h->d_Sval32; }
+    static const float *S(hdg_handle *h) { return h->d_Sval32; }
     static const float *D(hdg_handle *h) { return h->d_Dinv32; }
     static const float *H(hdg_handle *h) { return h->d_H32; }
     static const float *Dg(hdg_handle *h) { return h->d_D32; }
@@ -1295,7 +1295,7 @@ cudaError_t apply_dots_b(hdg_handle *h, unsigned nb, const T *x, T *y, const T *
                          unsigned int *counter, double *hdots, T *hneg) {
     constexpr int BB = sizeof(T) == 8 ? 4 : B;
     HDG_DISPATCH_PF(h->pf, T, (apply_dots_kernel_go<P, T, T, BB>(nb, 256, 0, h->stream, 
-                             h->NF, Ops<T>::S(h, false), h->d_nbr, x, y, V, ld, k, partial, counter, hdots, hneg)));
+                             h->NF, Ops<T>::S(h), h->d_nbr, x, y, V, ld, k, partial, counter, hdots, hneg)));
     return cudaGetLastError();
 }
 template <typename T>
@@ -1322,14 +1322,13 @@ cudaError_t launch_apply_dots_t(hdg_handle *h, const T *x, T *y, const T *V, siz
 }
 template <typename T>
 cudaError_t launch_apply_t(hdg_handle *h, const T *x, T *y) {
-    HDG_DISPATCH_PF(h->pf, T, (apply_kernel<P, T, T><<<blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream>>>(h->NF, Ops<T>::S(h, false), h->d_nbr, x, y)));
+    HDG_DISPATCH_PF(h->pf, T, (apply_kernel<P, T, T><<<blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream>>>(h->NF, Ops<T>::S(h), h->d_nbr, x, y)));
     return cudaGetLastError();
 }
-// residual / smoothing kernels serve the preconditioner (pre = true) or the
-// Krylov residual (pre = false)
+// res = b - S x, for the preconditioner and the Krylov residual
 template <typename T>
-cudaError_t launch_residual_t(hdg_handle *h, const T *b, const T *x, T *r, bool pre) {
-    HDG_DISPATCH_PF(h->pf, T, (residual_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, pre), h->d_nbr, b, x, r)));
+cudaError_t launch_residual_t(hdg_handle *h, const T *b, const T *x, T *r) {
+    HDG_DISPATCH_PF(h->pf, T, (residual_kernel_go<P, T, T>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h), h->d_nbr, b, x, r)));
     return cudaGetLastError();
 }
 // A sweep with b = D^-1 times the right-hand side where the handle's sweeps of this type
@@ -1344,7 +1343,7 @@ cudaError_t smooth_any(hdg_handle *h, const T *b, const T *x, T *xout, T om, T b
     if (Ops<T>::H(h)) {
         HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T, true, CHEB>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::H(h), nullptr, h->d_nbr, b, x, xout, om, beta, xprev)));
     } else {
-        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T, false, CHEB>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, xout, om, beta, xprev)));
+        HDG_DISPATCH_PF(h->pf, T, (smooth_kernel_go<P, T, T, false, CHEB>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h), Ops<T>::D(h), h->d_nbr, b, x, xout, om, beta, xprev)));
     }
     return cudaGetLastError();
 }
@@ -1397,7 +1396,7 @@ cudaError_t launch_residual_smooth_t(hdg_handle *h, const T *b, const T *x, T *r
     if (Ops<T>::H(h)) {
         HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T, true>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::H(h), Ops<T>::Dg(h), h->d_nbr, b, x, res, y, om)));
     } else {
-        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T, false>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h, true), Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
+        HDG_DISPATCH_P(h->p, (residual_smooth_kernel_go<P, T, T, false>(blocks(h->NF, h->bs_facet), h->bs_facet, 0, h->stream, h->NF, Ops<T>::S(h), Ops<T>::D(h), h->d_nbr, b, x, res, y, om)));
     }
     return cudaGetLastError();
 }
@@ -1426,8 +1425,8 @@ template cudaError_t launch_apply_dots_t<double>(hdg_handle *, const double *, d
 template cudaError_t launch_apply_dots_t<float>(hdg_handle *, const float *, float *, const float *, size_t, int,
                                                 double *, unsigned int *, double *, float *);
 template cudaError_t launch_apply_t<float>(hdg_handle *, const float *, float *);
-template cudaError_t launch_residual_t<double>(hdg_handle *, const double *, const double *, double *, bool);
-template cudaError_t launch_residual_t<float>(hdg_handle *, const float *, const float *, float *, bool);
+template cudaError_t launch_residual_t<double>(hdg_handle *, const double *, const double *, double *);
+template cudaError_t launch_residual_t<float>(hdg_handle *, const float *, const float *, float *);
 template cudaError_t launch_smooth_t<double>(hdg_handle *, const double *, const double *, double *);
 template cudaError_t launch_smooth_t<float>(hdg_handle *, const float *, const float *, float *);
 template cudaError_t launch_smooth_cheb_t<double>(hdg_handle *, const double *, const double *, double *, double,
