@@ -482,14 +482,14 @@ def step13_bytes(arm: dict):
     in step 1: its cell kernel reads the h rows of R_M (and the inverse velocity
     block where f varies over the cells), r and the cell weights (15 float pairs)
     and writes z and the cell rows; the recovery reads X_B, z and lambda and
-    writes u, h.  FP64 handles read W_K, r in step 1 and R_M, X_B (where f is
-    constant on every cell: their h rows), r, lambda in step 3."""
+    writes u, h.  FP64 handles read W_K, r in step 1 and the h rows of R_M and X_B
+    (and three matrices of the velocity block where f varies), r, lambda in step 3."""
     N, n, nK, m = arm["n_cells"], arm["n_p"], 3 * arm["n_p"], 3 * arm["pp"]
     if arm.get("keep_z"):
         mats = n * nK + (0 if arm.get("f_const", True) else 2 * n * n)
         return 8.0 * N * (mats + 2 * nK + m + 15), 8.0 * N * (nK * m + 2 * nK + m)
-    rows = n if arm.get("f_const", True) else nK
-    return 8.0 * N * (m * nK + nK + m), 8.0 * N * (rows * (nK + m) + 3 * nK + m)
+    vel = 0 if arm.get("f_const", True) else 3 * n * n
+    return 8.0 * N * (m * nK + nK + m), 8.0 * N * (n * (nK + m) + vel + 3 * nK + m)
 
 
 def whole_solve(arm: dict, peaks: dict, steps: int) -> dict:

@@ -500,7 +500,19 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
             o[size_t(14) * kFFCells] = split(fk);
         }
     }
-    // ---- R_M and W_K (two-float handles: the h rows of R_M): the columns of the unit
+    if constexpr (!FF && !FC) {
+        // Q, P - Q and P + Q for step 3, in the place of R_M's velocity rows
+        for (int idx = t; idx < NP * NP * CC; idx += kCondThreads) {
+            const int Kc = blockIdx.x * CC + idx % CC;
+            if (Kc >= a.N) continue;
+            const double p = Ps[idx], q = Qs[idx];
+            double *o = a.Rm + size_t(idx / CC) * N + Kc;
+            o[0] = q;
+            o[size_t(NP * NP) * N] = p - q;
+            o[size_t(2 * NP * NP) * N] = p + q;
+        }
+    }
+    // ---- The h rows of R_M and (FP64 handles) W_K: the columns of the unit
     // vectors in u_x, u_y and h, spread over all the block's threads.  The h columns' h is
     // a column of S^-1 itself.
     for (int it = t; it < 3 * NP * CC; it += kCondThreads) {
@@ -552,13 +564,7 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                 a.Hr2[2 * ff_pair_index(size_t(K), size_t(i) * CPk + kap_ / 2, size_t(NP) * CPk) + kap_ % 2] = split(h[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                if constexpr (!FC) {            // (f constant: step 3 takes the h rows only)
-                    a.Rm[(size_t(i) * NK + kap_) * N + K] = wx[i];
-                    a.Rm[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
-                }
-                a.Rm[(size_t(2 * NP + i) * NK + kap_) * N + K] = h[i];
-            }
+            for (int i = 0; i < NP; ++i) a.Rm[(size_t(2 * NP + i) * NK + kap_) * N + K] = h[i];
             double wn[3][3];
 #pragma unroll
             for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, K, e, wn[e]);

@@ -1033,42 +1033,20 @@ void rhs_gather_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStr
 }
 
 
-// step 3: q_K = R_M r_K - X_B lambda_K, written in the caller's u / h layout
-template <int P>
-__global__ void recover_kernel(int N, int NF, const double *__restrict__ Rm, const double *__restrict__ Xb,
-                               const double *__restrict__ r_u, const double *__restrict__ r_h,
-                               const double *__restrict__ lam, const int32_t *__restrict__ facet_of,
-                               const int32_t *__restrict__ flip, double *__restrict__ u, double *__restrict__ hout) {
-    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP;
-    const size_t idx = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (idx >= size_t(N) * NK) return;
-    const int rho = int(idx / N), K = int(idx % N);
-    double acc = 0.0;
-#pragma unroll 5
-    for (int kap = 0; kap < NK; ++kap)
-        acc = fma(__ldg(Rm + size_t(rho * NK + kap) * N + K), cell_rhs<NP>(r_u, r_h, K, kap), acc);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const int f = facet_of[3 * K + i], fl = flip[3 * K + i];
-#pragma unroll
-        for (int j = 0; j < PP; ++j)
-            acc = fma(-__ldg(Xb + size_t(rho * M + i * PP + j) * N + K), lam[size_t(fl ? P - j : j) * NF + f], acc);
-    }
-    if (rho < 2 * NP) u[size_t(K) * 2 * NP + rho] = acc;
-    else hout[size_t(K) * NP + rho - 2 * NP] = acc;
-}
-
-// Step 3 where f is constant on every cell: h by the rows of R_M and X_B, the velocity from
-// the momentum equations,
-//   u = R (r_u - tau g (grad h + sum_e n_e lift_e (lambda - h))),   R = (1 + tau^2 f^2)^-1 [1 tau f; -tau f 1],
+// Step 3, q_K = R_M r_K - X_B lambda_K: h by the rows of R_M and X_B, the velocity from the
+// momentum equations,
+//   u = R w,   w = r_u - tau g (grad h + sum_e n_e lift_e (lambda - h)),   R = [P Q; -Q P],
 // the weak gradient with the trace terms taken as the nodal one (whose vanishing entries are
-// left out) plus the lifted jumps.  The FP64 pipe is the bound: at p = 3 about 860 FMAs per
-// cell instead of 1260, and a third of the bytes: 192 instead of 314 us on 131,072 cells,
-// 19.5 instead of 24 on 18,432 at p = 2.
+// left out) plus the lifted jumps.  P and Q are numbers where f is constant on every cell
+// (FC); else n_p x n_p matrices, kept as Q, P - Q and P + Q, so that R w takes three products,
+//   k = Q (w_x + w_y),   u_x = (P - Q) w_x + k,   u_y = (P + Q) w_y - k.
+// The FP64 pipe is the bound: at p = 3 about 860 (FC) and 1,120 FMAs per cell instead of
+// the 1,260 of all rows of R_M and X_B: 192 instead of 314 us on 131,072 cells, 19.5 instead
+// of 24 on 18,432 at p = 2; f varying 169 instead of 185 on 81,920.
 // 32 cells per block (lane = cell), the warps take the nodes in turn.
 template <int P> constexpr int kRecWarps = P == 1 ? 3 : P == 2 ? 6 : 5;
-template <int P>
-__global__ void __launch_bounds__(32 * kRecWarps<P>) recover_const_f_kernel(int N, int NF, const double *__restrict__ Rm,
+template <int P, bool FC>
+__global__ void __launch_bounds__(32 * kRecWarps<P>) recover_kernel(int N, int NF, const double *__restrict__ Rm,
                                                                             const double *__restrict__ Xb,
                                                                             const double *__restrict__ nref,
                                                                             const double *__restrict__ X,
@@ -1158,12 +1136,47 @@ __global__ void __launch_bounds__(32 * kRecWarps<P>) recover_const_f_kernel(int 
                 wx = fma(-geo[4 + 2 * e][lane], l, wx);
                 wy = fma(-geo[5 + 2 * e][lane], l, wy);
             }
-            const double kap = geo[10][lane], fk = geo[11][lane];
-            sV[i][lane] = fma(kap, wx, fk * wy);
-            sV[NP + i][lane] = fma(kap, wy, -fk * wx);
+            if constexpr (FC) {
+                const double kap = geo[10][lane], fk = geo[11][lane];
+                sV[i][lane] = fma(kap, wx, fk * wy);
+                sV[NP + i][lane] = fma(kap, wy, -fk * wx);
+            } else {
+                sV[i][lane] = wx;
+                sV[NP + i][lane] = wy;
+            }
         });
     }
     __syncthreads();
+    if constexpr (!FC) {
+        if (on)
+            for (int i = w; i < NP; i += NW) sL[i][lane] = sV[i][lane] + sV[NP + i][lane];   // (the jumps have been read)
+        __syncthreads();
+        double ux[NP / NW], uy[NP / NW];
+        if (on) {
+#pragma unroll
+            for (int t = 0; t < NP / NW; ++t) {
+                const size_t i = size_t(w + t * NW), NN = NP * NP;
+                double a = 0.0, b = 0.0, c = 0.0;
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                    c = fma(__ldg(Rm + (i * NP + k) * N + K), sL[k][lane], c);
+                    a = fma(__ldg(Rm + (NN + i * NP + k) * N + K), sV[k][lane], a);
+                    b = fma(__ldg(Rm + (2 * NN + i * NP + k) * N + K), sV[NP + k][lane], b);
+                }
+                ux[t] = a + c;
+                uy[t] = b - c;
+            }
+        }
+        __syncthreads();                        // every warp has read w
+        if (on) {
+#pragma unroll
+            for (int t = 0; t < NP / NW; ++t) {
+                sV[w + t * NW][lane] = ux[t];
+                sV[NP + w + t * NW][lane] = uy[t];
+            }
+        }
+        __syncthreads();
+    }
     for (int j = threadIdx.x; j < nc * 2 * NP; j += 32 * NW) u[size_t(K0) * 2 * NP + j] = sV[j % (2 * NP)][j / (2 * NP)];
     for (int j = threadIdx.x; j < nc * NP; j += 32 * NW) hout[size_t(K0) * NP + j] = sV[2 * NP + j % NP][j / NP];
 }
@@ -1490,14 +1503,17 @@ cudaError_t launch_rhs(hdg_handle *h, const double *r_u, const double *r_h, doub
 cudaError_t launch_recover(hdg_handle *h, const double *r_u, const double *r_h, const double *lam, double *u,
                            double *hout) {
     if (h->prm.flux == 1) return launch_recover_lf(h, r_u, r_h, lam, u, hout);
-    size_t n = size_t(h->N) * h->nK;
+    const unsigned nb = blocks(h->N, 32);
+    const double tau = h->prm.tau, tg = tau * h->prm.g;
     if (h->f_const) {
-        HDG_DISPATCH_P(h->p, (recover_const_f_kernel<P><<<blocks(h->N, 32), 32 * kRecWarps<P>, 0, h->stream>>>(
-                                 h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, h->prm.tau,
-                                 h->prm.tau * h->prm.g, r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout)));
-        return cudaGetLastError();
+        HDG_DISPATCH_P(h->p, (recover_kernel<P, true><<<nb, 32 * kRecWarps<P>, 0, h->stream>>>(
+                                 h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, tau, tg, r_u, r_h, lam,
+                                 h->d_facet_of, h->d_flip, u, hout)));
+    } else {
+        HDG_DISPATCH_P(h->p, (recover_kernel<P, false><<<nb, 32 * kRecWarps<P>, 0, h->stream>>>(
+                                 h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, tau, tg, r_u, r_h, lam,
+                                 h->d_facet_of, h->d_flip, u, hout)));
     }
-    HDG_DISPATCH_P(h->p, (recover_kernel<P><<<blocks(n, 256), 256, 0, h->stream>>>(h->N, h->NF, h->d_Rm, h->d_Xb, r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout)));
     return cudaGetLastError();
 }
 

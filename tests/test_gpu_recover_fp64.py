@@ -1,6 +1,6 @@
-"""The FP64 recovery where f is constant on every cell (csrc/k_trace.cu): h by the rows of
-R_M and X_B, the velocity from the momentum equations, against the oracle, p = 1..4, with
-and without rotation, on a mesh whose cell count (242) leaves a ragged block of 32 cells.
+"""The FP64 recovery (csrc/k_trace.cu): h by the rows of R_M and X_B, the velocity from the
+momentum equations, against the oracle, p = 1..4, without rotation, with f constant on
+every cell and varying, on a mesh whose cell count (242) leaves a ragged block of 32 cells.
 
 1e-12 relative, the suite's tolerance for the FP64 steps."""
 import numpy as np
@@ -23,14 +23,14 @@ def _built():
 
 
 @pytest.mark.parametrize("p", [1, 2, 3, 4])
-@pytest.mark.parametrize("f0", [0.0, 1.0])
+@pytest.mark.parametrize("f0", [0.0, 1.0, "varying"])
 def test_recovery_matches_oracle(p, f0):
     from paper_2004_09389_gb300 import HDG_FP64, HDG_MIXED_FGMRES64, HDGSolver
     mesh = I.periodic_square_hierarchy(11, n_coarsest=4)
-    f = I.coriolis_flat(mesh, f0)
+    rng = np.random.default_rng(p)
+    f = rng.uniform(-1.0, 1.0, mesh.n_vertices) if f0 == "varying" else I.coriolis_flat(mesh, f0)
     tau, g, H = 12 * mesh.h, 1.3, 0.7
     prob = HDGProblem(mesh, p, tau=tau, g=g, H=H, f_vertex=f)
-    rng = np.random.default_rng(p)
     ru = rng.standard_normal((mesh.n_cells, 2, prob.np))
     rh = rng.standard_normal((mesh.n_cells, prob.np))
     lam = rng.standard_normal((prob.n_facets, p + 1))
