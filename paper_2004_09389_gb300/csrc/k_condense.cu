@@ -48,10 +48,12 @@ struct Sz {
 // measured, one warp instruction in about 77 cycles per scheduler), so the split is
 // the one that keeps the warps full (at p = 3 8 x 10 columns up to S, 8 x 12 for X_B
 // and all 8 x 30 of R_M dealt to the 96 threads) and what need not be FP64 is not: the
-// conversions to float pairs, the correction of the refinement, pivot tests.  The h
-// columns of R_M are S^-1 as it stands, and R_M's h rows are not refined (step 1 and
-// the recovery of the two-float handles are as exact either way, 1e-14 to 7e-14 of the
-// oracle at p = 1 .. 4, Courant 8 and 16).  20,480 cells at p = 3, two-float, f varying:
+// conversions to float pairs, the correction of the refinement, pivot tests.  The columns
+// of R_M are refined like those of X_B where W_K = C R_M follows from them (FP64 handles:
+// without, the condensed right-hand side of smooth data was 1.3e-14 off at p = 3 and 1.1e-13
+// at p = 4, Courant 16, instead of 1.0e-15 and 3.8e-15); the two-float handles' h rows are
+// not (their right-hand side is 4e-14 and 2.5e-13 off either way).  20,480 cells at p = 3,
+// two-float, f varying:
 // 1,345 us instead of 1,773 (one pass of 10 of 12 columns per component of R_M, all of
 // them refined in FP64, a full division per pivot and column, two products where column
 // k meets the pivot's); 18,432 cells at p = 2 in FP64: 384 instead of 419, against 1,466
@@ -179,16 +181,9 @@ __device__ __forceinline__ void add_div(const double *ref, double g00, double g0
     });
 }
 
-// h = S^-1 rh and (wx, wy) -= T h (Ts null: h alone), cell c of the block's matrices.  So
-// non-null: S itself, for one step of iterative refinement of h, the residual in FP64 and
-// its correction, 1e-14 of h, with the inverse rounded to FP32 (Sf).  The explicit inverse alone
-// leaves S_K about 20 times less exact than an elimination of the whole cell system
-// (p = 3, Courant 16: S_K applied to a nearly constant trace off by 1e-12 instead of
-// 7e-14); one step brings it to 2e-14.
+// h = S^-1 rh for cell c of the block's matrices, the explicit inverse
 template <int NP, int CC>
-__device__ __forceinline__ void back_substitute(const double *Ss, const double *So, const float *Sf, const double *Ts,
-                                                int c, const double (&rh)[NP], double (&wx)[NP], double (&wy)[NP],
-                                                double (&h)[NP]) {
+__device__ __forceinline__ void inverse_product(const double *Ss, int c, const double (&rh)[NP], double (&h)[NP]) {
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
         row_fence();
@@ -197,26 +192,39 @@ __device__ __forceinline__ void back_substitute(const double *Ss, const double *
         for (int k = 0; k < NP; ++k) v = fma(Ss[(i * NP + k) * CC + c], rh[k], v);
         h[i] = v;
     }
-    if (So) {
-        float res[NP];
+}
+
+// One step of iterative refinement of h = S^-1 rh: the residual in FP64 from S itself (So)
+// and its correction, 1e-14 of h, with the inverse rounded to FP32 (Sf).  The explicit inverse
+// alone leaves S_K about 20 times less exact than an elimination of the whole cell system
+// (p = 3, Courant 16: S_K applied to a nearly constant trace off by 1e-12 instead of
+// 7e-14; one step brings it to 2e-14), and W_K up to 24 times.
+template <int NP, int CC>
+__device__ __forceinline__ void refine(const double *So, const float *Sf, int c, const double (&rh)[NP],
+                                       double (&h)[NP]) {
+    float res[NP];
 #pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            row_fence();
-            double v = rh[i];
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+        double v = rh[i];
 #pragma unroll
-            for (int k = 0; k < NP; ++k) v = fma(-So[(i * NP + k) * CC + c], h[k], v);
-            res[i] = to_float(v);
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            row_fence();
-            float v = 0.0f;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) v = fmaf(Sf[(i * NP + k) * CC + c], res[k], v);
-            h[i] += join(make_float2(v, 0.0f));
-        }
+        for (int k = 0; k < NP; ++k) v = fma(-So[(i * NP + k) * CC + c], h[k], v);
+        res[i] = to_float(v);
     }
-    if (!Ts) return;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+        float v = 0.0f;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) v = fmaf(Sf[(i * NP + k) * CC + c], res[k], v);
+        h[i] += join(make_float2(v, 0.0f));
+    }
+}
+
+// (wx, wy) -= T h
+template <int NP, int CC>
+__device__ __forceinline__ void subtract_gradient(const double *Ts, int c, const double (&h)[NP], double (&wx)[NP],
+                                                  double (&wy)[NP]) {
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
         row_fence();
@@ -456,7 +464,9 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
             }
         }
         add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
-        back_substitute<NP, CC>(Ss, So, Sf, Ts, c, rh, wx, wy, h);
+        inverse_product<NP, CC>(Ss, c, rh, h);
+        refine<NP, CC>(So, Sf, c, rh, h);
+        subtract_gradient<NP, CC>(Ts, c, h, wx, wy);
         if constexpr (FF) {
             constexpr int CPb = (M + 1) / 2;
 #pragma unroll
@@ -514,15 +524,14 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
     }
     // ---- The h rows of R_M and (FP64 handles) W_K: the columns of the unit
     // vectors in u_x, u_y and h, spread over all the block's threads.  The h columns' h is
-    // a column of S^-1 itself.
+    // a column of S^-1, refined on FP64 handles.
     for (int it = t; it < 3 * NP * CC; it += kCondThreads) {
         const int c = it % CC, kap_ = it / CC, comp = kap_ / NP, j = kap_ % NP, K = blockIdx.x * CC + c;
         if (K >= a.N) continue;
         const double j00 = geo[0 * CC + c], j01 = geo[1 * CC + c], j10 = geo[2 * CC + c], j11 = geo[3 * CC + c];
-        double wx[NP], wy[NP], h[NP];
+        double wx[NP], wy[NP], rh[NP], h[NP];
         if (comp < 2) {
             const double kap = geo[13 * CC + c], fk = geo[14 * CC + c];
-            double rh[NP];
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
                 double p, q;
@@ -538,24 +547,18 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                 rh[i] = 0.0;
             }
             add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
-            back_substitute<NP, CC>(Ss, nullptr, nullptr, FF ? nullptr : Ts, c, rh, wx, wy, h);
+            inverse_product<NP, CC>(Ss, c, rh, h);
         } else {
 #pragma unroll
-            for (int i = 0; i < NP; ++i) h[i] = Ss[(i * NP + j) * CC + c];
-            if constexpr (!FF) {
-#pragma unroll
-                for (int i = 0; i < NP; ++i) {
-                    row_fence();
-                    double vx = 0.0, vy = 0.0;
-#pragma unroll
-                    for (int k = 0; k < NP; ++k) {
-                        vx = fma(-Ts[(i * NP + k) * CC + c], h[k], vx);
-                        vy = fma(-Ts[((NP + i) * NP + k) * CC + c], h[k], vy);
-                    }
-                    wx[i] = vx;
-                    wy[i] = vy;
-                }
+            for (int i = 0; i < NP; ++i) {
+                wx[i] = wy[i] = 0.0;
+                rh[i] = i == j ? 1.0 : 0.0;
+                h[i] = Ss[(i * NP + j) * CC + c];
             }
+        }
+        if constexpr (!FF) {
+            refine<NP, CC>(So, Sf, c, rh, h);
+            subtract_gradient<NP, CC>(Ts, c, h, wx, wy);
         }
         if constexpr (FF) {
             constexpr int CPk = (NK + 1) / 2;
