@@ -1522,7 +1522,7 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(dalloc(&h->d_nbr, 4 * NF));
     if (!mode_ff(*prm)) {
         TRY(dalloc(&h->d_Xb, nK * m * N));
-        TRY(dalloc(&h->d_Rm, nK * nK * N));
+        TRY(dalloc(&h->d_Rm, (prm->flux == 1 ? nK * nK : size_t(rm_offsets(h->p, h->f_const).total)) * N));
         TRY(dalloc(&h->d_W, m * nK * N));
     }
     TRY(dalloc(&h->d_Scell, N * m * m));

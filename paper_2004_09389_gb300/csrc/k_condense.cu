@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
         }
     }
     if constexpr (!FF && !FC) {
-        // Q, P - Q and P + Q for step 3, in the place of R_M's velocity rows
+        // Q, P - Q and P + Q for step 3
         for (int idx = t; idx < NP * NP * CC; idx += kCondThreads) {
             const int Kc = blockIdx.x * CC + idx % CC;
             if (Kc >= a.N) continue;
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                 a.Hr2[2 * ff_pair_index(size_t(K), size_t(i) * CPk + kap_ / 2, size_t(NP) * CPk) + kap_ % 2] = split(h[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < NP; ++i) a.Rm[(size_t(2 * NP + i) * NK + kap_) * N + K] = h[i];
+            for (int i = 0; i < NP; ++i) a.Rm[(size_t(rm_offsets(P, FC).h) + i * NK + kap_) * N + K] = h[i];
             double wn[3][3];
 #pragma unroll
             for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, K, e, wn[e]);

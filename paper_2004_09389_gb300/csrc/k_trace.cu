@@ -1096,12 +1096,13 @@ __global__ void __launch_bounds__(32 * kRecWarps<P>) recover_kernel(int N, int N
     if (on) {
 #pragma unroll
         for (int t = 0; t < NP / NW; ++t) {
-            const size_t row = size_t(2 * NP + w + t * NW);
+            const size_t i = size_t(w + t * NW);
             double acc = 0.0;
 #pragma unroll 10
-            for (int kap = 0; kap < NK; ++kap) acc = fma(__ldg(Rm + (row * NK + kap) * N + K), sV[kap][lane], acc);
+            for (int kap = 0; kap < NK; ++kap)
+                acc = fma(__ldg(Rm + (rm_offsets(P, FC).h + i * NK + kap) * N + K), sV[kap][lane], acc);
 #pragma unroll
-            for (int q = 0; q < M; ++q) acc = fma(-__ldg(Xb + (row * M + q) * N + K), sL[q][lane], acc);
+            for (int q = 0; q < M; ++q) acc = fma(-__ldg(Xb + ((2 * NP + i) * M + q) * N + K), sL[q][lane], acc);
             hv[t] = acc;
         }
     }
