@@ -1485,6 +1485,20 @@ bool hat_pays32(const hdg_params &prm, size_t NF, size_t pp, size_t l2) {
     return mode_pre32(prm) || 14 * blk <= l2 / 3 || 6 * blk > l2 / 3 * 2;
 }
 
+// The recovery of FP64 handles by the rows of R_M and X_B (n_K (n_K + m) FMAs per cell, one
+// dependent sum per thread) or by the h rows and the momentum equations (0.7 to 0.9 of the
+// FMAs from p = 2 on, but a chain of five barriers): by rows until they take the FP64 pipe
+// about as long as that chain.  In us, rows / momentum, f constant per cell: p = 1 512 cells
+// 4.1 / 7.4, 131,072 35 / 43; p = 2 8,192 10.2 / 11.8, 18,432 21.0 / 18.0; p = 3 2,048 8.9 / 14.7, 4,608
+// 14.6 / 14.8, 8,192 24.8 / 20.0; p = 4 2,048 14.5 / 23.6, 8,192 49 / 34.  Where f varies the
+// momentum form has three products more: p = 1 131,072 35 / 52, p = 2 113 / 121, p = 4 32,768
+// 157 / 182; p = 3 2,048 8.8 / 17.7, 8,192 23.7 / 24.9, 18,432 48.8 / 45.1, 73,728 165 / 158.
+bool recover_by_rows(int p, size_t N, bool f_const) {
+    const size_t n = size_t(p + 1) * (p + 2) / 2, fmas = N * 9 * n * (n + size_t(p) + 1);
+    if (f_const) return p == 1 || fmas <= 7000000;
+    return p != 3 || fmas <= 15000000;
+}
+
 int setup_device(hdg_handle *h, const hdg_params *prm) {
     cudaStream_t s = h->stream;
     const HostMesh &hm = h->hm;
@@ -1522,7 +1536,8 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(dalloc(&h->d_nbr, 4 * NF));
     if (!mode_ff(*prm)) {
         TRY(dalloc(&h->d_Xb, nK * m * N));
-        TRY(dalloc(&h->d_Rm, (prm->flux == 1 ? nK * nK : size_t(rm_offsets(h->p, h->f_const).total)) * N));
+        h->rec_rows = prm->flux == 1 || recover_by_rows(h->p, N, h->f_const);
+        TRY(dalloc(&h->d_Rm, size_t(rm_offsets(h->p, h->f_const, h->rec_rows).total) * N));
         TRY(dalloc(&h->d_W, m * nK * N));
     }
     TRY(dalloc(&h->d_Scell, N * m * m));

@@ -72,15 +72,15 @@ __host__ __device__ constexpr NodalOffsets nodal_offsets(int p) {
     const int l = 3 * n * (p + 1);
     return NodalOffsets{0, nn, 2 * nn, 2 * nn + l, 3 * nn + l, 4 * nn + l, 5 * nn + l, 6 * nn + l};
 }
-// What the recovery of FP64 handles keeps of R_M = A^-1 Mass per cell (upwind flux): where f
-// varies over a cell, Q, P - Q and P + Q of the inverse velocity block [n][n]; the h rows
-// [n][3 n].  315 MB where f is constant, instead of the 944 of all rows, on 131,072 cells at
-// p = 3.
+// What the recovery of FP64 handles keeps of R_M = A^-1 Mass per cell (upwind flux): the h
+// rows [n][3 n], behind the velocity rows [2 n][3 n] (rows) or, where f varies over a cell,
+// Q, P - Q and P + Q of the inverse velocity block [n][n].  315 MB where f is constant,
+// instead of the 944 of all rows, on 131,072 cells at p = 3.
 struct RmOffsets {
     int h, total;
 };
-__host__ __device__ constexpr RmOffsets rm_offsets(int p, bool f_const) {
-    const int n = (p + 1) * (p + 2) / 2, v = f_const ? 0 : 3 * n * n;
+__host__ __device__ constexpr RmOffsets rm_offsets(int p, bool f_const, bool rows) {
+    const int n = (p + 1) * (p + 2) / 2, v = rows ? 6 * n * n : f_const ? 0 : 3 * n * n;
     return RmOffsets{v, v + 3 * n * n};
 }
 // lattice index b (row) of cell node k of degree p; a = k - row start, c = p - a - b
@@ -872,6 +872,7 @@ struct hdg_handle {
     std::vector<double> cheb_c_omega, cheb_c_beta;
     bool has_f = false;               // a non-zero Coriolis field was given to hdg_setup
     bool f_const = true;              // the field is constant on every cell (none, or an f-plane)
+    bool rec_rows = false;            // FP64 recovery by the rows of R_M (recover_by_rows)
     // Chebyshev smoother (smoother 1): the ellipse, the Ritz values it was
     // fitted to, and per step k the sweep coefficients omega_k (of D^-1 r)
     // and beta_k (of x_k - x_{k-1})

@@ -68,7 +68,9 @@ struct NodalArgs {
     const double *M1;       // [PP][PP] edge mass matrix
     const double *X;        // [N][3][2]
     const double *fcell;    // [N][3]
-    double *Xb, *Rm, *W, *Scell;       // FP64 handles (Scell: both)
+    double *Xb, *W, *Scell;            // FP64 handles (Scell: both)
+    double *Rh, *Ru, *PQ;              // FP64 handles: the h rows of R_M, its velocity rows (or null) or
+                                       // else (f varying over a cell) Q, P - Q, P + Q
     float2 *Xb2, *Hr2, *lgeo;          // two-float handles: X_B, the h rows of R_M, the cell
     float4 *PQ2;                       // weights and (f varying over a cell) P, Q
     int32_t *status;
@@ -512,11 +514,11 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
     }
     if constexpr (!FF && !FC) {
         // Q, P - Q and P + Q for step 3
-        for (int idx = t; idx < NP * NP * CC; idx += kCondThreads) {
+        for (int idx = t; a.PQ && idx < NP * NP * CC; idx += kCondThreads) {
             const int Kc = blockIdx.x * CC + idx % CC;
             if (Kc >= a.N) continue;
             const double p = Ps[idx], q = Qs[idx];
-            double *o = a.Rm + size_t(idx / CC) * N + Kc;
+            double *o = a.PQ + size_t(idx / CC) * N + Kc;
             o[0] = q;
             o[size_t(NP * NP) * N] = p - q;
             o[size_t(2 * NP * NP) * N] = p + q;
@@ -567,7 +569,14 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
                 a.Hr2[2 * ff_pair_index(size_t(K), size_t(i) * CPk + kap_ / 2, size_t(NP) * CPk) + kap_ % 2] = split(h[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < NP; ++i) a.Rm[(size_t(rm_offsets(P, FC).h) + i * NK + kap_) * N + K] = h[i];
+            for (int i = 0; i < NP; ++i) a.Rh[(size_t(i) * NK + kap_) * N + K] = h[i];
+            if (a.Ru) {
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    a.Ru[(size_t(i) * NK + kap_) * N + K] = wx[i];
+                    a.Ru[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
+                }
+            }
             double wn[3][3];
 #pragma unroll
             for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, K, e, wn[e]);
@@ -935,7 +944,10 @@ cudaError_t condense_nodal_p(hdg_handle *h) {
     NodalArgs a;
     a.N = h->N; a.tau = h->prm.tau; a.g = h->prm.g; a.H = h->prm.H; a.ts = h->tau_s;
     a.nref = h->d_nref; a.M1 = h->d_ref + ref_offsets(P).M1; a.X = h->d_X; a.fcell = h->d_fcell;
-    a.Xb = h->d_Xb; a.Rm = h->d_Rm; a.W = h->d_W; a.Scell = h->d_Scell; a.status = h->d_status;
+    a.Xb = h->d_Xb; a.W = h->d_W; a.Scell = h->d_Scell; a.status = h->d_status;
+    a.Rh = FF ? nullptr : h->d_Rm + size_t(rm_offsets(P, FC, h->rec_rows).h) * h->N;
+    a.Ru = h->rec_rows ? h->d_Rm : nullptr;
+    a.PQ = h->rec_rows ? nullptr : h->d_Rm;
     a.Xb2 = h->d_Xb2; a.Hr2 = h->d_Hr2; a.lgeo = h->d_lgeo; a.PQ2 = reinterpret_cast<float4 *>(h->d_PQ2);
     k<<<(h->N + kCondCells<P> - 1) / kCondCells<P>, kCondThreads, smem, h->stream>>>(a);
     return cudaGetLastError();

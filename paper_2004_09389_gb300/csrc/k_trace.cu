@@ -1033,7 +1033,34 @@ void rhs_gather_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStr
 }
 
 
-// Step 3, q_K = R_M r_K - X_B lambda_K: h by the rows of R_M and X_B, the velocity from the
+// Step 3, q_K = R_M r_K - X_B lambda_K, by the rows of both, one thread per row and cell
+// (recover_by_rows in api.cu: small meshes)
+template <int P>
+__global__ void recover_rows_kernel(int N, int NF, const double *__restrict__ Rm, const double *__restrict__ Xb,
+                                    const double *__restrict__ r_u, const double *__restrict__ r_h,
+                                    const double *__restrict__ lam, const int32_t *__restrict__ facet_of,
+                                    const int32_t *__restrict__ flip, double *__restrict__ u,
+                                    double *__restrict__ hout) {
+    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP;
+    const size_t idx = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (idx >= size_t(N) * NK) return;
+    const int rho = int(idx / N), K = int(idx % N);
+    double acc = 0.0;
+#pragma unroll 5
+    for (int kap = 0; kap < NK; ++kap)
+        acc = fma(__ldg(Rm + size_t(rho * NK + kap) * N + K), cell_rhs<NP>(r_u, r_h, K, kap), acc);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int f = facet_of[3 * K + i], fl = flip[3 * K + i];
+#pragma unroll
+        for (int j = 0; j < PP; ++j)
+            acc = fma(-__ldg(Xb + size_t(rho * M + i * PP + j) * N + K), lam[size_t(fl ? P - j : j) * NF + f], acc);
+    }
+    if (rho < 2 * NP) u[size_t(K) * 2 * NP + rho] = acc;
+    else hout[size_t(K) * NP + rho - 2 * NP] = acc;
+}
+
+// The same on larger meshes: h by the rows of R_M and X_B, the velocity from the
 // momentum equations,
 //   u = R w,   w = r_u - tau g (grad h + sum_e n_e lift_e (lambda - h)),   R = [P Q; -Q P],
 // the weak gradient with the trace terms taken as the nodal one (whose vanishing entries are
@@ -1041,10 +1068,10 @@ void rhs_gather_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStr
 // (FC); else n_p x n_p matrices, kept as Q, P - Q and P + Q, so that R w takes three products,
 //   k = Q (w_x + w_y),   u_x = (P - Q) w_x + k,   u_y = (P + Q) w_y - k.
 // The FP64 pipe is the bound: at p = 3 about 860 (FC) and 1,120 FMAs per cell instead of
-// the 1,260 of all rows of R_M and X_B: 192 instead of 314 us on 131,072 cells, 19.5 instead
-// of 24 on 18,432 at p = 2; f varying 169 instead of 185 on 81,920.
+// the 1,260 of all rows of R_M and X_B: 192 instead of 314 us on 131,072 cells, 18.0 instead
+// of 21.0 on 18,432 at p = 2; f varying 169 instead of 185 on 81,920.
 // 32 cells per block (lane = cell), the warps take the nodes in turn.
-template <int P> constexpr int kRecWarps = P == 1 ? 3 : P == 2 ? 6 : 5;
+template <int P> constexpr int kRecWarps = P == 2 ? 6 : 5;
 template <int P, bool FC>
 __global__ void __launch_bounds__(32 * kRecWarps<P>) recover_kernel(int N, int NF, const double *__restrict__ Rm,
                                                                             const double *__restrict__ Xb,
@@ -1100,7 +1127,7 @@ __global__ void __launch_bounds__(32 * kRecWarps<P>) recover_kernel(int N, int N
             double acc = 0.0;
 #pragma unroll 10
             for (int kap = 0; kap < NK; ++kap)
-                acc = fma(__ldg(Rm + (rm_offsets(P, FC).h + i * NK + kap) * N + K), sV[kap][lane], acc);
+                acc = fma(__ldg(Rm + (rm_offsets(P, FC, false).h + i * NK + kap) * N + K), sV[kap][lane], acc);
 #pragma unroll
             for (int q = 0; q < M; ++q) acc = fma(-__ldg(Xb + ((2 * NP + i) * M + q) * N + K), sL[q][lane], acc);
             hv[t] = acc;
@@ -1504,17 +1531,23 @@ cudaError_t launch_rhs(hdg_handle *h, const double *r_u, const double *r_h, doub
 cudaError_t launch_recover(hdg_handle *h, const double *r_u, const double *r_h, const double *lam, double *u,
                            double *hout) {
     if (h->prm.flux == 1) return launch_recover_lf(h, r_u, r_h, lam, u, hout);
+    if (h->rec_rows) {
+        HDG_DISPATCH_P(h->p, (recover_rows_kernel<P><<<blocks(size_t(h->N) * h->nK, 256), 256, 0, h->stream>>>(
+                                 h->N, h->NF, h->d_Rm, h->d_Xb, r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout)));
+        return cudaGetLastError();
+    }
+    // (recover_by_rows leaves these)
     const unsigned nb = blocks(h->N, 32);
     const double tau = h->prm.tau, tg = tau * h->prm.g;
-    if (h->f_const) {
-        HDG_DISPATCH_P(h->p, (recover_kernel<P, true><<<nb, 32 * kRecWarps<P>, 0, h->stream>>>(
-                                 h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, tau, tg, r_u, r_h, lam,
-                                 h->d_facet_of, h->d_flip, u, hout)));
-    } else {
-        HDG_DISPATCH_P(h->p, (recover_kernel<P, false><<<nb, 32 * kRecWarps<P>, 0, h->stream>>>(
-                                 h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, tau, tg, r_u, r_h, lam,
-                                 h->d_facet_of, h->d_flip, u, hout)));
-    }
+    auto momentum = [&](auto kernel, int warps) {
+        kernel<<<nb, 32 * warps, 0, h->stream>>>(h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, tau, tg,
+                                                 r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout);
+    };
+    if (h->f_const && h->p == 2) momentum(&recover_kernel<2, true>, kRecWarps<2>);
+    else if (h->f_const && h->p == 3) momentum(&recover_kernel<3, true>, kRecWarps<3>);
+    else if (h->f_const && h->p == 4) momentum(&recover_kernel<4, true>, kRecWarps<4>);
+    else if (!h->f_const && h->p == 3) momentum(&recover_kernel<3, false>, kRecWarps<3>);
+    else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
