@@ -1502,9 +1502,9 @@ bool recover_by_rows(int p, size_t N, bool f_const) {
 int setup_device(hdg_handle *h, const hdg_params *prm) {
     cudaStream_t s = h->stream;
     const HostMesh &hm = h->hm;
-    RefElem re = build_ref_elem(h->p);
+    RefElem re;
+    const NodalRef nr = build_nodal_ref(h->p, &re);
     TRY(upload(&h->d_ref, re.packed(), s));
-    const NodalRef nr = build_nodal_ref(h->p);
     TRY(upload(&h->d_nref, nr.packed(), s));
     TRY(upload(&h->d_X, hm.X, s));
     std::vector<double> fcell(size_t(h->N) * 3, 0.0);
