@@ -631,7 +631,7 @@ __device__ __forceinline__ double block_sum_warp0(double v) {
 // pdl_launch may be scheduled while the previous kernel in the stream drains
 // its last blocks, which hides most of the launch and dispatch latency of
 // short kernels.  Such a kernel calls pdl_wait() before it touches any global
-// memory: the wait returns once the previous kernel has completed and its
+// memory that the previous kernel may write: the wait returns once that has completed and its
 // writes are visible (for a kernel launched without the attribute it returns
 // at once).  pdl_wait() then lets the next kernel be scheduled in turn.
 __device__ __forceinline__ void pdl_wait() {

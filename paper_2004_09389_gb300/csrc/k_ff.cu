@@ -31,8 +31,9 @@ inline unsigned blocks(size_t n, int bs) { return unsigned((n + bs - 1) / bs); }
 // The cell kernels take 32 consecutive cells per block (lane = cell): the
 // cells' right-hand sides r_K = (r_u, r_h) are read as contiguous chunks,
 // split once into shared memory and shared by the warps, which take the output
-// rows in turn; per-cell matrices, split into pairs of row entries
-// ([row][col pair][N], split_pairs_kernel), load coalesced, 16 bytes per lane.
+// rows in turn; per-cell matrices are float pairs of two row entries in tiles of 32 cells
+// ([tile][row][col pair][32], ff_pair_index, written by the condensation) and load
+// coalesced, 16 bytes per lane.
 constexpr int kCells = kFFCells;
 constexpr int kCellsPad = kCells + 1;
 
@@ -488,17 +489,6 @@ __device__ __forceinline__ void stage_cell_rhs(int N, int K0, const double *__re
         if (ch) ch[k] = v;
         sIn[2 * NP + j % NP][j / NP] = split(v);
     }
-}
-
-// the product of two pairs as a normalised pair (leading product by FMA with
-// its exact error, the cross terms added to it; about 2^-46 relative)
-__device__ __forceinline__ float2 ff_mul(const float2 a, const float2 b) {
-    const float p = __fmul_rn(a.x, b.x);
-    float e = __fmaf_rn(a.x, b.x, -p);
-    e = __fmaf_rn(a.x, b.y, e);
-    e = __fmaf_rn(a.y, b.x, e);
-    const float hi = __fadd_rn(p, e);
-    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, p)));
 }
 
 // ---------------------------------------------------------------- the cell solve

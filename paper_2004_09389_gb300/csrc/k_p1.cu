@@ -876,9 +876,11 @@ __device__ __forceinline__ void coarse_product(const double *inv, int n, const T
 // 32.  The FP64 pipe bounds it (n^2 FMAs over 152 SMs: 2 us at n = 1,024), so the rows
 // go evenly over the SMs (R: about n / 152), each value of b is widened once per warp
 // for R rows, and the lanes' R sums are added by halving exchanges (R adds instead of
-// 5 R) before the eight warps' sums.  The operator is static during a solve: the first
-// kDensePre columns' entries per lane are loaded before the wait for the previous kernel.
-constexpr int kDenseWarps = 8, kDensePre = 4;
+// 5 R) before the eight warps' sums.  The operator is static during a solve: a lane's
+// entries (up to kDensePre columns) are loaded before the wait for the previous kernel, by
+// when every kernel before that one has completed.
+constexpr int kDenseWarps = 8, kDensePre = 4, kDenseMax = 32 * kDenseWarps * kDensePre;
+static_assert(kTailOpMax <= kDenseMax, "every tail operator's columns fit the lanes");
 template <int R>
 __device__ __forceinline__ void dense_loads(const double *op, int n, int row0, int j, int jend, double (&a)[R]) {
 #pragma unroll
@@ -906,13 +908,6 @@ __device__ __forceinline__ void dense_kernel_impl(int bid_, int nb_, const doubl
         const double bd = double(bv[u]);
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[r] = fma(a[u][r], bd, acc[r]);
-    }
-    for (int j = j0 + 32 * kDensePre; j - lane < jend; j += 32) {   // n above 1,024
-        double v[R];
-        dense_loads<R>(op, n, row0, j, jend, v);
-        const double bd = j < jend ? double(b[j]) : 0.0;
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = fma(v[r], bd, acc[r]);
     }
     int keep;
     const double t = warp_sums<R>(acc, keep);
@@ -1191,6 +1186,7 @@ cudaError_t launch_p1_up_fused(const DevLevel &fine, const DevLevel &coarse, con
 }
 template <typename T>
 cudaError_t launch_p1_dense(const double *op, int n, const T *b, T *x, cudaStream_t s) {
+    if (n > kDenseMax) return cudaErrorInvalidValue;       // (set-up admits 1,024 coarsest vertices at most)
     // rows per block: about one block per SM
     constexpr unsigned bs = 32 * kDenseWarps;
     if (n <= 152) dense_kernel_go<T, 1>(blocks(n, 1), bs, 0, s, op, n, b, x);
