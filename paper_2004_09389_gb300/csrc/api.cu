@@ -1492,11 +1492,12 @@ bool hat_pays32(const hdg_params &prm, size_t NF, size_t pp, size_t l2) {
 // 4.1 / 7.4, 131,072 35 / 43; p = 2 8,192 10.2 / 11.8, 18,432 21.0 / 18.0; p = 3 2,048 8.9 / 14.7, 4,608
 // 14.6 / 14.8, 8,192 24.8 / 20.0; p = 4 2,048 14.5 / 23.6, 8,192 49 / 34.  Where f varies the
 // momentum form has three products more: p = 1 131,072 35 / 52, p = 2 113 / 121, p = 4 32,768
-// 157 / 182; p = 3 2,048 8.8 / 17.7, 8,192 23.7 / 24.9, 18,432 48.8 / 45.1, 73,728 165 / 158.
+// 157 / 182; p = 3 2,048 8.8 / 17.7, 8,192 23.7 / 24.9, then by how evenly its blocks fill the SMs
+// 18,432 48.8 / 45.1, 20,480 52.7 / 56.7, 32,768 78 / 83, 73,728 165 / 158, 81,920 185 / 169.
 bool recover_by_rows(int p, size_t N, bool f_const) {
     const size_t n = size_t(p + 1) * (p + 2) / 2, fmas = N * 9 * n * (n + size_t(p) + 1);
     if (f_const) return p == 1 || fmas <= 7000000;
-    return p != 3 || fmas <= 15000000;
+    return p != 3 || fmas <= 62000000;
 }
 
 int setup_device(hdg_handle *h, const hdg_params *prm) {

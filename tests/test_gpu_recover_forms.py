@@ -25,7 +25,7 @@ def _built():
 
 # the two sides of each line: by rows, by the momentum equations
 @pytest.mark.parametrize("p,n,varying", [(2, 84, False), (2, 88, False), (3, 52, False), (3, 62, False),
-                                         (4, 36, False), (4, 38, False), (3, 76, True), (3, 80, True),
+                                         (4, 36, False), (4, 38, False), (3, 152, True), (3, 160, True),
                                          (2, 88, True), (1, 128, False)])
 def test_recovery_on_either_side_of_the_line(p, n, varying):
     from paper_2004_09389_gb300 import HDG_FP64, HDGSolver
