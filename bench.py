@@ -490,7 +490,7 @@ def step13_bytes(arm: dict):
         mats = n * nK + (0 if arm.get("f_const", True) else 2 * n * n)
         return 8.0 * N * (mats + 2 * nK + m + 15), 8.0 * N * (nK * m + 2 * nK + m)
     const, p, fmas = arm.get("f_const", True), arm["pp"] - 1, N * nK * (nK + m)
-    if (p == 1 or fmas <= 7_000_000) if const else (p != 3 or fmas <= 62_000_000):
+    if p == 1 or fmas <= 7_000_000:
         step3 = nK * (nK + m)
     else:
         step3 = n * (nK + m) + (0 if const else 3 * n * n)
@@ -612,15 +612,16 @@ def roofline(arm: dict, peaks: dict, fma: dict | None = None, bf16_pre: bool = F
 
 def condense_rate(arm: dict, fma: dict) -> dict:
     """FP64 flop rate of the condensation against the measured FP64 FMA rate.
-    Per cell, with f constant on every cell (an FP64 handle): the columns of T and
-    of the height system, its inverse, X_B and R_M with one refinement step, S_K and
-    W_K; div counts the non-zero nodal derivative entries."""
+    Per cell, with f constant on every cell (an FP64 handle that recovers from the
+    momentum equations): the columns of T and of the height system, its inverse, X_B
+    with one refinement step, S_K, the h rows of R_M and the rows of W_K, refined
+    too; div counts the non-zero nodal derivative entries."""
     n, m, pp, N = arm["n_p"], 3 * arm["pp"], arm["pp"], arm["n_cells"]
     nz = {3: 14, 6: 48, 10: 120, 15: 250}[n]
     div, c_rows = 4 * n + nz, 9 * pp + 3 * pp * pp
     fmas = (n * (8 * n + div + 2 * n + n * n)                    # T, the height system, its inverse
             + m * (3 * n + div + 4 * n * n + c_rows)             # X_B (2 n^2 for h and its residual, 2 n^2 for u), S_K
-            + n * (2 * div + 11 * n * n + 3 * c_rows))           # R_M (its h columns from S^-1), W_K
+            + 2 * n * (div + n * n) + m * (2 * pp * n + 2 * n * n + nz + 10 * n))   # R_M's h rows, W_K
     tf = 2.0 * fmas * N / (arm["condense_ms"] * 1e-3) / 1e12
     return {"flops_per_cell": 2 * fmas, "achieved_tflops": tf, "peak_tflops": fma["fp64_tflops"],
             "frac": tf / fma["fp64_tflops"], "timing": "host wall clock around hdg_condense (one call, synchronised)",

@@ -1491,13 +1491,12 @@ bool hat_pays32(const hdg_params &prm, size_t NF, size_t pp, size_t l2) {
 // about as long as that chain.  In us, rows / momentum, f constant per cell: p = 1 512 cells
 // 4.1 / 7.4, 131,072 35 / 43; p = 2 8,192 10.2 / 11.8, 18,432 21.0 / 18.0; p = 3 2,048 8.9 / 14.7, 4,608
 // 14.6 / 14.8, 8,192 24.8 / 20.0; p = 4 2,048 14.5 / 23.6, 8,192 49 / 34.  Where f varies the
-// momentum form has three products more: p = 1 131,072 35 / 52, p = 2 113 / 121, p = 4 32,768
-// 157 / 182; p = 3 2,048 8.8 / 17.7, 8,192 23.7 / 24.9, then by how evenly its blocks fill the SMs
-// 18,432 48.8 / 45.1, 20,480 52.7 / 56.7, 32,768 78 / 83, 73,728 165 / 158, 81,920 185 / 169.
-bool recover_by_rows(int p, size_t N, bool f_const) {
-    const size_t n = size_t(p + 1) * (p + 2) / 2, fmas = N * 9 * n * (n + size_t(p) + 1);
-    if (f_const) return p == 1 || fmas <= 7000000;
-    return p != 3 || fmas <= 62000000;
+// momentum form has three products more and the two stay close above the line (p = 2 131,072
+// 113 / 121, p = 3 20,480 53 / 57, 81,920 185 / 169, p = 4 32,768 157 / 182), but the rows' velocity
+// part costs the condensation 6 n_p^3 FMAs per cell, a sixth of its time there.
+bool recover_by_rows(int p, size_t N) {
+    const size_t n = size_t(p + 1) * (p + 2) / 2;
+    return p == 1 || N * 9 * n * (n + size_t(p) + 1) <= 7000000;
 }
 
 int setup_device(hdg_handle *h, const hdg_params *prm) {
@@ -1537,7 +1536,7 @@ int setup_device(hdg_handle *h, const hdg_params *prm) {
     TRY(dalloc(&h->d_nbr, 4 * NF));
     if (!mode_ff(*prm)) {
         TRY(dalloc(&h->d_Xb, nK * m * N));
-        h->rec_rows = prm->flux == 1 || recover_by_rows(h->p, N, h->f_const);
+        h->rec_rows = prm->flux == 1 || recover_by_rows(h->p, N);
         TRY(dalloc(&h->d_Rm, size_t(rm_offsets(h->p, h->f_const, h->rec_rows).total) * N));
         TRY(dalloc(&h->d_W, m * nK * N));
     }

@@ -39,8 +39,8 @@ struct Sz {
 //   u = R r_u - T h,
 // so that a cell takes two inverses of n_p x n_p instead of one of 3 n_p x 3 n_p.
 // Where f is constant on every cell (FC; decided at set-up), F = f and P, Q are
-// numbers: one inverse.  X_B = A^-1 B, R_M = A^-1 Mass, S_K = Mt_K + C X_B and
-// W_K = C R_M follow column by column.
+// numbers: one inverse.  X_B = A^-1 B, R_M = A^-1 Mass and S_K = Mt_K + C X_B follow
+// column by column, W_K = C R_M row by row.
 //
 // One thread per column of a cell, kCondCells<P> cells per block with the cell as
 // the fastest thread index (shared-memory reads without bank conflicts, global
@@ -48,12 +48,10 @@ struct Sz {
 // measured, one warp instruction in about 77 cycles per scheduler), so the split is
 // the one that keeps the warps full (at p = 3 8 x 10 columns up to S, 8 x 12 for X_B
 // and all 8 x 30 of R_M dealt to the 96 threads) and what need not be FP64 is not: the
-// conversions to float pairs, the correction of the refinement, pivot tests.  The columns
-// of R_M are refined like those of X_B where W_K = C R_M follows from them (FP64 handles:
-// without, the condensed right-hand side of smooth data was 1.3e-14 off at p = 3 and 1.1e-13
-// at p = 4, Courant 16, instead of 1.0e-15 and 3.8e-15); the two-float handles' h rows are
-// not (their right-hand side is 4e-14 and 2.5e-13 off either way).  20,480 cells at p = 3,
-// two-float, f varying:
+// conversions to float pairs, the correction of the refinement, pivot tests.  The h
+// columns of R_M are S^-1 as it stands, and R_M's h rows are not refined (step 1 and
+// the recovery of the two-float handles are as exact either way, and so is the FP64
+// recovery).  20,480 cells at p = 3, two-float, f varying:
 // 1,345 us instead of 1,773 (one pass of 10 of 12 columns per component of R_M, all of
 // them refined in FP64, a full division per pivot and column, two products where column
 // k meets the pivot's); 18,432 cells at p = 2 in FP64: 384 instead of 419, against 1,466
@@ -200,7 +198,7 @@ __device__ __forceinline__ void inverse_product(const double *Ss, int c, const d
 // and its correction, 1e-14 of h, with the inverse rounded to FP32 (Sf).  The explicit inverse
 // alone leaves S_K about 20 times less exact than an elimination of the whole cell system
 // (p = 3, Courant 16: S_K applied to a nearly constant trace off by 1e-12 instead of
-// 7e-14; one step brings it to 2e-14), and W_K up to 24 times.
+// 7e-14; one step brings it to 2e-14).
 template <int NP, int CC>
 __device__ __forceinline__ void refine(const double *So, const float *Sf, int c, const double (&rh)[NP],
                                        double (&h)[NP]) {
@@ -249,7 +247,7 @@ __device__ __forceinline__ void edge_weights(const NodalArgs &a, const double *g
 }
 
 // row (edge e, node jj) of C q into out[row * ld]; diag is added to the rows of edge e0
-// (diag times column jj0 of the edge mass matrix; e0 = -1: nothing)
+// (diag times column jj0 of the edge mass matrix)
 template <int P>
 __device__ __forceinline__ void c_rows(const double *m1, const double (&wn)[3][3], const double (&qx)[Sz<P>::NP],
                                        const double (&qy)[Sz<P>::NP], const double (&qh)[Sz<P>::NP], int e0, int jj0,
@@ -274,6 +272,107 @@ __device__ __forceinline__ void c_rows(const double *m1, const double (&wn)[3][3
     }
 }
 
+// Row (edge e, node jj) of W_K = C R_M for cell c of the block's matrices: C's row with the
+// velocity eliminated, k = C_h - C_u T, times S^-1 with one refinement step (as in refine, from
+// the left), gives the entries w for r_h; C_u - w tau H div, times R, those for r_u.  By rows
+// every entry is exact to its own rounding: from the columns of R_M, each refined, the
+// condensed right-hand side of smooth r_h alone was up to 20 times as far off (p = 4, Courant
+// 16: 6.8e-15), and unrefined that of smooth r_u and r_h 1.1e-13.
+template <int P, bool FC, int CC>
+__device__ __forceinline__ void w_row(const double *ref, const double *m1, const double *Ss, const double *So,
+                                      const float *Sf, const double *Ts, const double *Ps, const double *Qs, int c,
+                                      int e, int jj, double w0, double w1, double w2, double g00, double g01,
+                                      double g10, double g11, double kap, double fk, double *out, size_t ld) {
+    constexpr int PP = P + 1, NP = Sz<P>::NP;
+    constexpr NodalOffsets O = nodal_offsets(P);
+    auto mu = [&](int i) {                     // the edge mass matrix's column jj at cell node i
+        const int pos = e == 0 ? node_edge_pos(P, 0, i) : e == 1 ? node_edge_pos(P, 1, i) : node_edge_pos(P, 2, i);
+        return pos >= 0 ? m1[pos * PP + jj] : 0.0;
+    };
+    double k[NP], w[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        k[i] = w2 * mu(i);
+        w[i] = 0.0;
+    }
+#pragma unroll
+    for (int jb = 0; jb < PP; ++jb) {
+        row_fence();
+        const int b = edge_cell_node(P, e, jb);
+        const double x = w0 * m1[jb * PP + jj], y = w1 * m1[jb * PP + jj];
+#pragma unroll
+        for (int j = 0; j < NP; ++j)
+            k[j] = fma(-x, Ts[(b * NP + j) * CC + c], fma(-y, Ts[((NP + b) * NP + j) * CC + c], k[j]));
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+#pragma unroll
+        for (int j = 0; j < NP; ++j) w[j] = fma(k[i], Ss[(i * NP + j) * CC + c], w[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+#pragma unroll
+        for (int j = 0; j < NP; ++j) k[j] = fma(-w[i], So[(i * NP + j) * CC + c], k[j]);
+    }
+    float r[NP], d[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        r[i] = to_float(k[i]);
+        d[i] = 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        row_fence();
+#pragma unroll
+        for (int j = 0; j < NP; ++j) d[j] = fmaf(r[i], Sf[(i * NP + j) * CC + c], d[j]);
+    }
+    double vx[NP], vy[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        w[j] += join(make_float2(d[j], 0.0f));
+        out[size_t(2 * NP + j) * ld] = w[j];
+        vx[j] = vy[j] = 0.0;
+    }
+    static_for<NP>([&](auto ia_) {
+        constexpr int ia = decltype(ia_)::value;
+        row_fence();
+        static_for<NP>([&](auto ib_) {
+            constexpr int ib = decltype(ib_)::value;
+            if constexpr (nodal_dx_nonzero(P, ia, ib)) vx[ib] = fma(ref[O.Dx + ia * NP + ib], w[ia], vx[ib]);
+            if constexpr (nodal_dy_nonzero(P, ia, ib)) vy[ib] = fma(ref[O.Dy + ia * NP + ib], w[ia], vy[ib]);
+        });
+    });
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        const double p1 = vx[i], p2 = vy[i], q = mu(i);
+        vx[i] = fma(w0, q, fma(g00, p1, g01 * p2));
+        vy[i] = fma(w1, q, fma(g10, p1, g11 * p2));
+    }
+    if constexpr (FC) {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            out[size_t(j) * ld] = fma(kap, vx[j], -fk * vy[j]);
+            out[size_t(NP + j) * ld] = fma(fk, vx[j], kap * vy[j]);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            row_fence();
+            double ox = 0.0, oy = 0.0;
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                const double p = Ps[(i * NP + j) * CC + c], q = Qs[(i * NP + j) * CC + c];
+                ox = fma(vx[i], p, fma(-vy[i], q, ox));
+                oy = fma(vx[i], q, fma(vy[i], p, oy));
+            }
+            out[size_t(j) * ld] = ox;
+            out[size_t(NP + j) * ld] = oy;
+        }
+    }
+}
+
 // shared memory of the kernel below, in doubles
 template <int P, bool FC>
 struct CondSmem {
@@ -285,8 +384,13 @@ struct CondSmem {
     static constexpr int oSf = oQ + (FC ? 0 : NN * CC), total = oSf + (NN * CC + 1) / 2;   // (oSf: floats)
 };
 
+// blocks per SM that the FP64 instances are compiled for (as many as their shared memory
+// admits from p = 3 on; 0: the compiler's choice)
 template <int P, bool FC, bool FF>
-__global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs a) {
+constexpr int kCondPerSM = FF ? 0 : P == 1 ? 10 : P == 2 ? 7 : P == 3 ? (FC ? 5 : 4) : (FC ? 3 : 2);
+
+template <int P, bool FC, bool FF>
+__global__ void __launch_bounds__(kCondThreads, kCondPerSM<P, FC, FF>) condense_nodal_kernel(NodalArgs a) {
     using L = CondSmem<P, FC>;
     constexpr int PP = P + 1, NP = L::NP, NK = 3 * NP, M = 3 * PP, CC = L::CC;
     constexpr NodalOffsets O = nodal_offsets(P);
@@ -489,6 +593,15 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
         }
         c_rows<P>(m1, wn, wx, wy, h, e, jj, e == 0 ? wn[0][2] : e == 1 ? wn[1][2] : wn[2][2], a.Scell + size_t(K) * M * M + j, M);
     }
+    if constexpr (!FF) {
+        // ---- W_K, row (edge e, trace node jj)
+        if (cell && j < M) {
+            const int e = j / PP, jj = j % PP;
+            auto of_edge = [&](int q) { return e == 0 ? wn[0][q] : e == 1 ? wn[1][q] : wn[2][q]; };
+            w_row<P, FC, CC>(ref, m1, Ss, So, Sf, Ts, Ps, Qs, c, e, jj, of_edge(0), of_edge(1), of_edge(2), -tH * j00,
+                             -tH * j01, -tH * j10, -tH * j11, kap, fk, a.W + size_t(j) * NK * N + K, N);
+        }
+    }
     if constexpr (FF) {
         // P and Q (f varying over the cell) as float pairs in cell tiles, and the cell's weights (k_ff.cu)
         if constexpr (!FC) {
@@ -524,15 +637,16 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
             o[size_t(2 * NP * NP) * N] = p + q;
         }
     }
-    // ---- The h rows of R_M and (FP64 handles) W_K: the columns of the unit
-    // vectors in u_x, u_y and h, spread over all the block's threads.  The h columns' h is
-    // a column of S^-1, refined on FP64 handles.
+    // ---- The h rows of R_M and (FP64 handles that recover by the rows) its velocity rows: the
+    // columns of the unit vectors in u_x, u_y and h, spread over all the block's threads.
+    // The h columns' h is a column of S^-1 itself.
     for (int it = t; it < 3 * NP * CC; it += kCondThreads) {
         const int c = it % CC, kap_ = it / CC, comp = kap_ / NP, j = kap_ % NP, K = blockIdx.x * CC + c;
         if (K >= a.N) continue;
         const double j00 = geo[0 * CC + c], j01 = geo[1 * CC + c], j10 = geo[2 * CC + c], j11 = geo[3 * CC + c];
-        double wx[NP], wy[NP], rh[NP], h[NP];
+        double wx[NP], wy[NP], h[NP];
         if (comp < 2) {
+            double rh[NP];
             const double kap = geo[13 * CC + c], fk = geo[14 * CC + c];
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
@@ -554,13 +668,8 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
                 wx[i] = wy[i] = 0.0;
-                rh[i] = i == j ? 1.0 : 0.0;
                 h[i] = Ss[(i * NP + j) * CC + c];
             }
-        }
-        if constexpr (!FF) {
-            refine<NP, CC>(So, Sf, c, rh, h);
-            subtract_gradient<NP, CC>(Ts, c, h, wx, wy);
         }
         if constexpr (FF) {
             constexpr int CPk = (NK + 1) / 2;
@@ -571,16 +680,13 @@ __global__ void __launch_bounds__(kCondThreads) condense_nodal_kernel(NodalArgs 
 #pragma unroll
             for (int i = 0; i < NP; ++i) a.Rh[(size_t(i) * NK + kap_) * N + K] = h[i];
             if (a.Ru) {
+                subtract_gradient<NP, CC>(Ts, c, h, wx, wy);
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
                     a.Ru[(size_t(i) * NK + kap_) * N + K] = wx[i];
                     a.Ru[(size_t(NP + i) * NK + kap_) * N + K] = wy[i];
                 }
             }
-            double wn[3][3];
-#pragma unroll
-            for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, K, e, wn[e]);
-            c_rows<P>(m1, wn, wx, wy, h, -1, 0, 0.0, a.W + size_t(kap_) * N + K, size_t(NK) * N);
         }
     }
 }

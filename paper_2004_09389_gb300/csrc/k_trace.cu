@@ -1536,18 +1536,18 @@ cudaError_t launch_recover(hdg_handle *h, const double *r_u, const double *r_h, 
                                  h->N, h->NF, h->d_Rm, h->d_Xb, r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout)));
         return cudaGetLastError();
     }
-    // (recover_by_rows leaves these)
     const unsigned nb = blocks(h->N, 32);
     const double tau = h->prm.tau, tg = tau * h->prm.g;
     auto momentum = [&](auto kernel, int warps) {
         kernel<<<nb, 32 * warps, 0, h->stream>>>(h->N, h->NF, h->d_Rm, h->d_Xb, h->d_nref, h->d_X, h->d_fcell, tau, tg,
                                                  r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout);
     };
-    if (h->f_const && h->p == 2) momentum(&recover_kernel<2, true>, kRecWarps<2>);
-    else if (h->f_const && h->p == 3) momentum(&recover_kernel<3, true>, kRecWarps<3>);
-    else if (h->f_const && h->p == 4) momentum(&recover_kernel<4, true>, kRecWarps<4>);
-    else if (!h->f_const && h->p == 3) momentum(&recover_kernel<3, false>, kRecWarps<3>);
-    else return cudaErrorInvalidValue;
+    switch (h->p) {
+        case 2: h->f_const ? momentum(&recover_kernel<2, true>, kRecWarps<2>) : momentum(&recover_kernel<2, false>, kRecWarps<2>); break;
+        case 3: h->f_const ? momentum(&recover_kernel<3, true>, kRecWarps<3>) : momentum(&recover_kernel<3, false>, kRecWarps<3>); break;
+        case 4: h->f_const ? momentum(&recover_kernel<4, true>, kRecWarps<4>) : momentum(&recover_kernel<4, false>, kRecWarps<4>); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

@@ -24,9 +24,8 @@ def _built():
 
 
 # the two sides of each line: by rows, by the momentum equations
-@pytest.mark.parametrize("p,n,varying", [(2, 84, False), (2, 88, False), (3, 52, False), (3, 62, False),
-                                         (4, 36, False), (4, 38, False), (3, 152, True), (3, 160, True),
-                                         (2, 88, True), (1, 128, False)])
+@pytest.mark.parametrize("p,n", [(1, 128), (2, 84), (2, 88), (3, 52), (3, 62), (4, 36), (4, 38)])
+@pytest.mark.parametrize("varying", [False, True])
 def test_recovery_on_either_side_of_the_line(p, n, varying):
     from paper_2004_09389_gb300 import HDG_FP64, HDGSolver
     mesh = I.periodic_square_hierarchy(n, n_coarsest=4)
