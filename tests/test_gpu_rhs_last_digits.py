@@ -46,3 +46,26 @@ def test_condensed_rhs_is_exact_to_rounding(p, varying):
         s.close()
         d = gd.cpu().numpy().ravel() - exact
         assert np.sqrt((d * d).sum()) <= 3 * prob.np * 2.0 ** -52 * np.sqrt((exact * exact).sum())
+
+
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_condensed_rhs_of_r_h_alone(p):
+    """r_u = 0, f = 0: sums of n_p products of entries that are exact to their own rounding,
+    (n_p + 2) 2^-53 relative (each product and addition rounds once, an entry twice)."""
+    import extended
+    from paper_2004_09389_gb300 import HDG_FP64, HDGSolver
+    mesh = I.periodic_square_hierarchy(11, n_coarsest=4)
+    f, g, H = np.zeros(mesh.n_vertices), 1.3, 0.7
+    tau = 16 * mesh.h / np.sqrt(g * H)
+    prob = HDGProblem(mesh, p, tau=tau, g=g, H=H, f_vertex=f)
+    x, y = np.moveaxis(I.dg_node_positions(mesh, p), -1, 0) * 2.0 * np.pi
+    rh = 0.2 + np.cos(2 * x - y) + 0.5 * np.sin(x + 0.4)
+    ru = np.zeros((mesh.n_cells, 2, prob.np))
+    exact = extended.condensed_rhs(prob, ru, rh)
+    s = HDGSolver(mesh, p, tau, g, H, f_vertex=f, precision=HDG_FP64)
+    gd = torch.empty(prob.n_facets, p + 1, dtype=torch.float64, device="cuda")
+    s.condensed_rhs_dev(torch.from_numpy(ru).cuda(), torch.from_numpy(rh).cuda(), gd)
+    torch.cuda.synchronize()
+    s.close()
+    d = gd.cpu().numpy().ravel() - exact
+    assert np.sqrt((d * d).sum()) <= (prob.np + 2) * 2.0 ** -53 * np.sqrt((exact * exact).sum())
