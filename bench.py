@@ -489,8 +489,8 @@ def step13_bytes(arm: dict):
     if arm.get("keep_z"):
         mats = n * nK + (0 if arm.get("f_const", True) else 2 * n * n)
         return 8.0 * N * (mats + 2 * nK + m + 15), 8.0 * N * (nK * m + 2 * nK + m)
-    const, p, fmas = arm.get("f_const", True), arm["pp"] - 1, N * nK * (nK + m)
-    if p == 1 or fmas <= 7_000_000:
+    const = arm.get("f_const", True)
+    if arm["pp"] == 2 or 8 * N * nK * nK <= 8 << 20:
         step3 = nK * (nK + m)
     else:
         step3 = n * (nK + m) + (0 if const else 3 * n * n)
