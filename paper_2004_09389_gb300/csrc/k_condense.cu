@@ -51,11 +51,12 @@ struct Sz {
 // conversions to float pairs, the correction of the refinement, pivot tests.  The h
 // columns of R_M are S^-1 as it stands, and R_M's h rows are not refined (step 1 and
 // the recovery of the two-float handles are as exact either way, and so is the FP64
-// recovery).  20,480 cells at p = 3, two-float, f varying:
-// 1,345 us instead of 1,773 (one pass of 10 of 12 columns per component of R_M, all of
-// them refined in FP64, a full division per pivot and column, two products where column
-// k meets the pivot's); 18,432 cells at p = 2 in FP64: 384 instead of 419, against 1,466
-// by elimination of the whole augmented cell system [A | B | Mass], one cell per block.
+// recovery).  20,480 cells at p = 3, two-float, f varying: 1,345 us instead of 1,773 (one pass
+// of 10 of 12 columns per component of R_M, all of them refined in FP64, a full division
+// per pivot and column, two products where column k meets the pivot's).  FP64, 32,768 cells at
+// p = 2, 3, 4: 518, 1,561 and 4,194 us (f varying 700, 2,324, 6,458), with W_K from the columns of
+// R_M 559, 1,708 and 4,752 (712, 2,385, 6,763), by elimination of the whole augmented cell
+// system [A | B | Mass], one cell per block, 2,587, 6,629 and 16,949.
 template <int P> constexpr int kCondCells = P == 1 ? 16 : P == 2 ? 10 : P == 3 ? 8 : 6;
 constexpr int kCondThreads = 96;
 
@@ -274,22 +275,23 @@ __device__ __forceinline__ void c_rows(const double *m1, const double (&wn)[3][3
 
 // Row (edge e, node jj) of W_K = C R_M for cell c of the block's matrices: C's row with the
 // velocity eliminated, k = C_h - C_u T, times S^-1 with one refinement step (as in refine, from
-// the left), gives the entries w for r_h; C_u - w tau H div, times R, those for r_u.  By rows
+// the left), gives the entries w for r_h; (C_u - w tau H div) R is those for r_u, formed here where
+// R is two numbers (FC), else column by column from w (w_column).  By rows
 // every entry is exact to its own rounding: from the columns of R_M, each refined, the
 // condensed right-hand side of smooth r_h alone was up to 20 times as far off (p = 4, Courant
 // 16: 6.8e-15), and unrefined that of smooth r_u and r_h 1.1e-13.
 template <int P, bool FC, int CC>
 __device__ __forceinline__ void w_row(const double *ref, const double *m1, const double *Ss, const double *So,
-                                      const float *Sf, const double *Ts, const double *Ps, const double *Qs, int c,
-                                      int e, int jj, double w0, double w1, double w2, double g00, double g01,
-                                      double g10, double g11, double kap, double fk, double *out, size_t ld) {
+                                      const float *Sf, const double *Ts, int c, int e, int jj, double w0, double w1,
+                                      double w2, double g00, double g01, double g10, double g11, double kap, double fk,
+                                      double *out, size_t ld, double (&w)[Sz<P>::NP]) {
     constexpr int PP = P + 1, NP = Sz<P>::NP;
     constexpr NodalOffsets O = nodal_offsets(P);
     auto mu = [&](int i) {                     // the edge mass matrix's column jj at cell node i
         const int pos = e == 0 ? node_edge_pos(P, 0, i) : e == 1 ? node_edge_pos(P, 1, i) : node_edge_pos(P, 2, i);
         return pos >= 0 ? m1[pos * PP + jj] : 0.0;
     };
-    double k[NP], w[NP];
+    double k[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
         k[i] = w2 * mu(i);
@@ -328,47 +330,57 @@ __device__ __forceinline__ void w_row(const double *ref, const double *m1, const
 #pragma unroll
         for (int j = 0; j < NP; ++j) d[j] = fmaf(r[i], Sf[(i * NP + j) * CC + c], d[j]);
     }
-    double vx[NP], vy[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
         w[j] += join(make_float2(d[j], 0.0f));
         out[size_t(2 * NP + j) * ld] = w[j];
-        vx[j] = vy[j] = 0.0;
-    }
-    static_for<NP>([&](auto ia_) {
-        constexpr int ia = decltype(ia_)::value;
-        row_fence();
-        static_for<NP>([&](auto ib_) {
-            constexpr int ib = decltype(ib_)::value;
-            if constexpr (nodal_dx_nonzero(P, ia, ib)) vx[ib] = fma(ref[O.Dx + ia * NP + ib], w[ia], vx[ib]);
-            if constexpr (nodal_dy_nonzero(P, ia, ib)) vy[ib] = fma(ref[O.Dy + ia * NP + ib], w[ia], vy[ib]);
-        });
-    });
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        const double p1 = vx[i], p2 = vy[i], q = mu(i);
-        vx[i] = fma(w0, q, fma(g00, p1, g01 * p2));
-        vy[i] = fma(w1, q, fma(g10, p1, g11 * p2));
     }
     if constexpr (FC) {
+        double vx[NP], vy[NP];
 #pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            out[size_t(j) * ld] = fma(kap, vx[j], -fk * vy[j]);
-            out[size_t(NP + j) * ld] = fma(fk, vx[j], kap * vy[j]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
+        for (int j = 0; j < NP; ++j) vx[j] = vy[j] = 0.0;
+        static_for<NP>([&](auto ia_) {
+            constexpr int ia = decltype(ia_)::value;
             row_fence();
-            double ox = 0.0, oy = 0.0;
+            static_for<NP>([&](auto ib_) {
+                constexpr int ib = decltype(ib_)::value;
+                if constexpr (nodal_dx_nonzero(P, ia, ib)) vx[ib] = fma(ref[O.Dx + ia * NP + ib], w[ia], vx[ib]);
+                if constexpr (nodal_dy_nonzero(P, ia, ib)) vy[ib] = fma(ref[O.Dy + ia * NP + ib], w[ia], vy[ib]);
+            });
+        });
 #pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                const double p = Ps[(i * NP + j) * CC + c], q = Qs[(i * NP + j) * CC + c];
-                ox = fma(vx[i], p, fma(-vy[i], q, ox));
-                oy = fma(vx[i], q, fma(vy[i], p, oy));
-            }
-            out[size_t(j) * ld] = ox;
-            out[size_t(NP + j) * ld] = oy;
+        for (int j = 0; j < NP; ++j) {
+            const double q = mu(j), x = fma(w0, q, fma(g00, vx[j], g01 * vy[j])), y = fma(w1, q, fma(g10, vx[j], g11 * vy[j]));
+            out[size_t(j) * ld] = fma(kap, x, -fk * y);
+            out[size_t(NP + j) * ld] = fma(fk, x, kap * y);
+        }
+    }
+}
+
+// Column of W_K for a unit vector in r_u: C_u (wx, wy) + w rh with (wx, wy) its velocity R e and rh =
+// -tau H div R e, the rows w of the cell from shared memory ([M][NP][CC])
+template <int P, int CC>
+__device__ __forceinline__ void w_column(const double *m1, const double *ws, int c, const double (&wn)[3][3],
+                                         const double (&wx)[Sz<P>::NP], const double (&wy)[Sz<P>::NP],
+                                         const double (&rh)[Sz<P>::NP], double *out, size_t ld) {
+    constexpr int PP = P + 1, NP = Sz<P>::NP;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        row_fence();
+        double fl[PP];
+#pragma unroll
+        for (int jb = 0; jb < PP; ++jb) {
+            const int b = edge_cell_node(P, e, jb);
+            fl[jb] = fma(wn[e][0], wx[b], wn[e][1] * wy[b]);
+        }
+#pragma unroll
+        for (int jj = 0; jj < PP; ++jj) {
+            double v = 0.0;
+#pragma unroll
+            for (int jb = 0; jb < PP; ++jb) v = fma(m1[jb * PP + jj], fl[jb], v);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) v = fma(ws[((e * PP + jj) * NP + i) * CC + c], rh[i], v);
+            out[size_t(e * PP + jj) * ld] = v;
         }
     }
 }
@@ -379,9 +391,11 @@ struct CondSmem {
     static constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NN = NP * NP, CC = kCondCells<P>;
     static constexpr int oRef = 0, oM1 = nodal_offsets(P).total, oGeo = oM1 + PP * PP;
     static constexpr int nGeo = 4 + 9 + 2 + 3;                     // j, edge weights, R (FC), f
-    static constexpr int oS = oGeo + nGeo * CC, oT = oS + NN * CC, oSo = oT + 2 * NN * CC, oP = oSo + NN * CC;
-    static constexpr int oQ = oP + (FC ? 0 : NN * CC);
-    static constexpr int oSf = oQ + (FC ? 0 : NN * CC), total = oSf + (NN * CC + 1) / 2;   // (oSf: floats)
+    static constexpr int oS = oGeo + nGeo * CC, oT = oS + NN * CC, oSo = oT + 2 * NN * CC;
+    static constexpr int oSf = oSo + NN * CC, nSf = (NN * CC + 1) / 2;                     // (oSf: floats)
+    // the rows w of W_K take the place of So and Sf (which they outgrow at p = 1)
+    static constexpr int nW = FC ? 0 : 3 * PP * NP * CC, oP = oSo + (nW > NN * CC + nSf ? nW : NN * CC + nSf);
+    static constexpr int oQ = oP + (FC ? 0 : NN * CC), total = oQ + (FC ? 0 : NN * CC);
 };
 
 // blocks per SM that the FP64 instances are compiled for (as many as their shared memory
@@ -595,11 +609,20 @@ __global__ void __launch_bounds__(kCondThreads, kCondPerSM<P, FC, FF>) condense_
     }
     if constexpr (!FF) {
         // ---- W_K, row (edge e, trace node jj)
+        double wr[NP];
         if (cell && j < M) {
             const int e = j / PP, jj = j % PP;
             auto of_edge = [&](int q) { return e == 0 ? wn[0][q] : e == 1 ? wn[1][q] : wn[2][q]; };
-            w_row<P, FC, CC>(ref, m1, Ss, So, Sf, Ts, Ps, Qs, c, e, jj, of_edge(0), of_edge(1), of_edge(2), -tH * j00,
-                             -tH * j01, -tH * j10, -tH * j11, kap, fk, a.W + size_t(j) * NK * N + K, N);
+            w_row<P, FC, CC>(ref, m1, Ss, So, Sf, Ts, c, e, jj, of_edge(0), of_edge(1), of_edge(2), -tH * j00,
+                             -tH * j01, -tH * j10, -tH * j11, kap, fk, a.W + size_t(j) * NK * N + K, N, wr);
+        }
+        if constexpr (!FC) {
+            __syncthreads();                   // So and Sf have been read
+            if (cell && j < M) {
+#pragma unroll
+                for (int i = 0; i < NP; ++i) So[(j * NP + i) * CC + c] = wr[i];
+            }
+            __syncthreads();
         }
     }
     if constexpr (FF) {
@@ -639,7 +662,7 @@ __global__ void __launch_bounds__(kCondThreads, kCondPerSM<P, FC, FF>) condense_
     }
     // ---- The h rows of R_M and (FP64 handles that recover by the rows) its velocity rows: the
     // columns of the unit vectors in u_x, u_y and h, spread over all the block's threads.
-    // The h columns' h is a column of S^-1 itself.
+    // The h columns' h is a column of S^-1 itself.  Where f varies, W_K's entries for r_u too.
     for (int it = t; it < 3 * NP * CC; it += kCondThreads) {
         const int c = it % CC, kap_ = it / CC, comp = kap_ / NP, j = kap_ % NP, K = blockIdx.x * CC + c;
         if (K >= a.N) continue;
@@ -663,6 +686,12 @@ __global__ void __launch_bounds__(kCondThreads, kCondPerSM<P, FC, FF>) condense_
                 rh[i] = 0.0;
             }
             add_div<P>(ref, -tH * j00, -tH * j01, -tH * j10, -tH * j11, wx, wy, rh);
+            if constexpr (!FF && !FC) {
+                double wn[3][3];
+#pragma unroll
+                for (int e = 0; e < 3; ++e) edge_weights(a, geo, CC, c, K, e, wn[e]);
+                w_column<P, CC>(m1, So, c, wn, wx, wy, rh, a.W + size_t(kap_) * N + K, size_t(NK) * N);
+            }
             inverse_product<NP, CC>(Ss, c, rh, h);
         } else {
 #pragma unroll
