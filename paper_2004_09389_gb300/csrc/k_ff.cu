@@ -630,9 +630,9 @@ __device__ __forceinline__ void stage_tab(float4 *tab, const float4 *src) {
 // Step 1: z_K = A_K^-1 M_K r_K by the cell solve, stored as normalised pairs (z2
 // [NK][N], when given) for step 3, and the cell rows ycell = C_K z_K: on edge i the
 // flux H t_y u_x - H t_x u_y + tau_s |e| h at its p + 1 cell nodes, times the edge mass
-// matrix.  Bound by HBM and FP32 issue together: 98 us on 131,072 cells at p = 3 with f
-// constant per cell (430 MB, 4.4 TB/s), 118 us on 327,680 at p = 2 with f varying,
-// against 188 and 178 us with the rows of the stored A_K^-1 M_K (1,029 MB, HBM-bound).
+// matrix.  Bound by HBM and FP32 issue together: 90 us on 131,072 cells at p = 3 with f
+// constant per cell (430 MB, 4.8 TB/s), 123 us on 327,680 at p = 2 with f varying,
+// against 186 and 176 us with the rows of the stored A_K^-1 M_K (1,029 MB, HBM-bound).
 template <int P, bool FC>
 __device__ __forceinline__ void rhs_cell_z_kernel_impl(int bid_, int nb_, int N, const SolveMat &m,
                                                        const double *__restrict__ r_u,

@@ -1212,11 +1212,11 @@ __global__ void __launch_bounds__(32 * kRecWarps<P>) recover_kernel(int N, int N
 // P1 restriction rho = pi^T: r_c[v] = sum over facet ends at v of the nodal
 // weights of the linear interpolant (1 - t_r at the lower vertex, t_r at the higher).
 // Latency bounds it (list, facet id, p + 1 values, one after the other), so in FP32 eight
-// lanes (L) share a vertex's facet ends where that still is about one wave of threads: 5.4
-// instead of 6.5 us for 40,962 vertices at p = 3, 3.4 instead of 3.7 for 20,736 at p = 2, but
-// 6.5 instead of 5.3 for 65,536 and 12.0 instead of 7.8 for 163,842 (kRestrictShared).  In
-// FP64, where the lanes' additions would take the pipe longer than the loads, and on the
-// larger meshes one thread takes them all.
+// lanes (L) share a vertex's facet ends up to kRestrictShared vertices (1.3 times the threads
+// that 152 SMs hold; a line between the measured 40,962 and 65,536): 5.4 instead of 6.5 us for
+// 40,962 vertices at p = 3, 3.4 instead of 3.7 for 20,736 at p = 2, but 6.5 instead of 5.3 for
+// 65,536 and 12.0 instead of 7.8 for 163,842.  In FP64, where the lanes' additions would take
+// the pipe longer than the loads, and on the larger meshes one thread takes them all.
 constexpr int kRestrictShared = 49152;
 template <int P, typename T, int L>
 __device__ __forceinline__ void restrict_kernel_impl(int bid_, int nb_, int nv, int NF,
