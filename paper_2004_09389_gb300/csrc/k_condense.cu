@@ -398,10 +398,11 @@ struct CondSmem {
     static constexpr int oQ = oP + (FC ? 0 : NN * CC), total = oQ + (FC ? 0 : NN * CC);
 };
 
-// blocks per SM that the FP64 instances are compiled for (as many as their shared memory
-// admits from p = 3 on; 0: the compiler's choice)
+// blocks per SM that the kernel is compiled for (as many as the shared memory admits from p = 3
+// on; 0: the compiler's choice, which suits the two-float instances but the one at p = 3 with f
+// varying: 1,377 instead of 1,398 us on 20,480 cells, by how the last of its blocks fall)
 template <int P, bool FC, bool FF>
-constexpr int kCondPerSM = FF ? 0 : P == 1 ? 10 : P == 2 ? 7 : P == 3 ? (FC ? 5 : 4) : (FC ? 3 : 2);
+constexpr int kCondPerSM = FF ? (P == 3 && !FC ? 4 : 0) : P == 1 ? 10 : P == 2 ? 7 : P == 3 ? (FC ? 5 : 4) : (FC ? 3 : 2);
 
 template <int P, bool FC, bool FF>
 __global__ void __launch_bounds__(kCondThreads, kCondPerSM<P, FC, FF>) condense_nodal_kernel(NodalArgs a) {
