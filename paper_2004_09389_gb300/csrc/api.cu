@@ -1488,12 +1488,12 @@ bool hat_pays32(const hdg_params &prm, size_t NF, size_t pp, size_t l2) {
 // The recovery of FP64 handles by the rows of R_M and X_B (n_K (n_K + m) FMAs per cell, one
 // dependent sum per thread) or by the h rows and the momentum equations (0.7 to 0.9 of the
 // FMAs from p = 2 on, but a chain of five barriers).  In us, rows / momentum, f constant per cell
-// (f varying): p = 1 512 cells 4.1 / 7.4, 131,072 35 / 43 (35 / 52); p = 2 512 5.2 / 8.8, 8,192 10.2 / 11.8,
-// 18,432 21.0 / 18.0; p = 3 512 7.4 / 14.6 (7.4 / 17.6), 4,608 14.6 / 14.8, 8,192 24.8 / 20.0 (23.7 / 24.9); p = 4
-// 512 9.1 / 23.5, 4,608 32 / 24, 32,768 157 / 102 (157 / 182).  But the rows take three times R_M's
-// bytes, which displace the solve's operators from L2 between steps (p = 4, 1,152 cells, 19 MB
-// of R_M, three handles in turn: 1,010 us per step instead of 972), and 6 n_p^3 FMAs per cell of
-// the condensation, a sixth of its time on large meshes where f varies: so up to 8 MB.
+// (f varying): p = 1 512 cells 4.2 / 7.4 (7.8), 131,072 35 / 43 (52); p = 2 512 5.3 / 8.8 (10.2), 3,200
+// 7.4 / 9.1; p = 3 512 6.1 / 14.6 (17.6), 1,152 6.4 / 14.7; p = 4 512 9.8 / 23.5 (29.2).  On one handle the
+// rows win up to about 14,000, 5,000 and 2,600 cells, but they take three times R_M's bytes, which
+// displace the solve's operators from L2 between steps (p = 4, 1,152 cells, 19 MB of R_M, three
+// handles in turn: 1,010 us per step instead of 972), and 6 n_p^3 FMAs per cell of the condensation,
+// a sixth of its time on large meshes where f varies: so up to 8 MB.
 bool recover_by_rows(int p, size_t N) {
     const size_t n = size_t(p + 1) * (p + 2) / 2;
     return p == 1 || N * 9 * n * n * sizeof(double) <= size_t(8) << 20;

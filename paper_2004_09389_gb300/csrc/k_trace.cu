@@ -1033,29 +1033,42 @@ void rhs_gather_kernel_go(unsigned grid_, unsigned block_, size_t smem_, cudaStr
 }
 
 
-// Step 3, q_K = R_M r_K - X_B lambda_K, by the rows of both, one thread per row and cell
-// (recover_by_rows in api.cu: small meshes)
+// Step 3, q_K = R_M r_K - X_B lambda_K, by the rows of both (recover_by_rows in api.cu), one
+// thread per row and cell.  A block takes whole cells and stages their r and lambda before it writes,
+// so that u and h_out may be r_u and r_h, as in the kernels below.  Latency bounds it on small
+// meshes: a thread issues the loads of its row of R_M first (512 cells with a cold cache, p = 1 .. 4:
+// 5.6, 6.8, 8.2 and 11.4 us, instead of 6.8, 9.0, 13.8 and 18.2 with r and lambda read by every
+// thread).  At p = 1, which takes it at every size, the FP64 pipe does, and seven blocks per SM
+// instead of early loads: 34.6 us on 131,072 cells, 43.0 with them.
+template <int P> constexpr int kRowCells = P == 1 ? 32 : P == 2 ? 16 : 8;
 template <int P>
-__global__ void recover_rows_kernel(int N, int NF, const double *__restrict__ Rm, const double *__restrict__ Xb,
-                                    const double *__restrict__ r_u, const double *__restrict__ r_h,
-                                    const double *__restrict__ lam, const int32_t *__restrict__ facet_of,
-                                    const int32_t *__restrict__ flip, double *__restrict__ u,
-                                    double *__restrict__ hout) {
-    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP;
-    const size_t idx = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (idx >= size_t(N) * NK) return;
-    const int rho = int(idx / N), K = int(idx % N);
-    double acc = 0.0;
-#pragma unroll 5
-    for (int kap = 0; kap < NK; ++kap)
-        acc = fma(__ldg(Rm + size_t(rho * NK + kap) * N + K), cell_rhs<NP>(r_u, r_h, K, kap), acc);
+__global__ void __launch_bounds__(kRowCells<P> * 3 * (P + 1) * (P + 2) / 2, P == 1 ? 7 : 1)
+    recover_rows_kernel(int N, int NF, const double *__restrict__ Rm, const double *__restrict__ Xb, const double *r_u,
+                        const double *r_h, const double *__restrict__ lam, const int32_t *__restrict__ facet_of,
+                        const int32_t *__restrict__ flip, double *u, double *hout) {
+    constexpr int PP = P + 1, NP = (P + 1) * (P + 2) / 2, NK = 3 * NP, M = 3 * PP, CC = kRowCells<P>, NT = CC * NK;
+    __shared__ double sR[NK][CC + 1], sL[M][CC + 1];
+    const int t = threadIdx.x, c = t % CC, rho = t / CC, K0 = blockIdx.x * CC, K = K0 + c, nc = min(CC, N - K0);
+    const double *rm = Rm + size_t(rho) * NK * N + K, *xb = Xb + size_t(rho) * M * N + K;
+    double a[NK];
+    if (P > 1 && K < N) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const int f = facet_of[3 * K + i], fl = flip[3 * K + i];
-#pragma unroll
-        for (int j = 0; j < PP; ++j)
-            acc = fma(-__ldg(Xb + size_t(rho * M + i * PP + j) * N + K), lam[size_t(fl ? P - j : j) * NF + f], acc);
+        for (int kap = 0; kap < NK; ++kap) a[kap] = __ldg(rm + size_t(kap) * N);
     }
+    for (int j = t; j < nc * 2 * NP; j += NT) sR[j % (2 * NP)][j / (2 * NP)] = r_u[size_t(K0) * 2 * NP + j];
+    for (int j = t; j < nc * NP; j += NT) sR[2 * NP + j % NP][j / NP] = r_h[size_t(K0) * NP + j];
+    for (int j = t; j < nc * M; j += NT) {
+        const int cell = j / M, q = j % M, i = q / PP, jj = q % PP;
+        const int f = facet_of[3 * (K0 + cell) + i], fl = flip[3 * (K0 + cell) + i];
+        sL[q][cell] = lam[size_t(fl ? P - jj : jj) * NF + f];
+    }
+    __syncthreads();
+    if (K >= N) return;
+    double acc = 0.0;
+#pragma unroll
+    for (int kap = 0; kap < NK; ++kap) acc = fma(P > 1 ? a[kap] : __ldg(rm + size_t(kap) * N), sR[kap][c], acc);
+#pragma unroll
+    for (int q = 0; q < M; ++q) acc = fma(-__ldg(xb + size_t(q) * N), sL[q][c], acc);
     if (rho < 2 * NP) u[size_t(K) * 2 * NP + rho] = acc;
     else hout[size_t(K) * NP + rho - 2 * NP] = acc;
 }
@@ -1532,7 +1545,7 @@ cudaError_t launch_recover(hdg_handle *h, const double *r_u, const double *r_h, 
                            double *hout) {
     if (h->prm.flux == 1) return launch_recover_lf(h, r_u, r_h, lam, u, hout);
     if (h->rec_rows) {
-        HDG_DISPATCH_P(h->p, (recover_rows_kernel<P><<<blocks(size_t(h->N) * h->nK, 256), 256, 0, h->stream>>>(
+        HDG_DISPATCH_P(h->p, (recover_rows_kernel<P><<<blocks(h->N, kRowCells<P>), kRowCells<P> * h->nK, 0, h->stream>>>(
                                  h->N, h->NF, h->d_Rm, h->d_Xb, r_u, r_h, lam, h->d_facet_of, h->d_flip, u, hout)));
         return cudaGetLastError();
     }
